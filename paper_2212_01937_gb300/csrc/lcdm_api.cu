@@ -23,6 +23,10 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // largest batch whose root preparation uses four lanes per cosmology
 #define LCDM_PREP_GROUP_MAX_B 16384
 
+// Row records: those of the core (NCORE floats or doubles per row), or those
+// of the X-tangent kernel, in the same memory (a plan that needs both prepares
+// one after the other).
+static_assert(NCORE <= NREC + NREC, "the core's record fits the workspace of the X-tangent kernel's two");
 size_t ws_bytes_for(int64_t B) {
     return align256((size_t)B * NREC * sizeof(double)) + align256((size_t)B * NREC * sizeof(float2));
 }
@@ -49,6 +53,7 @@ size_t det_bytes() {
 struct Carved {
     double* recD;
     float2* recF;
+    char* core;                  // the core's records (the same memory)
     double* part = nullptr;      // deterministic mode: [warps][2][DET_NV]
     int64_t* wrow = nullptr;     // [warps][2]
 };
@@ -57,6 +62,7 @@ lcdm_status carve(void* ws, size_t ws_bytes, int64_t B, Carved& c, int det = 0) 
     if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < ws_bytes_for(B) + (det ? det_bytes() : 0))
         return LCDM_ERR_WORKSPACE;
     c.recD = (double*)ws;
+    c.core = (char*)ws;
     c.recF = (float2*)((char*)ws + align256((size_t)B * NREC * sizeof(double)));
     if (det) {
         c.part = (double*)((char*)ws + ws_bytes_for(B));
@@ -109,6 +115,9 @@ int log2_bucket(int64_t n) {
 
 struct Plan {
     PairArgs args;
+    const void* core;       // the core's records
+    int legacy;             // the tangent launch is the X-tangent kernel's
+    int absorb;             // the core's records need the absorption distance's constants
     int prec, K, wt, wx;
     int64_t npairs;
     TuneKey key;
@@ -136,6 +145,7 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     memset(&a, 0, sizeof(a));
     a.recD = cv.recD;
     a.recF = cv.recF;
+    P.core = cv.core;
     a.part = cv.part;
     a.wrow = cv.wrow;
     a.det_cap = cv.part ? (int64_t)det_warps() : 0;
@@ -180,11 +190,25 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     }
     P.wt = wt;
     P.wx = wx;
+    P.legacy = P.K > 0 && wx;
+    P.absorb = (P.split_mask >> LCDM_X) & 1 || (P.K == 0 && wx);
     P.key = TuneKey(current_device(), P.prec, P.K, wt, wx, opts->layout, log2_bucket(P.npairs));
     return LCDM_OK;
 }
 
 lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s);
+
+// index of the plan's kernel in its table (4 and up: per-pair Jacobians)
+int entry_index(const Plan& P) {
+    bool jac = false;
+    for (int i = 0; i < LCDM_NOUT; i++) jac = jac || P.args.jac[i];
+    return (P.wt ? 2 : 0) + (P.wx ? 1 : 0) + (jac ? 4 : 0);
+}
+const PairsEntry& plan_entry(const Plan& P) {
+    const int i = entry_index(P);
+    const PairsTable& t = table(P.prec, P.K);
+    return i < 4 ? t.e[i] : t.jac[i - 4];
+}
 
 }  // namespace
 
@@ -212,44 +236,44 @@ cudaError_t launch_det_fixup(const PairArgs& a, int64_t nwarps, cudaStream_t s) 
 
 namespace {
 
-// The plan's launches: the value-only outputs of split_mask first (K = 0,
-// their tracks only, no reductions), then the tangent launch without them.
-lcdm_status launch_plan(Plan& P, int block, int bps, int lane_map, cudaStream_t s) {
-    if (P.split_mask) {
-        Plan V = P;
-        PairArgs& v = V.args;
-        v.outmask = 0;
-        for (int i = 0; i < LCDM_NOUT; i++) {
-            v.jac[i] = nullptr;
-            v.cot[i] = nullptr;
-            if (!(P.split_mask & (1 << i))) v.out[i] = nullptr;
-            if (v.out[i]) v.outmask |= 1 << i;
-        }
-        v.mobs = nullptr;
-        v.grad = nullptr;
-        v.loglike = nullptr;
-        V.K = 0;
-        V.wt = (P.split_mask >> LCDM_T) & 1;
-        V.wx = (P.split_mask >> LCDM_X) & 1;
-        V.split_mask = 0;
-        std::get<2>(V.key) = 0;
-        std::get<3>(V.key) = V.wt;
-        std::get<4>(V.key) = V.wx;
-        lcdm_status st = launch_one(V, 0, 0, lane_map, s);
-        if (st != LCDM_OK) return st;
-        Plan T = P;
-        for (int i = 0; i < LCDM_NOUT; i++)
-            if (P.split_mask & (1 << i)) { T.args.out[i] = nullptr; T.args.outmask &= ~(1 << i); }
-        T.split_mask = 0;
-        return launch_one(T, block, bps, lane_map, s);
+// The value-only outputs of split_mask: a launch of their own (K = 0, their
+// tracks only, no reductions).
+lcdm_status launch_values(const Plan& P, int lane_map, cudaStream_t s) {
+    Plan V = P;
+    PairArgs& v = V.args;
+    v.outmask = 0;
+    for (int i = 0; i < LCDM_NOUT; i++) {
+        v.jac[i] = nullptr;
+        v.cot[i] = nullptr;
+        if (!(P.split_mask & (1 << i))) v.out[i] = nullptr;
+        if (v.out[i]) v.outmask |= 1 << i;
     }
-    return launch_one(P, block, bps, lane_map, s);
+    v.mobs = nullptr;
+    v.grad = nullptr;
+    v.loglike = nullptr;
+    V.K = 0;
+    V.legacy = 0;
+    V.wt = (P.split_mask >> LCDM_T) & 1;
+    V.wx = (P.split_mask >> LCDM_X) & 1;
+    V.split_mask = 0;
+    std::get<2>(V.key) = 0;
+    std::get<3>(V.key) = V.wt;
+    std::get<4>(V.key) = V.wx;
+    return launch_one(V, 0, 0, lane_map, s);
+}
+// The plan's main launch, without the outputs of split_mask.
+lcdm_status launch_main(const Plan& P, int block, int bps, int lane_map, cudaStream_t s) {
+    Plan T = P;
+    for (int i = 0; i < LCDM_NOUT; i++)
+        if (P.split_mask & (1 << i)) { T.args.out[i] = nullptr; T.args.outmask &= ~(1 << i); }
+    T.split_mask = 0;
+    return launch_one(T, block, bps, lane_map, s);
 }
 
 // Resident blocks per SM of a pair kernel, queried once per (device, kernel,
 // block size): the query is host work on every launch otherwise (the chunked
 // host entry point launches twice per chunk).
-int cached_occ(const PairsTable& t, int idx, int prec, int K, int block) {
+int cached_occ(const PairsEntry& t, int idx, int prec, int K, int block) {
     static std::mutex mu;
     static std::map<std::tuple<int, int, int, int, int>, int> cache;
     const auto key = std::make_tuple(current_device(), prec, K, idx, block);
@@ -258,16 +282,16 @@ int cached_occ(const PairsTable& t, int idx, int prec, int K, int block) {
         auto it = cache.find(key);
         if (it != cache.end()) return it->second;
     }
-    const int occ = t.occ[idx](block);
+    const int occ = t.occ(block);
     if (occ > 0) {
         std::lock_guard<std::mutex> lk(mu);
         cache[key] = occ;
     }
     return occ;
 }
+
 lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s) {
-    const PairsTable& t = table(P.prec, P.K);
-    int idx = (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
+    const PairsEntry& t = plan_entry(P);
     if (block == 0 || bps == 0 || lane_map == LCDM_MAP_TUNED) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(P.key);
@@ -279,7 +303,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     }
     P.args.interleave = lane_map == LCDM_MAP_INTERLEAVED ? 1 : 0;
     if (block == 0) block = 256;   // full-size blocks (the largest kernels step in lockstep, see pairs_kernel)
-    int occ = cached_occ(t, idx, P.prec, P.K, block);
+    int occ = cached_occ(t, entry_index(P), P.prec, P.K, block);
     if (occ <= 0) return LCDM_ERR_CUDA;
     if (bps == 0 || bps > occ) bps = occ;
     int64_t warps = (int64_t)num_sms() * bps * (block / 32);
@@ -291,7 +315,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     int64_t grid = (need_warps * 32 + block - 1) / block;
     if (grid < 1) grid = 1;
     if (P.npairs == 0) return LCDM_OK;
-    cudaError_t e = t.launch[idx](P.args, (int)grid, block, s);
+    cudaError_t e = t.launch(P.args, P.core, (int)grid, block, s);
     g_launches++;
     if (e != cudaSuccess) return LCDM_ERR_CUDA;
     if (P.args.part && (P.args.grad || P.args.loglike)) {
@@ -302,25 +326,66 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     return e == cudaSuccess ? LCDM_OK : LCDM_ERR_CUDA;
 }
 
-lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv, int32_t* status,
-                     double* grad, double* loglike, cudaStream_t s) {
+// What a call's records hold.
+struct PrepNeed {
+    bool legacy;     // the X-tangent kernel's records, else the core's
+    int prec;        // precision of the core's records
+    bool tangents, absorb;
+};
+
+lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv, const PrepNeed& need,
+                     int32_t* status, double* grad, double* loglike, cudaStream_t s) {
     // One warp per block, so that the FP64 work spreads over as many SMs as
     // possible.  Up to LCDM_PREP_GROUP_MAX_B cosmologies the solve is bound by
     // the latency of one cosmology's dependent FP64 chain and four lanes share
     // each root solve; beyond that the FP64 pipe is the bound and one lane per
     // cosmology does no repeated work.
+    PrepArgs a;
+    a.params = params;
+    a.B = B;
+    a.ncol = opts->ncol;
+    a.tangents = need.tangents;
+    a.absorb = need.absorb;
+    a.recD = need.legacy ? cv.recD : nullptr;
+    a.recF = need.legacy ? cv.recF : nullptr;
+    a.coreF = !need.legacy && need.prec == 1 ? (float*)cv.core : nullptr;
+    a.coreD = !need.legacy && need.prec == 0 ? (double*)cv.core : nullptr;
+    a.status = status;
+    a.grad = grad;
+    a.loglike = loglike;
     const int block = 32;
     if (B <= LCDM_PREP_GROUP_MAX_B) {
         const int64_t grid = (4 * B + block - 1) / block;
-        prep_kernel<4><<<(unsigned)grid, block, 0, s>>>(params, B, opts->ncol, cv.recD, cv.recF, status, grad,
-                                                       loglike);
+        prep_kernel<4><<<(unsigned)grid, block, 0, s>>>(a);
     } else {
         const int64_t grid = (B + block - 1) / block;
-        prep_kernel<1><<<(unsigned)grid, block, 0, s>>>(params, B, opts->ncol, cv.recD, cv.recF, status, grad,
-                                                       loglike);
+        prep_kernel<1><<<(unsigned)grid, block, 0, s>>>(a);
     }
     g_launches++;
     return cudaGetLastError() == cudaSuccess ? LCDM_OK : LCDM_ERR_CUDA;
+}
+
+// Preparation and launches of a plan.  A plan whose tangent launch is the
+// X-tangent kernel's and that also has value-only outputs prepares the core's
+// records for those first, then its own.
+lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv,
+                     int32_t* status, double* grad, double* loglike, int block, int bps, int lane_map, cudaStream_t s) {
+    lcdm_status st;
+    if (P.split_mask || !P.legacy) {
+        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.absorb != 0};
+        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
+        if (st != LCDM_OK) return st;
+    }
+    if (P.split_mask) {
+        st = launch_values(P, lane_map, s);
+        if (st != LCDM_OK) return st;
+    }
+    if (P.legacy) {
+        const PrepNeed need = {true, P.prec, true, true};
+        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
+        if (st != LCDM_OK) return st;
+    }
+    return launch_main(P, block, bps, lane_map, s);
 }
 
 __global__ void extract_roots(const double* __restrict__ recD, int64_t B, int ncol, double* roots, double* droots,
@@ -362,9 +427,8 @@ lcdm_status pairs_common(const double* params, int64_t B, const int64_t* offsets
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, jac, cot, mobs, M, sigma, grad, loglike, status, opts, cv, P);
     if (st != LCDM_OK) return st;
-    st = run_prep(params, B, opts, cv, status, grad, loglike, stream);
-    if (st != LCDM_OK) return st;
-    return launch_plan(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
+    return run_plan(P, params, B, opts, cv, status, grad, loglike, opts->block, opts->blocks_per_sm, opts->lane_map,
+                    stream);
 }
 
 // ----------------------------------------------------------------------------
@@ -444,6 +508,7 @@ HostCarve host_carve(char* base, int64_t B, int64_t n, int ncol, size_t es) {
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align256(bytes); return p; };
     char* rec = take(ws_bytes_for(B));
     c.rec.recD = (double*)rec;
+    c.rec.core = take((size_t)B * NCORE * es);
     c.rec.recF = rec ? (float2*)(rec + align256((size_t)B * NREC * sizeof(double))) : nullptr;
     c.params = (double*)take((size_t)B * ncol * sizeof(double));
     c.offsets = (int64_t*)take((size_t)(B + 1) * sizeof(int64_t));
@@ -479,6 +544,7 @@ BetweenCarve between_carve(char* base, int64_t B, int64_t npairs, int ncol, size
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align256(bytes); return p; };
     char* rec = take(ws_bytes_for(B));
     c.rec.recD = (double*)rec;
+    c.rec.core = rec;
     c.rec.recF = rec ? (float2*)(rec + align256((size_t)B * NREC * sizeof(double))) : nullptr;
     c.params4 = (double*)take((size_t)B * 4 * sizeof(double));
     c.jac = (double*)take((size_t)B * 4 * ncol * sizeof(double));
@@ -501,9 +567,9 @@ lcdm_status between_npairs(int64_t B, int64_t n, const lcdm_opts* opts, int64_t*
     return LCDM_OK;
 }
 
-// Shift every row to its lower limit and prepare the shifted records.
+// Shift every row to its lower limit.
 lcdm_status between_setup(const double* params, int64_t B, const double* z1, int ncol, const BetweenCarve& w,
-                          const lcdm_opts* opts4, int32_t* status, double* gradp, cudaStream_t stream) {
+                          cudaStream_t stream) {
     ShiftArgs sa;
     sa.params = params;
     sa.z1 = z1;
@@ -515,7 +581,7 @@ lcdm_status between_setup(const double* params, int64_t B, const double* z1, int
     sa.rowf = w.rowf;
     if (launch_shift(sa, stream) != cudaSuccess) return LCDM_ERR_CUDA;
     g_launches++;
-    return run_prep(w.params4, B, opts4, w.rec, status, gradp, nullptr, stream);
+    return LCDM_OK;
 }
 
 }  // namespace
@@ -548,7 +614,7 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
     if (ws_bytes < w.bytes) return LCDM_ERR_WORKSPACE;
     lcdm_opts o4 = *opts;
     o4.ncol = 4;
-    st = between_setup(params, B, z1, ncol, w, &o4, cosmo_status, grad ? w.gradp : nullptr, stream);
+    st = between_setup(params, B, z1, ncol, w, stream);
     if (st != LCDM_OK) return st;
     PairMapArgs m;
     memset(&m, 0, sizeof(m));
@@ -574,7 +640,8 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
     Plan P;
     make_plan(w.params4, B, offsets, w.zp, n, out, nullptr, grad ? cotk : nullptr, nullptr, 0, 1,
               grad ? w.gradp : nullptr, nullptr, cosmo_status, &o4, w.rec, P);
-    st = launch_plan(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
+    st = run_plan(P, w.params4, B, &o4, w.rec, cosmo_status, grad ? w.gradp : nullptr, nullptr, opts->block,
+                  opts->blocks_per_sm, opts->lane_map, stream);
     if (st != LCDM_OK) return st;
     if (out) {
         for (int i = 0; i < LCDM_NOUT; i++) m.out[i] = out[i];
@@ -620,9 +687,8 @@ lcdm_status lcdm_gauss_loglike_dz(const double* params, int64_t B, const int64_t
     st = make_plan(params, B, offsets, z, n, out, nullptr, nullptr, m_obs, M, sigma, grad, loglike, cosmo_status,
                    opts, cv, P);
     if (st != LCDM_OK) return st;
-    st = run_prep(params, B, opts, cv, cosmo_status, grad, loglike, stream);
-    if (st != LCDM_OK) return st;
-    st = launch_plan(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
+    st = run_plan(P, params, B, opts, cv, cosmo_status, grad, loglike, opts->block, opts->blocks_per_sm, opts->lane_map,
+                  stream);
     if (st != LCDM_OK) return st;
     DzArgs d;
     d.params = params;
@@ -670,9 +736,8 @@ lcdm_status lcdm_distances_vjp_dz(const double* params, int64_t B, const int64_t
     st = make_plan(params, B, offsets, z, n, outk, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad, nullptr,
                    cosmo_status, opts, cv, P);
     if (st != LCDM_OK) return st;
-    st = run_prep(params, B, opts, cv, cosmo_status, grad, nullptr, stream);
-    if (st != LCDM_OK) return st;
-    st = launch_plan(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
+    st = run_plan(P, params, B, opts, cv, cosmo_status, grad, nullptr, opts->block, opts->blocks_per_sm, opts->lane_map,
+                  stream);
     if (st != LCDM_OK) return st;
     DzArgs d;
     memset(&d, 0, sizeof(d));
@@ -708,11 +773,13 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     if (ws_bytes < w.bytes) return LCDM_ERR_WORKSPACE;
     lcdm_opts o4 = *opts;
     o4.ncol = 4;
-    lcdm_status st = between_setup(params, B, z1, ncol, w, &o4, cosmo_status, nullptr, stream);
+    lcdm_status st = between_setup(params, B, z1, ncol, w, stream);
+    if (st != LCDM_OK) return st;
+    const PrepNeed need = {false, 0, grad != nullptr, false};
+    st = run_prep(w.params4, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     LimitArgs la;
-    la.recD = w.rec.recD;
-    la.recF = w.rec.recF;
+    la.rec = (const double*)w.rec.core;
     la.status = cosmo_status;
     la.B = B;
     la.scale = w.scale;
@@ -783,8 +850,24 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
     chk(cudaEventRecord(ev[1], hs->up));
     chk(cudaStreamWaitEvent(stream, ev[1], 0));
     if (!ok) return LCDM_ERR_CUDA;
-    st = run_prep(d.params, B, opts, d.rec, d.status, d.grad, nullptr, stream);
-    if (st != LCDM_OK) return st;
+    // one preparation of all rows for every chunk (both kinds of records when a
+    // plan of X's tangents also has value-only outputs)
+    {
+        Plan P;
+        void* const* outs = out;
+        make_plan(d.params, B, d.offsets, d.z, n, outs, nullptr, cot, nullptr, 0, 1, d.grad, nullptr, d.status, opts,
+                  d.rec, P);
+        if (P.legacy) {
+            const PrepNeed need = {true, P.prec, true, true};
+            st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
+            if (st != LCDM_OK) return st;
+        }
+        if (P.split_mask || !P.legacy) {
+            const PrepNeed need = {false, P.prec, !P.legacy, P.absorb != 0};
+            st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
+            if (st != LCDM_OK) return st;
+        }
+    }
     // chunk c covers rows [rb[c], rb[c+1]); its share of the pairs ramps up and
     // down, weights min(c + 1, nchunks - c, 3) (1 2 3 ... 3 2 1): the first
     // chunk's input copy and the last chunk's output copy are the parts of the
@@ -830,11 +913,16 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
         Carved rc;
         rc.recD = d.rec.recD + r0 * NREC;
         rc.recF = d.rec.recF + r0 * NREC;
+        rc.core = d.rec.core + (size_t)r0 * NCORE * es;
         Plan P;
         make_plan(d.params + r0 * ncol, r1 - r0, d.offsets + r0, d.z, o1 - o0, outd, nullptr, cotd, nullptr, 0, 1,
                   d.grad + r0 * ncol, nullptr, d.status + r0, opts, rc, P);
         P.args.base = o0;
-        st = launch_plan(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
+        if (P.split_mask) {
+            st = launch_values(P, opts->lane_map, stream);
+            if (st != LCDM_OK) return st;
+        }
+        st = launch_main(P, opts->block, opts->blocks_per_sm, opts->lane_map, stream);
         if (st != LCDM_OK) return st;
         chk(cudaEventRecord(ev[3 + 2 * c], stream));
         chk(cudaStreamWaitEvent(hs->down, ev[3 + 2 * c], 0));
@@ -862,7 +950,8 @@ lcdm_status lcdm_roots(const double* params, int64_t B, const lcdm_opts* opts, d
     Carved cv;
     lcdm_status st = carve(ws, ws_bytes, B, cv);
     if (st != LCDM_OK) return st;
-    st = run_prep(params, B, opts, cv, cosmo_status, nullptr, nullptr, stream);
+    const PrepNeed need = {true, 0, true, false};
+    st = run_prep(params, B, opts, cv, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     extract_roots<<<(unsigned)((B + 127) / 128), 128, 0, stream>>>(cv.recD, B, opts->ncol, roots, droots, kind);
     g_launches++;
@@ -919,8 +1008,7 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
     st = make_plan(params, B, offsets, z, n, out, nullptr, cot, nullptr, 0, 1, grad, nullptr, cosmo_status, opts, cv,
                    P);
     if (st != LCDM_OK) return st;
-    const PairsTable& t = table(P.prec, P.K);
-    int idx = (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
+    const PairsEntry& t = plan_entry(P);
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return LCDM_ERR_CUDA;
     const int blocks[] = {64, 128, 256};
@@ -929,14 +1017,23 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
     for (int map = LCDM_MAP_CONTIGUOUS; map <= LCDM_MAP_INTERLEAVED; map++) {
         if (opts->lane_map != LCDM_MAP_TUNED && map != opts->lane_map) continue;
         for (int block : blocks) {
-            int occ = t.occ[idx](block);
+            int occ = t.occ(block);
             for (int bps = 1; bps <= occ; bps = (bps * 2 > occ && bps < occ) ? occ : bps * 2) {
                 float tot = 0;
                 for (int rep = 0; rep < 3; rep++) {
-                    if (run_prep(params, B, opts, cv, cosmo_status, grad, nullptr, stream) != LCDM_OK)
+                    // (the preparation is not timed, but where it comes between the launches)
+                    const bool both = P.legacy && P.split_mask;
+                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.absorb != 0};
+                    if (!both && run_prep(params, B, opts, cv, need, cosmo_status, grad, nullptr, stream) != LCDM_OK)
                         return LCDM_ERR_CUDA;
                     cudaEventRecord(e0, stream);
-                    if (launch_plan(P, block, bps, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
+                    if (both) {
+                        if (run_plan(P, params, B, opts, cv, cosmo_status, grad, nullptr, block, bps, map, stream) != LCDM_OK)
+                            return LCDM_ERR_CUDA;
+                    } else {
+                        if (P.split_mask && launch_values(P, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
+                        if (launch_main(P, block, bps, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
+                    }
                     cudaEventRecord(e1, stream);
                     cudaEventSynchronize(e1);
                     float ms = 0;

@@ -4,6 +4,7 @@
 #include <math_constants.h>
 
 #include "lcdm_between.cuh"
+#include "lcdm_core.cuh"
 #include "lcdm_kernels.cuh"
 
 namespace lcdm {
@@ -213,66 +214,35 @@ cudaError_t launch_chain(const double* jac, const double* gradp, int64_t B, int 
 
 // ------------------------------------------------- upper limit at infinity -
 // One thread per row of the shifted cosmology: chi'(0, inf) and t'(0, inf)
-// in FP64, with the closure tangents w.r.t. (Om', OL', Or') when K = 3.
-template <int K> struct LimitEval {
-    typedef PairEval<double, K, true, false> E;
-    typedef typename E::S S;
-
-    static __device__ void run(const double* rd, const float2* rf, int kind, S& Ichi, S& It, int* fail) {
-        S A = E::val(rd, rf, RF_A, RF_DA);
-        S amh = E::val(rd, rf, RF_AMH, RF_DAMH);
-        S Pre = E::val(rd, rf, RF_PRE, RF_DPRE), Pim = E::val(rd, rf, RF_PIM, RF_DPIM);
-        S qA = E::val(rd, rf, RF_QA, RF_DQA), nrm = E::val(rd, rf, RF_NRM, RF_DNRM);
-        S qPre = E::val(rd, rf, RF_QPRE, RF_DQPRE), qPim = E::val(rd, rf, RF_QPIM, RF_DQPIM);
-        if (kind == 0 || kind == 2) {
-            CPair<S> P = mkcp(mkcx<S>(Pre, Pim)), qP = mkcp(mkcx<S>(qPre, qPim));
-            if (kind == 0)
-                quartic_limits<S, CPair<S> >(E::val(rd, rf, RF_MA, RF_DMA), E::val(rd, rf, RF_EPSA, RF_DEPSA),
-                                             E::val(rd, rf, RF_B, RF_DB), P, qA, E::val(rd, rf, RF_QB, RF_DQB),
-                                             qP, nrm, Ichi, It, fail);
-            else
-                cubic_limits<S, CPair<S> >(A, amh, qA, qP, nrm, Ichi, It, fail);
-        } else {
-            RPair<S> P = mkrp<S>(Pre, Pim), qP = mkrp<S>(qPre, qPim);
-            if (kind == 1)
-                quartic_limits<S, RPair<S> >(E::val(rd, rf, RF_MA, RF_DMA), E::val(rd, rf, RF_EPSA, RF_DEPSA),
-                                             E::val(rd, rf, RF_B, RF_DB), P, qA, E::val(rd, rf, RF_QB, RF_DQB),
-                                             qP, nrm, Ichi, It, fail);
-            else
-                cubic_limits<S, RPair<S> >(A, amh, qA, qP, nrm, Ichi, It, fail);
-        }
-    }
-};
-
-template <int K> __global__ void __launch_bounds__(128) limits_kernel(LimitArgs a) {
+// in FP64, with the closure gradient w.r.t. (Om', OL', Or') by one reverse
+// pass when GRAD.  Bound by the FP64 pipe.
+template <bool GRAD> __global__ void __launch_bounds__(128) limits_kernel(LimitArgs a) {
     const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= a.B) return;
-    const double* rd = a.recD + b * NREC;
-    const float2* rf = a.recF + b * NREC;
+    const double* rec = a.rec + b * NCORE;
     const double nan = CUDART_NAN;
     double chi = nan, age = nan;
     int st = a.status[b];
     if (st == ST_OK) {
-        typedef typename LimitEval<K>::S S;
-        S Ichi, It;
+        CorePair<double, true, false, GRAD, true> e;
         int fail = 0;
-        LimitEval<K>::run(rd, rf, (int)rd[RF_KIND], Ichi, It, &fail);
-        const double s = a.scale[b], DH = rd[RF_DH], tH = rd[RF_TH], H0 = rd[RF_H0];
+        e.forward(1.0, rec, &fail);
+        const double s = a.scale[b], DH = rec[C_DH], tH = rec[C_TH];
         if (fail) {
             a.status[b] = st = ST_NOCONV;
-        } else if constexpr (K > 0) {
-            chi = s * DH * Ichi.v;
-            age = tH * It.v;
-            const double gc = a.cot_chi ? a.cot_chi[b] : 0.0, ga = a.cot_age ? a.cot_age[b] : 0.0;
-            double* g = a.gradp + b * 4;
-            g[0] = -(gc * chi + ga * age) / H0;
-            for (int k = 0; k < K; k++) g[1 + k] = gc * s * DH * Ichi.d[k] + ga * tH * It.d[k];
         } else {
-            chi = s * DH * Ichi;
-            age = tH * It;
+            chi = s * DH * e.Ichi;
+            age = tH * e.It;
+            if (GRAD) {
+                const double gc = a.cot_chi ? a.cot_chi[b] : 0.0, ga = a.cot_age ? a.cot_age[b] : 0.0;
+                double* g = a.gradp + b * 4;
+                g[0] = -(gc * chi + ga * age) / rec[C_H0];
+                e.reverse(gc * s * DH, ga * tH);
+                for (int k = 0; k < 3; k++) g[1 + k] = e.along(k);
+            }
         }
     }
-    if (st != ST_OK && K > 0 && a.gradp)
+    if (st != ST_OK && GRAD && a.gradp)
         for (int k = 0; k < 4; k++) a.gradp[b * 4 + k] = nan;
     if (a.chi) a.chi[b] = chi;
     if (a.age) a.age[b] = age;
@@ -281,8 +251,8 @@ template <int K> __global__ void __launch_bounds__(128) limits_kernel(LimitArgs 
 cudaError_t launch_limits(const LimitArgs& a, bool tangents, cudaStream_t s) {
     if (a.B <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((a.B + 127) / 128);
-    if (tangents) limits_kernel<3><<<grid, 128, 0, s>>>(a);
-    else limits_kernel<0><<<grid, 128, 0, s>>>(a);
+    if (tangents) limits_kernel<true><<<grid, 128, 0, s>>>(a);
+    else limits_kernel<false><<<grid, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -56,8 +56,7 @@ struct PairMapArgs {
 };
 
 struct LimitArgs {
-    const double* recD;     // records of the shifted cosmologies
-    const float2* recF;
+    const double* rec;      // [B][NCORE] core records of the shifted cosmologies
     int32_t* status;
     int64_t B;
     const double* scale;

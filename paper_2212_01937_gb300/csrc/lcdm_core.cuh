@@ -1,0 +1,736 @@
+// Distance integrals of one (cosmology, redshift) pair and their reverse-mode
+// derivatives, in either precision.
+//
+// The reduction is that of eqs. (3.7)-(3.9) / (B.1)-(B.3); it is written in
+// coordinates in which everything that does not depend on z is a constant of
+// the row.  Divided by N^2 (N = sqrt(E^2(0)) times the normalisation of the
+// roots), Carlson's arguments are
+//   s1 = n_A n_B + n_P n_P*,  u = n_P n_A + n_P* n_B (and u*),  n_j = sqrt(1 + z q_j),
+//   x1 = s1^2, y = u^2, and p = u_A5^2 for the third-kind integral of eq. (3.8),
+// and all their differences are constants of the row times z^2:
+//   the deviations X_i of (x1, y, y*) from their mean satisfy
+//     X^3 + e2 z^4 X - e3 z^6 = 0,  e2 = -I / (3 S0^2),  e3 = -J / (27 S0^3)
+//   with I, J the invariants of the quartic E^2(x) and S0 = E^2(x = 1);
+//   p = s5 - d,  s5 = (n_B |n_P|^2 + (1+z) n_A)^2 / (1+z),  d = OL/S0 z^2 (1+eps)^2 n_A^2 / (1+z);
+//   mean - p = m z^2,  (p - x1)(p - y)(p - y*) = -k^2 (OL/S0) z^6,
+//   k = 3 k2,  eps = -1/rho_A.
+// (p is a ratio of sums of positive numbers but for the subtraction of d, and
+// it is positive wherever E^2 > 0 between the limits: R_C(s5, p) diverges like
+// p^-1/2 while t is finite.  So no principal values occur.)
+// With eps = q_A = 0 and the cubic's real root in the place of B the same
+// formulas are those of App. B.1 (the radiationless case), so there is one
+// path for all root kinds.
+//
+// Consequences for the duplication (Carlson's algorithm, the paper's ref. [10]):
+//  * the sequence is carried without the division by four (x <- x + lambda):
+//    differences are then constant and the truncated series are polynomials
+//    in w = z^2 / A with constants of the row as coefficients (4 + 2 terms,
+//    to the 7th degree in the deviations);
+//  * the stopping rule is one multiplication: z^2 max|deviation| <= tol A;
+//  * y y* = x1 S^2 after the first step, so a step takes two square roots
+//    (one more per third-kind track) and no division by a difference;
+//  * the R_C(1, 1+e) argument of a third-kind track is const z^6 / d^2.
+// Gradients are taken in reverse through the stored sequence (s1, S, P and
+// sqrt(p) of each step): its cost does not depend on the number of
+// parameters, and nothing is divided by a difference of arguments.
+#pragma once
+#include "lcdm_math.cuh"
+
+namespace lcdm {
+
+// Row record of the core (T = float or double).  Tangent slots k = 0..5:
+// Om, OL, Or, Ok, Os, Ox (the first ncol - 1 used).
+enum CoreField {
+    C_QA = 0, C_QB, C_QR, C_QRL,          // q_j = -1/r_j; the pair: real and imaginary part, or the two reals
+    C_QI, C_QIL, C_C2, C_KIND,            // (QRL, QIL: low words in single precision); c2 = 2 / sqrt(S0);
+                                          // KIND: 1 for a complex pair, 0 for two reals
+    C_DH, C_TH, C_H0, C_OK,
+    C_DF, C_B2, C_B3, C_B4,               // DF: max deviation / z^2 from the mean of three; series of R_F
+    C_B5, C_B6, C_B7, C_RS,               // RS = -1 / (2 S0) with free S0, 0 under the closure
+    C_DJ, C_EPS, C_K2, C_K3,              // DJ: max deviation from the mean of five (t track)
+    C_A2, C_A3, C_A4, C_A5,               // series of the t track's R_J
+    C_A6, C_A7, C_FREE0, C_FREE1,
+    // absorption distance (values)
+    X_HX = 32, X_LX, X_PX, X_DX,          // p0 - x1 = -hx z^2; p0 = (..)^2 - lx z^2 w_B; pi/z^4; max deviation
+    X_C0, X_T1, X_G1, X_G2,
+    X_G3, X_G4, X_G5, X_SY,
+    X_N0, X_N1, X_N2, X_FREE,
+    X_AB, X_LAM, X_SQ, X_PQ,              // q_P + q_P*, q_P q_P*
+    X_A2 = 52,                            // a_j at p0 (6), a_j at x1 (6), divided differences (6)
+    X_D2 = 58, X_E2 = 64,
+    C_TAN = 72, C_TSTRIDE = 20,           // tangents of slot k at C_TAN + 20 k:
+    CT_QA = 0, CT_QB, CT_QR, CT_QI, CT_B2, CT_EPS = 10, CT_K2, CT_K3, CT_A2, CT_END = 19,
+    NCORE = C_TAN + 6 * C_TSTRIDE
+};
+
+// ------------------------------------------------------------- arithmetic ---
+// 1/sqrt and 1/x.  Single precision: the hardware approximations (within two
+// ulp).  Double precision: CUDA's rsqrt; the reciprocal by one third-order
+// step from the hardware's 20-bit approximation (error 2^-60 before rounding;
+// positive normal arguments), three fused multiply-adds where the division
+// issues about nine FP64 instructions.
+LCDM_HD float rsq(float x) { return srsqrt(x); }
+LCDM_HD double rsq(double x) {
+#ifdef __CUDA_ARCH__
+    return rsqrt(x);
+#else
+    return 1.0 / sqrt(x);
+#endif
+}
+LCDM_HD float rcp_(float x) {
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / x;
+#endif
+}
+LCDM_HD double rcp_(double x) {
+#ifdef __CUDA_ARCH__
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+#else
+    return 1.0 / x;
+#endif
+}
+
+template <class T> struct CoreTol;
+template <> struct CoreTol<float> {
+    // deviation at which a degree-7 series is used; relative deviation s of
+    // R_C's; largest z taken without scaling
+    static constexpr float dup = 0.15f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
+    enum { maxit = 24 };
+};
+template <> struct CoreTol<double> {
+    static constexpr double dup = 0.009, rc = 0.008, big = 1e30, e_series = 0.03;
+    enum { maxit = 40 };
+};
+
+// R_C(1, 1 + e) and its derivative by closed relations, for e beyond the
+// series; b = sqrt(1 + e)
+template <class T> struct RcE { T v, d; };
+template <class T> LCDM_NI RcE<T> rc1_far(T e, T b) {
+    T a = cst<T>(1.0), tm = cst<T>(1.0);
+    const T b0 = b;
+    T U = a * a + cst<T>(2.0) * b * b;
+#pragma unroll 1
+    for (int m = 0; m < CoreTol<T>::maxit && !(fabs(e) <= CoreTol<T>::rc * U); m++) {
+        const T n = a + b, q = cst<T>(2.0) * b * n;
+        a = n;
+        b = q * rsq(q);
+        U = a * a + cst<T>(2.0) * b * b;
+        tm = tm + tm;
+    }
+    const T s = e * rcp_(U);
+    const T ser = cst<T>(1.0) + s * s * (cst<T>(0.3) + s * (cst<T>(1.0 / 7) + s * (cst<T>(0.375)
+                  + s * (cst<T>(9.0 / 22) + s * (cst<T>(159.0 / 208) + s * cst<T>(1.125))))));
+    RcE<T> r;
+    r.v = tm * ser * rsq(U * cst<T>(1.0 / 3));
+    // 2 e dR_C/de = 1/(1+e) - R_C (from Euler's relation and the derivative along x and y together)
+    r.d = (rcp_(b0 * b0) - r.v) * cst<T>(0.5) / e;
+    return r;
+}
+// R_C(1, 1+e) = sum (-e)^n / (2n+1), with its derivative (GRAD)
+LCDM_HD RcE<float> rc1_core(float e, bool grad) {
+    if (fabsf(e) <= CoreTol<float>::e_series) {
+        RcE<float> r;
+        const float w = -e;
+        float s = 1.0f / 13, ds = 0.f;
+#pragma unroll
+        for (int n = 5; n >= 0; n--) { ds = ds * w + s; s = 1.0f / (2 * n + 1) + w * s; }
+        r.v = s;
+        r.d = -ds;
+        return r;
+    }
+    return rc1_far<float>(e, (1.0f + e) * rsq(1.0f + e));
+}
+LCDM_HD RcE<double> rc1_core(double e, bool grad) {
+    // e falls by 64 or more per step: most steps need a few terms only
+    const double w = -e;
+    const double ae = fabs(e);
+    RcE<double> r;
+    if (ae <= 3e-5) {
+        r.v = 1.0 + w * (1.0 / 3 + w * (0.2 + w * (1.0 / 7)));
+        r.d = grad ? -(1.0 / 3 + w * (0.4 + w * (3.0 / 7 + w * (4.0 / 9)))) : 0.0;
+        return r;
+    }
+    if (ae <= CoreTol<double>::e_series) {
+        double s = 1.0 / 25, ds = 0.0;
+#pragma unroll
+        for (int n = 11; n >= 0; n--) {
+            if (grad) ds = ds * w + s;
+            s = 1.0 / (2 * n + 1) + w * s;
+        }
+        r.v = s;
+        r.d = -ds;
+        return r;
+    }
+    return rc1_far<double>(e, (1.0 + e) * rsq(1.0 + e));
+}
+// (R_C(1, 1+e) - 1) / e
+template <class T> LCDM_HD T rc1m1_core(T e) {
+    constexpr int NT = sizeof(T) == 4 ? 6 : 12;
+    if (fabs(e) <= CoreTol<T>::e_series) {
+        const T w = -e;
+        T s = cst<T>(-1.0 / (2 * NT + 3));
+#pragma unroll
+        for (int n = NT; n >= 1; n--) s = cst<T>(-1.0 / (2 * n + 1)) + w * s;
+        return s;
+    }
+    return (rc1_far<T>(e, (cst<T>(1.0) + e) * rsq(cst<T>(1.0) + e)).v - cst<T>(1.0)) / e;
+}
+// [R_C(1, 1-w) - (1-w)^-1/2] / w  (see phi_rc) for 0 <= w < 1, so = sqrt(1-w)
+// (which cancels if formed from w near 1).  Beyond the series' range R_C's
+// duplication is carried on the difference itself: with a = sqrt(x), b =
+// sqrt(y), x - y = w, and b' = sqrt(2 b (a + b)) of the next step,
+//   F = R_C - 1/b = 2 F' - 2 w / ((a + b) b' (2 b + b')),
+// a sum of numbers of one sign.
+template <class T> LCDM_HD T phi_core(T w, T so) {
+    constexpr int NT = sizeof(T) == 4 ? 9 : 17;
+    T a = cst<T>(1.0), b = so, sum = cst<T>(0.0), t = cst<T>(1.0), ia = cst<T>(1.0), v = w;
+#pragma unroll 1
+    for (int m = 0; m < CoreTol<T>::maxit && v > cst<T>(0.1); m++) {
+        const T n = a + b, q = cst<T>(2.0) * b * n, c = q * rsq(q);
+        sum = sum - cst<T>(2.0) * t * rcp_(n * c * (cst<T>(2.0) * b + c));
+        a = n;
+        b = c;
+        t = t + t;
+        ia = rcp_(a);
+        v = w * (ia * ia);
+    }
+    constexpr double cs[17] = LCDM_PHI_CS;
+    T acc = cst<T>(cs[NT - 1]);
+#pragma unroll
+    for (int n = NT - 1; n >= 1; n--) acc = acc * v + cst<T>(cs[n - 1]);
+    return sum + t * acc * (ia * ia * ia);
+}
+
+// 1 + z q: rounded once in double precision; in single precision in
+// double-float arithmetic from q's two words (it cancels for the pair near
+// z = Re r_P close to the no-Big-Bang boundary)
+LCDM_HD double one_plus(double q, double, double z) { return fma(q, z, 1.0); }
+LCDM_HD float one_plus(float q, float ql, float z) {
+    const float p = q * z, e1 = fmaf(q, z, -p);
+    const df64 s = two_sum(1.0f, p);
+    return s.hi + (s.lo + fmaf(ql, z, e1));
+}
+// power of two near 1/z for very large z
+LCDM_HD float scale_of(float z) { return z < 1e38f ? pow2i<float>(-even_exponent(z)) : 0.0f; }
+LCDM_HD double scale_of(double z) {
+    int e;
+    frexp(z, &e);
+    return z < 1e300 ? pow2i<double>(-e) : 0.0;
+}
+
+// Four consecutive record entries from a multiple of four (records are 16-byte
+// aligned): one 128-bit load in single precision, two in double.
+template <class T> struct Quad { T v[4]; };
+LCDM_HD Quad<float> quad(const float* p) {
+    Quad<float> q;
+#ifdef __CUDA_ARCH__
+    const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+    q.v[0] = f.x; q.v[1] = f.y; q.v[2] = f.z; q.v[3] = f.w;
+#else
+    for (int i = 0; i < 4; i++) q.v[i] = p[i];
+#endif
+    return q;
+}
+LCDM_HD Quad<double> quad(const double* p) {
+    Quad<double> q;
+#ifdef __CUDA_ARCH__
+    const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    q.v[0] = a.x; q.v[1] = a.y; q.v[2] = b.x; q.v[3] = b.y;
+#else
+    for (int i = 0; i < 4; i++) q.v[i] = p[i];
+#endif
+    return q;
+}
+
+// ------------------------------------------------------------------- core ---
+// One pair.  WT: the time coordinate; WX: the absorption distance (values
+// only); REV: keep what the reverse pass needs; INF: the upper limit at
+// infinity.  There n_j / sqrt(z) -> sqrt(q_j), every u grows like z, and with
+// the homogeneity of R_F, R_C and R_J the powers of z cancel: z stands for 1
+// and 1 + z q_j for q_j, and eq. (3.8)'s R_C has the factor (1 + eps) n_A (in
+// the radiationless case n_A = 0: that term falls off like z^-1/2).
+template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair {
+    enum { ND = REV ? (int)CoreTol<T>::maxit : 1, NR = REV && WT ? (int)CoreTol<T>::maxit : 1 };
+    const T* rc;
+    T z, zh, z2, h, cz;
+    bool cplx, big;
+    // square roots of the linear factors and their reciprocals
+    T rA, nA, rB, nB, Pn, iP, wr, wi, nr, ni;   // real pair: nr, ni = n_1, n_2; wr, wi = their reciprocals
+    T s1, uR, uI;                               // real pair: u_1, u_2
+    int m;                                      // duplication steps taken
+    T tm;                                       // 2^m
+    T T3, RF, RJ, rF, wF, sF, rJ, wJ, sJs;      // 3 A, results, 1/sqrt(A), w, series
+    T p, izh, d5, a5, RCp, g, kB, ig;           // t
+    int mr;
+    T U, sc, rcr, tr;
+    T X;
+    T st1[ND], stS[ND], stP[ND], stq[ND];       // the sequence (local memory; only the steps taken are touched)
+    T ra[NR], rb[NR];
+    T Ichi, It;
+    // adjoints of the row's constants
+    T qA_, qB_, qR_, qI_, bF_, eps_, k2_, k3_, bJ_;
+
+    LCDM_HD void forward(T zin, const T* rec, int* fail) {
+        rc = rec;
+        z = zin;
+        const T one = cst<T>(1.0);
+        const Quad<T> k0 = quad(rc + C_QA), k1 = quad(rc + C_QI), kF = quad(rc + C_DF);
+        cplx = k1.v[3] != cst<T>(0.0);
+        const T wA = INF ? k0.v[0] : one + k0.v[0] * z, wB = INF ? k0.v[1] : one + k0.v[1] * z;
+        rA = INF && !(wA > cst<T>(0.0)) ? cst<T>(0.0) : rsq(wA);
+        nA = wA * rA;
+        rB = rsq(wB);
+        nB = wB * rB;
+        const T qR = k0.v[2], qI = k1.v[0], c2 = k1.v[2];
+        Quad<T> kT;
+        if (WT) kT = quad(rc + C_DJ);
+        T S, P, T30;
+        if (cplx) {
+            wr = INF ? qR : one_plus(qR, k0.v[3], z);
+            wi = qI * z;
+            const T r2 = wr * wr + wi * wi;
+            iP = rsq(r2);
+            Pn = r2 * iP;
+            // n_P: the larger part by a square root, the other by division
+            const T hh = (Pn + fabs(wr)) * cst<T>(0.5), rh = rsq(hh);
+            const T t = hh * rh, o = wi * cst<T>(0.5) * rh;
+            const bool pos = wr >= cst<T>(0.0);
+            nr = pos ? t : o;
+            ni = pos ? o : t;
+            uR = nr * (nA + nB);
+            uI = ni * (nA - nB);
+        } else {
+            const T w1 = INF ? qR : one_plus(qR, k0.v[3], z), w2 = INF ? qI : one_plus(qI, k1.v[1], z);
+            wr = rsq(w1);
+            wi = rsq(w2);
+            nr = w1 * wr;
+            ni = w2 * wi;
+            Pn = nr * ni;
+            uR = nr * nA + ni * nB;
+            uI = ni * nA + nr * nB;
+        }
+        s1 = nA * nB + Pn;
+        zh = z;
+        z2 = z * z;
+        const T z1 = INF ? one : one + z;
+        if (WT) {
+            izh = INF ? one : rsq(z1);
+            a5 = (nB * Pn + z1 * nA) * izh;
+        }
+        T aX = cst<T>(0.0), lX = cst<T>(0.0);
+        Quad<T> kX;
+        if (WX) {
+            kX = quad(rc + X_HX);
+            aX = nA * Pn + nB;
+            lX = kX.v[1] * wB;
+        }
+        // powers of z^6 and d^2 would leave the range for very large z:
+        // everything is homogeneous and is scaled by a power of two
+        big = z > CoreTol<T>::big;
+        h = one;
+        if (big) {
+            h = scale_of(z);
+            s1 = s1 * h; uR = uR * h; uI = uI * h;
+            if (WT) a5 = a5 * h;
+            if (WX) aX = aX * h;
+            zh = z * h;
+            z2 = zh * zh;
+            zh = z * h;
+        }
+        if (cplx) {
+            S = uR + uR;
+            P = uR * uR + uI * uI;
+            T30 = cst<T>(2.0) * (uR * uR - uI * uI);
+        } else {
+            S = uR + uI;
+            P = uR * uI;
+            T30 = uR * uR + uI * uI;
+        }
+        T x = s1 * s1;
+        T3 = x + T30;
+        T sJ = cst<T>(0.0), delta = cst<T>(0.0), opE = cst<T>(0.0);
+        p = cst<T>(0.0);
+        if (WT) {
+            opE = one + kT.v[1];
+            d5 = kT.v[3] * z2 * (opE * opE) * (wA * (izh * izh));
+            p = a5 * a5 - d5;
+            delta = cst<T>(-9.0) * kT.v[2] * kT.v[2] * kT.v[3] * (z2 * z2 * z2);
+        }
+        T p0 = cst<T>(0.0), dX = cst<T>(0.0), piX = cst<T>(0.0), sD = cst<T>(0.0), sDD = cst<T>(0.0), x0 = x, rp0 = cst<T>(0.0);
+        if (WX) {
+            p0 = aX * aX - lX * z2;
+            piX = kX.v[2] * (z2 * z2);
+            dX = -(kX.v[0] * z2) * piX;
+        }
+        T pX = p0;
+        const T dF = kF.v[0] * z2 * cst<T>(3.0), dJ = WT ? kT.v[0] * z2 * cst<T>(5.0) : cst<T>(0.0);
+        const T dD = WX ? kX.v[3] * z2 * cst<T>(5.0) : cst<T>(0.0);
+        T S1 = s1;
+        tm = one;
+        T q0 = cst<T>(0.0);
+        m = 0;
+#pragma unroll 1
+        for (; m < CoreTol<T>::maxit; m++) {
+            bool conv = dF <= CoreTol<T>::dup * T3;
+            if (WT) conv = conv && dJ <= CoreTol<T>::dup * (T3 + p + p);
+            if (WX) conv = conv && dD <= CoreTol<T>::dup * (T3 + pX + pX) && dD <= CoreTol<T>::dup * (T3 + x + x);
+            if (conv) break;
+            const T lam = S1 * S + P;
+            const T xl = x + lam;
+            if (WT) {
+                const T sq = p * rsq(p);
+                if (m == 0) q0 = sq;
+                const T gg = p + (sq * S + P);
+                const T id = rcp_((sq + S1) * gg);
+                const T e = (delta * id) * id;
+                sJ = sJ + tm * rc1_core(e, false).v * id;
+                if (REV) stq[m] = sq;
+                p = p + lam;
+            }
+            if (WX) {
+                // R_D: 1 / (s1 (x + lambda)); divided difference of the p0 track against it
+                const T ix = rcp_(S1 * xl);
+                sD = sD + tm * ix;
+                const T sq = pX * rsq(pX);
+                if (m == 0) rp0 = sq;
+                const T gg = pX + (sq * S + P), qs = sq + S1;
+                const T id = rcp_(qs * gg);
+                const T e = (dX * id) * id, eh = (piX * id) * id;
+                sDD = sDD + tm * (eh * rc1m1_core(e) * id
+                                  - (gg + cst<T>(2.0) * S1 * (qs + S)) * (id * id) * gg * ix * cst<T>(0.5));
+                pX = pX + lam;
+            }
+            if (REV) { st1[m] = S1; stS[m] = S; stP[m] = P; }
+            x = xl;
+            T3 = T3 + cst<T>(3.0) * lam;
+            const T n1 = x * rsq(x);
+            const T Q = S * (S + cst<T>(2.0) * (S1 + n1));
+            P = n1 * S;
+            S = Q * rsq(Q);
+            S1 = n1;
+            tm = tm + tm;
+        }
+        if (m == CoreTol<T>::maxit) *fail = 1;
+        // closing series in w = z^2 / A
+        {
+            const T A = T3 * cst<T>(1.0 / 3);
+            rF = rsq(A);
+            wF = z2 * (rF * rF);
+            const Quad<T> kB5 = quad(rc + C_B5);
+            T s = kB5.v[2];
+            s = s * wF + kB5.v[1];
+            s = s * wF + kB5.v[0];
+            s = s * wF + kF.v[3];
+            s = s * wF + kF.v[2];
+            s = s * wF + kF.v[1];
+            sF = one + s * (wF * wF);
+            RF = tm * sF * rF;
+        }
+        cz = c2 * zh;
+        Ichi = cz * RF;
+        if (WT) {
+            const T A = (T3 + p + p) * cst<T>(0.2);
+            rJ = rsq(A);
+            wJ = z2 * (rJ * rJ);
+            const Quad<T> kA = quad(rc + C_A2), kA6 = quad(rc + C_A6);
+            T s = kA6.v[1];
+            s = s * wJ + kA6.v[0];
+            s = s * wJ + kA.v[3];
+            s = s * wJ + kA.v[2];
+            s = s * wJ + kA.v[1];
+            s = s * wJ + kA.v[0];
+            sJs = one + s * (wJ * wJ);
+            RJ = tm * sJs * (rJ * rJ * rJ) + cst<T>(6.0) * sJ;
+            // R_C(s5, p), Carlson's duplication on the square roots a = sqrt(s5), b = sqrt(p)
+            T a = a5, b = m > 0 ? q0 : p * rsq(p);
+            U = a * a + cst<T>(2.0) * (b * b);
+            tr = one;
+            mr = 0;
+            const T ad = fabs(d5);
+#pragma unroll 1
+            for (; mr < CoreTol<T>::maxit; mr++) {
+                if (REV) { ra[mr < NR ? mr : 0] = a; rb[mr < NR ? mr : 0] = b; }
+                if (ad <= CoreTol<T>::rc * U) break;
+                const T n = a + b, q = cst<T>(2.0) * b * n;
+                a = n;
+                b = q * rsq(q);
+                U = a * a + cst<T>(2.0) * (b * b);
+                tr = tr + tr;
+            }
+            if (mr == CoreTol<T>::maxit) *fail = 1;
+            const T iA = cst<T>(3.0) * rcp_(U);
+            sc = -d5 * iA * cst<T>(1.0 / 3);
+            T ser = cst<T>(159.0 / 208) + sc * cst<T>(1.125);
+            ser = cst<T>(9.0 / 22) + sc * ser;
+            ser = cst<T>(0.375) + sc * ser;
+            ser = cst<T>(1.0 / 7) + sc * ser;
+            ser = cst<T>(0.3) + sc * ser;
+            ser = one + sc * sc * ser;
+            rcr = rsq(U * cst<T>(1.0 / 3));
+            RCp = tr * ser * rcr * izh;
+            const T eps = kT.v[1];
+            g = fabs(opE) * nA;
+            if (INF) {
+                It = cz * (RCp * g - eps * RF - kT.v[2] * z2 * RJ);
+            } else {
+                ig = rcp_(g + one);
+                kB = (one + (one + eps) * z1) * ig;
+                It = cz * (RCp + eps * (RCp * kB - RF) - kT.v[2] * z2 * RJ);
+            }
+        }
+        if (WX) {
+            const T iA2 = cst<T>(5.0) * rcp_(T3 + x + x);
+            const T A2 = (T3 + x + x) * cst<T>(0.2), A1 = (T3 + pX + pX) * cst<T>(0.2);
+            const T r1 = rsq(A1), r2 = rsq(A2);
+            const T i1 = r1 * r1, w1 = z2 * i1, w2 = z2 * iA2, ww = cst<T>(-0.4) * w1 * w2;
+            T q[20];   // a_j at p0, at x1, divided differences
+#pragma unroll
+            for (int j = 0; j < 5; j++) {
+                const Quad<T> f = quad(rc + X_A2 + 4 * j);
+#pragma unroll
+                for (int i = 0; i < 4; i++) q[4 * j + i] = f.v[i];
+            }
+            T v1 = q[5], v2 = q[11], e = -q[17];
+#pragma unroll
+            for (int j = 4; j >= 0; j--) {
+                e = e * w1 + v2 * ww - q[12 + j];
+                v1 = v1 * w1 + q[j];
+                v2 = v2 * w2 + q[6 + j];
+            }
+            const T ser1 = one + v1 * (w1 * w1);
+            const T dser = cst<T>(-0.4) * (w1 + w2) * z2 * i1 * iA2 * v1 + w2 * iA2 * e;
+            const T q1 = A1 * r1, q2 = A2 * r2;
+            const T r13 = r1 * i1, r23 = r2 * iA2;
+            const T dA = cst<T>(-0.4) * (A1 + q1 * q2 + A2) * rcp_(q1 + q2) * r13 * r23;
+            const T DJ = tm * (dA * ser1 + r23 * dser) + cst<T>(6.0) * sDD;
+            const T RD = tm * (one + v2 * (w2 * w2)) * r23 + cst<T>(3.0) * sD;
+            if (m == 0) rp0 = p0 * rsq(p0);
+            // the results belong to arguments scaled by h^2 (h = 1 but for very large z)
+            const T ih = big ? one / h : one;
+            const T s1u = s1 * ih, sp0 = rp0 * ih, zz = z * z, x1 = x0 * (ih * ih);
+            const T hRF = RF * h, hRD = RD * (h * h * h), hDJ = DJ * (h * h * h) * (h * h);
+            const Quad<T> c0 = quad(rc + X_C0), c3 = quad(rc + X_G3), cN = quad(rc + X_N0), cB = quad(rc + X_AB);
+            const T irA = rA, syd = c3.v[3] * (nA * Pn * rB + one), isy = rcp_(syd);
+            const T T0 = c0.v[0] * irA * (k0.v[1] * Pn * rcp_(nB + one) + (cB.v[2] + z * cB.v[3]) * rcp_(Pn + one)
+                                           - k0.v[0] * rcp_(nA + one));
+            const T t1 = zz * (c0.v[2] * hRD + c0.v[3] * zz * hDJ);
+            const T iyd = isy * isy;
+            // y / yd = S0 p0 / (yB^2 n_B^2 yd), the part of yd beside lam z^2
+            const T t2 = c3.v[0] * zz * phi_core(cB.v[1] * zz * iyd, sp0 * c3.v[3] * rB * isy) * iyd * isy;
+            const T as = nA * s1u;
+            const T num = x1 * (cN.v[1] * z + cN.v[0]) + cN.v[2] * zz;
+            const T t3 = c3.v[1] * nB * num * rcp_(sp0 * as * (as + cB.v[0] * sp0));
+            const T t4 = c3.v[2] * nB * irA * rcp_(s1u);
+            X = z * (T0 + c0.v[1] * hRF + t1 + t2 + t3 + t4);
+        }
+    }
+
+    // Adjoints of the row's constants for the cotangents ci, ti of Ichi, It.
+    LCDM_HD void reverse(T ci, T ti) {
+        const T one = cst<T>(1.0), two = cst<T>(2.0), half = cst<T>(0.5);
+        T RF_ = ci * cz, T_ = cst<T>(0.0), p_ = cst<T>(0.0), cJ = cst<T>(0.0), del_ = cst<T>(0.0), a_ = cst<T>(0.0),
+          b_ = cst<T>(0.0), d_ = cst<T>(0.0), nA_ = cst<T>(0.0), wA_ = cst<T>(0.0);
+        Quad<T> kT;
+        if (WT) kT = quad(rc + C_DJ);
+        const T eps = WT ? kT.v[1] : cst<T>(0.0), z1 = INF ? one : one + z;
+        eps_ = k2_ = k3_ = bJ_ = cst<T>(0.0);
+        if (WT) {
+            const T b = ti * cz;
+            const T RCp_ = INF ? b * g : b * (one + eps * kB);
+            RF_ = RF_ - b * eps;
+            const T bk = b * z2;
+            const T RJ_ = -bk * kT.v[2];
+            k2_ = -bk * RJ;
+            const T opE = one + eps, ao = fabs(opE), sA = opE < cst<T>(0.0) ? -nA : nA;
+            if (INF) {
+                eps_ = b * (RCp * sA - RF);
+                nA_ = b * RCp * ao;
+            } else {
+                // kB = (2 + z + eps (1+z)) / (|1+eps| n_A + 1)
+                const T er = b * eps * RCp * ig;
+                eps_ = b * (RCp * kB - RF) + er * (z1 - kB * sA);
+                nA_ = -er * kB * ao;
+            }
+            // R_C: series, then the steps in reverse
+            const T rcb = RCp_ * izh * tr * rcr;          // cotangent of the series
+            const T iU = cst<T>(1.0 / 3) * (rcr * rcr);   // 1 / U
+            T ser = cst<T>(1.125), ds = cst<T>(0.0);
+            ds = ser; ser = cst<T>(159.0 / 208) + sc * ser;
+            ds = ds * sc + ser; ser = cst<T>(9.0 / 22) + sc * ser;
+            ds = ds * sc + ser; ser = cst<T>(0.375) + sc * ser;
+            ds = ds * sc + ser; ser = cst<T>(1.0 / 7) + sc * ser;
+            ds = ds * sc + ser; ser = cst<T>(0.3) + sc * ser;
+            // f = 1 + s^2 q(s): f' = s (2 q + s q')
+            const T sd = sc * (two * ser + sc * ds), sv = one + sc * sc * ser;
+            d_ = -rcb * sd * iU;
+            const T U_ = -rcb * iU * (sc * sd + half * sv);
+            T ax = ra[mr < NR ? mr : 0], bx = rb[mr < NR ? mr : 0];
+            a_ = two * ax * U_;
+            b_ = cst<T>(4.0) * bx * U_;
+#pragma unroll 1
+            for (int i = mr - 1; i >= 0; i--) {
+                const T a0 = ra[i], b0 = rb[i];
+                const T Q_ = b_ * half * rcp_(bx);
+                const T n_ = a_ + two * b0 * Q_;
+                b_ = two * (a0 + b0) * Q_ + n_;
+                a_ = n_;
+                bx = b0;
+            }
+            p_ = b_ * half * rcp_(bx);                    // b = sqrt(p)
+            // R_J: closing series
+            const Quad<T> kA = quad(rc + C_A2), kA6 = quad(rc + C_A6);
+            T s = kA6.v[1], s2 = s;
+            s = s * wJ + kA6.v[0];
+            s2 = s2 * wJ + s; s = s * wJ + kA.v[3];
+            s2 = s2 * wJ + s; s = s * wJ + kA.v[2];
+            s2 = s2 * wJ + s; s = s * wJ + kA.v[1];
+            s2 = s2 * wJ + s; s = s * wJ + kA.v[0];
+            const T r2 = rJ * rJ, c = RJ_ * tm * r2 * rJ;
+            bJ_ = c;
+            const T A_ = -c * r2 * (wJ * wJ * (two * s + wJ * s2) + cst<T>(1.5) * sJs);
+            T_ = A_ * cst<T>(0.2);
+            // the sequence's final p: its cotangent joins the chain (p differs
+            // from the initial p by the sum of the lambdas)
+            cJ = cst<T>(6.0) * RJ_;
+            pf_ = A_ * cst<T>(0.4);
+        }
+        {
+            const Quad<T> kF = quad(rc + C_DF), kB5 = quad(rc + C_B5);
+            T s = kB5.v[2], s2 = s;
+            s = s * wF + kB5.v[1];
+            s2 = s2 * wF + s; s = s * wF + kB5.v[0];
+            s2 = s2 * wF + s; s = s * wF + kF.v[3];
+            s2 = s2 * wF + s; s = s * wF + kF.v[2];
+            s2 = s2 * wF + s; s = s * wF + kF.v[1];
+            const T c = RF_ * tm * rF;
+            bF_ = c;
+            T_ = T_ - c * (rF * rF) * cst<T>(1.0 / 3) * (wF * wF * (two * s + wF * s2) + half * sF);
+        }
+        // the duplication in reverse: cotangents of (s1, S, P), x and p
+        T s_ = cst<T>(0.0), S_ = cst<T>(0.0), P_ = cst<T>(0.0), x_ = cst<T>(0.0);
+        T ps_ = WT ? pf_ : cst<T>(0.0);
+        T delta = cst<T>(0.0), tk = tm;
+        if (WT) delta = cst<T>(-9.0) * kT.v[2] * kT.v[2] * kT.v[3] * (z2 * z2 * z2);
+        T n1, n1s;   // the next step's sqrt(x) and S
+#pragma unroll 1
+        for (int i = m - 1; i >= 0; i--) {
+            const T a = st1[i], Sm = stS[i], Pm = stP[i];
+            tk = tk * half;
+            T Sn_ = cst<T>(0.0), an_ = cst<T>(0.0);
+            if (i < m - 1) {
+                // next: n1 = sqrt(x'), P' = n1 S, S' = sqrt(S (S + 2 (a + n1)))
+                n1 = st1[i + 1];
+                n1s = stS[i + 1];
+                const T Q_ = S_ * half * rcp_(n1s);
+                const T t = two * Sm * Q_;
+                const T n_ = s_ + P_ * Sm + t;
+                Sn_ = P_ * n1 + Q_ * two * (Sm + a + n1);
+                an_ = t;
+                x_ = x_ + n_ * half * rcp_(n1);
+            }
+            const T lam_ = x_ + ps_ + cst<T>(3.0) * T_;
+            s_ = an_ + lam_ * Sm;
+            S_ = Sn_ + lam_ * a;
+            P_ = lam_;
+            if (WT) {
+                const T sq = stq[i], gg = sq * (sq + Sm) + Pm, qs = sq + a;
+                const T id = rcp_(qs * gg), e = (delta * id) * id;
+                const RcE<T> r = rc1_core(e, true);
+                const T c = cJ * tk * id;                 // cotangent of rc
+                del_ = del_ + c * r.d * id * id;
+                // 1/d: rc d(1/d) + rc' 2 delta id d(1/d), d(1/d) = -id^2 dd
+                const T dd = -c * id * (r.v + two * e * r.d);
+                const T g_ = dd * qs, q_ = dd * gg + g_ * Sm;
+                s_ = s_ + dd * gg;
+                S_ = S_ + g_ * sq;
+                P_ = P_ + g_;
+                ps_ = ps_ + g_ + q_ * half * rcp_(sq);
+            }
+        }
+        // initial values: x = s1^2, 3 A = x + y + y*, p = a5^2 - d5, delta = -9 k2^2 k3 z^6
+        s_ = s_ + two * s1 * (x_ + T_);
+        T nB_, Pn_ = cst<T>(0.0), h5_ = cst<T>(0.0);
+        if (WT) {
+            p_ = p_ + ps_;
+            a_ = a_ + two * a5 * p_;
+            d_ = d_ - p_;
+            const T z6 = z2 * z2 * z2, k2 = kT.v[2], k3 = kT.v[3];
+            k2_ = k2_ - cst<T>(18.0) * k2 * k3 * z6 * del_;
+            const T opE = one + eps, wA = nA * nA;
+            const T f = z2 * (izh * izh) * opE;
+            k3_ = -cst<T>(9.0) * k2 * k2 * z6 * del_ + d_ * f * opE * wA;
+            eps_ = eps_ + d_ * k3 * two * f * wA;
+            wA_ = d_ * k3 * f * opE;
+            h5_ = a_ * izh;
+            if (big) h5_ = h5_ * h;
+        }
+        T uR_, uI_;
+        if (cplx) {
+            uR_ = two * S_ + two * uR * P_ + cst<T>(4.0) * uR * T_;
+            uI_ = two * uI * P_ - cst<T>(4.0) * uI * T_;
+        } else {
+            uR_ = S_ + uI * P_ + two * uR * T_;
+            uI_ = S_ + uR * P_ + two * uI * T_;
+        }
+        if (big) { s_ = s_ * h; uR_ = uR_ * h; uI_ = uI_ * h; }
+        Pn_ = s_;
+        nA_ = nA_ + s_ * nB;
+        nB_ = s_ * nA;
+        if (WT) {
+            Pn_ = Pn_ + h5_ * nB;
+            nB_ = nB_ + h5_ * Pn;
+            nA_ = nA_ + h5_ * z1;
+        }
+        if (cplx) {
+            const T tr_ = uR_ * nr, ti_ = uI_ * ni;
+            nA_ = nA_ + tr_ + ti_;
+            nB_ = nB_ + tr_ - ti_;
+            const T r_ = uR_ * (nA + nB), i_ = uI_ * (nA - nB);
+            // n_P = sqrt(w_P), Pn = |w_P|
+            const T hp = half * iP;
+            qR_ = (Pn_ * wr * iP + hp * (nr * r_ - ni * i_)) * z;
+            qI_ = (Pn_ * wi * iP + hp * (ni * r_ + nr * i_)) * z;
+        } else {
+            nA_ = nA_ + uR_ * nr + uI_ * ni;
+            nB_ = nB_ + uR_ * ni + uI_ * nr;
+            qR_ = (uR_ * nA + uI_ * nB + Pn_ * ni) * half * wr * z;
+            qI_ = (uR_ * nB + uI_ * nA + Pn_ * nr) * half * wi * z;
+        }
+        qA_ = (nA_ * half * rA + wA_) * z;
+        qB_ = nB_ * half * rB * z;
+    }
+    T pf_;
+
+    // sum over the row's constants of adjoint times tangent, direction k
+    LCDM_HD T along(int k) const {
+        const T* t = rc + C_TAN + C_TSTRIDE * k;
+        const Quad<T> t0 = quad(t), t1 = quad(t + 4), t2 = quad(t + 8);
+        T b = t2.v[1];
+        b = b * wF + t2.v[0];
+        b = b * wF + t1.v[3];
+        b = b * wF + t1.v[2];
+        b = b * wF + t1.v[1];
+        b = b * wF + t1.v[0];
+        T r = qA_ * t0.v[0] + qB_ * t0.v[1] + (qR_ * t0.v[2] + qI_ * t0.v[3]) + bF_ * (wF * wF) * b;
+        if (WT) {
+            const Quad<T> t3 = quad(t + 12), t4 = quad(t + 16);
+            T a = t4.v[2];
+            a = a * wJ + t4.v[1];
+            a = a * wJ + t4.v[0];
+            a = a * wJ + t3.v[3];
+            a = a * wJ + t3.v[2];
+            a = a * wJ + t3.v[1];
+            r = r + (eps_ * t2.v[2] + k2_ * t2.v[3] + k3_ * t3.v[0]) + bJ_ * (wJ * wJ) * a;
+        }
+        return r;
+    }
+};
+
+}  // namespace lcdm

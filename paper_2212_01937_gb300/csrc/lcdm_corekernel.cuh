@@ -1,0 +1,283 @@
+// The pair kernel on the core (lcdm_core.cuh): values, vector-Jacobian
+// products, the Gaussian log-likelihood, and Jacobians.
+//
+// Bound by instruction issue (FP32) or by the FP64 pipe: per pair some 250
+// (values of d_C, t, mu) to 600 (with their gradient) instructions against
+// 8 to 32 bytes of memory traffic.  One thread per pair, warps over
+// contiguous ranges; a lane keeps its row's end and record pointer in
+// registers and looks the row up only when it leaves it.
+#pragma once
+#include "lcdm_core.cuh"
+#include "lcdm_kernels.cuh"
+
+namespace lcdm {
+
+// S_k(D) = D s(u), u = Ok D^2, s(u) = sum u^n / (2n+1)!; dS/dD = s + 2 u s',
+// dS/dOk = D^3 s'.  One Horner pass gives s and s'; beyond the series' range
+// (it cancels for u < -4, and needs more terms for large u) curv_map's closed
+// forms.
+template <class T> LCDM_HD void curv_core(T D, T Ok, bool want_d, T& S, T& SD, T& Sk) {
+    const T u = Ok * D * D;
+    constexpr bool F = sizeof(T) == 4;
+    constexpr int NT = F ? 9 : 11;
+    if (u <= (F ? (T)8 : (T)2) && u >= (F ? (T)-4 : (T)-2)) {
+        constexpr double cs[11] = {1.0, 1.0 / 6, 1.0 / 120, 1.0 / 5040, 1.0 / 362880, 1.0 / 39916800,
+                                   1.0 / 6227020800.0, 1.0 / 1307674368000.0, 1.0 / 355687428096000.0,
+                                   1.0 / 121645100408832000.0, 1.0 / 51090942171709440000.0};
+        T s = (T)cs[NT - 1], ds = 0;
+#pragma unroll
+        for (int i = NT - 2; i >= 0; i--) {
+            if (want_d) ds = ds * u + s;
+            s = (T)cs[i] + u * s;
+        }
+        S = D * s;
+        SD = s + (T)2 * u * ds;
+        Sk = D * D * D * ds;
+        return;
+    }
+    curv_map<T>(D, Ok, S, SD, Sk);
+}
+
+// acc += c.  Double-float: one error-free sum; its error joins the low word,
+// which is not renormalised (it stays far below the high word's last place
+// times the number of terms, and the flush adds both in double).
+__device__ __forceinline__ void acc_add(double& a, double c) { a += c; }
+__device__ __forceinline__ void acc_add(df64& a, float c) {
+    const df64 s = two_sum(a.hi, c);
+    a = mkdf(s.hi, LCDM_FADD(a.lo, s.lo));
+}
+
+struct CoreArgs {
+    PairArgs p;
+    const void* rec;    // [B][NCORE]
+};
+
+// registers per thread: blocks of 256 threads per SM the compiler aims at
+template <int PREC, int K, bool WT, bool WX, bool JAC> struct CoreBlocks { enum { value = PREC == 1 ? (K == 0 ? (WX ? 3 : 4) : (JAC ? 2 : 3)) : 2 }; };
+
+template <int PREC, int K, bool WT, bool WX, bool JAC>
+__global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, JAC>::value) core_kernel(CoreArgs ca) {
+    typedef typename std::conditional<PREC == 0, double, float>::type T;
+    typedef typename std::conditional<PREC == 0, double, df64>::type AccT;
+    constexpr int NV = K + 2;   // H0, K density directions, log-likelihood
+    const PairArgs& a = ca.p;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t start = warp * a.chunk;
+    const int64_t end = max(start, min(start + a.chunk, a.nnz));
+    const bool loglike = a.mobs != nullptr;
+    const bool reduce = !JAC && ((a.grad != nullptr) || (a.loglike != nullptr));
+    const T inv_sig = (T)(1.0 / a.sigma);
+    const T lnorm = (T)(-log(a.sigma * 2.5066282746310002));
+    const T Mobs = (T)a.M;
+    const T c5 = (T)(5.0 / 2.302585092994045684);
+    __shared__ AccT acc_s[JAC ? 1 : NV * ACC_STRIDE];
+    AccT* acc = acc_s + (JAC ? 0 : threadIdx.x);
+    if (reduce) {
+#pragma unroll
+        for (int i = 0; i < NV; i++) acc[i * ACC_STRIDE] = cst<AccT>(0.0);
+    }
+    int acc_row = -1;   // (a row's index fits 32 bits: its record alone takes 768 bytes)
+    int64_t wf = -1, wl = -1;
+    if (a.part && reduce && warp < a.det_cap) {
+        // deterministic reduction: the warp's first and last rows, its slots zeroed
+        if (start < end) {
+            wf = row_of(a, a.base + start);
+            wl = row_of(a, a.base + end - 1);
+        }
+        if (lane < 2 * DET_SLOT) a.part[warp * 2 * DET_SLOT + lane] = 0.0;
+        if (lane < 2) a.wrow[warp * 2 + lane] = lane == 0 ? wf : wl;
+        __syncwarp();
+        __threadfence_block();
+    }
+    const int64_t len = end - start, nb = (len + 31) / 32;
+    const int64_t s_lane = a.interleave ? nb : 1, s_it = a.interleave ? 1 : 32;
+    int64_t row = -1, rbeg = 0, rend = INT64_MIN;
+    const T* rec = nullptr;
+    int st = 0;
+    // outputs that need the curvature map
+    const bool map = loglike || (a.outmask & ((1 << O_DM) | (1 << O_DL) | (1 << O_MU))) ||
+                     (K > 0 && (a.cot[O_DM] || a.cot[O_DL] || a.cot[O_MU] || a.jac[O_DM] || a.jac[O_DL] || a.jac[O_MU]));
+    const bool want_mu = loglike || (a.outmask & (1 << O_MU));
+    for (int64_t it = 0; it < nb; it++) {
+        const int64_t off = (int64_t)lane * s_lane + it * s_it;
+        const bool active = off < len;
+        const int64_t pp = a.base + start + (active ? off : len - 1);
+        if (pp >= rend) {
+            if (a.layout == LAYOUT_CSR) {
+                if (row < 0) {
+                    row = row_search(a.offsets, a.B, pp);
+                } else {
+                    int steps = 0;
+                    while (row < a.B - 1 && __ldg(a.offsets + row + 1) <= pp && steps < 8) { row++; steps++; }
+                    if (row < a.B - 1 && __ldg(a.offsets + row + 1) <= pp) row = row_search(a.offsets, a.B, pp);
+                }
+                rend = row < a.B - 1 ? __ldg(a.offsets + row + 1) : INT64_MAX;
+            } else {
+                row = pp / a.nrow;
+                rbeg = row * a.nrow;
+                rend = rbeg + a.nrow;
+            }
+            rec = reinterpret_cast<const T*>(ca.rec) + row * NCORE;
+            st = a.status[row];
+        }
+        const int64_t zi = a.layout == LAYOUT_SHARED ? pp - rbeg : pp;
+        const T z = load_io<T>(a.z, zi);
+        T gcot[N_OUT];
+        T mob = (T)0;
+        if constexpr (K > 0 && !JAC) {
+            // loaded ahead of the evaluation, which hides their latency
+#pragma unroll
+            for (int i = 0; i < N_OUT; i++)
+                gcot[i] = (reduce && !loglike && a.cot[i] && i != O_X) ? load_io<T>(a.cot[i], pp) : (T)0;
+        }
+        if (!JAC && loglike) mob = load_io<T>(a.mobs, zi);
+        int fail = 0;
+        const bool zero = z == (T)0;
+        const bool ok = st == ST_OK;
+        T c[NV];
+#pragma unroll
+        for (int i = 0; i < NV; i++) c[i] = 0;
+        if (ok) {
+            CorePair<T, WT, WX, (K > 0)> e;
+            e.forward(zero ? (T)1 : z, rec, &fail);
+            const T D = zero ? (T)0 : e.Ichi;
+            const Quad<T> ku = quad(rec + C_DH);   // DH TH H0 OK
+            const T DH = ku.v[0], tH = ku.v[1];
+            const T z1 = (T)1 + z;
+            T S = 0, SD = 0, Sk = 0;
+            if (map) curv_core<T>(D, ku.v[3], K > 0, S, SD, Sk);
+            T v[N_OUT];
+            v[O_DC] = DH * D;
+            v[O_T] = WT ? (zero ? (T)0 : tH * e.It) : (T)0;
+            v[O_X] = WX ? (zero ? (T)0 : DH * e.X) : (T)0;
+            v[O_DM] = DH * S;
+            v[O_DL] = z1 * v[O_DM];
+            v[O_MU] = want_mu ? (T)5 * log10(v[O_DL]) + (T)25 : (T)0;
+            if (fail) {
+                const T nan = (T)CUDART_NAN;
+#pragma unroll
+                for (int i = 0; i < N_OUT; i++) v[i] = nan;
+                if (active) atomicMax(a.status + row, (int)ST_NOCONV);
+            }
+            if (active) {
+#pragma unroll
+                for (int i = 0; i < N_OUT; i++)
+                    if ((a.outmask & (1 << i)) && (i != O_X || WX || K == 0) && (i != O_T || WT))
+                        reinterpret_cast<T*>(a.out[i])[pp] = v[i];
+            }
+            if constexpr (JAC) {
+                // one reverse pass per integral, contracted with the tangents
+                const T iH0 = rcp_(ku.v[2]);
+                const T bad = fail ? (T)CUDART_NAN : (T)0;
+                T dc[K];
+                const bool jchi = a.jac[O_DC] || a.jac[O_DM] || a.jac[O_DL] || a.jac[O_MU];
+                if (jchi) {
+                    e.reverse((T)1, (T)0);
+                    const T fr = e.Ichi * rec[C_RS];
+#pragma unroll
+                    for (int k = 0; k < K; k++) dc[k] = zero ? (T)0 : e.along(k) + fr;
+                    const T ism = c5 / S;
+#pragma unroll
+                    for (int i = 0; i < N_OUT; i++) {
+                        if (i == O_T || i == O_X || !a.jac[i] || !active) continue;
+                        T* jp = reinterpret_cast<T*>(a.jac[i]) + pp * a.ncol;
+                        jp[0] = (i == O_MU ? -c5 * iH0 : -v[i] * iH0) + bad;
+#pragma unroll
+                        for (int k = 0; k < K; k++) {
+                            const T dOk = a.ncol == 4 ? (T)-1 : (k == 3 ? (T)1 : (T)0);
+                            T d = i == O_DC ? dc[k] : SD * dc[k] + Sk * dOk;
+                            d = i == O_MU ? (zero ? (T)0 : d * ism) : d * (i == O_DL ? z1 * DH : DH);
+                            jp[1 + k] = d + bad;
+                        }
+                    }
+                }
+                if (WT && a.jac[O_T]) {
+                    e.reverse((T)0, (T)1);
+                    const T fr = e.It * rec[C_RS];
+                    T* jp = reinterpret_cast<T*>(a.jac[O_T]) + pp * a.ncol;
+                    T dt[K];
+#pragma unroll
+                    for (int k = 0; k < K; k++) dt[k] = zero ? (T)0 : tH * (e.along(k) + fr);
+                    if (active) {
+                        jp[0] = -v[O_T] * iH0 + bad;
+#pragma unroll
+                        for (int k = 0; k < K; k++) jp[1 + k] = dt[k] + bad;
+                    }
+                }
+                continue;
+            }
+            if (reduce && active && !fail) {
+                T lin = 0, gm = 0;   // cotangent sums: of H0's linear outputs, of mu
+                T ci = 0, cs = 0, ti = 0;
+                if (loglike) {
+                    const T r = (mob - v[O_MU] - Mobs) * inv_sig;
+                    gm = r * inv_sig;
+                    c[K + 1] = (T)-0.5 * r * r + lnorm;
+                }
+                if constexpr (K > 0) {
+                    if (!loglike) {
+                        gm = gcot[O_MU];
+                        cs = DH * (gcot[O_DM] + z1 * gcot[O_DL]);
+                        ci = DH * gcot[O_DC];
+                        if (WT) ti = tH * gcot[O_T];
+                        lin = gcot[O_DC] * v[O_DC] + gcot[O_DM] * v[O_DM] + gcot[O_DL] * v[O_DL] + gcot[O_T] * v[O_T];
+                    }
+                    const T iH0 = rcp_(ku.v[2]);
+                    c[0] = -(lin + c5 * gm) * iH0;
+                    if (!zero) {
+                        if (gm != (T)0) cs = cs + gm * (c5 / S);
+                        ci = ci + cs * SD;
+                        e.reverse(ci, ti);
+                        const T fr = (e.Ichi * ci + (WT ? e.It * ti : (T)0)) * rec[C_RS];
+                        const T co = cs * Sk;
+#pragma unroll
+                        for (int k = 0; k < K; k++) {
+                            const T dOk = a.ncol == 4 ? (T)-1 : (k == 3 ? (T)1 : (T)0);
+                            c[1 + k] = e.along(k) + fr + co * dOk;
+                        }
+                    }
+                }
+            }
+        } else if (active) {
+            const T nan = (T)CUDART_NAN;
+#pragma unroll
+            for (int i = 0; i < N_OUT; i++) {
+                if (a.outmask & (1 << i)) reinterpret_cast<T*>(a.out[i])[pp] = nan;
+                if (JAC && a.jac[i]) {
+                    T* jp = reinterpret_cast<T*>(a.jac[i]) + pp * a.ncol;
+                    for (int k = 0; k <= K; k++) jp[k] = nan;
+                }
+            }
+        }
+        if (!reduce) continue;
+        // per-lane accumulation while the whole warp stays on one row
+        const int r32 = (int)row, r0 = __shfl_sync(0xffffffffu, r32, 0);
+        const bool uniform = __all_sync(0xffffffffu, r32 == r0);
+        if (uniform && r0 == acc_row) {
+            if (K > 0 && a.grad) {
+#pragma unroll
+                for (int i = 0; i <= K; i++) acc_add(acc[i * ACC_STRIDE], c[i]);
+            }
+            if (loglike) acc_add(acc[(K + 1) * ACC_STRIDE], c[K + 1]);
+            continue;
+        }
+        if (acc_row >= 0) flush_row<NV, K>(acc, acc_row, a, lane, warp, wf, wl);
+        if (uniform) {
+#pragma unroll
+            for (int i = 0; i < NV; i++) acc[i * ACC_STRIDE] = cst<AccT>(0.0) + c[i];
+            acc_row = r0;
+        } else {
+            double cd_[NV];
+#pragma unroll
+            for (int i = 0; i < NV; i++) cd_[i] = (double)c[i];
+            if (seg_reduce<NV>(cd_, row) && active) add_row(a, row, cd_, K + 1, warp, wf, wl);
+#pragma unroll
+            for (int i = 0; i < NV; i++) acc[i * ACC_STRIDE] = cst<AccT>(0.0);
+            acc_row = -1;
+        }
+    }
+    if (reduce && acc_row >= 0) flush_row<NV, K>(acc, acc_row, a, lane, warp, wf, wl);
+}
+
+}  // namespace lcdm

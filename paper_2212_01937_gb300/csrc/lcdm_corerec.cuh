@@ -1,0 +1,225 @@
+// The row record of the core (lcdm_core.cuh) from a cosmology's roots.
+#pragma once
+#include "lcdm_core.cuh"
+
+namespace lcdm {
+
+// Roots of E^2(x), x = 1 + z, as classified by the preparation: the big root A
+// (quartic only), B, and the pair (conjugate: P = (pr, +-pi); two reals: pr, pi),
+// with derivatives along the K density directions.
+struct RowRoots {
+    double H0, Om, OL, Or, Ok, Os, Ox;
+    int ncol, quartic, cpair;
+    double A, B, pr, pi;
+    // set by finish(): q_j = -1/(rho_j - 1) (0 for the cubic's absent root; the
+    // pair: real and imaginary part, or the two), eps = -1/rho_A, 1/S0
+    double qA, qB, q1, q2, eps, S0, iS0;
+
+    // (for a valid row: every real root below 1, S0 > 0)
+    LCDM_HD void finish() {
+        qA = quartic ? rcp_(1.0 - A) : 0.0;
+        eps = quartic ? -1.0 / A : 0.0;
+        qB = rcp_(1.0 - B);
+        // one reciprocal for the pair
+        const double a = pr - 1.0, b = cpair ? pi : pi - 1.0;
+        const double i = -rcp_(cpair ? a * a + b * b : a * b);
+        q1 = (cpair ? a : b) * i;
+        q2 = (cpair ? -b : a) * i;
+        S0 = ncol == 4 ? 1.0 : Om + OL + Or + Ok + Os + Ox;
+        iS0 = ncol == 4 ? 1.0 : rcp_(S0);
+    }
+};
+
+// derivative of the density parameters (Om, OL, Or, Ok + Os, Ox) along direction k
+struct RowDir { double dOm, dOL, dOr, dOk, dOx, dS; };
+LCDM_HD RowDir row_dir(int ncol, int k) {
+    RowDir d;
+    d.dOm = k == 0; d.dOL = k == 1; d.dOr = k == 2; d.dOx = k == 5;
+    d.dOk = k == 3 || k == 4 ? 1.0 : (ncol == 4 ? -1.0 : 0.0);
+    d.dS = ncol == 4 ? 0.0 : 1.0;
+    return d;
+}
+
+// The closing series' coefficients (single precision records: in single
+// precision; they enter the results times the squared deviation and higher
+// powers, at most a fiftieth).
+// R_F in w: b_2 .. b_7 from (e2, e3)
+template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, S* b) {
+    typedef typename Base<S>::type B;
+    b[0] = e2 * cst<B>(-0.1);
+    b[1] = e3 * cst<B>(1.0 / 14);
+    b[2] = e2 * e2 * cst<B>(1.0 / 24);
+    b[3] = e2 * e3 * cst<B>(-3.0 / 44);
+    b[4] = e2 * e2 * e2 * cst<B>(-5.0 / 208) + e3 * e3 * cst<B>(3.0 / 104);
+    b[5] = e2 * e2 * e3 * cst<B>(1.0 / 16);
+}
+// closing series of R_J: a_2 .. a_7; m = (mean of three - p) / z^2
+template <class S> struct SeriesBase { typedef typename Base<S>::type type; };
+template <class T> struct SeriesBase<DD<T> > { typedef T type; };
+template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, S* a) {
+    typedef typename SeriesBase<S>::type B;
+    const S m2 = m * m;
+    const S E2 = e2 - m2 * cst<B>(0.6);
+    const S Q = e3 - m * e2 * cst<B>(0.4) - m2 * m * cst<B>(0.064);
+    const S P = m * cst<B>(0.6), P2 = P * P, P3 = P2 * P;
+    const S E3 = Q + E2 * P * cst<B>(2.0) + P3 * cst<B>(4.0);
+    const S E4 = (Q * cst<B>(2.0) + E2 * P + P3 * cst<B>(3.0)) * P;
+    const S E5 = Q * P2;
+    const S E22 = E2 * E2;
+    a[0] = E2 * cst<B>(-3.0 / 14);
+    a[1] = E3 * cst<B>(1.0 / 6);
+    a[2] = E22 * cst<B>(9.0 / 88) - E4 * cst<B>(3.0 / 22);
+    a[3] = E5 * cst<B>(3.0 / 26) - E2 * E3 * cst<B>(9.0 / 52);
+    a[4] = E22 * E2 * cst<B>(-1.0 / 16) + E3 * E3 * cst<B>(3.0 / 40) + E2 * E4 * cst<B>(3.0 / 20);
+    a[5] = E22 * E3 * cst<B>(45.0 / 272) - (E3 * E4 + E2 * E5) * cst<B>(9.0 / 68);
+}
+// largest deviation of the three, and of the five, arguments from their mean, over z^2
+LCDM_HD float dev3(double e2, double e3) {
+    const float a = sqrtf((float)fabs(e2)), b = cbrtf(4.0f * (float)fabs(e3));
+    return a > b ? a : b;
+}
+LCDM_HD float dev5(float d3, double m) {
+    const float am = (float)fabs(m);
+    const float a = 0.6f * am, b = d3 + 0.4f * am;
+    return a > b ? a : b;
+}
+
+template <class T> LCDM_HD void put(T* rec, int i, double v) { rec[i] = (T)v; }
+LCDM_HD void put_lo(float* rec, int i, double v) { rec[i] = (float)(v - (double)(float)v); }
+LCDM_HD void put_lo(double* rec, int i, double) { rec[i] = 0.0; }
+
+// values (directions are added by core_tangent)
+template <class T> LCDM_HD void core_values(const RowRoots& r, bool absorb, T* rec) {
+    const double Oks = r.Ok + r.Os, S0 = r.S0, iS0 = r.iS0, sS = r.ncol == 4 ? 1.0 : sqrt(S0), isS = sS * iS0;
+    const double qA = r.qA, qB = r.qB, q1 = r.q1, q2 = r.q2, eps = r.eps;
+    put(rec, C_QA, qA); put(rec, C_QB, qB);
+    put(rec, C_QR, q1); put_lo(rec, C_QRL, q1);
+    put(rec, C_QI, q2); put_lo(rec, C_QIL, q2);
+    put(rec, C_C2, 2.0 * isS);
+    put(rec, C_OK, r.Ok);
+    put(rec, C_KIND, r.cpair ? 1.0 : 0.0);
+    put(rec, C_RS, r.ncol == 4 ? 0.0 : -0.5 * iS0);
+    put(rec, C_FREE0, 0.0); put(rec, C_FREE1, 0.0);
+    // invariants
+    const double I = 12.0 * r.Or * r.OL - 3.0 * r.Om * r.Ox + Oks * Oks;
+    const double J = 2.0 * Oks * Oks * Oks - 9.0 * r.Om * Oks * r.Ox + 27.0 * r.Or * r.Ox * r.Ox
+                     + 27.0 * r.Om * r.Om * r.OL - 72.0 * r.Or * Oks * r.OL;
+    const double e2 = I * (-1.0 / 3) * (iS0 * iS0), e3 = J * (-1.0 / 27) * (iS0 * iS0 * iS0);
+    const T f2 = (T)e2, f3 = (T)e3;
+    T b[6], a[6];
+    rf_coefs<T>(f2, f3, b);
+    for (int j = 0; j < 6; j++) rec[C_B2 + j] = b[j];
+    const float d3 = dev3(e2, e3);
+    rec[C_DF] = (T)d3;
+    // t: E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
+    const double g0 = r.OL, g1 = r.Ox - eps * g0, g2 = Oks - eps * g1, g3 = r.Om - eps * g2;
+    const double k = (-g3 + eps * (g2 - eps * (g1 - eps * g0))) * iS0;
+    const double m = (g2 + eps * (3.0 * eps * g0 - 2.0 * g1)) * (iS0 * (1.0 / 3));
+    put(rec, C_EPS, eps);
+    put(rec, C_K2, k * (1.0 / 3));
+    put(rec, C_K3, r.OL * iS0);
+    rj_coefs<T>((T)m, f2, f3, a);
+    for (int j = 0; j < 6; j++) rec[C_A2 + j] = a[j];
+    rec[C_DJ] = (T)dev5(d3, m);
+    if (!absorb) return;
+    const double S = r.cpair ? 2.0 * r.pr : r.pr + r.pi, Q = r.cpair ? r.pr * r.pr + r.pi * r.pi : r.pr * r.pi;
+    const double pB = r.cpair ? (r.pr - r.B) * (r.pr - r.B) + r.pi * r.pi : (r.pr - r.B) * (r.pi - r.B);
+    const double yB = 1.0 - r.B, mA = r.quartic ? r.Or * r.A : -r.Om, rs = r.B + S, iS3 = iS0 * isS;
+    const double X1 = mA * iS0 * (1.0 / 3) * ((S - 2.0 * r.B) + eps * (2.0 * Q - r.B * S));
+    double hx = 0.0;
+    if (r.quartic) {
+        const double aA = -r.Or * (r.A - 1.0), iaA = rcp_(aA), aB = aA - r.Or * yB, c = 1.0 - eps * rs;
+        const double rE1 = -(mA * (2.0 * S + eps * (Q + r.B * r.B + r.B * S)));
+        hx = r.Or * pB * iS0;
+        put(rec, X_LX, r.Or * yB * yB * iS0);
+        put(rec, X_PX, pB * aB * aB * (iS0 * iS0));
+        put(rec, X_C0, sS * iaA);
+        put(rec, X_T1, (2.0 * r.B * r.B - pB) * isS);
+        put(rec, X_G1, pB * rE1 * (1.0 / 3) * iS3);
+        put(rec, X_G2, -c * aB * mA * pB * pB * (1.0 / 3) * (iS3 * iS0));
+        put(rec, X_G3, c * mA);
+        put(rec, X_G4, c * yB * mA * iS3 * (iaA * iaA));
+        put(rec, X_G5, rE1 * yB * isS * iaA);
+        put(rec, X_SY, sS * rcp_(yB));
+        put(rec, X_N0, S0 * (2.0 * aA * yB - r.Or * yB * yB));
+        put(rec, X_N1, S0 * aA);
+        put(rec, X_N2, aB * aB * pB);
+        put(rec, X_AB, aB * iaA);
+        put(rec, X_LAM, r.Or);
+    } else {
+        put(rec, X_LX, 0.0); put(rec, X_PX, 0.0);
+        put(rec, X_C0, (2.0 / 3) * sS / r.Om);
+        put(rec, X_T1, (2.0 / 3) * (3.0 * r.B * r.B - pB) * isS);
+        put(rec, X_G1, (4.0 / 9) * rs * pB * r.Om * iS3);
+        put(rec, X_G2, 0.0); put(rec, X_G3, 0.0); put(rec, X_G4, 0.0);
+        put(rec, X_G5, (4.0 / 3) * rs * yB * isS);
+        put(rec, X_SY, 1.0);
+        put(rec, X_N0, 0.0); put(rec, X_N1, 0.0); put(rec, X_N2, 0.0);
+        put(rec, X_AB, 0.0); put(rec, X_LAM, 0.0);
+    }
+    put(rec, X_FREE, 0.0);
+    put(rec, X_HX, hx);
+    const float dA = dev5(d3, X1 + hx), dD = dev5(d3, X1);
+    rec[X_DX] = (T)(dA > dD ? dA : dD);
+    if (r.cpair) { put(rec, X_SQ, 2.0 * q1); put(rec, X_PQ, q1 * q1 + q2 * q2); }
+    else { put(rec, X_SQ, q1 + q2); put(rec, X_PQ, q1 * q2); }
+    // the series at p0 (offset X1 + hx) and at x1 (offset X1), and their divided differences
+    DD<T> ad[6];
+    rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx), (T)X1, (T)1), mkdd<T>(f2, f2, (T)0), mkdd<T>(f3, f3, (T)0), ad);
+    for (int j = 0; j < 6; j++) {
+        rec[X_A2 + j] = ad[j].v1;
+        rec[X_D2 + j] = ad[j].v2;
+        rec[X_E2 + j] = ad[j].d;
+    }
+}
+
+// tangents of direction k; dA, dB, (dpr, dpi): the roots' derivatives along it
+template <class T>
+LCDM_HD void core_tangent(const RowRoots& r, int k, double dA, double dB, double dpr, double dpi, T* rec) {
+    T* t = rec + C_TAN + C_TSTRIDE * k;
+    const RowDir d = row_dir(r.ncol, k);
+    const double Oks = r.Ok + r.Os, iS0 = r.iS0, eps = r.eps;
+    put(t, CT_QA, r.quartic ? dA * (r.qA * r.qA) : 0.0);
+    put(t, CT_QB, dB * (r.qB * r.qB));
+    if (r.cpair) {
+        // dq = q^2 dr
+        const double s1 = r.q1 * r.q1 - r.q2 * r.q2, s2 = 2.0 * r.q1 * r.q2;
+        put(t, CT_QR, s1 * dpr - s2 * dpi);
+        put(t, CT_QI, s1 * dpi + s2 * dpr);
+    } else {
+        put(t, CT_QR, dpr * (r.q1 * r.q1));
+        put(t, CT_QI, dpi * (r.q2 * r.q2));
+    }
+    // the third-kind integral's constants in double
+    typedef Dual<double, 1> D;
+    D Om, OL, Or, c, Ox, is, ep;
+    Om.v = r.Om; Om.d[0] = d.dOm;
+    OL.v = r.OL; OL.d[0] = d.dOL;
+    Or.v = r.Or; Or.d[0] = d.dOr;
+    c.v = Oks; c.d[0] = d.dOk;
+    Ox.v = r.Ox; Ox.d[0] = d.dOx;
+    is.v = iS0; is.d[0] = -d.dS * iS0 * iS0;
+    ep.v = eps; ep.d[0] = r.quartic ? dA * (eps * eps) : 0.0;
+    const D g1 = Ox - ep * OL, g2 = c - ep * g1, g3 = Om - ep * g2;
+    const D kk = (ep * (g2 - ep * (g1 - ep * OL)) - g3) * is;
+    put(t, CT_EPS, ep.d[0]);
+    put(t, CT_K2, kk.d[0] * (1.0 / 3));
+    put(t, CT_K3, (OL * is).d[0]);
+    // the series in the record's precision
+    typedef Dual<T, 1> F;
+    auto to = [](const D& x) { F f; f.v = (T)x.v; f.d[0] = (T)x.d[0]; return f; };
+    const F fm = to(Om), fl = to(OL), fr = to(Or), fc = to(c), fx = to(Ox), fs = to(is), fe = to(ep), f1 = to(g1), f2 = to(g2);
+    const F I = fr * fl * cst<T>(12.0) - fm * fx * cst<T>(3.0) + fc * fc;
+    const F J = fc * fc * fc * cst<T>(2.0) - fm * fc * fx * cst<T>(9.0) + fr * fx * fx * cst<T>(27.0)
+                + fm * fm * fl * cst<T>(27.0) - fr * fc * fl * cst<T>(72.0);
+    const F e2 = I * fs * fs * cst<T>(-1.0 / 3), e3 = J * fs * fs * fs * cst<T>(-1.0 / 27);
+    F b[6], a[6];
+    rf_coefs<F>(e2, e3, b);
+    for (int j = 0; j < 6; j++) t[CT_B2 + j] = b[j].d[0];
+    const F m = (f2 + fe * (fe * fl * cst<T>(3.0) - f1 * cst<T>(2.0))) * fs * cst<T>(1.0 / 3);
+    rj_coefs<F>(m, e2, e3, a);
+    for (int j = 0; j < 6; j++) t[CT_A2 + j] = a[j].d[0];
+    put(t, CT_END, 0.0);
+}
+
+}  // namespace lcdm

@@ -129,12 +129,6 @@ template <class T, int K> LCDM_HD Dual<T, K> rc_any(const Dual<T, K>& x, const D
 // Phi(w) = [R_C(1, 1-w) - (1-w)^-1/2] / w: the part of R_C(y + d, y) - y^-1/2
 // that is linear in w = d / (y + d), as a series for small w (coefficients
 // 1/(2n+1) - C(2n,n)/4^n, n >= 1) and directly otherwise.
-// The coefficients 1/(2n+1) - C(2n,n)/4^n, n = 1 .. 17 (exact rationals rounded).
-#define LCDM_PHI_CS {-0.16666666666666666, -0.175, -0.16964285714285715, -0.1623263888888889,                   \
-                     -0.1551846590909091, -0.14866286057692307, -0.14280598958333332, -0.13755708582261028,      \
-                     -0.13283900210731908, -0.1285780043829055, -0.12470983422320822, -0.12118025779724122,      \
-                     -0.1179439800756949, -0.11496322216658757, -0.11220638357823895, -0.10964690378838868,      \
-                     -0.10726233098788986}
 template <class S> LCDM_HD S phi_rc(const S& w, int* fail) {
     typedef typename Base<S>::type T;
     constexpr int NT = sizeof(T) == 4 ? 9 : 17;
@@ -326,57 +320,6 @@ LCDM_HD void cubic_integrals_any(typename Base<S>::type z, const S& A, const PS&
                                  int* fail) {
     if constexpr (CALL) cubic_integrals_call<S, PS, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
     else cubic_integrals<S, PS, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
-}
-
-// ------------------------------------------------------ z -> infinity ------
-// The upper limit at infinity (Sec. 2.1.1: the age t(0, inf); the comoving
-// distance to the particle horizon chi(0, inf)) of the quantities above, with
-// the same root labels and scalings.  As z grows, n_j / sqrt(z) -> sqrt(q_j),
-// every u grows like z, and with the homogeneity of R_F, R_C (degree -1/2)
-// and R_J (degree -3/2) every power of z cancels; in eq. (3.8)
-// (1+z) / (1 + eps_A (1+z)) -> 1 / eps_A.  In (B.2) the R_C term falls off
-// like z^-1/2 and drops out.  Ichi and It are in the units of their
-// finite-z counterparts (c/H0 and 1/H0 after the record's prefactors).
-template <class S, class PS>
-LCDM_NI void quartic_limits(const S& mA, const S& epsA, const S& B, const PS& P, const S& qA, const S& qB,
-                            const PS& qP, const S& nrm, S& Ichi, S& It, int* fail) {
-    typedef typename Base<S>::type T;
-    const T one = cst<T>(1.0), third = cst<T>(1.0 / 3.0);
-    S nA = ssqrt(qA), nB = ssqrt(qB);
-    PS nP = psqrt(qP);
-    S uAB = nrm * (nA * nB + pprod(nP));
-    PS uAP = pscale(pscale(nP, nA) + pscale(pswap(nP), nB), nrm);
-    S x1 = uAB * uAB;
-    S rhoB = B + one;
-    PS rhoP = padd(P, one);
-    S ppPA = pprod(padd(pscale(rhoP, epsA), one));
-    S p[1];
-    p[0] = -(mA * ppPA * rhoB);
-    S RF, RD1, RJ[1];
-    carlson_any<1, false, false>(uAB, uAP, p, RF, RD1, RJ, fail);
-    Ichi = RF * cst<T>(2.0);                                   // eq. (3.7), z -> inf
-    S kq5 = (x1 + p[0]) / ((one + epsA) * epsA);
-    S ks5 = kq5 + mA * pprod(rhoP) * rhoB;
-    It = (rc_any(ks5, kq5, fail) - epsA * RF - mA * (one + epsA * rhoB) * ppPA * RJ[0] * third)
-         * cst<T>(2.0);                                        // eq. (3.8), z -> inf
-}
-
-template <class S, class PS>
-LCDM_NI void cubic_limits(const S& A, const S& amh, const S& qA, const PS& qP, const S& nrm, S& Ichi, S& It,
-                          int* fail) {
-    typedef typename Base<S>::type T;
-    const T one = cst<T>(1.0);
-    S nA = ssqrt(qA);
-    PS nP = psqrt(qP);
-    // u_A / z -> N n_P n_P*,  u_P / z -> N n_P* n_A  (the plain u_i -> Y_i = sqrt(-r_i))
-    S uA = nrm * pprod(nP);
-    PS uP = pscale(pswap(nP), nA * nrm);
-    S p[1];
-    p[0] = A + one;                                            // u_A5^2 - u_A^2 = rho_A
-    S RF, RD1, RJ[1];
-    carlson_any<1, false, false>(uA, uP, p, RF, RD1, RJ, fail);
-    Ichi = amh * RF * cst<T>(2.0);                             // eq. (B.1), z -> inf
-    It = amh * RJ[0] * cst<T>(2.0 / 3.0);                      // eq. (B.2), z -> inf
 }
 
 }  // namespace lcdm

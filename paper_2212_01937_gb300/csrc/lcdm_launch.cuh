@@ -1,55 +1,84 @@
 // Launch helpers for the pair kernel instantiations (one translation unit per
 // precision and tangent count, so they compile in parallel).
 #pragma once
-#include "lcdm_kernels.cuh"
+#include "lcdm_corekernel.cuh"
 
 namespace lcdm {
 
-typedef cudaError_t (*pairs_launch_fn)(const PairArgs&, int grid, int block, cudaStream_t);
-typedef int (*pairs_occ_fn)(int block);
-
-template <int PREC, int K, bool WT, bool WX>
-cudaError_t launch_pairs(const PairArgs& a, int grid, int block, cudaStream_t s) {
-    pairs_kernel<PREC, K, WT, WX><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
-}
-template <int PREC, int K, bool WT, bool WX>
-int occupancy_pairs(int block) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pairs_kernel<PREC, K, WT, WX>, block, 0) != cudaSuccess)
-        return 0;
-    return n;
-}
-
-// table entry for (WT, WX) = index (WT ? 2 : 0) + (WX ? 1 : 0)
-struct PairsTable {
-    pairs_launch_fn launch[4];
-    pairs_occ_fn occ[4];
+// One pair kernel: its launch and its resident blocks per SM.  `rec` is the
+// core's record; the kernel of X's tangents reads the records in the arguments.
+struct PairsEntry {
+    cudaError_t (*launch)(const PairArgs& a, const void* rec, int grid, int block, cudaStream_t s);
+    int (*occ)(int block);
 };
 
-#define LCDM_DEFINE_TABLE(NAME, PREC, K)                                                     \
-    PairsTable NAME() {                                                                      \
-        PairsTable t;                                                                        \
-        t.launch[0] = launch_pairs<PREC, K, false, false>;                                   \
-        t.launch[1] = launch_pairs<PREC, K, false, true>;                                    \
-        t.launch[2] = launch_pairs<PREC, K, true, false>;                                    \
-        t.launch[3] = launch_pairs<PREC, K, true, true>;                                     \
-        t.occ[0] = occupancy_pairs<PREC, K, false, false>;                                   \
-        t.occ[1] = occupancy_pairs<PREC, K, false, true>;                                    \
-        t.occ[2] = occupancy_pairs<PREC, K, true, false>;                                    \
-        t.occ[3] = occupancy_pairs<PREC, K, true, true>;                                     \
-        return t;                                                                            \
+template <int PREC, int K, bool WT> struct TangentX {
+    static cudaError_t launch(const PairArgs& a, const void*, int grid, int block, cudaStream_t s) {
+        pairs_kernel<PREC, K, WT, true><<<grid, block, 0, s>>>(a);
+        return cudaGetLastError();
     }
+    static int occ(int block) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pairs_kernel<PREC, K, WT, true>, block, 0) != cudaSuccess)
+            return 0;
+        return n;
+    }
+};
+template <int PREC, int K, bool WT, bool WX, bool JAC> struct Core {
+    static cudaError_t launch(const PairArgs& a, const void* rec, int grid, int block, cudaStream_t s) {
+        CoreArgs c;
+        c.p = a;
+        c.rec = rec;
+        core_kernel<PREC, K, WT, WX, JAC><<<grid, block, 0, s>>>(c);
+        return cudaGetLastError();
+    }
+    static int occ(int block) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core_kernel<PREC, K, WT, WX, JAC>, block, 0) != cudaSuccess)
+            return 0;
+        return n;
+    }
+};
+
+// entries by (WT ? 2 : 0) + (WX ? 1 : 0); jac: the kernels of per-pair
+// Jacobians (without X's, whose tangents have a kernel of their own)
+struct PairsTable {
+    PairsEntry e[4], jac[4];
+};
+
+template <class E> PairsEntry entry() { PairsEntry e; e.launch = E::launch; e.occ = E::occ; return e; }
+
+template <int PREC> PairsTable value_table() {
+    PairsTable t;
+    t.e[0] = entry<Core<PREC, 0, false, false, false> >();
+    t.e[1] = entry<Core<PREC, 0, false, true, false> >();
+    t.e[2] = entry<Core<PREC, 0, true, false, false> >();
+    t.e[3] = entry<Core<PREC, 0, true, true, false> >();
+    for (int i = 0; i < 4; i++) t.jac[i] = t.e[i];
+    return t;
+}
+template <int PREC, int K> PairsTable tangent_table() {
+    PairsTable t;
+    t.e[0] = entry<Core<PREC, K, false, false, false> >();
+    t.e[1] = entry<TangentX<PREC, K, false> >();
+    t.e[2] = entry<Core<PREC, K, true, false, false> >();
+    t.e[3] = entry<TangentX<PREC, K, true> >();
+    t.jac[0] = entry<Core<PREC, K, false, false, true> >();
+    t.jac[1] = t.e[1];
+    t.jac[2] = entry<Core<PREC, K, true, false, true> >();
+    t.jac[3] = t.e[3];
+    return t;
+}
 
 PairsTable table_f64_k0();
 PairsTable table_f64_k3();
 PairsTable table_f64_k4();
+PairsTable table_f64_k6();
 PairsTable table_mix_k0();
 PairsTable table_mix_k3();
 PairsTable table_mix_k4();
-PairsTable table_f64_k6();
+PairsTable table_mix_k6();
 // second pass of the deterministic reduction (defined with the other kernels)
 cudaError_t launch_det_fixup(const PairArgs& a, int64_t nwarps, cudaStream_t s);
-PairsTable table_mix_k6();
 
 }  // namespace lcdm

@@ -707,6 +707,14 @@ LCDM_HD SymResult<T, NJ> carlson_sym(T s1, T S, T P, bool cplx, const T* pj, con
     return R;
 }
 
+// [R_C(1, 1-w) - (1-w)^-1/2] / w as a series in w.
+// The coefficients 1/(2n+1) - C(2n,n)/4^n, n = 1 .. 17 (exact rationals rounded).
+#define LCDM_PHI_CS {-0.16666666666666666, -0.175, -0.16964285714285715, -0.1623263888888889,                   \
+                     -0.1551846590909091, -0.14866286057692307, -0.14280598958333332, -0.13755708582261028,      \
+                     -0.13283900210731908, -0.1285780043829055, -0.12470983422320822, -0.12118025779724122,      \
+                     -0.1179439800756949, -0.11496322216658757, -0.11220638357823895, -0.10964690378838868,      \
+                     -0.10726233098788986}
+
 // Square roots' sum S and product P of the pair whose members are the squares
 // of u (the callers' u's: y = u^2, principal roots |u| resp. +-u with Re >= 0).
 template <class S> LCDM_HD S proot_sum(const CPair<S>& u) { return sabs(u.c.re) * cst_like(u.c.re, 2.0); }

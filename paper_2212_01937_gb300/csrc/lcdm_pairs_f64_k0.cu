@@ -1,5 +1,5 @@
 // Pair-kernel instantiations: precision f64, 0 tangent directions.
 #include "lcdm_launch.cuh"
 namespace lcdm {
-LCDM_DEFINE_TABLE(table_f64_k0, 0, 0)
+PairsTable table_f64_k0() { return value_table<0>(); }
 }

@@ -1,5 +1,5 @@
 // Pair-kernel instantiations: precision mix, 4 tangent directions.
 #include "lcdm_launch.cuh"
 namespace lcdm {
-LCDM_DEFINE_TABLE(table_mix_k4, 1, 4)
+PairsTable table_mix_k4() { return tangent_table<1, 4>(); }
 }

@@ -2,6 +2,7 @@
 // classify the roots, choose the root labels, precompute the per-cosmology
 // constants and the root tangents (App. A, eqs. A.1-A.4).
 #pragma once
+#include "lcdm_corerec.cuh"
 #include "lcdm_kernels.cuh"
 
 namespace lcdm {
@@ -99,6 +100,42 @@ LCDM_HD void polish_root(const double* a, int n, cd& x) {
     }
 }
 
+// One Newton step from one compensated evaluation, the quotient in single
+// precision: enough for a root known to about 1e-15 / separation (the step
+// leaves 1e-7 of that error), without polish_root's confirming evaluations.
+LCDM_HD void polish_once(const double* a, int n, cd& x) {
+    cd p, dp;
+    horner_comp(a, n, x, p, dp);
+    const float pr = (float)p.re, pi = (float)p.im, dr = (float)dp.re, di = (float)dp.im;
+    const float i = 1.0f / (dr * dr + di * di);
+    const float wr = (pr * dr + pi * di) * i, wi = (pi * dr - pr * di) * i;
+    if (!(fabsf(wr) + fabsf(wi) < 1e30f)) return;
+    x = cmk(x.re - (double)wr, x.im - (double)wi);
+}
+
+// A double as a float after division by 2^e (by its bits: no FP64 instruction),
+// 0 or a huge number beyond the float's range; and a double's binary exponent.
+// With e = the larger exponent of a number's parts, ratios of its size can be
+// compared in single precision wherever it lies.
+LCDM_HD int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
+LCDM_HD float scaled(double v, int e) {
+    const long long b = __double_as_longlong(v);
+    const int k = (int)((b >> 52) & 0x7ff) - e;   // biased exponent of the quotient
+    if (k < 1023 - 100) return 0.0f;
+    if (k > 1023 + 100) return 1e30f;
+    return (float)__longlong_as_double((b & ~(0x7ffLL << 52)) | ((long long)k << 52));
+}
+LCDM_HD int exponent_of(cd z) {
+    const int a = exponent_of(z.re), b = exponent_of(z.im);
+    return a > b ? a : b;
+}
+// |Im z| <= 1e-12 |z|
+LCDM_HD bool negligible_im(cd z) {
+    const int e = exponent_of(z);
+    const float x = scaled(z.re, e), y = scaled(z.im, e);
+    return fabsf(y) <= 1e-12f * sqrtf(x * x + y * y);
+}
+
 // Single-precision elementary functions for the starting circles only (no
 // accuracy needed there): the fast hardware approximations on the device.
 LCDM_HD float flog(float x) {
@@ -133,13 +170,13 @@ LCDM_HD float fsin(float x) {
 // Starting points of the root iteration for the monic polynomial c (degree
 // n <= 4): circles whose radii come from the Newton polygon of log|c_k|, so
 // that a root near -Om/Or and the O(1) roots both start close.
-LCDM_HD void start_points(const double* c, int n, cd* z) {
+LCDM_HD void start_points(const float* c, int n, float* zr, float* zi) {
     // upper convex hull of (k, log|c_k|); single precision is enough for the start
     float lg[5];
     int idx[5], m = 0;
-    for (int k = 0; k <= n; k++) lg[k] = c[k] != 0 ? flog((float)fabs(c[k])) : -1e30f;
+    for (int k = 0; k <= n; k++) lg[k] = c[k] != 0.f ? flog(fabsf(c[k])) : -1e30f;
     for (int k = 0; k <= n; k++) {
-        if (c[k] == 0) continue;
+        if (c[k] == 0.f) continue;
         while (m >= 2) {
             int a = idx[m - 2], b = idx[m - 1];
             // remove b if it lies below the segment a-k
@@ -153,10 +190,11 @@ LCDM_HD void start_points(const double* c, int n, cd* z) {
         float rad = fexp((lg[a] - lg[b]) / w);
         for (int j = 0; j < w && r < 4; j++) {
             float ang = 6.2831853f * j / w + 6.2831853f * a / n + 0.4f;
-            z[r++] = cmk(rad * fcos(ang), rad * fsin(ang));
+            zr[r] = rad * fcos(ang);
+            zi[r++] = rad * fsin(ang);
         }
     }
-    for (; r < 4; r++) z[r] = cmk(0.5 * r + 0.1, 0.3);  // (zero constant term etc.)
+    for (; r < 4; r++) { zr[r] = 0.5f * r + 0.1f; zi[r] = 0.3f; }  // (zero constant term etc.)
 }
 
 // Roots of the monic polynomial c (degree n <= 4) by the simultaneous
@@ -166,27 +204,52 @@ LCDM_HD void start_points(const double* c, int n, cd* z) {
 // cosmology (few cosmologies: latency-bound); one lane does no repeated work
 // (many cosmologies: bound by the FP64 pipe).  Every lane of the warp must
 // call this (groups with active == false take part in the shuffles without
-// updating).  Single precision first, to about 1e-6 relative (short latency
-// chains), then double precision from there (cubic convergence: two or three
-// sweeps), stopping after a sweep with every correction below 1e-15 relative
-// or once the corrections stop shrinking (rounding level of a near-multiple
-// root); one Newton step per root at the end.  On return every lane of the
-// group holds all n roots in z.
-template <int G> __device__ void group_roots(const double* c, const double* alpha, int n, bool active, cd* z) {
+// updating).
+//
+// On this part every FP64 instruction of a warp holds its sub-partition for
+// 64 cycles (19 per SM when all four issue), whatever the number of active
+// lanes or independent operations, so what counts is the number of FP64
+// instructions.  Hence: single precision first, to about 1e-6; then sweeps in
+// which only what decides the accuracy is double, the polynomial's and its
+// derivative's values (26 instructions) and the differences of the roots; the
+// correction itself, a number known to 1e-7 of its size, is single.  A sweep
+// leaves 1e-7 of the error (or its cube), so two usually end it; comparisons
+// are made in single precision or on the bits.  (4096 rows: 0.070 ms with
+// double corrections, confirmations and hypot; see DESIGN for the rest.)
+// Coefficients outside single precision's range (Or0 below about 1e-10, OL0 =
+// 0) take the sweeps in double throughout.
+//
+// A root closer than a tenth of its modulus to another (near-multiple roots,
+// as near the no-Big-Bang boundary) is polished on the original coefficients
+// (the monic ones carry the rounding of the division by alpha_n) by the
+// compensated scheme; an isolated one is within an ulp or two after the
+// sweeps.  For single-precision distances the polish starts at a hundredth
+// (`near`): the roots' error there is 1e-13 without it.
+// On return every lane of the group holds all n roots in z.
+template <int G>
+__device__ void group_roots(const double* c, const double* alpha, int n, bool active, float near, cd* z) {
     constexpr int R = 4 / G;   // roots per lane
     const unsigned full = 0xffffffffu;
     const int s = threadIdx.x & (G - 1);
-    cd z0[4];
-    start_points(c, n, z0);
+    float cf[5], zr[R], zi[R];
+    bool usual = true;
+#pragma unroll
+    for (int k = 0; k <= 4; k++) {
+        cf[k] = k <= n ? (float)c[k] : 0.f;
+        usual = usual && fabsf(cf[k]) < 1e6f;
+    }
+    usual = usual && fabsf(cf[0]) > 1e-20f;
+    float st_r[4], st_i[4];
+    start_points(cf, n, st_r, st_i);
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        zr[r] = G == 1 ? st_r[r] : (s == 0 ? st_r[0] : s == 1 ? st_r[1] : s == 2 ? st_r[2] : st_r[3]);
+        zi[r] = G == 1 ? st_i[r] : (s == 0 ? st_i[0] : s == 1 ? st_i[1] : s == 2 ? st_i[2] : st_i[3]);
+    }
     double zre[R], zim[R];
 #pragma unroll
-    for (int r = 0; r < R; r++) { zre[r] = z0[r * G + s].re; zim[r] = z0[r * G + s].im; }
+    for (int r = 0; r < R; r++) { zre[r] = zr[r]; zim[r] = zi[r]; }
     {
-        float cf[5];
-        for (int k = 0; k <= 4; k++) cf[k] = k <= n ? (float)c[k] : 0.f;
-        float zr[R], zi[R];
-#pragma unroll
-        for (int r = 0; r < R; r++) { zr[r] = (float)zre[r]; zi[r] = (float)zim[r]; }
         bool done = !active;
 #pragma unroll 1
         for (int itf = 0; itf < 100; itf++) {
@@ -202,9 +265,9 @@ template <int G> __device__ void group_roots(const double* c, const double* alph
                 const int j = r * G + s;
                 if (done || j >= n) continue;
                 const float xr0 = ar[j], xi0 = ai[j];
-                float pr = cf[n], pi = 0.f, dr = 0.f, di = 0.f;
-#pragma unroll 1
-                for (int k = n - 1; k >= 0; k--) {
+                float pr = cf[4], pi = 0.f, dr = 0.f, di = 0.f;   // (cf[4] = 0 for a cubic)
+#pragma unroll
+                for (int k = 3; k >= 0; k--) {
                     float ndr = dr * xr0 - di * xi0 + pr, ndi = dr * xi0 + di * xr0 + pi;
                     float npr = pr * xr0 - pi * xi0 + cf[k], npi = pr * xi0 + pi * xr0;
                     dr = ndr; di = ndi; pr = npr; pi = npi;
@@ -241,43 +304,64 @@ template <int G> __device__ void group_roots(const double* c, const double* alph
         for (int r = 0; r < R; r++)
             if (isfinite(zr[r]) && isfinite(zi[r])) { zre[r] = zr[r]; zim[r] = zi[r]; }
     }
-    // Single precision can merge a complex pair of nearly double roots (near
-    // the no-Big-Bang boundary) into two points on or near the real axis, and
-    // for a real polynomial the iteration keeps real approximations real.
-    // Two such approximations within 1e-3 of each other get imaginary
-    // offsets of opposite sign (far above double precision, far below the
-    // spacing), which lets the double-precision sweeps move them back into
-    // the complex plane if the roots are complex; real ones return to the axis.
+    // the roots' separation relative to their moduli (float): isolated or not
+    float sep = 1.0f;
     {
-        double cr[4], ci[4];
+        float ar[4], ai[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            cr[k] = G == 1 ? zre[k / G] : __shfl_sync(full, zre[k / G], k % G, G);
-            ci[k] = G == 1 ? zim[k / G] : __shfl_sync(full, zim[k / G], k % G, G);
+            ar[k] = G == 1 ? (float)zre[k / G] : __shfl_sync(full, (float)zre[k / G], k % G, G);
+            ai[k] = G == 1 ? (float)zim[k / G] : __shfl_sync(full, (float)zim[k / G], k % G, G);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (k == j || j >= n || k >= n) continue;
+                const float dr = ar[j] - ar[k], di = ai[j] - ai[k], q = dr * dr + di * di, mj = ar[j] * ar[j] + ai[j] * ai[j];
+                if (!(q > sep * sep * mj)) sep = sqrtf(q / mj);
+            }
+        }
+        if (!(sep > 0.f)) sep = 0.f;
+    }
+    const bool iso = sep > 0.1f;
+    // (a group's lanes agree; the others take the next block for nothing)
+    if (!__all_sync(full, iso || !active)) {
+        // Single precision can merge a complex pair of nearly double roots (near
+        // the no-Big-Bang boundary) into two points on or near the real axis, and
+        // for a real polynomial the iteration keeps real approximations real.
+        // Two such approximations within 1e-3 of each other get imaginary
+        // offsets of opposite sign (far above double precision, far below the
+        // spacing), which lets the double-precision sweeps move them back into
+        // the complex plane if the roots are complex; real ones return to the axis.
+        float cr[4], ci[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            cr[k] = G == 1 ? (float)zre[k / G] : __shfl_sync(full, (float)zre[k / G], k % G, G);
+            ci[k] = G == 1 ? (float)zim[k / G] : __shfl_sync(full, (float)zim[k / G], k % G, G);
         }
 #pragma unroll
         for (int r = 0; r < R; r++) {
             const int j = r * G + s;
             if (j >= n) continue;
-            const double m = fabs(cr[j]) + fabs(ci[j]);
-            if (!(fabs(ci[j]) < 1e-6 * m)) continue;
-#pragma unroll 1
-            for (int k = 0; k < n; k++) {
-                if (k == j || !(fabs(ci[k]) < 1e-6 * m)) continue;
-                if (fabs(cr[k] - cr[j]) < 1e-3 * m) { zim[r] += (j < k ? 1e-6 : -1e-6) * m; break; }
+            float xj = 0.f, yj = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (k == j) { xj = cr[k]; yj = ci[k]; }
+            const float m = fabsf(xj) + fabsf(yj);
+            if (!(fabsf(yj) < 1e-6f * m)) continue;
+            float off = 0.f;
+#pragma unroll
+            for (int k = 3; k >= 0; k--) {
+                if (k == j || k >= n || !(fabsf(ci[k]) < 1e-6f * m)) continue;
+                if (fabsf(cr[k] - xj) < 1e-3f * m) off = j < k ? 1e-6f : -1e-6f;
             }
+            if (off != 0.f) zim[r] = (double)(yj + off * m);
         }
     }
     {
-        int settled = 0;
-        double prev = 1e300;
         bool done = !active;
-        // Isolated roots (every one more than a tenth of its modulus from the
-        // others, judged on the single-precision approximations): the
-        // iteration converges cubically from ~1e-6, so one FP64 sweep whose
-        // corrections are all below 1e-6 leaves them within rounding and no
-        // confirming sweep is needed.
-        bool iso = true;
+        float prev = 3e38f;
 #pragma unroll 1
         for (int it = 0; it < 200; it++) {
             double br[4], bi[4];
@@ -286,62 +370,81 @@ template <int G> __device__ void group_roots(const double* c, const double* alph
                 br[k] = G == 1 ? zre[k / G] : __shfl_sync(full, zre[k / G], k % G, G);
                 bi[k] = G == 1 ? zim[k / G] : __shfl_sync(full, zim[k / G], k % G, G);
             }
-            if (it == 0) {
-#pragma unroll 1
-                for (int j = 0; j < n; j++) {
-                    const float mj = sqrtf((float)(br[j] * br[j] + bi[j] * bi[j]));
-#pragma unroll 1
-                    for (int k = 0; k < n; k++) {
-                        if (k == j) continue;
-                        const float dr_ = (float)(br[j] - br[k]), di_ = (float)(bi[j] - bi[k]);
-                        if (!(sqrtf(dr_ * dr_ + di_ * di_) > 0.1f * mj)) iso = false;
-                    }
-                }
-            }
-            double worst = 0.0;
+            float worst = 0.f;
 #pragma unroll
             for (int r = 0; r < R; r++) {
                 const int j = r * G + s;
                 if (done || j >= n) continue;
-                cd zj = cmk(br[j], bi[j]), p, dp;
-                horner(c, n, zj, p, dp);
-                if (p.re == 0 && p.im == 0) continue;
-                cd ratio = cmul(p, crcp(dp));
-                cd sm = cmk(0, 0);
+                const double x = br[j], y = bi[j];
+                if (usual) {
+                    // value and derivative by Horner's rule (the monic quartic's first two steps by hand)
+                    cd p, dp;
+                    if (n == 4) {
+                        p = cmk(x + c[3], y);
+                        dp = cmk(x + p.re, y + y);
+                    } else {
+                        p = cmk(1.0, 0.0);
+                        dp = cmk(0.0, 0.0);
+                    }
+#pragma unroll
+                    for (int k = 2; k >= 0; k--) {
+                        if (n == 4 ? k < 2 : true)
+                            dp = cmk(fma(dp.re, x, fma(-dp.im, y, p.re)), fma(dp.re, y, fma(dp.im, x, p.im)));
+                        p = cmk(fma(p.re, x, fma(-p.im, y, c[k])), fma(p.re, y, p.im * x));
+                    }
+                    const float pr = (float)p.re, pi = (float)p.im, dr = (float)dp.re, di = (float)dp.im;
+                    float sr = 0.f, si = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        if (k == j || k >= n) continue;
+                        const float xr = (float)(x - br[k]), xi = (float)(y - bi[k]), x2 = xr * xr + xi * xi;
+                        if (!(x2 > 0.f)) continue;
+                        const float ix = 1.0f / x2;
+                        sr += xr * ix;
+                        si -= xi * ix;
+                    }
+                    // w = p / (p' - p S)
+                    const float er = dr - (pr * sr - pi * si), ei = di - (pr * si + pi * sr), ie = 1.0f / (er * er + ei * ei);
+                    const float wr = (pr * er + pi * ei) * ie, wi = (pi * er - pr * ei) * ie;
+                    if (pr == 0.f && pi == 0.f) continue;
+                    zre[r] = x - (double)wr;
+                    zim[r] = y - (double)wi;
+                    const float xf = (float)x, yf = (float)y, rel = (wr * wr + wi * wi) / (xf * xf + yf * yf);
+                    if (!(rel <= worst)) worst = rel;   // a NaN counts as the worst
+                } else {
+                    cd zj = cmk(x, y), p, dp;
+                    horner(c, n, zj, p, dp);
+                    if (p.re == 0 && p.im == 0) continue;
+                    cd ratio = cmul(p, crcp(dp));
+                    cd sm = cmk(0, 0);
 #pragma unroll 1
-                for (int k = 0; k < n; k++)
-                    if (k != j) sm = cadd(sm, crcp(csub(zj, cmk(br[k], bi[k]))));
-                cd w = cmul(ratio, crcp(csub(cmk(1, 0), cmul(ratio, sm))));
-                zj = csub(zj, w);
-                zre[r] = zj.re; zim[r] = zj.im;
-                const double rel = cnorm(w) * ddiv(1.0, cnorm(zj) + 1e-300);
-                if (!(rel <= worst)) worst = rel;   // a NaN counts as the worst
+                    for (int k = 0; k < n; k++)
+                        if (k != j) sm = cadd(sm, crcp(csub(zj, cmk(br[k], bi[k]))));
+                    cd w = cmul(ratio, crcp(csub(cmk(1, 0), cmul(ratio, sm))));
+                    zj = csub(zj, w);
+                    zre[r] = zj.re; zim[r] = zj.im;
+                    const float rel = (float)(cnorm(w) * ddiv(1.0, cnorm(zj) + 1e-300));
+                    if (!(rel <= worst)) worst = rel;
+                }
             }
             if (G > 1) {
 #pragma unroll
                 for (int o = 1; o < G; o <<= 1) {
-                    double v = __shfl_xor_sync(full, worst, o, G);
+                    const float v = __shfl_xor_sync(full, worst, o, G);
                     if (!(v <= worst)) worst = v;
                 }
             }
             if (!done) {
-                if (worst < 1e-30 || (it == 0 && iso && worst < 1e-12)) { if (++settled >= 1) done = true; }
-                else if (it >= 4 && worst >= 0.25 * prev && worst < 1e-24) done = true;
+                // |w| below 1e-9 |z| (usual: 1e-7 of it is left), or no longer shrinking
+                if (worst < (usual ? 1e-18f : 1e-30f)) done = true;
+                else if (it >= 4 && worst >= 0.25f * prev && worst < 1e-16f) done = true;
                 prev = worst;
             }
             if (__all_sync(full, done)) break;
         }
     }
     // A root whose imaginary part is negligible (|Im| <= 1e-12 |z|: the
-    // classification's test) is put on the real axis.  Roots closer than a
-    // tenth of their modulus to another root (near-multiple roots, as near
-    // the no-Big-Bang boundary) are then polished by Newton steps on the
-    // original coefficients (the monic ones carry the rounding of the
-    // division by alpha_n), evaluated by the compensated scheme, each by the
-    // lane that owns it; an isolated root is already within an ulp or two
-    // after the sweeps (the rounding of the monic coefficients moves it by
-    // its condition number, small when it is isolated), so it skips the
-    // polish and its FP64 work.
+    // classification's test) is put on the real axis; then the polish.
     {
         double cr[4], ci[4];
 #pragma unroll
@@ -354,13 +457,20 @@ template <int G> __device__ void group_roots(const double* c, const double* alph
             const int j = r * G + s;
             if (!active || j >= n) continue;
             cd zj = cmk(zre[r], zim[r]);
-            const double mz = cabs_(zj);
-            if (fabs(zj.im) <= 1e-12 * mz) zj.im = 0.0;
-            bool isolated = true;
-#pragma unroll 1
-            for (int k = 0; k < n; k++)
-                if (k != j && !(cabs_(csub(cmk(cr[k], ci[k]), cmk(cr[j], ci[j]))) > 0.1 * mz)) isolated = false;
-            if (!isolated) polish_root(alpha, n, zj);
+            const int ez = exponent_of(zj);
+            const float mx = scaled(zj.re, ez), my = scaled(zj.im, ez), mz = sqrtf(mx * mx + my * my);
+            if (fabsf(my) <= 1e-12f * mz) zj.im = 0.0;
+            float d = 1.0f;   // distance to the nearest other root over the modulus
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (k == j || k >= n) continue;
+                const float xr = scaled(cr[k] - cr[j], ez), xi = scaled(ci[k] - ci[j], ez);
+                const float q = sqrtf(xr * xr + xi * xi) / mz;
+                if (!(q >= d)) d = q;
+            }
+            if (!(d > near)) {
+                if (d > 1e-4f) polish_once(alpha, n, zj); else polish_root(alpha, n, zj);
+            }
             zre[r] = zj.re; zim[r] = zj.im;
         }
     }
@@ -370,30 +480,41 @@ template <int G> __device__ void group_roots(const double* c, const double* alph
                       : cmk(__shfl_sync(full, zre[k / G], k % G, G), __shfl_sync(full, zim[k / G], k % G, G));
 }
 
-// Record of one cosmology from its parameter row p[ncol] = (H0, Om, OL, Or[, Ok]);
-// returns the status code.  Called by the G lanes of a group together (see
-// group_roots); `active` is false for lanes past the last cosmology.
-template <int G> __device__ int prep_one(const double* p, int ncol, double* rec, bool active) {
-    double H0 = p[0], Om = p[1], OL = p[2], Or = p[3];
-    double Ok = ncol >= 5 ? p[4] : 1.0 - Om - OL - Or;
+// Root solve and classification of one cosmology, parameter row p[ncol] =
+// (H0, Om, OL, Or[, Ok[, Os, Ox]]): the labelled roots in r and, with
+// `tangents`, their derivatives dr[slot][k] (slots: A and B of a quartic, B of
+// a cubic, then the pair; 1: each lane of a group gets the directions k equal
+// to its own number modulo G, 2: every lane gets all).  Returns the status code.  Called by the G lanes of
+// a group together (see group_roots); `active` is false for lanes past the
+// last cosmology.
+template <int G>
+__device__ int prep_roots(const double* p, int ncol, bool active, int tangents, float near, RowRoots& r,
+                          cd (*dr)[RF_KT], bool& labelled) {
+    r.H0 = p[0]; r.Om = p[1]; r.OL = p[2]; r.Or = p[3];
+    r.Ok = ncol >= 5 ? p[4] : 1.0 - r.Om - r.OL - r.Or;
     // the further components of fn4 (7-column rows): Os (w = -1/3) scales as
     // (1+z)^2 like curvature but stays out of the curvature map, Ox (w = -2/3)
     // as (1+z); with them every density is an independent direction
-    const double Os = ncol >= 7 ? p[5] : 0.0, Ox = ncol >= 7 ? p[6] : 0.0;
-    for (int i = 0; i < NREC; i++) rec[i] = 0;
-    int st = ST_OK, kind = 0;
+    r.Os = ncol >= 7 ? p[5] : 0.0;
+    r.Ox = ncol >= 7 ? p[6] : 0.0;
+    r.ncol = ncol;
+    const double Om = r.Om, OL = r.OL, Or = r.Or, Ok = r.Ok, Os = r.Os, Ox = r.Ox;
+    labelled = false;
+    int st = ST_OK;
     const int K = ncol - 1;
-    bool finite = isfinite(H0) && isfinite(Om) && isfinite(OL) && isfinite(Or) && isfinite(Ok) &&
-                  isfinite(Os) && isfinite(Ox);
-    int n = Or > 0 ? 4 : 3;
-    if (!finite || !(H0 > 0) || Or < 0 || (n == 3 && !(Om > 0))) st = ST_INVALID;
+    const bool finite = isfinite(r.H0) && isfinite(Om) && isfinite(OL) && isfinite(Or) && isfinite(Ok) &&
+                        isfinite(Os) && isfinite(Ox);
+    const int n = Or > 0 ? 4 : 3;
+    r.quartic = n == 4;
+    r.cpair = 0;
+    if (!finite || !(r.H0 > 0) || Or < 0 || (n == 3 && !(Om > 0))) st = ST_INVALID;
     cd z[4];
     double alpha[5] = {OL, Ox, Ok + Os, Om, Or};
     double an = alpha[n];
     double c[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     c[n] = 1.0;
     if (st == ST_OK) {
-        const double ian = ddiv(1.0, an);
+        const double ian = an < 1e-280 ? ddiv(1.0, an) : rcp_(an);
         for (int k = 0; k <= n; k++) c[k] = alpha[k] * ian;
         c[n] = 1.0;
     }
@@ -408,17 +529,19 @@ template <int G> __device__ int prep_one(const double* p, int ncol, double* rec,
     // tangent slots of such a row are NaN (no gradient).
     const double dtol = 8.0 * 2.220446049250313e-16 * (fabs(Om) + fabs(Or) + fabs(OL) + fabs(Ok) + 1.0);
     const bool triple0 = st == ST_OK && fabs(OL) <= dtol && fabs(Ox) <= dtol && fabs(Ok + Os) <= dtol;
-    group_roots<G>(c, alpha, n, active && st == ST_OK && !triple0, z);   // every lane, outside any divergent branch
+    group_roots<G>(c, alpha, n, active && st == ST_OK && !triple0, near, z);   // every lane, outside any divergent branch
     if (triple0) {
         z[0] = cmk(n == 4 ? -Om / Or : 0.0, 0.0);
         for (int i = 1; i < 4; i++) z[i] = cmk(0.0, 0.0);
     }
     if (st == ST_OK) {
-        // classification: real when the imaginary part is negligible
+        // classification: real when the imaginary part is negligible (compared
+        // in single precision; other comparisons on the bits: a double's
+        // comparison holds the FP64 pipe like any other FP64 instruction)
         int nreal = 0, ir[4], ic[4], ncx = 0;
         #pragma unroll 1
         for (int i = 0; i < n; i++) {
-            if (triple0 || fabs(z[i].im) <= 1e-12 * cabs_(z[i])) {   // (polished on the axis already)
+            if (triple0 || negligible_im(z[i])) {   // (polished on the axis already)
                 z[i].im = 0;
                 ir[nreal++] = i;
             }
@@ -426,169 +549,222 @@ template <int G> __device__ int prep_one(const double* p, int ncol, double* rec,
         }
         #pragma unroll 1
         for (int i = 0; i < nreal; i++)
-            if (z[ir[i]].re >= 1.0) st = ST_NO_BIG_BANG;   // real root at z >= 0 (Sec. 3, Fig. 1)
+            if (__double_as_longlong(z[ir[i]].re) >= __double_as_longlong(1.0)) st = ST_NO_BIG_BANG;   // real root at z >= 0 (Sec. 3, Fig. 1)
         // order reals by decreasing |rho| (fn15: largest roots of E^2(z+1))
         #pragma unroll 1
         for (int i = 0; i < nreal; i++)
             for (int j = i + 1; j < nreal; j++)
-                if (fabs(z[ir[j]].re) > fabs(z[ir[i]].re)) { int t = ir[i]; ir[i] = ir[j]; ir[j] = t; }
-        cd A, Bv, P1, P2;
+                if ((__double_as_longlong(z[ir[j]].re) & INT64_MAX) > (__double_as_longlong(z[ir[i]].re) & INT64_MAX)) { int t = ir[i]; ir[i] = ir[j]; ir[j] = t; }
+        cd A = cmk(0, 0), Bv = cmk(0, 0), P1 = cmk(0, 0), P2 = cmk(0, 0);
         bool cpair = false;
         if (n == 4 && nreal == 2 && ncx == 2) {
-            kind = 0; A = z[ir[0]]; Bv = z[ir[1]]; cpair = true;
+            A = z[ir[0]]; Bv = z[ir[1]]; cpair = true;
             P1 = z[ic[0]].im > 0 ? z[ic[0]] : z[ic[1]];
             P1.im = 0.5 * (fabs(z[ic[0]].im) + fabs(z[ic[1]].im));
             P1.re = 0.5 * (z[ic[0]].re + z[ic[1]].re);
         } else if (n == 4 && nreal == 4) {
-            kind = 1; A = z[ir[0]]; Bv = z[ir[1]]; P1 = z[ir[2]]; P2 = z[ir[3]];
+            A = z[ir[0]]; Bv = z[ir[1]]; P1 = z[ir[2]]; P2 = z[ir[3]];
         } else if (n == 3 && nreal == 1 && ncx == 2) {
-            kind = 2; A = z[ir[0]]; Bv = cmk(0, 0); cpair = true;
+            Bv = z[ir[0]]; cpair = true;
             P1 = z[ic[0]].im > 0 ? z[ic[0]] : z[ic[1]];
             P1.im = 0.5 * (fabs(z[ic[0]].im) + fabs(z[ic[1]].im));
             P1.re = 0.5 * (z[ic[0]].re + z[ic[1]].re);
         } else if (n == 3 && nreal == 3) {
-            kind = 3; A = z[ir[0]]; Bv = cmk(0, 0); P1 = z[ir[1]]; P2 = z[ir[2]];
+            Bv = z[ir[0]]; P1 = z[ir[1]]; P2 = z[ir[2]];
         } else if (st == ST_OK) {
             st = ST_UNSUPPORTED;   // e.g. two complex pairs (no real root)
         }
-        if (st == ST_OK || st == ST_NO_BIG_BANG) {
-            // roots in x = 1+z for the derivatives; stored in z
-            cd rho[4];
-            int nr = 0;
-            rho[nr++] = A;
-            if (n == 4) rho[nr++] = Bv;
-            rho[nr++] = P1;
-            rho[nr++] = cpair ? cmk(P1.re, -P1.im) : P2;
-            if (A.re == 0.0 && !triple0) st = st == ST_OK ? ST_DEGENERATE : st;   // division by rho_A in eq. (3.8)
-            rec[RF_A] = A.re - 1.0;
-            rec[RF_B] = (n == 4 ? Bv.re : 1.0) - 1.0;
-            if (cpair) { rec[RF_PRE] = P1.re - 1.0; rec[RF_PIM] = P1.im; }
-            else { rec[RF_PRE] = P1.re - 1.0; rec[RF_PIM] = P2.re - 1.0; }
-            rec[RF_YA] = sqrt(-rec[RF_A]);
-            rec[RF_YB] = sqrt(-rec[RF_B]);
-            if (cpair) { cd y = csqrt_(cmk(-rec[RF_PRE], -rec[RF_PIM])); rec[RF_YPRE] = y.re; rec[RF_YPIM] = y.im; }
-            else { rec[RF_YPRE] = sqrt(-rec[RF_PRE]); rec[RF_YPIM] = sqrt(-rec[RF_PIM]); }
-            // App. A (eqs. A.2-A.4): d rho_j / d c_i = -rho_j^i / prod_{m != j} (rho_j - rho_m).
-            // Summed over the coefficients c_i = alpha_i / alpha_n of the monic
-            // polynomial this is
-            //   d rho_j / d theta_k = -(dE^2/dtheta_k)(rho_j) / (alpha_n prod_{m != j} (rho_j - rho_m)),
-            // with dE^2/dOm = x^3, dE^2/dOL = 1, dE^2/dOr = x^4, dE^2/dOk = dE^2/dOs = x^2,
-            // dE^2/dOx = x, and -x^2 added to the first three under the closure.
-            // With G lanes per cosmology, lane j of the group takes root j and
-            // the group exchanges the results (the G lanes of a group take the
-            // same branches: one cosmology).
-            cd dr[4][RF_KT];
-            const int sg = G > 1 ? (int)(threadIdx.x & (G - 1)) : 0;
-            int degen = 0;
+        if (st != ST_OK && st != ST_NO_BIG_BANG) return st;
+        labelled = true;
+        r.cpair = cpair;
+        r.A = A.re;
+        r.B = Bv.re;
+        r.pr = P1.re;
+        r.pi = cpair ? P1.im : P2.re;
+        // division by rho_A in eq. (3.8)
+        if (n == 4 && A.re == 0.0 && !triple0) st = st == ST_OK ? ST_DEGENERATE : st;
+        if (n == 3 && Bv.re == 0.0 && !triple0) st = st == ST_OK ? ST_DEGENERATE : st;
+        cd rho[4];
+        int nr = 0;
+        if (n == 4) rho[nr++] = A;
+        rho[nr++] = Bv;
+        rho[nr++] = P1;
+        rho[nr++] = cpair ? cmk(P1.re, -P1.im) : P2;
+        int degen = 0;
+        if (!tangents) {
+            // (two equal labelled roots: the reduction's differences vanish)
             #pragma unroll 1
-            for (int j = 0; j < nr; j++) {
-                if (G > 1 && j != sg) continue;
-                const cd x = rho[j], x2 = cmul(x, x);
-                cd e2p = cmk(an, 0);
-                #pragma unroll 1
-                for (int m2 = 0; m2 < nr; m2++)
-                    if (m2 != j) e2p = cmul(e2p, csub(x, rho[m2]));
-                const bool degenerate = e2p.re == 0 && e2p.im == 0;
-                if (degenerate) degen = 1;
-                const cd inv = degenerate ? cmk(nan(""), nan("")) : crcp(e2p);
-                const cd x3 = cmul(x2, x);
-                const cd cx2 = ncol == 4 ? x2 : cmk(0, 0);
-                #pragma unroll 1
-                for (int k = 0; k < K; k++) {
-                    const cd g = k == 0 ? csub(x3, cx2) : k == 1 ? csub(cmk(1, 0), cx2)
-                               : k == 2 ? csub(cmul(x3, x), cx2) : k == 5 ? x : x2;
-                    cd d = cmul(g, inv);
-                    dr[j][k] = cmk(-d.re, -d.im);
-                    if (n == 3 && k == 2) dr[j][k] = cmk(nan(""), nan(""));  // no Or direction in a cubic
-                }
+            for (int j = 0; j < nr; j++)
+                for (int m2 = 0; m2 < j; m2++)
+                    if (rho[j].re == rho[m2].re && rho[j].im == rho[m2].im) degen = 1;
+            if (degen && !triple0) st = (st == ST_OK) ? ST_DEGENERATE : st;
+            return st;
+        }
+        // App. A (eqs. A.2-A.4): d rho_j / d c_i = -rho_j^i / prod_{m != j} (rho_j - rho_m).
+        // Summed over the coefficients c_i = alpha_i / alpha_n of the monic
+        // polynomial this is
+        //   d rho_j / d theta_k = -(dE^2/dtheta_k)(rho_j) / (alpha_n prod_{m != j} (rho_j - rho_m)),
+        // with dE^2/dOm = x^3, dE^2/dOL = 1, dE^2/dOr = x^4, dE^2/dOk = dE^2/dOs = x^2,
+        // dE^2/dOx = x, and -x^2 added to the first three under the closure.
+        // With G lanes per cosmology, lane j of the group takes root j and
+        // the group exchanges the results (the G lanes of a group take the
+        // same branches: one cosmology).
+        const int sg = G > 1 ? (int)(threadIdx.x & (G - 1)) : 0;
+        cd mine[RF_KT];
+        #pragma unroll
+        for (int k = 0; k < RF_KT; k++) mine[k] = cmk(0, 0);
+        #pragma unroll 1
+        for (int j = 0; j < nr; j++) {
+            if (G > 1 && j != sg) continue;
+            const cd x = rho[j];
+            cd e2p = cmk(-an, 0);
+            #pragma unroll 1
+            for (int m2 = 0; m2 < nr; m2++)
+                if (m2 != j) e2p = cmul(e2p, csub(x, rho[m2]));
+            const bool degenerate = e2p.re == 0 && e2p.im == 0;
+            if (degenerate) degen = 1;
+            // inv = -1 / (alpha_n prod), y = x^2 inv
+            const double ie = rcp_(cnorm(e2p));
+            const cd inv = degenerate ? cmk(nan(""), nan("")) : cmk(e2p.re * ie, -(e2p.im * ie));
+            const cd y = cmul(x, cmul(x, inv));
+            if (ncol == 4) {
+                // x^3 - x^2 = x^2 (x-1), 1 - x^2 = -(x-1)(x+1), x^4 - x^2 = x^2 (x-1)(x+1)
+                const cd u = cmk(x.re - 1.0, x.im), t = cmul(u, cmk(x.re + 1.0, x.im)), w = cmul(t, inv);
+                mine[0] = cmul(y, u);
+                mine[1] = cmk(-w.re, -w.im);
+                mine[2] = cmul(y, t);
+            } else {
+                const cd y3 = cmul(y, x);
+                mine[0] = y3;
+                mine[1] = inv;
+                mine[2] = cmul(y3, x);
+                mine[3] = y;
+                mine[4] = y;
+                mine[5] = cmul(x, inv);
             }
-            if (G > 1) {
-                const unsigned gmask = ((1u << G) - 1) << ((threadIdx.x & 31) & ~(G - 1));
-                #pragma unroll
-                for (int o = 1; o < G; o <<= 1) degen |= __shfl_xor_sync(gmask, degen, o, G);
+            if (n == 3) mine[2] = cmk(nan(""), nan(""));  // no Or direction in a cubic
+            if (G == 1)
+                for (int k = 0; k < K; k++) dr[j][k] = mine[k];
+        }
+        if (G > 1) {
+            const unsigned gmask = ((1u << G) - 1) << ((threadIdx.x & 31) & ~(G - 1));
+            #pragma unroll
+            for (int o = 1; o < G; o <<= 1) degen |= __shfl_xor_sync(gmask, degen, o, G);
+            if (tangents == 1) {
+                // transposed: at step d lane l reads lane l + d's direction l
+                #pragma unroll 1
+                for (int h = 0; h < K; h += G)
+                    #pragma unroll 1
+                    for (int d = 0; d < G; d++) {
+                        const int from = (sg + d) & (G - 1), give = h + ((sg - d) & (G - 1));
+                        const cd v = give < K ? mine[give] : cmk(0, 0);
+                        const cd g = cmk(__shfl_sync(gmask, v.re, from, G), __shfl_sync(gmask, v.im, from, G));
+                        if (h + sg < K) dr[from][h + sg] = g;
+                    }
+            } else {
                 #pragma unroll 1
                 for (int j = 0; j < nr; j++)
                     #pragma unroll 1
-                    for (int k = 0; k < K; k++) {
-                        dr[j][k].re = __shfl_sync(gmask, dr[j][k].re, j, G);
-                        dr[j][k].im = __shfl_sync(gmask, dr[j][k].im, j, G);
-                    }
+                    for (int k = 0; k < K; k++)
+                        dr[j][k] = cmk(__shfl_sync(gmask, mine[k].re, j, G), __shfl_sync(gmask, mine[k].im, j, G));
             }
-            if (degen && !triple0) st = (st == ST_OK) ? ST_DEGENERATE : st;
-            // big-root quantities of the quartic, scaled by lam = Or (see quartic_integrals)
-            if (n == 4) {
-                double rA = A.re;                  // rho_A
-                rec[RF_LAM] = Or;
-                rec[RF_AA] = -Or * (rA - 1.0);
-                rec[RF_MA] = Or * rA;
-                const double irA = ddiv(1.0, rA);
-                rec[RF_EPSA] = -irA;
-                rec[RF_RHOA] = rA;
-                // Tangents of m_A = lam rho_A = y from the scaled quartic
-                //   F(y) = y^4 + Om y^3 + (Ok + Os) Or y^2 + Ox Or^2 y + OL Or^3 = Or^3 E^2(rho_A) = 0,
-                // dy = -(dF/dtheta) / (dF/dy), a ratio of O(1) terms: in the Or
-                // direction rho_A d lam and lam d rho_A are each O(Om/Or) and cancel.
-                // a_A = -lam (rho_A - 1) = -y + lam.
-                const double y = Or * rA, Oks = Ok + Os;
-                const double iFy = ddiv(1.0, y * y * (4.0 * y + 3.0 * Om) + 2.0 * Oks * Or * y + Ox * Or * Or);
-                const double cl = ncol == 4 ? 1.0 : 0.0, FOk = Or * y * y;
-                const double Fth[RF_KT] = {y * y * y - cl * FOk, Or * Or * Or - cl * FOk,
-                                           Oks * y * y + 2.0 * Ox * Or * y + 3.0 * OL * Or * Or - cl * FOk, FOk, FOk,
-                                           Or * Or * y};
-                #pragma unroll 1
-                for (int k = 0; k < K; k++) {
-                    double dl = (k == 2) ? 1.0 : 0.0, dA = dr[0][k].re;
-                    const double dy = -Fth[k] * iFy;
-                    rec[RF_DLAM + k] = dl;
-                    rec[RF_DAA + k] = dl - dy;
-                    rec[RF_DMA + k] = dy;
-                    rec[RF_DEPSA + k] = dA * (irA * irA);
-                    rec[RF_DRHOA + k] = dA;
-                }
-            }
-            // q_j = -1/r_j (dq_j = dr_j / r_j^2) for the normalised Carlson arguments
-            {
-                double rA = A.re - 1.0;
-                const double iA = rA != 0.0 ? ddiv(1.0, rA) : 0.0;
-                rec[RF_QA] = -iA;
-                for (int k = 0; k < K; k++) rec[RF_DQA + k] = dr[0][k].re * (iA * iA);
-                if (n == 4) {
-                    double rB = Bv.re - 1.0;
-                    const double iB = rB != 0.0 ? ddiv(1.0, rB) : 0.0;
-                    rec[RF_QB] = -iB;
-                    for (int k = 0; k < K; k++) rec[RF_DQB + k] = dr[1][k].re * (iB * iB);
-                }
-                const int jq = n == 4 ? 2 : 1;
-                if (cpair) {
-                    cd r = cmk(P1.re - 1.0, P1.im);
-                    cd q = cdiv(cmk(-1.0, 0.0), r);
-                    rec[RF_QPRE] = q.re;
-                    rec[RF_QPIM] = q.im;
-                    const cd q2 = cmul(q, q);   // dq = dr / r^2 = q^2 dr
-                    for (int k = 0; k < K; k++) {
-                        cd dq = cmul(dr[jq][k], q2);
-                        rec[RF_DQPRE + k] = dq.re;
-                        rec[RF_DQPIM + k] = dq.im;
-                    }
-                } else {
-                    double r1 = P1.re - 1.0, r2 = P2.re - 1.0;
-                    const double i1 = r1 != 0.0 ? ddiv(1.0, r1) : 0.0, i2 = r2 != 0.0 ? ddiv(1.0, r2) : 0.0;
-                    rec[RF_QPRE] = -i1;
-                    rec[RF_QPIM] = -i2;
-                    for (int k = 0; k < K; k++) {
-                        rec[RF_DQPRE + k] = dr[jq][k].re * (i1 * i1);
-                        rec[RF_DQPIM + k] = dr[jq + 1][k].re * (i2 * i2);
-                    }
-                }
-            }
+        }
+        if (degen && !triple0) st = (st == ST_OK) ? ST_DEGENERATE : st;
+    }
+    return st;
+}
+
+// The record of the X-tangent kernel (RecField) from the labelled roots.
+__device__ __noinline__ void legacy_record(const RowRoots& r, const cd (*dr)[RF_KT], bool labelled, double* rec) {
+    const double H0 = r.H0, Om = r.Om, OL = r.OL, Or = r.Or, Ok = r.Ok, Os = r.Os, Ox = r.Ox;
+    const int ncol = r.ncol, K = ncol - 1, n = r.quartic ? 4 : 3;
+    const bool cpair = r.cpair;
+    // slot A of this record is the cubic's only special root
+    const cd A = cmk(r.quartic ? r.A : r.B, 0.0), Bv = cmk(r.quartic ? r.B : 0.0, 0.0);
+    const cd P1 = cmk(r.pr, cpair ? r.pi : 0.0), P2 = cmk(cpair ? 0.0 : r.pi, 0.0);
+    for (int i = 0; i < NREC; i++) rec[i] = 0;
+    if (labelled) {
+        rec[RF_A] = A.re - 1.0;
+        rec[RF_B] = (n == 4 ? Bv.re : 1.0) - 1.0;
+        if (cpair) { rec[RF_PRE] = P1.re - 1.0; rec[RF_PIM] = P1.im; }
+        else { rec[RF_PRE] = P1.re - 1.0; rec[RF_PIM] = P2.re - 1.0; }
+        rec[RF_YA] = sqrt(-rec[RF_A]);
+        rec[RF_YB] = sqrt(-rec[RF_B]);
+        if (cpair) { cd y = csqrt_(cmk(-rec[RF_PRE], -rec[RF_PIM])); rec[RF_YPRE] = y.re; rec[RF_YPIM] = y.im; }
+        else { rec[RF_YPRE] = sqrt(-rec[RF_PRE]); rec[RF_YPIM] = sqrt(-rec[RF_PIM]); }
+        // big-root quantities of the quartic, scaled by lam = Or (see quartic_integrals)
+        if (n == 4) {
+            double rA = A.re;                  // rho_A
+            rec[RF_LAM] = Or;
+            rec[RF_AA] = -Or * (rA - 1.0);
+            rec[RF_MA] = Or * rA;
+            const double irA = ddiv(1.0, rA);
+            rec[RF_EPSA] = -irA;
+            rec[RF_RHOA] = rA;
+            // Tangents of m_A = lam rho_A = y from the scaled quartic
+            //   F(y) = y^4 + Om y^3 + (Ok + Os) Or y^2 + Ox Or^2 y + OL Or^3 = Or^3 E^2(rho_A) = 0,
+            // dy = -(dF/dtheta) / (dF/dy), a ratio of O(1) terms: in the Or
+            // direction rho_A d lam and lam d rho_A are each O(Om/Or) and cancel.
+            // a_A = -lam (rho_A - 1) = -y + lam.
+            const double y = Or * rA, Oks = Ok + Os;
+            const double iFy = ddiv(1.0, y * y * (4.0 * y + 3.0 * Om) + 2.0 * Oks * Or * y + Ox * Or * Or);
+            const double cl = ncol == 4 ? 1.0 : 0.0, FOk = Or * y * y;
+            const double Fth[RF_KT] = {y * y * y - cl * FOk, Or * Or * Or - cl * FOk,
+                                       Oks * y * y + 2.0 * Ox * Or * y + 3.0 * OL * Or * Or - cl * FOk, FOk, FOk,
+                                       Or * Or * y};
             #pragma unroll 1
             for (int k = 0; k < K; k++) {
-                rec[RF_DA + k] = dr[0][k].re;
-                rec[RF_DB + k] = n == 4 ? dr[1][k].re : 0.0;
-                int jp = n == 4 ? 2 : 1;
-                if (cpair) { rec[RF_DPRE + k] = dr[jp][k].re; rec[RF_DPIM + k] = dr[jp][k].im; }
-                else { rec[RF_DPRE + k] = dr[jp][k].re; rec[RF_DPIM + k] = dr[jp + 1][k].re; }
+                double dl = (k == 2) ? 1.0 : 0.0, dA = dr[0][k].re;
+                const double dy = -Fth[k] * iFy;
+                rec[RF_DLAM + k] = dl;
+                rec[RF_DAA + k] = dl - dy;
+                rec[RF_DMA + k] = dy;
+                rec[RF_DEPSA + k] = dA * (irA * irA);
+                rec[RF_DRHOA + k] = dA;
             }
+        }
+        // q_j = -1/r_j (dq_j = dr_j / r_j^2) for the normalised Carlson arguments
+        {
+            double rA = A.re - 1.0;
+            const double iA = rA != 0.0 ? ddiv(1.0, rA) : 0.0;
+            rec[RF_QA] = -iA;
+            for (int k = 0; k < K; k++) rec[RF_DQA + k] = dr[0][k].re * (iA * iA);
+            if (n == 4) {
+                double rB = Bv.re - 1.0;
+                const double iB = rB != 0.0 ? ddiv(1.0, rB) : 0.0;
+                rec[RF_QB] = -iB;
+                for (int k = 0; k < K; k++) rec[RF_DQB + k] = dr[1][k].re * (iB * iB);
+            }
+            const int jq = n == 4 ? 2 : 1;
+            if (cpair) {
+                cd r = cmk(P1.re - 1.0, P1.im);
+                cd q = cdiv(cmk(-1.0, 0.0), r);
+                rec[RF_QPRE] = q.re;
+                rec[RF_QPIM] = q.im;
+                const cd q2 = cmul(q, q);   // dq = dr / r^2 = q^2 dr
+                for (int k = 0; k < K; k++) {
+                    cd dq = cmul(dr[jq][k], q2);
+                    rec[RF_DQPRE + k] = dq.re;
+                    rec[RF_DQPIM + k] = dq.im;
+                }
+            } else {
+                double r1 = P1.re - 1.0, r2 = P2.re - 1.0;
+                const double i1 = r1 != 0.0 ? ddiv(1.0, r1) : 0.0, i2 = r2 != 0.0 ? ddiv(1.0, r2) : 0.0;
+                rec[RF_QPRE] = -i1;
+                rec[RF_QPIM] = -i2;
+                for (int k = 0; k < K; k++) {
+                    rec[RF_DQPRE + k] = dr[jq][k].re * (i1 * i1);
+                    rec[RF_DQPIM + k] = dr[jq + 1][k].re * (i2 * i2);
+                }
+            }
+        }
+        #pragma unroll 1
+        for (int k = 0; k < K; k++) {
+            rec[RF_DA + k] = dr[0][k].re;
+            rec[RF_DB + k] = n == 4 ? dr[1][k].re : 0.0;
+            int jp = n == 4 ? 2 : 1;
+            if (cpair) { rec[RF_DPRE + k] = dr[jp][k].re; rec[RF_DPIM + k] = dr[jp][k].im; }
+            else { rec[RF_DPRE + k] = dr[jp][k].re; rec[RF_DPIM + k] = dr[jp + 1][k].re; }
         }
     }
     // prefactors: alpha_m^-1/2 (Or for the quartic, Om for the cubic, eq. 3.2 / fn13)
@@ -599,7 +775,7 @@ template <int G> __device__ int prep_one(const double* p, int ncol, double* rec,
     const double iH0 = ddiv(1.0, H0);
     rec[RF_DH] = LCDM_C_KMS * iH0;
     rec[RF_TH] = LCDM_HUBBLE_GYR * iH0;
-    rec[RF_KIND] = kind;
+    rec[RF_KIND] = n == 4 ? (cpair ? 0 : 1) : (cpair ? 2 : 3);
     // N = sqrt(E^2(0) / alpha_n): E^2(0) = Om + OL + Or + Ok (+ Os + Ox), exactly 1 under the closure
     const double S0 = ncol == 4 ? 1.0 : Om + OL + Or + Ok + Os + Ox;
     const double iOm = ddiv(1.0, Om);
@@ -620,39 +796,81 @@ template <int G> __device__ int prep_one(const double* p, int ncol, double* rec,
         if (n == 3 && k == 2) rec[RF_DAMH + k] = nan("");
         rec[RF_DOK + k] = ncol == 4 ? -1.0 : (k == 3 ? 1.0 : 0.0);
     }
-    return st;
 }
 
-// G lanes per cosmology (see group_roots); grad / loglike (optional): rows
-// initialised to 0 (NaN for a bad status).  Launched with 32-thread blocks
+// The core's record of one cosmology: lane 0 of the group writes the values,
+// lane k mod G the tangents of direction k.
+template <int G, class T>
+__device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, bool absorb, bool tangents, T* rec) {
+    if (lane == 0) {
+        core_values<T>(r, absorb, rec);
+        const double iH0 = r.H0 < 1e-280 ? ddiv(1.0, r.H0) : rcp_(r.H0);
+        put(rec, C_DH, LCDM_C_KMS * iH0);
+        put(rec, C_TH, LCDM_HUBBLE_GYR * iH0);
+        put(rec, C_H0, r.H0);
+    }
+    if (!tangents) return;
+    const int b = r.quartic ? 1 : 0;
+    #pragma unroll 1
+    for (int k = lane; k < r.ncol - 1; k += G)
+        core_tangent<T>(r, k, dr[0][k].re, dr[b][k].re, dr[b + 1][k].re, r.cpair ? dr[b + 1][k].im : dr[b + 2][k].re,
+                        rec);
+}
+
+struct PrepArgs {
+    const double* params;   // [B][ncol]
+    int64_t B;
+    int ncol;
+    int tangents;           // the root derivatives are needed
+    int absorb;             // the absorption distance's constants are needed
+    double* recD;           // [B][NREC] record of the X-tangent kernel, and its (hi, lo) copy (optional)
+    float2* recF;
+    float* coreF;           // [B][NCORE] record of the core, single or double precision (optional)
+    double* coreD;
+    int32_t* status;
+    double* grad;           // [B][ncol], [B]: initialised to 0 (NaN for a bad status), optional
+    double* loglike;
+};
+
+// G lanes per cosmology (see group_roots).  Launched with 32-thread blocks
 // over G B threads.
-template <int G>
-__global__ void prep_kernel(const double* __restrict__ params, int64_t B, int ncol, double* __restrict__ recD,
-                            float2* __restrict__ recF, int32_t* __restrict__ status, double* __restrict__ grad,
-                            double* __restrict__ loglike) {
+template <int G> __global__ void prep_kernel(PrepArgs a) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t b = t / G;
     const int j = (int)(t % G);
-    const bool inb = b < B;
+    const bool inb = b < a.B;
+    const int ncol = a.ncol;
     // lanes past the end work on a copy of the last row and write nothing
-    const double* prow = params + (inb ? b : B - 1) * ncol;
-    double rec[NREC];
-    const int st = prep_one<G>(prow, ncol, rec, inb);
+    const double* prow = a.params + (inb ? b : a.B - 1) * ncol;
+    RowRoots r;
+    cd dr[4][RF_KT];
+    bool labelled;
+    const int st = prep_roots<G>(prow, ncol, inb, a.tangents ? (a.recD ? 2 : 1) : 0, a.coreF ? 0.01f : 0.1f, r, dr,
+                                 labelled);
     if (!inb) return;
-    double* rd = recD + b * NREC;
-    float2* rf = recF + b * NREC;
-    #pragma unroll 1
-    for (int i = j; i < NREC; i += G) {
-        rd[i] = rec[i];
-        float h = (float)rec[i];
-        rf[i] = make_float2(h, (float)(rec[i] - (double)h));
+    if (a.recD) {
+        double rec[NREC];
+        legacy_record(r, dr, labelled, rec);
+        double* rd = a.recD + b * NREC;
+        float2* rf = a.recF + b * NREC;
+        #pragma unroll 1
+        for (int i = j; i < NREC; i += G) {
+            rd[i] = rec[i];
+            float h = (float)rec[i];
+            rf[i] = make_float2(h, (float)(rec[i] - (double)h));
+        }
+    }
+    if (st == ST_OK && (a.coreF || a.coreD)) {
+        r.finish();
+        if (a.coreF) write_core<G, float>(r, dr, j, a.absorb, a.tangents, a.coreF + b * NCORE);
+        else write_core<G, double>(r, dr, j, a.absorb, a.tangents, a.coreD + b * NCORE);
     }
     if (j != 0) return;
-    status[b] = st;
+    a.status[b] = st;
     double init = st == ST_OK ? 0.0 : nan("");
-    if (grad)
-        for (int k = 0; k < ncol; k++) grad[b * ncol + k] = init;
-    if (loglike) loglike[b] = init;
+    if (a.grad)
+        for (int k = 0; k < ncol; k++) a.grad[b * ncol + k] = init;
+    if (a.loglike) a.loglike[b] = init;
 }
 
 }  // namespace lcdm
