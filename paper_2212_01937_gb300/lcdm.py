@@ -10,6 +10,7 @@ Precision ``"fp32"`` (LCDM_FP32_MIXED: float32 I/O and per-pair arithmetic,
 FP64 root preparation and reductions) or ``"fp64"``.
 """
 import ctypes
+import functools
 import os
 
 import torch
@@ -92,7 +93,27 @@ def _ptr(t):
 
 
 def _stream(device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    # the raw handle: a Stream object costs as much host time as a launch
+    index = device.index if device.index is not None else torch.cuda.current_device()
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(index))
+
+
+def _as(t, dtype, device):
+    """t with the given type and device, contiguous (t itself where it is: a
+    call of .to() that has nothing to do still costs microseconds)."""
+    if t.dtype is not dtype or t.device != device:
+        t = t.to(device=device, dtype=dtype)
+    return t if t.is_contiguous() else t.contiguous()
+
+
+@functools.lru_cache(maxsize=256)
+def _workspace_bytes(B, ncol, precision, layout, deterministic):
+    """lcdm_workspace_size: a function of its arguments alone (but for the
+    deterministic mode, whose part depends on the current device)."""
+    nbytes = ctypes.c_size_t()
+    opts = Opts(ncol, precision, layout, 0, 0, 0, deterministic)
+    _check(load().lcdm_workspace_size(B, ctypes.byref(opts), ctypes.byref(nbytes)))
+    return nbytes.value
 
 
 def launch_count():
@@ -128,23 +149,24 @@ class Call:
 
     def __init__(self, params, z, offsets=None, layout=None, precision="fp32", block=0, blocks_per_sm=0,
                  workspace=None, lane_map="tuned", deterministic=False):
-        lib = load()
         if not params.is_cuda:
             raise ValueError("params must be a CUDA tensor")
         self.device = params.device
-        self.params = params.to(torch.float64).contiguous()
+        self.params = _as(params, torch.float64, self.device)
         self.B, ncol = self.params.shape
         if layout is None:
             layout = "csr" if offsets is not None else "dense"
         self.layout = layout
         self.precision = precision
         self.dtype = torch.float64 if precision == "fp64" else torch.float32
-        self.z = z.to(device=self.device, dtype=self.dtype).contiguous().reshape(-1)
+        self.z = _as(z, self.dtype, self.device)
+        if self.z.dim() != 1:
+            self.z = self.z.reshape(-1)
         self.offsets = None
         if layout == "csr":
             if offsets is None:
                 raise ValueError("csr layout needs offsets")
-            self.offsets = offsets.to(device=self.device, dtype=torch.int64).contiguous()
+            self.offsets = _as(offsets, torch.int64, self.device)
             self.n = self.z.numel()
             self.npairs = self.n
         elif layout == "dense":
@@ -157,12 +179,12 @@ class Call:
             self.npairs = self.B * self.n
         self.opts = Opts(ncol, PRECISION[precision], LAYOUT[layout], block, blocks_per_sm, LANE_MAP[lane_map],
                          1 if deterministic else 0)
-        nbytes = ctypes.c_size_t()
-        _check(lib.lcdm_workspace_size(self.B, ctypes.byref(self.opts), ctypes.byref(nbytes)))
-        if workspace is not None and workspace.numel() >= nbytes.value:
+        size = _workspace_bytes.__wrapped__ if deterministic else _workspace_bytes
+        nbytes = size(self.B, ncol, PRECISION[precision], LAYOUT[layout], 1 if deterministic else 0)
+        if workspace is not None and workspace.numel() >= nbytes:
             self.ws = workspace
         else:
-            self.ws = torch.empty(nbytes.value, dtype=torch.uint8, device=self.device)
+            self.ws = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
         self.ws_bytes = self.ws.numel()
         self.status = torch.empty(self.B, dtype=torch.int32, device=self.device)
 
@@ -229,7 +251,7 @@ def distances_vjp(params, z, cot, offsets=None, outputs=(), call=None, grad_z=Fa
     (lcdm_distances_vjp_dz; ``workspace`` as for gauss_loglike)."""
     c = call if call is not None else Call(params, z, offsets, **kw)
     out, vp = c.out_buffers(outputs)
-    cots = {n: v.to(device=c.device, dtype=c.dtype).contiguous() for n, v in cot.items() if v is not None}
+    cots = {n: _as(v, c.dtype, c.device) for n, v in cot.items() if v is not None}
     cp = _VP6(*[(cots[n].data_ptr() if n in cots else None) for n in OUTS])
     grad = torch.empty(c.B, c.ncol, dtype=torch.float64, device=c.device)
     if grad_z:
@@ -409,20 +431,26 @@ class Distances(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, params, z, offsets, outputs, layout, precision):
-        res = distances(params, z, offsets, outputs=outputs, layout=layout, precision=precision)
-        ctx.save_for_backward(params, z, offsets if offsets is not None else torch.empty(0))
-        ctx.meta = (outputs, layout, precision, offsets is not None)
+        # an output that the loss does not use arrives in backward as None, not as
+        # a tensor of zeros: it adds no integral to the tangent kernel
+        ctx.set_materialize_grads(False)
+        # the double-precision rows are saved beside the parameters, so that
+        # backward does not convert them again
+        rows = _as(params, torch.float64, params.device)
+        res = distances(rows, z, offsets, outputs=outputs, layout=layout, precision=precision)
+        ctx.save_for_backward(params, z, offsets, None if rows is params else rows)
+        ctx.meta = (outputs, layout, precision)
         return tuple(res[n] for n in outputs)
 
     @staticmethod
     def backward(ctx, *grads):
-        params, z, offsets = ctx.saved_tensors
-        outputs, layout, precision, has_off = ctx.meta
+        params, z, offsets, rows = ctx.saved_tensors
+        outputs, layout, precision = ctx.meta
         cot = {n: g for n, g in zip(outputs, grads) if g is not None}
         want_z = ctx.needs_input_grad[1]
         if want_z and layout == "shared":
             raise ValueError("redshift gradients need the csr or dense layout")
-        res = distances_vjp(params, z, cot, offsets if has_off else None, layout=layout, precision=precision,
+        res = distances_vjp(params if rows is None else rows, z, cot, offsets, layout=layout, precision=precision,
                             grad_z=want_z)
         gz = res["grad_z"].reshape(z.shape).to(z.dtype) if want_z else None
         return res["grad"].to(params.dtype), gz, None, None, None, None
