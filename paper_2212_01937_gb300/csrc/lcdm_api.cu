@@ -10,7 +10,6 @@
 #include "lcdm_between.cuh"
 #include "lcdm_launch.cuh"
 #include "lcdm_prep.cuh"
-#include "lcdm_redshift.cuh"
 
 using namespace lcdm;
 
@@ -116,6 +115,7 @@ int log2_bucket(int64_t n) {
 struct Plan {
     PairArgs args;
     const void* core;       // the core's records
+    void* grad_z;           // [npairs] derivatives with respect to the redshifts, optional
     int legacy;             // the tangent launch is the X-tangent kernel's
     int absorb;             // the core's records need the absorption distance's constants
     int prec, K, wt, wx;
@@ -146,6 +146,7 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     a.recD = cv.recD;
     a.recF = cv.recF;
     P.core = cv.core;
+    P.grad_z = nullptr;
     a.part = cv.part;
     a.wrow = cv.wrow;
     a.det_cap = cv.part ? (int64_t)det_warps() : 0;
@@ -198,16 +199,18 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
 
 lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s);
 
-// index of the plan's kernel in its table (4 and up: per-pair Jacobians)
+// index of the plan's kernel in its table (4 and up: per-pair Jacobians, 8 and
+// up: with the redshift derivatives)
 int entry_index(const Plan& P) {
     bool jac = false;
     for (int i = 0; i < LCDM_NOUT; i++) jac = jac || P.args.jac[i];
+    if (P.grad_z && !P.wx && !P.legacy) return 8 + (P.wt ? 1 : 0);
     return (P.wt ? 2 : 0) + (P.wx ? 1 : 0) + (jac ? 4 : 0);
 }
 const PairsEntry& plan_entry(const Plan& P) {
     const int i = entry_index(P);
     const PairsTable& t = table(P.prec, P.K);
-    return i < 4 ? t.e[i] : t.jac[i - 4];
+    return i < 4 ? t.e[i] : i < 8 ? t.jac[i - 4] : t.dz[i - 8];
 }
 
 }  // namespace
@@ -242,6 +245,7 @@ lcdm_status launch_values(const Plan& P, int lane_map, cudaStream_t s) {
     Plan V = P;
     PairArgs& v = V.args;
     v.outmask = 0;
+    V.grad_z = nullptr;
     for (int i = 0; i < LCDM_NOUT; i++) {
         v.jac[i] = nullptr;
         v.cot[i] = nullptr;
@@ -261,13 +265,36 @@ lcdm_status launch_values(const Plan& P, int lane_map, cudaStream_t s) {
     std::get<4>(V.key) = V.wx;
     return launch_one(V, 0, 0, lane_map, s);
 }
+// The redshift derivatives alone: a value launch of chi without outputs.
+lcdm_status launch_dz(const Plan& P, int lane_map, cudaStream_t s) {
+    Plan D = P;
+    for (int i = 0; i < LCDM_NOUT; i++) D.args.out[i] = D.args.jac[i] = nullptr;
+    D.args.outmask = 0;
+    D.args.grad = nullptr;
+    D.K = D.legacy = D.wt = D.wx = D.split_mask = 0;
+    std::get<2>(D.key) = std::get<3>(D.key) = std::get<4>(D.key) = 0;
+    return launch_one(D, 0, 0, lane_map, s);
+}
+// The redshift derivatives come with the plan's main launch, unless that is
+// the X-tangent kernel or a value launch with t or X.
+bool separate_dz(const Plan& P) { return P.grad_z && (P.legacy || (P.K == 0 && (P.wt || P.wx))); }
 // The plan's main launch, without the outputs of split_mask.
 lcdm_status launch_main(const Plan& P, int block, int bps, int lane_map, cudaStream_t s) {
     Plan T = P;
+    if (separate_dz(P)) T.grad_z = nullptr;
     for (int i = 0; i < LCDM_NOUT; i++)
         if (P.split_mask & (1 << i)) { T.args.out[i] = nullptr; T.args.outmask &= ~(1 << i); }
     T.split_mask = 0;
     return launch_one(T, block, bps, lane_map, s);
+}
+
+lcdm_status launch_nan_rows(const Plan& P, cudaStream_t s) {
+    if (P.npairs == 0) return LCDM_OK;
+    const unsigned grid = (unsigned)((P.args.B * 32 + 127) / 128);
+    if (P.prec == 0) nan_rows_kernel<double><<<grid, 128, 0, s>>>(P.args, (double*)P.grad_z);
+    else nan_rows_kernel<float><<<grid, 128, 0, s>>>(P.args, (float*)P.grad_z);
+    g_launches++;
+    return cudaGetLastError() == cudaSuccess ? LCDM_OK : LCDM_ERR_CUDA;
 }
 
 // Resident blocks per SM of a pair kernel, queried once per (device, kernel,
@@ -315,7 +342,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     int64_t grid = (need_warps * 32 + block - 1) / block;
     if (grid < 1) grid = 1;
     if (P.npairs == 0) return LCDM_OK;
-    cudaError_t e = t.launch(P.args, P.core, (int)grid, block, s);
+    cudaError_t e = t.launch(P.args, P.core, P.grad_z, (int)grid, block, s);
     g_launches++;
     if (e != cudaSuccess) return LCDM_ERR_CUDA;
     if (P.args.part && (P.args.grad || P.args.loglike)) {
@@ -371,13 +398,18 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
 lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv,
                      int32_t* status, double* grad, double* loglike, int block, int bps, int lane_map, cudaStream_t s) {
     lcdm_status st;
-    if (P.split_mask || !P.legacy) {
+    const bool dz = separate_dz(P);
+    if (P.split_mask || dz || !P.legacy) {
         const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.absorb != 0};
         st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
         if (st != LCDM_OK) return st;
     }
     if (P.split_mask) {
         st = launch_values(P, lane_map, s);
+        if (st != LCDM_OK) return st;
+    }
+    if (dz) {
+        st = launch_dz(P, lane_map, s);
         if (st != LCDM_OK) return st;
     }
     if (P.legacy) {
@@ -679,39 +711,16 @@ lcdm_status lcdm_gauss_loglike_dz(const double* params, int64_t B, const int64_t
     const size_t es = opts->precision == LCDM_FP64 ? 8 : 4;
     Carved cv;
     carve(ws, ws_bytes, B, cv);
-    char* dC = (char*)ws + align256(ws_bytes_for(B));
-    char* mu = dC + align256((size_t)npairs * es);
-    if (mu_out) mu = (char*)mu_out;
-    void* out[LCDM_NOUT] = {dC, nullptr, nullptr, nullptr, nullptr, mu};
+    void* out[LCDM_NOUT] = {nullptr, nullptr, nullptr, nullptr, nullptr, mu_out};
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, nullptr, nullptr, m_obs, M, sigma, grad, loglike, cosmo_status,
                    opts, cv, P);
     if (st != LCDM_OK) return st;
+    P.grad_z = grad_z;
     st = run_plan(P, params, B, opts, cv, cosmo_status, grad, loglike, opts->block, opts->blocks_per_sm, opts->lane_map,
                   stream);
     if (st != LCDM_OK) return st;
-    DzArgs d;
-    d.params = params;
-    d.ncol = opts->ncol;
-    d.status = cosmo_status;
-    d.offsets = offsets;
-    d.layout = opts->layout;
-    d.nrow = n;
-    d.nnz = npairs;
-    d.B = B;
-    d.fp64 = opts->precision == LCDM_FP64;
-    d.z = z;
-    d.mobs = m_obs;
-    d.dC = dC;
-    d.mu = mu;
-    d.M = M;
-    d.sigma = sigma;
-    for (int i = 0; i < LCDM_NOUT; i++) d.cot[i] = nullptr;
-    d.vjp = 0;
-    d.grad_z = grad_z;
-    if (launch_loglike_dz(d, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-    g_launches++;
-    return LCDM_OK;
+    return launch_nan_rows(P, stream);
 }
 
 lcdm_status lcdm_distances_vjp_dz(const double* params, int64_t B, const int64_t* offsets, const void* z,
@@ -726,39 +735,19 @@ lcdm_status lcdm_distances_vjp_dz(const double* params, int64_t B, const int64_t
     size_t need = 0;
     lcdm_loglike_dz_workspace_size(B, n, opts, &need);
     if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < need) return LCDM_ERR_WORKSPACE;
-    const int64_t npairs = opts->layout == LCDM_LAYOUT_CSR ? n : B * n;
     Carved cv;
     carve(ws, ws_bytes, B, cv);
-    void* outk[LCDM_NOUT];
-    for (int i = 0; i < LCDM_NOUT; i++) outk[i] = out ? out[i] : nullptr;
-    if (!outk[LCDM_DC]) outk[LCDM_DC] = (char*)ws + align256(ws_bytes_for(B));   // d_C feeds the z-derivatives
     Plan P;
-    st = make_plan(params, B, offsets, z, n, outk, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad, nullptr,
+    st = make_plan(params, B, offsets, z, n, out, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad, nullptr,
                    cosmo_status, opts, cv, P);
     if (st != LCDM_OK) return st;
+    P.grad_z = grad_z;
+    if (!grad)   // values and redshift derivatives: the cotangents carry no parameter gradient
+        for (int i = 0; i < LCDM_NOUT; i++) P.args.cot[i] = cot[i];
     st = run_plan(P, params, B, opts, cv, cosmo_status, grad, nullptr, opts->block, opts->blocks_per_sm, opts->lane_map,
                   stream);
     if (st != LCDM_OK) return st;
-    DzArgs d;
-    memset(&d, 0, sizeof(d));
-    d.params = params;
-    d.ncol = opts->ncol;
-    d.status = cosmo_status;
-    d.offsets = offsets;
-    d.layout = opts->layout;
-    d.nrow = n;
-    d.nnz = npairs;
-    d.B = B;
-    d.fp64 = opts->precision == LCDM_FP64;
-    d.z = z;
-    d.dC = outk[LCDM_DC];
-    d.sigma = 1.0;
-    for (int i = 0; i < LCDM_NOUT; i++) d.cot[i] = cot[i];
-    d.vjp = 1;
-    d.grad_z = grad_z;
-    if (launch_loglike_dz(d, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-    g_launches++;
-    return LCDM_OK;
+    return launch_nan_rows(P, stream);
 }
 
 lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, double* chi_inf, double* t_inf,

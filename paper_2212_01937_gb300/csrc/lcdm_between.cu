@@ -224,9 +224,11 @@ template <bool GRAD> __global__ void __launch_bounds__(128) limits_kernel(LimitA
     double chi = nan, age = nan;
     int st = a.status[b];
     if (st == ST_OK) {
-        CorePair<double, true, false, GRAD, true> e;
+        typedef CorePair<double, true, false, GRAD, true> E;
+        E e;
+        typename E::Tape tape;
         int fail = 0;
-        e.forward(1.0, rec, &fail);
+        e.forward(1.0, rec, tape, &fail);
         const double s = a.scale[b], DH = rec[C_DH], tH = rec[C_TH];
         if (fail) {
             a.status[b] = st = ST_NOCONV;
@@ -236,8 +238,8 @@ template <bool GRAD> __global__ void __launch_bounds__(128) limits_kernel(LimitA
             if (GRAD) {
                 const double gc = a.cot_chi ? a.cot_chi[b] : 0.0, ga = a.cot_age ? a.cot_age[b] : 0.0;
                 double* g = a.gradp + b * 4;
-                g[0] = -(gc * chi + ga * age) / rec[C_H0];
-                e.reverse(gc * s * DH, ga * tH);
+                g[0] = -(gc * chi + ga * age) * rec[C_IH0];
+                e.reverse(gc * s * DH, ga * tH, tape);
                 for (int k = 0; k < 3; k++) g[1 + k] = e.along(k);
             }
         }

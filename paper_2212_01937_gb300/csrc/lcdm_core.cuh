@@ -44,7 +44,7 @@ enum CoreField {
     C_QA = 0, C_QB, C_QR, C_QRL,          // q_j = -1/r_j; the pair: real and imaginary part, or the two reals
     C_QI, C_QIL, C_C2, C_KIND,            // (QRL, QIL: low words in single precision); c2 = 2 / sqrt(S0);
                                           // KIND: 1 for a complex pair, 0 for two reals
-    C_DH, C_TH, C_H0, C_OK,
+    C_DH, C_TH, C_IH0, C_OK,              // c/H0 [Mpc], 1/H0 [Gyr], 1/H0, Omega_k0
     C_DF, C_B2, C_B3, C_B4,               // DF: max deviation / z^2 from the mean of three; series of R_F
     C_B5, C_B6, C_B7, C_RS,               // RS = -1 / (2 S0) with free S0, 0 under the closure
     C_DJ, C_EPS, C_K2, C_K3,              // DJ: max deviation from the mean of five (t track)
@@ -250,6 +250,16 @@ LCDM_HD Quad<double> quad(const double* p) {
 }
 
 // ------------------------------------------------------------------- core ---
+// The steps taken, for the reverse pass: s1, S and P of the duplication (sqrt(p)
+// of the t track), and R_C's a and b.  Apart from the pair's other state: it is
+// indexed by the step and lives in local memory (of which only the steps taken
+// are touched), where it would take everything in the same object with it (51
+// local loads and stores per pair instead of 8).
+template <class T, bool REV, bool WT> struct CoreTape {
+    enum { N = REV ? (int)CoreTol<T>::maxit : 1, NR = REV && WT ? (int)CoreTol<T>::maxit : 1, NQ = NR };
+    T s1[N], S[N], P[N], q[NQ], ra[NR], rb[NR];
+};
+
 // One pair.  WT: the time coordinate; WX: the absorption distance (values
 // only); REV: keep what the reverse pass needs; INF: the upper limit at
 // infinity.  There n_j / sqrt(z) -> sqrt(q_j), every u grows like z, and with
@@ -257,7 +267,7 @@ LCDM_HD Quad<double> quad(const double* p) {
 // and 1 + z q_j for q_j, and eq. (3.8)'s R_C has the factor (1 + eps) n_A (in
 // the radiationless case n_A = 0: that term falls off like z^-1/2).
 template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair {
-    enum { ND = REV ? (int)CoreTol<T>::maxit : 1, NR = REV && WT ? (int)CoreTol<T>::maxit : 1 };
+    typedef CoreTape<T, REV, WT> Tape;
     const T* rc;
     T z, zh, z2, h, cz;
     bool cplx, big;
@@ -271,13 +281,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     int mr;
     T U, sc, rcr, tr;
     T X;
-    T st1[ND], stS[ND], stP[ND], stq[ND];       // the sequence (local memory; only the steps taken are touched)
-    T ra[NR], rb[NR];
     T Ichi, It;
     // adjoints of the row's constants
     T qA_, qB_, qR_, qI_, bF_, eps_, k2_, k3_, bJ_;
 
-    LCDM_HD void forward(T zin, const T* rec, int* fail) {
+    LCDM_HD void forward(T zin, const T* rec, Tape& tape, int* fail) {
         rc = rec;
         z = zin;
         const T one = cst<T>(1.0);
@@ -313,6 +321,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             nr = w1 * wr;
             ni = w2 * wi;
             Pn = nr * ni;
+            iP = wr * wi;
             uR = nr * nA + ni * nB;
             uI = ni * nA + nr * nB;
         }
@@ -391,7 +400,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 const T id = rcp_((sq + S1) * gg);
                 const T e = (delta * id) * id;
                 sJ = sJ + tm * rc1_core(e, false).v * id;
-                if (REV) stq[m] = sq;
+                if (REV) tape.q[m] = sq;
                 p = p + lam;
             }
             if (WX) {
@@ -407,7 +416,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                                   - (gg + cst<T>(2.0) * S1 * (qs + S)) * (id * id) * gg * ix * cst<T>(0.5));
                 pX = pX + lam;
             }
-            if (REV) { st1[m] = S1; stS[m] = S; stP[m] = P; }
+            if (REV) {
+                tape.s1[m] = S1;
+                tape.S[m] = S;
+                if (WT) tape.P[m] = P;
+            }
             x = xl;
             T3 = T3 + cst<T>(3.0) * lam;
             const T n1 = x * rsq(x);
@@ -456,7 +469,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T ad = fabs(d5);
 #pragma unroll 1
             for (; mr < CoreTol<T>::maxit; mr++) {
-                if (REV) { ra[mr < NR ? mr : 0] = a; rb[mr < NR ? mr : 0] = b; }
+                if (REV) { tape.ra[mr] = a; tape.rb[mr] = b; }
                 if (ad <= CoreTol<T>::rc * U) break;
                 const T n = a + b, q = cst<T>(2.0) * b * n;
                 a = n;
@@ -532,8 +545,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         }
     }
 
+    // 1 / E(z) = E(0)^-1 / (n_A n_B |n_P|^2)
+    LCDM_HD T inv_E() const { return rc[C_C2] * cst<T>(0.5) * (rA * rB * iP); }
+
     // Adjoints of the row's constants for the cotangents ci, ti of Ichi, It.
-    LCDM_HD void reverse(T ci, T ti) {
+    LCDM_HD void reverse(T ci, T ti, const Tape& tape) {
         const T one = cst<T>(1.0), two = cst<T>(2.0), half = cst<T>(0.5);
         T RF_ = ci * cz, T_ = cst<T>(0.0), p_ = cst<T>(0.0), cJ = cst<T>(0.0), del_ = cst<T>(0.0), a_ = cst<T>(0.0),
           b_ = cst<T>(0.0), d_ = cst<T>(0.0), nA_ = cst<T>(0.0), wA_ = cst<T>(0.0);
@@ -571,12 +587,12 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T sd = sc * (two * ser + sc * ds), sv = one + sc * sc * ser;
             d_ = -rcb * sd * iU;
             const T U_ = -rcb * iU * (sc * sd + half * sv);
-            T ax = ra[mr < NR ? mr : 0], bx = rb[mr < NR ? mr : 0];
+            T ax = tape.ra[mr < Tape::NR ? mr : 0], bx = tape.rb[mr < Tape::NR ? mr : 0];
             a_ = two * ax * U_;
             b_ = cst<T>(4.0) * bx * U_;
 #pragma unroll 1
             for (int i = mr - 1; i >= 0; i--) {
-                const T a0 = ra[i], b0 = rb[i];
+                const T a0 = tape.ra[i], b0 = tape.rb[i];
                 const T Q_ = b_ * half * rcp_(bx);
                 const T n_ = a_ + two * b0 * Q_;
                 b_ = two * (a0 + b0) * Q_ + n_;
@@ -618,16 +634,14 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         T ps_ = WT ? pf_ : cst<T>(0.0);
         T delta = cst<T>(0.0), tk = tm;
         if (WT) delta = cst<T>(-9.0) * kT.v[2] * kT.v[2] * kT.v[3] * (z2 * z2 * z2);
-        T n1, n1s;   // the next step's sqrt(x) and S
+        T n1 = one, n1s = one;   // the next step's sqrt(x) and S
 #pragma unroll 1
         for (int i = m - 1; i >= 0; i--) {
-            const T a = st1[i], Sm = stS[i], Pm = stP[i];
+            const T a = tape.s1[i], Sm = tape.S[i], Pm = WT ? tape.P[i] : cst<T>(0.0);
             tk = tk * half;
             T Sn_ = cst<T>(0.0), an_ = cst<T>(0.0);
             if (i < m - 1) {
                 // next: n1 = sqrt(x'), P' = n1 S, S' = sqrt(S (S + 2 (a + n1)))
-                n1 = st1[i + 1];
-                n1s = stS[i + 1];
                 const T Q_ = S_ * half * rcp_(n1s);
                 const T t = two * Sm * Q_;
                 const T n_ = s_ + P_ * Sm + t;
@@ -635,12 +649,14 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 an_ = t;
                 x_ = x_ + n_ * half * rcp_(n1);
             }
+            n1 = a;
+            n1s = Sm;
             const T lam_ = x_ + ps_ + cst<T>(3.0) * T_;
             s_ = an_ + lam_ * Sm;
             S_ = Sn_ + lam_ * a;
             P_ = lam_;
             if (WT) {
-                const T sq = stq[i], gg = sq * (sq + Sm) + Pm, qs = sq + a;
+                const T sq = tape.q[i], gg = sq * (sq + Sm) + Pm, qs = sq + a;
                 const T id = rcp_(qs * gg), e = (delta * id) * id;
                 const RcE<T> r = rc1_core(e, true);
                 const T c = cJ * tk * id;                 // cotangent of rc

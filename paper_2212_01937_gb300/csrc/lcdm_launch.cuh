@@ -8,12 +8,12 @@ namespace lcdm {
 // One pair kernel: its launch and its resident blocks per SM.  `rec` is the
 // core's record; the kernel of X's tangents reads the records in the arguments.
 struct PairsEntry {
-    cudaError_t (*launch)(const PairArgs& a, const void* rec, int grid, int block, cudaStream_t s);
+    cudaError_t (*launch)(const PairArgs& a, const void* rec, void* grad_z, int grid, int block, cudaStream_t s);
     int (*occ)(int block);
 };
 
 template <int PREC, int K, bool WT> struct TangentX {
-    static cudaError_t launch(const PairArgs& a, const void*, int grid, int block, cudaStream_t s) {
+    static cudaError_t launch(const PairArgs& a, const void*, void*, int grid, int block, cudaStream_t s) {
         pairs_kernel<PREC, K, WT, true><<<grid, block, 0, s>>>(a);
         return cudaGetLastError();
     }
@@ -24,49 +24,56 @@ template <int PREC, int K, bool WT> struct TangentX {
         return n;
     }
 };
-template <int PREC, int K, bool WT, bool WX, bool JAC> struct Core {
-    static cudaError_t launch(const PairArgs& a, const void* rec, int grid, int block, cudaStream_t s) {
+template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
+    static cudaError_t launch(const PairArgs& a, const void* rec, void* grad_z, int grid, int block, cudaStream_t s) {
         CoreArgs c;
         c.p = a;
         c.rec = rec;
-        core_kernel<PREC, K, WT, WX, JAC><<<grid, block, 0, s>>>(c);
+        c.grad_z = grad_z;
+        core_kernel<PREC, K, WT, WX, MODE><<<grid, block, 0, s>>>(c);
         return cudaGetLastError();
     }
     static int occ(int block) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core_kernel<PREC, K, WT, WX, JAC>, block, 0) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core_kernel<PREC, K, WT, WX, MODE>, block, 0) != cudaSuccess)
             return 0;
         return n;
     }
 };
 
 // entries by (WT ? 2 : 0) + (WX ? 1 : 0); jac: the kernels of per-pair
-// Jacobians (without X's, whose tangents have a kernel of their own)
+// Jacobians (without X's, whose tangents have a kernel of their own); dz: those
+// that also give the redshift derivatives, by WT (four- and five-column rows;
+// of the value kernels only the one without t and X)
 struct PairsTable {
-    PairsEntry e[4], jac[4];
+    PairsEntry e[4], jac[4], dz[2];
 };
 
 template <class E> PairsEntry entry() { PairsEntry e; e.launch = E::launch; e.occ = E::occ; return e; }
 
 template <int PREC> PairsTable value_table() {
-    PairsTable t;
-    t.e[0] = entry<Core<PREC, 0, false, false, false> >();
-    t.e[1] = entry<Core<PREC, 0, false, true, false> >();
-    t.e[2] = entry<Core<PREC, 0, true, false, false> >();
-    t.e[3] = entry<Core<PREC, 0, true, true, false> >();
-    for (int i = 0; i < 4; i++) t.jac[i] = t.e[i];
+    PairsTable t = {};
+    t.e[0] = entry<Core<PREC, 0, false, false> >();
+    t.e[1] = entry<Core<PREC, 0, false, true> >();
+    t.e[2] = entry<Core<PREC, 0, true, false> >();
+    t.e[3] = entry<Core<PREC, 0, true, true> >();
+    t.dz[0] = entry<Core<PREC, 0, false, false, CORE_DZ> >();
     return t;
 }
 template <int PREC, int K> PairsTable tangent_table() {
-    PairsTable t;
-    t.e[0] = entry<Core<PREC, K, false, false, false> >();
+    PairsTable t = {};
+    t.e[0] = entry<Core<PREC, K, false, false> >();
     t.e[1] = entry<TangentX<PREC, K, false> >();
-    t.e[2] = entry<Core<PREC, K, true, false, false> >();
+    t.e[2] = entry<Core<PREC, K, true, false> >();
     t.e[3] = entry<TangentX<PREC, K, true> >();
-    t.jac[0] = entry<Core<PREC, K, false, false, true> >();
+    t.jac[0] = entry<Core<PREC, K, false, false, CORE_JAC> >();
     t.jac[1] = t.e[1];
-    t.jac[2] = entry<Core<PREC, K, true, false, true> >();
+    t.jac[2] = entry<Core<PREC, K, true, false, CORE_JAC> >();
     t.jac[3] = t.e[3];
+    if constexpr (K < 6) {
+        t.dz[0] = entry<Core<PREC, K, false, false, CORE_DZ> >();
+        t.dz[1] = entry<Core<PREC, K, true, false, CORE_DZ> >();
+    }
     return t;
 }
 

@@ -807,7 +807,7 @@ __device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, b
         const double iH0 = r.H0 < 1e-280 ? ddiv(1.0, r.H0) : rcp_(r.H0);
         put(rec, C_DH, LCDM_C_KMS * iH0);
         put(rec, C_TH, LCDM_HUBBLE_GYR * iH0);
-        put(rec, C_H0, r.H0);
+        put(rec, C_IH0, iH0);
     }
     if (!tangents) return;
     const int b = r.quartic ? 1 : 0;
