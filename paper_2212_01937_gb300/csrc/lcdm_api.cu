@@ -23,12 +23,14 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 #define LCDM_PREP_GROUP_MAX_B 16384
 
 // Row records: those of the core (NCORE floats or doubles per row), or those
-// of the X-tangent kernel, in the same memory (a plan that needs both prepares
-// one after the other).
-static_assert(NCORE <= NREC + NREC, "the core's record fits the workspace of the X-tangent kernel's two");
-size_t ws_bytes_for(int64_t B) {
-    return align256((size_t)B * NREC * sizeof(double)) + align256((size_t)B * NREC * sizeof(float2));
-}
+// of the X-tangent kernel (FP64 and its (hi, lo) copy), in the same memory (a
+// plan that needs both prepares one after the other).
+#define LCDM_RECORD_BYTES(B)                                                                              \
+    (((size_t)(B) * NCORE * sizeof(double) + 255) / 256 * 256 >                                           \
+             ((size_t)(B) * NREC * sizeof(double) + 255) / 256 * 256 + ((size_t)(B) * NREC * sizeof(float2) + 255) / 256 * 256 \
+         ? ((size_t)(B) * NCORE * sizeof(double) + 255) / 256 * 256                                       \
+         : ((size_t)(B) * NREC * sizeof(double) + 255) / 256 * 256 + ((size_t)(B) * NREC * sizeof(float2) + 255) / 256 * 256)
+size_t ws_bytes_for(int64_t B) { return LCDM_RECORD_BYTES(B); }
 
 bool opts_ok(const lcdm_opts* o) {
     return o && (o->ncol == 4 || o->ncol == 5 || o->ncol == 7) &&
@@ -117,7 +119,7 @@ struct Plan {
     const void* core;       // the core's records
     void* grad_z;           // [npairs] derivatives with respect to the redshifts, optional
     int legacy;             // the tangent launch is the X-tangent kernel's
-    int absorb;             // the core's records need the absorption distance's constants
+    int time, absorb;       // the core's records need the constants of t, of the absorption distance
     int prec, K, wt, wx;
     int64_t npairs;
     TuneKey key;
@@ -192,6 +194,7 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     P.wt = wt;
     P.wx = wx;
     P.legacy = P.K > 0 && wx;
+    P.time = (P.split_mask >> LCDM_T) & 1 || (!P.legacy && wt);
     P.absorb = (P.split_mask >> LCDM_X) & 1 || (P.K == 0 && wx);
     P.key = TuneKey(current_device(), P.prec, P.K, wt, wx, opts->layout, log2_bucket(P.npairs));
     return LCDM_OK;
@@ -357,7 +360,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
 struct PrepNeed {
     bool legacy;     // the X-tangent kernel's records, else the core's
     int prec;        // precision of the core's records
-    bool tangents, absorb;
+    bool tangents, time, absorb;
 };
 
 lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv, const PrepNeed& need,
@@ -372,6 +375,7 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
     a.B = B;
     a.ncol = opts->ncol;
     a.tangents = need.tangents;
+    a.time = need.time;
     a.absorb = need.absorb;
     a.recD = need.legacy ? cv.recD : nullptr;
     a.recF = need.legacy ? cv.recF : nullptr;
@@ -400,7 +404,7 @@ lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_
     lcdm_status st;
     const bool dz = separate_dz(P);
     if (P.split_mask || dz || !P.legacy) {
-        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.absorb != 0};
+        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.time != 0, P.absorb != 0};
         st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
         if (st != LCDM_OK) return st;
     }
@@ -413,7 +417,7 @@ lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_
         if (st != LCDM_OK) return st;
     }
     if (P.legacy) {
-        const PrepNeed need = {true, P.prec, true, true};
+        const PrepNeed need = {true, P.prec, true, true, true};
         st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
         if (st != LCDM_OK) return st;
     }
@@ -469,8 +473,7 @@ lcdm_status pairs_common(const double* params, int64_t B, const int64_t* offsets
 // cudaGetSymbolAddress (the host-side name is only a stand-in and must never
 // be handed to a kernel).
 // ----------------------------------------------------------------------------
-#define LCDM_STATIC_WS_BYTES (((size_t)LCDM_STATIC_MAX_COSMOLOGIES * NREC * sizeof(double) + 255) / 256 * 256 + \
-                              ((size_t)LCDM_STATIC_MAX_COSMOLOGIES * NREC * sizeof(float2) + 255) / 256 * 256)
+#define LCDM_STATIC_WS_BYTES LCDM_RECORD_BYTES(LCDM_STATIC_MAX_COSMOLOGIES)
 static __device__ __align__(256) unsigned char g_static_ws[LCDM_STATIC_WS_BYTES];
 
 static void* g_static_ptr[LCDM_MAX_DEVICES];
@@ -764,7 +767,7 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     o4.ncol = 4;
     lcdm_status st = between_setup(params, B, z1, ncol, w, stream);
     if (st != LCDM_OK) return st;
-    const PrepNeed need = {false, 0, grad != nullptr, false};
+    const PrepNeed need = {false, 0, grad != nullptr, true, false};
     st = run_prep(w.params4, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     LimitArgs la;
@@ -847,12 +850,12 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
         make_plan(d.params, B, d.offsets, d.z, n, outs, nullptr, cot, nullptr, 0, 1, d.grad, nullptr, d.status, opts,
                   d.rec, P);
         if (P.legacy) {
-            const PrepNeed need = {true, P.prec, true, true};
+            const PrepNeed need = {true, P.prec, true, true, true};
             st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
             if (st != LCDM_OK) return st;
         }
         if (P.split_mask || !P.legacy) {
-            const PrepNeed need = {false, P.prec, !P.legacy, P.absorb != 0};
+            const PrepNeed need = {false, P.prec, !P.legacy, P.time != 0, P.absorb != 0};
             st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
             if (st != LCDM_OK) return st;
         }
@@ -939,7 +942,7 @@ lcdm_status lcdm_roots(const double* params, int64_t B, const lcdm_opts* opts, d
     Carved cv;
     lcdm_status st = carve(ws, ws_bytes, B, cv);
     if (st != LCDM_OK) return st;
-    const PrepNeed need = {true, 0, true, false};
+    const PrepNeed need = {true, 0, true, true, false};
     st = run_prep(params, B, opts, cv, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     extract_roots<<<(unsigned)((B + 127) / 128), 128, 0, stream>>>(cv.recD, B, opts->ncol, roots, droots, kind);
@@ -1012,7 +1015,7 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
                 for (int rep = 0; rep < 3; rep++) {
                     // (the preparation is not timed, but where it comes between the launches)
                     const bool both = P.legacy && P.split_mask;
-                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.absorb != 0};
+                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.time != 0, P.absorb != 0};
                     if (!both && run_prep(params, B, opts, cv, need, cosmo_status, grad, nullptr, stream) != LCDM_OK)
                         return LCDM_ERR_CUDA;
                     cudaEventRecord(e0, stream);

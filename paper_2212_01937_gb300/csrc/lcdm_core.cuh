@@ -24,8 +24,8 @@
 // Consequences for the duplication (Carlson's algorithm, the paper's ref. [10]):
 //  * the sequence is carried without the division by four (x <- x + lambda):
 //    differences are then constant and the truncated series are polynomials
-//    in w = z^2 / A with constants of the row as coefficients (4 + 2 terms,
-//    to the 7th degree in the deviations);
+//    in w = z^2 / A with constants of the row as coefficients, so a degree more
+//    costs one multiply-add (and a larger deviation may be left: fewer steps);
 //  * the stopping rule is one multiplication: z^2 max|deviation| <= tol A;
 //  * y y* = x1 S^2 after the first step, so a step takes two square roots
 //    (one more per third-kind track) and no division by a difference;
@@ -45,36 +45,55 @@ enum CoreField {
     C_QI, C_QIL, C_C2, C_KIND,            // (QRL, QIL: low words in single precision); c2 = 2 / sqrt(S0);
                                           // KIND: 1 for a complex pair, 0 for two reals
     C_DH, C_TH, C_IH0, C_OK,              // c/H0 [Mpc], 1/H0 [Gyr], 1/H0, Omega_k0
-    C_DF, C_B2, C_B3, C_B4,               // DF: max deviation / z^2 from the mean of three; series of R_F
-    C_B5, C_B6, C_B7, C_RS,               // RS = -1 / (2 S0) with free S0, 0 under the closure
-    C_DJ, C_EPS, C_K2, C_K3,              // DJ: max deviation from the mean of five (t track)
-    C_A2, C_A3, C_A4, C_A5,               // series of the t track's R_J
-    C_A6, C_A7, C_FREE0, C_FREE1,
+    C_DF, C_B = 13,                       // DF: max deviation / z^2 from the mean of three; B: series of R_F (10)
+    C_RS = 23,                            // -1 / (2 S0) with free S0, 0 under the closure
+    C_DJ = 24, C_EPS, C_K2, C_K3,         // DJ: max deviation from the mean of five (t track)
+    C_A = 28,                             // series of the t track's R_J (10)
+    C_FREE0 = 38, C_FREE1,
     // absorption distance (values)
-    X_HX = 32, X_LX, X_PX, X_DX,          // p0 - x1 = -hx z^2; p0 = (..)^2 - lx z^2 w_B; pi/z^4; max deviation
+    X_HX = 40, X_LX, X_PX, X_DX,          // p0 - x1 = -hx z^2; p0 = (..)^2 - lx z^2 w_B; pi/z^4; max deviation
     X_C0, X_T1, X_G1, X_G2,
     X_G3, X_G4, X_G5, X_SY,
     X_N0, X_N1, X_N2, X_FREE,
     X_AB, X_LAM, X_SQ, X_PQ,              // q_P + q_P*, q_P q_P*
-    X_A2 = 52,                            // a_j at p0 (6), a_j at x1 (6), divided differences (6)
-    X_D2 = 58, X_E2 = 64,
-    C_TAN = 72, C_TSTRIDE = 20,           // tangents of slot k at C_TAN + 20 k:
-    CT_QA = 0, CT_QB, CT_QR, CT_QI, CT_B2, CT_EPS = 10, CT_K2, CT_K3, CT_A2, CT_END = 19,
+    X_S = 60,                             // series at p0, at x1, and their divided differences, by degree (3 x 10)
+    C_TAN = 92, C_TSTRIDE = 28,           // tangents of slot k at C_TAN + 28 k:
+    CT_QA = 0, CT_QB, CT_QR, CT_QI, CT_B, CT_EPS = 14, CT_K2, CT_K3, CT_A = 17, CT_END = 27,
     NCORE = C_TAN + 6 * C_TSTRIDE
 };
+enum { CORE_NS = 10 };   // series coefficients in the record: degrees 2 to 11
 
 // ------------------------------------------------------------- arithmetic ---
-// 1/sqrt and 1/x.  Single precision: the hardware approximations (within two
-// ulp).  Double precision: CUDA's rsqrt; the reciprocal by one third-order
-// step from the hardware's 20-bit approximation (error 2^-60 before rounding;
-// positive normal arguments), three fused multiply-adds where the division
-// issues about nine FP64 instructions.
+// 1/sqrt, sqrt and 1/x of positive normal numbers.  Single precision: the
+// hardware approximations (within two ulp).  Double precision: one step of
+// Householder's third-order method from the hardware's 20-bit approximation
+// (error 2^-60 before rounding), written out for each: with y ~ x^-1/2, t = x y
+// and e = 1 - t y,  x^-1/2 = y + y e (1/2 + 3 e / 8),  x^1/2 = t + t e (1/2 + 3 e / 8);
+// with y ~ 1/x, e = 1 - x y,  1/x = y + y (e + e^2).  Five, five and three FP64
+// instructions; CUDA's square root issues about 9, its division 9, rsqrt 5.5.
 LCDM_HD float rsq(float x) { return srsqrt(x); }
+LCDM_HD float sqt(float x) { return x * srsqrt(x); }
+#ifdef __CUDA_ARCH__
+LCDM_HD double rsq_seed(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+#endif
 LCDM_HD double rsq(double x) {
 #ifdef __CUDA_ARCH__
-    return rsqrt(x);
+    const double y = rsq_seed(x), e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 #else
     return 1.0 / sqrt(x);
+#endif
+}
+LCDM_HD double sqt(double x) {
+#ifdef __CUDA_ARCH__
+    const double y = rsq_seed(x), t = x * y, e = fma(-t, y, 1.0);
+    return fma(t * e, fma(0.375, e, 0.5), t);
+#else
+    return sqrt(x);
 #endif
 }
 LCDM_HD float rcp_(float x) {
@@ -99,14 +118,15 @@ LCDM_HD double rcp_(double x) {
 
 template <class T> struct CoreTol;
 template <> struct CoreTol<float> {
-    // deviation at which a degree-7 series is used; relative deviation s of
-    // R_C's; largest z taken without scaling
-    static constexpr float dup = 0.15f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
-    enum { maxit = 24 };
+    // largest deviation left to the series of degree ns + 1 (its truncation:
+    // about dup^(ns + 2) / 100); relative deviation s of R_C's; largest z taken
+    // without scaling
+    static constexpr float dup = 0.25f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
+    enum { maxit = 24, ns = 8 };
 };
 template <> struct CoreTol<double> {
-    static constexpr double dup = 0.009, rc = 0.008, big = 1e30, e_series = 0.03;
-    enum { maxit = 40 };
+    static constexpr double dup = 0.05, rc = 0.008, big = 1e30, e_series = 0.03;
+    enum { maxit = 40, ns = 10 };
 };
 
 // R_C(1, 1 + e) and its derivative by closed relations, for e beyond the
@@ -120,7 +140,7 @@ template <class T> LCDM_NI RcE<T> rc1_far(T e, T b) {
     for (int m = 0; m < CoreTol<T>::maxit && !(fabs(e) <= CoreTol<T>::rc * U); m++) {
         const T n = a + b, q = cst<T>(2.0) * b * n;
         a = n;
-        b = q * rsq(q);
+        b = sqt(q);
         U = a * a + cst<T>(2.0) * b * b;
         tm = tm + tm;
     }
@@ -145,7 +165,7 @@ LCDM_HD RcE<float> rc1_core(float e, bool grad) {
         r.d = -ds;
         return r;
     }
-    return rc1_far<float>(e, (1.0f + e) * rsq(1.0f + e));
+    return rc1_far<float>(e, sqt(1.0f + e));
 }
 LCDM_HD RcE<double> rc1_core(double e, bool grad) {
     // e falls by 64 or more per step: most steps need a few terms only
@@ -168,19 +188,21 @@ LCDM_HD RcE<double> rc1_core(double e, bool grad) {
         r.d = -ds;
         return r;
     }
-    return rc1_far<double>(e, (1.0 + e) * rsq(1.0 + e));
+    return rc1_far<double>(e, sqt(1.0 + e));
 }
 // (R_C(1, 1+e) - 1) / e
 template <class T> LCDM_HD T rc1m1_core(T e) {
     constexpr int NT = sizeof(T) == 4 ? 6 : 12;
+    const T w = -e;
+    if (sizeof(T) == 8 && fabs(e) <= cst<T>(3e-5))
+        return cst<T>(-1.0 / 3) + w * (cst<T>(-0.2) + w * (cst<T>(-1.0 / 7) + w * cst<T>(-1.0 / 9)));
     if (fabs(e) <= CoreTol<T>::e_series) {
-        const T w = -e;
         T s = cst<T>(-1.0 / (2 * NT + 3));
 #pragma unroll
         for (int n = NT; n >= 1; n--) s = cst<T>(-1.0 / (2 * n + 1)) + w * s;
         return s;
     }
-    return (rc1_far<T>(e, (cst<T>(1.0) + e) * rsq(cst<T>(1.0) + e)).v - cst<T>(1.0)) / e;
+    return (rc1_far<T>(e, sqt(cst<T>(1.0) + e)).v - cst<T>(1.0)) / e;
 }
 // [R_C(1, 1-w) - (1-w)^-1/2] / w  (see phi_rc) for 0 <= w < 1, so = sqrt(1-w)
 // (which cancels if formed from w near 1).  Beyond the series' range R_C's
@@ -193,7 +215,7 @@ template <class T> LCDM_HD T phi_core(T w, T so) {
     T a = cst<T>(1.0), b = so, sum = cst<T>(0.0), t = cst<T>(1.0), ia = cst<T>(1.0), v = w;
 #pragma unroll 1
     for (int m = 0; m < CoreTol<T>::maxit && v > cst<T>(0.1); m++) {
-        const T n = a + b, q = cst<T>(2.0) * b * n, c = q * rsq(q);
+        const T n = a + b, q = cst<T>(2.0) * b * n, c = sqt(q);
         sum = sum - cst<T>(2.0) * t * rcp_(n * c * (cst<T>(2.0) * b + c));
         a = n;
         b = c;
@@ -250,6 +272,31 @@ LCDM_HD Quad<double> quad(const double* p) {
 }
 
 // ------------------------------------------------------------------- core ---
+// A closing series 1 + w^2 (c_2 + c_3 w + ...) from ns coefficients at rec[i],
+// i = 0 or 1 modulo 4, and with it (D) the derivative of the bracket.
+template <class T> struct SerVal { T v, d; };
+template <bool D, class T> LCDM_HD SerVal<T> series(const T* rec, int i, T w) {
+    constexpr int N = CoreTol<T>::ns;
+    T c[12];
+    const int skip = i & 3;
+#pragma unroll
+    for (int q = 0; q < (N + skip + 3) / 4; q++) {
+        const Quad<T> k = quad(rec + (i - skip) + 4 * q);
+#pragma unroll
+        for (int l = 0; l < 4; l++)
+            if (4 * q + l >= skip && 4 * q + l - skip < 12) c[4 * q + l - skip] = k.v[l];
+    }
+    SerVal<T> r;
+    r.v = c[N - 1];
+    r.d = cst<T>(0.0);
+#pragma unroll
+    for (int j = N - 2; j >= 0; j--) {
+        if (D) r.d = r.d * w + r.v;
+        r.v = r.v * w + c[j];
+    }
+    return r;
+}
+
 // The steps taken, for the reverse pass: s1, S and P of the duplication (sqrt(p)
 // of the t track), and R_C's a and b.  Apart from the pair's other state: it is
 // indexed by the step and lives in local memory (of which only the steps taken
@@ -289,7 +336,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         rc = rec;
         z = zin;
         const T one = cst<T>(1.0);
-        const Quad<T> k0 = quad(rc + C_QA), k1 = quad(rc + C_QI), kF = quad(rc + C_DF);
+        const Quad<T> k0 = quad(rc + C_QA), k1 = quad(rc + C_QI);
         cplx = k1.v[3] != cst<T>(0.0);
         const T wA = INF ? k0.v[0] : one + k0.v[0] * z, wB = INF ? k0.v[1] : one + k0.v[1] * z;
         rA = INF && !(wA > cst<T>(0.0)) ? cst<T>(0.0) : rsq(wA);
@@ -379,22 +426,25 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             dX = -(kX.v[0] * z2) * piX;
         }
         T pX = p0;
-        const T dF = kF.v[0] * z2 * cst<T>(3.0), dJ = WT ? kT.v[0] * z2 * cst<T>(5.0) : cst<T>(0.0);
-        const T dD = WX ? kX.v[3] * z2 * cst<T>(5.0) : cst<T>(0.0);
+        const float it = (float)(1.0 / CoreTol<T>::dup), z2f = (float)z2 * it;
+        const float dF = (float)rc[C_DF] * z2f * 3.0f, dJ = WT ? (float)kT.v[0] * z2f * 5.0f : 0.0f;
+        const float dD = WX ? (float)kX.v[3] * z2f * 5.0f : 0.0f;
         T S1 = s1;
         tm = one;
         T q0 = cst<T>(0.0);
         m = 0;
 #pragma unroll 1
         for (; m < CoreTol<T>::maxit; m++) {
-            bool conv = dF <= CoreTol<T>::dup * T3;
-            if (WT) conv = conv && dJ <= CoreTol<T>::dup * (T3 + p + p);
-            if (WX) conv = conv && dD <= CoreTol<T>::dup * (T3 + pX + pX) && dD <= CoreTol<T>::dup * (T3 + x + x);
+            // (compared in single precision: in double each comparison would hold
+            // the FP64 pipe)
+            bool conv = dF <= (float)T3;
+            if (WT) conv = conv && dJ <= (float)(T3 + p + p);
+            if (WX) conv = conv && dD <= (float)(T3 + pX + pX) && dD <= (float)(T3 + x + x);
             if (conv) break;
             const T lam = S1 * S + P;
             const T xl = x + lam;
             if (WT) {
-                const T sq = p * rsq(p);
+                const T sq = sqt(p);
                 if (m == 0) q0 = sq;
                 const T gg = p + (sq * S + P);
                 const T id = rcp_((sq + S1) * gg);
@@ -407,7 +457,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 // R_D: 1 / (s1 (x + lambda)); divided difference of the p0 track against it
                 const T ix = rcp_(S1 * xl);
                 sD = sD + tm * ix;
-                const T sq = pX * rsq(pX);
+                const T sq = sqt(pX);
                 if (m == 0) rp0 = sq;
                 const T gg = pX + (sq * S + P), qs = sq + S1;
                 const T id = rcp_(qs * gg);
@@ -423,10 +473,10 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             }
             x = xl;
             T3 = T3 + cst<T>(3.0) * lam;
-            const T n1 = x * rsq(x);
+            const T n1 = sqt(x);
             const T Q = S * (S + cst<T>(2.0) * (S1 + n1));
             P = n1 * S;
-            S = Q * rsq(Q);
+            S = sqt(Q);
             S1 = n1;
             tm = tm + tm;
         }
@@ -436,13 +486,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T A = T3 * cst<T>(1.0 / 3);
             rF = rsq(A);
             wF = z2 * (rF * rF);
-            const Quad<T> kB5 = quad(rc + C_B5);
-            T s = kB5.v[2];
-            s = s * wF + kB5.v[1];
-            s = s * wF + kB5.v[0];
-            s = s * wF + kF.v[3];
-            s = s * wF + kF.v[2];
-            s = s * wF + kF.v[1];
+            const T s = series<false>(rc, C_B, wF).v;
             sF = one + s * (wF * wF);
             RF = tm * sF * rF;
         }
@@ -452,17 +496,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T A = (T3 + p + p) * cst<T>(0.2);
             rJ = rsq(A);
             wJ = z2 * (rJ * rJ);
-            const Quad<T> kA = quad(rc + C_A2), kA6 = quad(rc + C_A6);
-            T s = kA6.v[1];
-            s = s * wJ + kA6.v[0];
-            s = s * wJ + kA.v[3];
-            s = s * wJ + kA.v[2];
-            s = s * wJ + kA.v[1];
-            s = s * wJ + kA.v[0];
+            const T s = series<false>(rc, C_A, wJ).v;
             sJs = one + s * (wJ * wJ);
             RJ = tm * sJs * (rJ * rJ * rJ) + cst<T>(6.0) * sJ;
             // R_C(s5, p), Carlson's duplication on the square roots a = sqrt(s5), b = sqrt(p)
-            T a = a5, b = m > 0 ? q0 : p * rsq(p);
+            T a = a5, b = m > 0 ? q0 : sqt(p);
             U = a * a + cst<T>(2.0) * (b * b);
             tr = one;
             mr = 0;
@@ -473,7 +511,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 if (ad <= CoreTol<T>::rc * U) break;
                 const T n = a + b, q = cst<T>(2.0) * b * n;
                 a = n;
-                b = q * rsq(q);
+                b = sqt(q);
                 U = a * a + cst<T>(2.0) * (b * b);
                 tr = tr + tr;
             }
@@ -503,19 +541,22 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T A2 = (T3 + x + x) * cst<T>(0.2), A1 = (T3 + pX + pX) * cst<T>(0.2);
             const T r1 = rsq(A1), r2 = rsq(A2);
             const T i1 = r1 * r1, w1 = z2 * i1, w2 = z2 * iA2, ww = cst<T>(-0.4) * w1 * w2;
-            T q[20];   // a_j at p0, at x1, divided differences
+            // series at p0 and at x1, and the divided difference of the brackets
+            // (coefficients by degree: at p0, at x1, their divided difference)
+            constexpr int N = CoreTol<T>::ns;
+            T v1 = cst<T>(0.0), v2 = cst<T>(0.0), e = cst<T>(0.0);
+            T q[3 * CORE_NS + 2];
 #pragma unroll
-            for (int j = 0; j < 5; j++) {
-                const Quad<T> f = quad(rc + X_A2 + 4 * j);
+            for (int j = 0; j < (3 * N + 3) / 4; j++) {
+                const Quad<T> f = quad(rc + X_S + 4 * j);
 #pragma unroll
                 for (int i = 0; i < 4; i++) q[4 * j + i] = f.v[i];
             }
-            T v1 = q[5], v2 = q[11], e = -q[17];
 #pragma unroll
-            for (int j = 4; j >= 0; j--) {
-                e = e * w1 + v2 * ww - q[12 + j];
-                v1 = v1 * w1 + q[j];
-                v2 = v2 * w2 + q[6 + j];
+            for (int j = N - 1; j >= 0; j--) {
+                e = e * w1 + v2 * ww - q[3 * j + 2];
+                v1 = v1 * w1 + q[3 * j];
+                v2 = v2 * w2 + q[3 * j + 1];
             }
             const T ser1 = one + v1 * (w1 * w1);
             const T dser = cst<T>(-0.4) * (w1 + w2) * z2 * i1 * iA2 * v1 + w2 * iA2 * e;
@@ -524,7 +565,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T dA = cst<T>(-0.4) * (A1 + q1 * q2 + A2) * rcp_(q1 + q2) * r13 * r23;
             const T DJ = tm * (dA * ser1 + r23 * dser) + cst<T>(6.0) * sDD;
             const T RD = tm * (one + v2 * (w2 * w2)) * r23 + cst<T>(3.0) * sD;
-            if (m == 0) rp0 = p0 * rsq(p0);
+            if (m == 0) rp0 = sqt(p0);
             // the results belong to arguments scaled by h^2 (h = 1 but for very large z)
             const T ih = big ? one / h : one;
             const T s1u = s1 * ih, sp0 = rp0 * ih, zz = z * z, x1 = x0 * (ih * ih);
@@ -601,13 +642,8 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             }
             p_ = b_ * half * rcp_(bx);                    // b = sqrt(p)
             // R_J: closing series
-            const Quad<T> kA = quad(rc + C_A2), kA6 = quad(rc + C_A6);
-            T s = kA6.v[1], s2 = s;
-            s = s * wJ + kA6.v[0];
-            s2 = s2 * wJ + s; s = s * wJ + kA.v[3];
-            s2 = s2 * wJ + s; s = s * wJ + kA.v[2];
-            s2 = s2 * wJ + s; s = s * wJ + kA.v[1];
-            s2 = s2 * wJ + s; s = s * wJ + kA.v[0];
+            const SerVal<T> sv2 = series<true>(rc, C_A, wJ);
+            const T s = sv2.v, s2 = sv2.d;
             const T r2 = rJ * rJ, c = RJ_ * tm * r2 * rJ;
             bJ_ = c;
             const T A_ = -c * r2 * (wJ * wJ * (two * s + wJ * s2) + cst<T>(1.5) * sJs);
@@ -618,13 +654,8 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             pf_ = A_ * cst<T>(0.4);
         }
         {
-            const Quad<T> kF = quad(rc + C_DF), kB5 = quad(rc + C_B5);
-            T s = kB5.v[2], s2 = s;
-            s = s * wF + kB5.v[1];
-            s2 = s2 * wF + s; s = s * wF + kB5.v[0];
-            s2 = s2 * wF + s; s = s * wF + kF.v[3];
-            s2 = s2 * wF + s; s = s * wF + kF.v[2];
-            s2 = s2 * wF + s; s = s * wF + kF.v[1];
+            const SerVal<T> sv2 = series<true>(rc, C_B, wF);
+            const T s = sv2.v, s2 = sv2.d;
             const T c = RF_ * tm * rF;
             bF_ = c;
             T_ = T_ - c * (rF * rF) * cst<T>(1.0 / 3) * (wF * wF * (two * s + wF * s2) + half * sF);
@@ -727,23 +758,12 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     // sum over the row's constants of adjoint times tangent, direction k
     LCDM_HD T along(int k) const {
         const T* t = rc + C_TAN + C_TSTRIDE * k;
-        const Quad<T> t0 = quad(t), t1 = quad(t + 4), t2 = quad(t + 8);
-        T b = t2.v[1];
-        b = b * wF + t2.v[0];
-        b = b * wF + t1.v[3];
-        b = b * wF + t1.v[2];
-        b = b * wF + t1.v[1];
-        b = b * wF + t1.v[0];
+        const Quad<T> t0 = quad(t);
+        const T b = series<false>(t, CT_B, wF).v;
         T r = qA_ * t0.v[0] + qB_ * t0.v[1] + (qR_ * t0.v[2] + qI_ * t0.v[3]) + bF_ * (wF * wF) * b;
         if (WT) {
-            const Quad<T> t3 = quad(t + 12), t4 = quad(t + 16);
-            T a = t4.v[2];
-            a = a * wJ + t4.v[1];
-            a = a * wJ + t4.v[0];
-            a = a * wJ + t3.v[3];
-            a = a * wJ + t3.v[2];
-            a = a * wJ + t3.v[1];
-            r = r + (eps_ * t2.v[2] + k2_ * t2.v[3] + k3_ * t3.v[0]) + bJ_ * (wJ * wJ) * a;
+            const T a = series<false>(t, CT_A, wJ).v;
+            r = r + (eps_ * t[CT_EPS] + k2_ * t[CT_K2] + k3_ * t[CT_K3]) + bJ_ * (wJ * wJ) * a;
         }
         return r;
     }

@@ -40,38 +40,52 @@ LCDM_HD RowDir row_dir(int ncol, int k) {
     return d;
 }
 
-// The closing series' coefficients (single precision records: in single
-// precision; they enter the results times the squared deviation and higher
-// powers, at most a fiftieth).
-// R_F in w: b_2 .. b_7 from (e2, e3)
-template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, S* b) {
-    typedef typename Base<S>::type B;
-    b[0] = e2 * cst<B>(-0.1);
-    b[1] = e3 * cst<B>(1.0 / 14);
-    b[2] = e2 * e2 * cst<B>(1.0 / 24);
-    b[3] = e2 * e3 * cst<B>(-3.0 / 44);
-    b[4] = e2 * e2 * e2 * cst<B>(-5.0 / 208) + e3 * e3 * cst<B>(3.0 / 104);
-    b[5] = e2 * e2 * e3 * cst<B>(1.0 / 16);
-}
-// closing series of R_J: a_2 .. a_7; m = (mean of three - p) / z^2
+// The closing series' coefficients, degrees 2 to 11 (single-precision records:
+// in single precision; they enter the results times the squared deviation and
+// higher powers, at most a twentieth).  With the arguments' deviations X_i from
+// their mean (sum 0) the series are sum_N c_N T_N, c_N = 1/(2N+1) for R_F and
+// 3/(2N+3) for R_J (DLMF 19.19), where sum_N T_N t^N = prod_i (1 - t X_i)^-1/2
+// = Q(t)^-1/2, Q = 1 + E2 t^2 - E3 t^3 + E4 t^4 - E5 t^5; from 2 Q S' = -Q' S,
+//   N T_N = - sum_j (N - j/2) q_j T_{N-j}.
 template <class S> struct SeriesBase { typedef typename Base<S>::type type; };
 template <class T> struct SeriesBase<DD<T> > { typedef T type; };
+template <class S> LCDM_HD S zero_like(const S& a) { return a * typename SeriesBase<S>::type(0); }
+// R_F: b_2 .. b_11 from (e2, e3)
+template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, S* b) {
+    typedef typename SeriesBase<S>::type B;
+    S t[CORE_NS + 2];
+    t[0] = zero_like(e2) + B(1);
+    t[1] = zero_like(e2);
+#pragma unroll
+    for (int n = 2; n < CORE_NS + 2; n++) {
+        S v = t[n - 2] * e2 * B(-(n - 1.0) / n);
+        if (n >= 3) v = v + t[n - 3] * e3 * B((n - 1.5) / n);
+        t[n] = v;
+        b[n - 2] = v * B(1.0 / (2 * n + 1));
+    }
+}
+// R_J: a_2 .. a_11; m = (mean of three - p) / z^2
 template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, S* a) {
     typedef typename SeriesBase<S>::type B;
     const S m2 = m * m;
-    const S E2 = e2 - m2 * cst<B>(0.6);
-    const S Q = e3 - m * e2 * cst<B>(0.4) - m2 * m * cst<B>(0.064);
-    const S P = m * cst<B>(0.6), P2 = P * P, P3 = P2 * P;
-    const S E3 = Q + E2 * P * cst<B>(2.0) + P3 * cst<B>(4.0);
-    const S E4 = (Q * cst<B>(2.0) + E2 * P + P3 * cst<B>(3.0)) * P;
+    const S E2 = e2 - m2 * B(0.6);
+    const S Q = e3 - m * e2 * B(0.4) - m2 * m * B(0.064);
+    const S P = m * B(0.6), P2 = P * P, P3 = P2 * P;
+    const S E3 = Q + E2 * P * B(2.0) + P3 * B(4.0);
+    const S E4 = (Q * B(2.0) + E2 * P + P3 * B(3.0)) * P;
     const S E5 = Q * P2;
-    const S E22 = E2 * E2;
-    a[0] = E2 * cst<B>(-3.0 / 14);
-    a[1] = E3 * cst<B>(1.0 / 6);
-    a[2] = E22 * cst<B>(9.0 / 88) - E4 * cst<B>(3.0 / 22);
-    a[3] = E5 * cst<B>(3.0 / 26) - E2 * E3 * cst<B>(9.0 / 52);
-    a[4] = E22 * E2 * cst<B>(-1.0 / 16) + E3 * E3 * cst<B>(3.0 / 40) + E2 * E4 * cst<B>(3.0 / 20);
-    a[5] = E22 * E3 * cst<B>(45.0 / 272) - (E3 * E4 + E2 * E5) * cst<B>(9.0 / 68);
+    S t[CORE_NS + 2];
+    t[0] = zero_like(E2) + B(1);
+    t[1] = zero_like(E2);
+#pragma unroll
+    for (int n = 2; n < CORE_NS + 2; n++) {
+        S v = t[n - 2] * E2 * B(-(n - 1.0) / n);
+        if (n >= 3) v = v + t[n - 3] * E3 * B((n - 1.5) / n);
+        if (n >= 4) v = v - t[n - 4] * E4 * B((n - 2.0) / n);
+        if (n >= 5) v = v + t[n - 5] * E5 * B((n - 2.5) / n);
+        t[n] = v;
+        a[n - 2] = v * B(3.0 / (2 * n + 3));
+    }
 }
 // largest deviation of the three, and of the five, arguments from their mean, over z^2
 LCDM_HD float dev3(double e2, double e3) {
@@ -89,7 +103,7 @@ LCDM_HD void put_lo(float* rec, int i, double v) { rec[i] = (float)(v - (double)
 LCDM_HD void put_lo(double* rec, int i, double) { rec[i] = 0.0; }
 
 // values (directions are added by core_tangent)
-template <class T> LCDM_HD void core_values(const RowRoots& r, bool absorb, T* rec) {
+template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool absorb, T* rec) {
     const double Oks = r.Ok + r.Os, S0 = r.S0, iS0 = r.iS0, sS = r.ncol == 4 ? 1.0 : sqrt(S0), isS = sS * iS0;
     const double qA = r.qA, qB = r.qB, q1 = r.q1, q2 = r.q2, eps = r.eps;
     put(rec, C_QA, qA); put(rec, C_QB, qB);
@@ -106,21 +120,25 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool absorb, T* r
                      + 27.0 * r.Om * r.Om * r.OL - 72.0 * r.Or * Oks * r.OL;
     const double e2 = I * (-1.0 / 3) * (iS0 * iS0), e3 = J * (-1.0 / 27) * (iS0 * iS0 * iS0);
     const T f2 = (T)e2, f3 = (T)e3;
-    T b[6], a[6];
+    T b[CORE_NS];
     rf_coefs<T>(f2, f3, b);
-    for (int j = 0; j < 6; j++) rec[C_B2 + j] = b[j];
+#pragma unroll
+    for (int j = 0; j < CORE_NS; j++) rec[C_B + j] = b[j];
     const float d3 = dev3(e2, e3);
     rec[C_DF] = (T)d3;
-    // t: E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
-    const double g0 = r.OL, g1 = r.Ox - eps * g0, g2 = Oks - eps * g1, g3 = r.Om - eps * g2;
-    const double k = (-g3 + eps * (g2 - eps * (g1 - eps * g0))) * iS0;
-    const double m = (g2 + eps * (3.0 * eps * g0 - 2.0 * g1)) * (iS0 * (1.0 / 3));
-    put(rec, C_EPS, eps);
-    put(rec, C_K2, k * (1.0 / 3));
-    put(rec, C_K3, r.OL * iS0);
-    rj_coefs<T>((T)m, f2, f3, a);
-    for (int j = 0; j < 6; j++) rec[C_A2 + j] = a[j];
-    rec[C_DJ] = (T)dev5(d3, m);
+    if (time) {
+        // t: E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
+        const double g0 = r.OL, g1 = r.Ox - eps * g0, g2 = Oks - eps * g1, g3 = r.Om - eps * g2;
+        const double k = (-g3 + eps * (g2 - eps * (g1 - eps * g0))) * iS0;
+        const double m = (g2 + eps * (3.0 * eps * g0 - 2.0 * g1)) * (iS0 * (1.0 / 3));
+        put(rec, C_EPS, eps);
+        put(rec, C_K2, k * (1.0 / 3));
+        put(rec, C_K3, r.OL * iS0);
+        rj_coefs<T>((T)m, f2, f3, b);
+#pragma unroll
+        for (int j = 0; j < CORE_NS; j++) rec[C_A + j] = b[j];
+        rec[C_DJ] = (T)dev5(d3, m);
+    }
     if (!absorb) return;
     const double S = r.cpair ? 2.0 * r.pr : r.pr + r.pi, Q = r.cpair ? r.pr * r.pr + r.pi * r.pi : r.pr * r.pi;
     const double pB = r.cpair ? (r.pr - r.B) * (r.pr - r.B) + r.pi * r.pi : (r.pr - r.B) * (r.pi - r.B);
@@ -164,18 +182,20 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool absorb, T* r
     if (r.cpair) { put(rec, X_SQ, 2.0 * q1); put(rec, X_PQ, q1 * q1 + q2 * q2); }
     else { put(rec, X_SQ, q1 + q2); put(rec, X_PQ, q1 * q2); }
     // the series at p0 (offset X1 + hx) and at x1 (offset X1), and their divided differences
-    DD<T> ad[6];
+    DD<T> ad[CORE_NS];
     rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx), (T)X1, (T)1), mkdd<T>(f2, f2, (T)0), mkdd<T>(f3, f3, (T)0), ad);
-    for (int j = 0; j < 6; j++) {
-        rec[X_A2 + j] = ad[j].v1;
-        rec[X_D2 + j] = ad[j].v2;
-        rec[X_E2 + j] = ad[j].d;
+#pragma unroll
+    for (int j = 0; j < CORE_NS; j++) {
+        rec[X_S + 3 * j] = ad[j].v1;
+        rec[X_S + 3 * j + 1] = ad[j].v2;
+        rec[X_S + 3 * j + 2] = ad[j].d;
     }
+    rec[X_S + 3 * CORE_NS] = rec[X_S + 3 * CORE_NS + 1] = (T)0;
 }
 
 // tangents of direction k; dA, dB, (dpr, dpi): the roots' derivatives along it
 template <class T>
-LCDM_HD void core_tangent(const RowRoots& r, int k, double dA, double dB, double dpr, double dpi, T* rec) {
+LCDM_HD void core_tangent(const RowRoots& r, bool time, int k, double dA, double dB, double dpr, double dpi, T* rec) {
     T* t = rec + C_TAN + C_TSTRIDE * k;
     const RowDir d = row_dir(r.ncol, k);
     const double Oks = r.Ok + r.Os, iS0 = r.iS0, eps = r.eps;
@@ -190,7 +210,6 @@ LCDM_HD void core_tangent(const RowRoots& r, int k, double dA, double dB, double
         put(t, CT_QR, dpr * (r.q1 * r.q1));
         put(t, CT_QI, dpi * (r.q2 * r.q2));
     }
-    // the third-kind integral's constants in double
     typedef Dual<double, 1> D;
     D Om, OL, Or, c, Ox, is, ep;
     Om.v = r.Om; Om.d[0] = d.dOm;
@@ -199,26 +218,32 @@ LCDM_HD void core_tangent(const RowRoots& r, int k, double dA, double dB, double
     c.v = Oks; c.d[0] = d.dOk;
     Ox.v = r.Ox; Ox.d[0] = d.dOx;
     is.v = iS0; is.d[0] = -d.dS * iS0 * iS0;
-    ep.v = eps; ep.d[0] = r.quartic ? dA * (eps * eps) : 0.0;
-    const D g1 = Ox - ep * OL, g2 = c - ep * g1, g3 = Om - ep * g2;
-    const D kk = (ep * (g2 - ep * (g1 - ep * OL)) - g3) * is;
-    put(t, CT_EPS, ep.d[0]);
-    put(t, CT_K2, kk.d[0] * (1.0 / 3));
-    put(t, CT_K3, (OL * is).d[0]);
     // the series in the record's precision
     typedef Dual<T, 1> F;
     auto to = [](const D& x) { F f; f.v = (T)x.v; f.d[0] = (T)x.d[0]; return f; };
-    const F fm = to(Om), fl = to(OL), fr = to(Or), fc = to(c), fx = to(Ox), fs = to(is), fe = to(ep), f1 = to(g1), f2 = to(g2);
+    const F fm = to(Om), fl = to(OL), fr = to(Or), fc = to(c), fx = to(Ox), fs = to(is);
     const F I = fr * fl * cst<T>(12.0) - fm * fx * cst<T>(3.0) + fc * fc;
     const F J = fc * fc * fc * cst<T>(2.0) - fm * fc * fx * cst<T>(9.0) + fr * fx * fx * cst<T>(27.0)
                 + fm * fm * fl * cst<T>(27.0) - fr * fc * fl * cst<T>(72.0);
     const F e2 = I * fs * fs * cst<T>(-1.0 / 3), e3 = J * fs * fs * fs * cst<T>(-1.0 / 27);
-    F b[6], a[6];
+    F b[CORE_NS];
     rf_coefs<F>(e2, e3, b);
-    for (int j = 0; j < 6; j++) t[CT_B2 + j] = b[j].d[0];
-    const F m = (f2 + fe * (fe * fl * cst<T>(3.0) - f1 * cst<T>(2.0))) * fs * cst<T>(1.0 / 3);
-    rj_coefs<F>(m, e2, e3, a);
-    for (int j = 0; j < 6; j++) t[CT_A2 + j] = a[j].d[0];
+#pragma unroll
+    for (int j = 0; j < CORE_NS; j++) t[CT_B + j] = b[j].d[0];
+    if (time) {
+        // the third-kind integral's constants in double
+        ep.v = eps; ep.d[0] = r.quartic ? dA * (eps * eps) : 0.0;
+        const D g1 = Ox - ep * OL, g2 = c - ep * g1, g3 = Om - ep * g2;
+        const D kk = (ep * (g2 - ep * (g1 - ep * OL)) - g3) * is;
+        put(t, CT_EPS, ep.d[0]);
+        put(t, CT_K2, kk.d[0] * (1.0 / 3));
+        put(t, CT_K3, (OL * is).d[0]);
+        const F fe = to(ep), f1 = to(g1), f2 = to(g2);
+        const F m = (f2 + fe * (fe * fl * cst<T>(3.0) - f1 * cst<T>(2.0))) * fs * cst<T>(1.0 / 3);
+        rj_coefs<F>(m, e2, e3, b);
+#pragma unroll
+        for (int j = 0; j < CORE_NS; j++) t[CT_A + j] = b[j].d[0];
+    }
     put(t, CT_END, 0.0);
 }
 

@@ -801,9 +801,9 @@ __device__ __noinline__ void legacy_record(const RowRoots& r, const cd (*dr)[RF_
 // The core's record of one cosmology: lane 0 of the group writes the values,
 // lane k mod G the tangents of direction k.
 template <int G, class T>
-__device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, bool absorb, bool tangents, T* rec) {
+__device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, bool time, bool absorb, bool tangents, T* rec) {
     if (lane == 0) {
-        core_values<T>(r, absorb, rec);
+        core_values<T>(r, time, absorb, rec);
         const double iH0 = r.H0 < 1e-280 ? ddiv(1.0, r.H0) : rcp_(r.H0);
         put(rec, C_DH, LCDM_C_KMS * iH0);
         put(rec, C_TH, LCDM_HUBBLE_GYR * iH0);
@@ -813,7 +813,7 @@ __device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, b
     const int b = r.quartic ? 1 : 0;
     #pragma unroll 1
     for (int k = lane; k < r.ncol - 1; k += G)
-        core_tangent<T>(r, k, dr[0][k].re, dr[b][k].re, dr[b + 1][k].re, r.cpair ? dr[b + 1][k].im : dr[b + 2][k].re,
+        core_tangent<T>(r, time, k, dr[0][k].re, dr[b][k].re, dr[b + 1][k].re, r.cpair ? dr[b + 1][k].im : dr[b + 2][k].re,
                         rec);
 }
 
@@ -822,6 +822,7 @@ struct PrepArgs {
     int64_t B;
     int ncol;
     int tangents;           // the root derivatives are needed
+    int time;               // the time coordinate's constants are needed
     int absorb;             // the absorption distance's constants are needed
     double* recD;           // [B][NREC] record of the X-tangent kernel, and its (hi, lo) copy (optional)
     float2* recF;
@@ -862,8 +863,8 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
     }
     if (st == ST_OK && (a.coreF || a.coreD)) {
         r.finish();
-        if (a.coreF) write_core<G, float>(r, dr, j, a.absorb, a.tangents, a.coreF + b * NCORE);
-        else write_core<G, double>(r, dr, j, a.absorb, a.tangents, a.coreD + b * NCORE);
+        if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, a.tangents, a.coreF + b * NCORE);
+        else write_core<G, double>(r, dr, j, a.time, a.absorb, a.tangents, a.coreD + b * NCORE);
     }
     if (j != 0) return;
     a.status[b] = st;
