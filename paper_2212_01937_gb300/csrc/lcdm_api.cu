@@ -118,6 +118,9 @@ struct Plan {
     PairArgs args;
     const void* core;       // the core's records
     void* grad_z;           // [npairs] derivatives with respect to the redshifts, optional
+    const float4* rowf;     // general limits: the rows' maps (null: limits from 0)
+    const double* z1;
+    const double* scale;
     int legacy;             // the tangent launch is the X-tangent kernel's
     int time, absorb;       // the core's records need the constants of t, of the absorption distance
     int prec, K, wt, wx;
@@ -149,6 +152,8 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     a.recF = cv.recF;
     P.core = cv.core;
     P.grad_z = nullptr;
+    P.rowf = nullptr;
+    P.z1 = P.scale = nullptr;
     a.part = cv.part;
     a.wrow = cv.wrow;
     a.det_cap = cv.part ? (int64_t)det_warps() : 0;
@@ -203,17 +208,28 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
 lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s);
 
 // index of the plan's kernel in its table (4 and up: per-pair Jacobians, 8 and
-// up: with the redshift derivatives)
+// up: with the redshift derivatives, 10 and up: general limits)
 int entry_index(const Plan& P) {
     bool jac = false;
     for (int i = 0; i < LCDM_NOUT; i++) jac = jac || P.args.jac[i];
+    if (P.rowf) return 10 + (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
     if (P.grad_z && !P.wx && !P.legacy) return 8 + (P.wt ? 1 : 0);
     return (P.wt ? 2 : 0) + (P.wx ? 1 : 0) + (jac ? 4 : 0);
+}
+CoreArgs core_args(const Plan& P) {
+    CoreArgs c;
+    c.p = P.args;
+    c.rec = P.core;
+    c.grad_z = P.grad_z;
+    c.rowf = P.rowf;
+    c.z1 = P.z1;
+    c.scale = P.scale;
+    return c;
 }
 const PairsEntry& plan_entry(const Plan& P) {
     const int i = entry_index(P);
     const PairsTable& t = table(P.prec, P.K);
-    return i < 4 ? t.e[i] : i < 8 ? t.jac[i - 4] : t.dz[i - 8];
+    return i < 4 ? t.e[i] : i < 8 ? t.jac[i - 4] : i < 10 ? t.dz[i - 8] : t.bt[i - 10];
 }
 
 }  // namespace
@@ -345,7 +361,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     int64_t grid = (need_warps * 32 + block - 1) / block;
     if (grid < 1) grid = 1;
     if (P.npairs == 0) return LCDM_OK;
-    cudaError_t e = t.launch(P.args, P.core, P.grad_z, (int)grid, block, s);
+    cudaError_t e = t.launch(core_args(P), (int)grid, block, s);
     g_launches++;
     if (e != cudaSuccess) return LCDM_ERR_CUDA;
     if (P.args.part && (P.args.grad || P.args.loglike)) {
@@ -356,11 +372,13 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     return e == cudaSuccess ? LCDM_OK : LCDM_ERR_CUDA;
 }
 
+int core_ns(int prec) { return prec == 0 ? (int)CoreTol<double>::ns : (int)CoreTol<float>::ns; }
 // What a call's records hold.
 struct PrepNeed {
     bool legacy;     // the X-tangent kernel's records, else the core's
     int prec;        // precision of the core's records
     bool tangents, time, absorb;
+    int ns;          // series coefficients of the core's records
 };
 
 lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv, const PrepNeed& need,
@@ -375,6 +393,7 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
     a.B = B;
     a.ncol = opts->ncol;
     a.tangents = need.tangents;
+    a.ns = need.ns;
     a.time = need.time;
     a.absorb = need.absorb;
     a.recD = need.legacy ? cv.recD : nullptr;
@@ -404,7 +423,7 @@ lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_
     lcdm_status st;
     const bool dz = separate_dz(P);
     if (P.split_mask || dz || !P.legacy) {
-        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.time != 0, P.absorb != 0};
+        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.time != 0, P.absorb != 0, core_ns(P.prec)};
         st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
         if (st != LCDM_OK) return st;
     }
@@ -417,7 +436,7 @@ lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_
         if (st != LCDM_OK) return st;
     }
     if (P.legacy) {
-        const PrepNeed need = {true, P.prec, true, true, true};
+        const PrepNeed need = {true, P.prec, true, true, true, 0};
         st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
         if (st != LCDM_OK) return st;
     }
@@ -651,34 +670,42 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
     o4.ncol = 4;
     st = between_setup(params, B, z1, ncol, w, stream);
     if (st != LCDM_OK) return st;
+    Plan P;
+    make_plan(w.params4, B, offsets, z2, n, out, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad ? w.gradp : nullptr,
+              nullptr, cosmo_status, &o4, w.rec, P);
     PairMapArgs m;
     memset(&m, 0, sizeof(m));
-    m.offsets = opts->layout == LCDM_LAYOUT_CSR ? offsets : nullptr;
-    m.nrow = n;
-    m.nnz = npairs;
-    m.B = B;
-    m.fp64 = opts->precision == LCDM_FP64;
-    m.z1 = z1;
-    m.scale = w.scale;
-    m.rowf = w.rowf;
-    m.z2 = z2;
-    m.zp = w.zp;
-    const void* cotk[LCDM_NOUT] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    if (grad)
+    if (!P.legacy) {
+        P.rowf = w.rowf;
+        P.z1 = z1;
+        P.scale = w.scale;
+    } else {
+        // the kernel of X's tangents takes mapped redshifts and cotangents
+        m.offsets = opts->layout == LCDM_LAYOUT_CSR ? offsets : nullptr;
+        m.nrow = n;
+        m.nnz = npairs;
+        m.B = B;
+        m.fp64 = opts->precision == LCDM_FP64;
+        m.z1 = z1;
+        m.scale = w.scale;
+        m.rowf = w.rowf;
+        m.z2 = z2;
+        m.zp = w.zp;
+        const void* cotk[LCDM_NOUT];
         for (int i = 0; i < LCDM_NOUT; i++) {
             m.cot[i] = cot[i];
             cotk[i] = cot[i];
             if (cot[i] && w.cotp[i]) { m.cotp[i] = w.cotp[i]; cotk[i] = w.cotp[i]; }
         }
-    if (launch_pair_pre(m, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-    g_launches++;
-    Plan P;
-    make_plan(w.params4, B, offsets, w.zp, n, out, nullptr, grad ? cotk : nullptr, nullptr, 0, 1,
-              grad ? w.gradp : nullptr, nullptr, cosmo_status, &o4, w.rec, P);
+        if (launch_pair_pre(m, stream) != cudaSuccess) return LCDM_ERR_CUDA;
+        g_launches++;
+        make_plan(w.params4, B, offsets, w.zp, n, out, nullptr, cotk, nullptr, 0, 1, w.gradp, nullptr, cosmo_status, &o4,
+                  w.rec, P);
+    }
     st = run_plan(P, w.params4, B, &o4, w.rec, cosmo_status, grad ? w.gradp : nullptr, nullptr, opts->block,
                   opts->blocks_per_sm, opts->lane_map, stream);
     if (st != LCDM_OK) return st;
-    if (out) {
+    if (out && P.legacy) {
         for (int i = 0; i < LCDM_NOUT; i++) m.out[i] = out[i];
         if (launch_pair_post(m, stream) != cudaSuccess) return LCDM_ERR_CUDA;
         g_launches++;
@@ -767,7 +794,7 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     o4.ncol = 4;
     lcdm_status st = between_setup(params, B, z1, ncol, w, stream);
     if (st != LCDM_OK) return st;
-    const PrepNeed need = {false, 0, grad != nullptr, true, false};
+    const PrepNeed need = {false, 0, grad != nullptr, true, false, CORE_NS_ONCE};
     st = run_prep(w.params4, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     LimitArgs la;
@@ -850,12 +877,12 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
         make_plan(d.params, B, d.offsets, d.z, n, outs, nullptr, cot, nullptr, 0, 1, d.grad, nullptr, d.status, opts,
                   d.rec, P);
         if (P.legacy) {
-            const PrepNeed need = {true, P.prec, true, true, true};
+            const PrepNeed need = {true, P.prec, true, true, true, 0};
             st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
             if (st != LCDM_OK) return st;
         }
         if (P.split_mask || !P.legacy) {
-            const PrepNeed need = {false, P.prec, !P.legacy, P.time != 0, P.absorb != 0};
+            const PrepNeed need = {false, P.prec, !P.legacy, P.time != 0, P.absorb != 0, core_ns(P.prec)};
             st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
             if (st != LCDM_OK) return st;
         }
@@ -942,7 +969,7 @@ lcdm_status lcdm_roots(const double* params, int64_t B, const lcdm_opts* opts, d
     Carved cv;
     lcdm_status st = carve(ws, ws_bytes, B, cv);
     if (st != LCDM_OK) return st;
-    const PrepNeed need = {true, 0, true, true, false};
+    const PrepNeed need = {true, 0, true, true, false, 0};
     st = run_prep(params, B, opts, cv, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     extract_roots<<<(unsigned)((B + 127) / 128), 128, 0, stream>>>(cv.recD, B, opts->ncol, roots, droots, kind);
@@ -1015,7 +1042,7 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
                 for (int rep = 0; rep < 3; rep++) {
                     // (the preparation is not timed, but where it comes between the launches)
                     const bool both = P.legacy && P.split_mask;
-                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.time != 0, P.absorb != 0};
+                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.time != 0, P.absorb != 0, core_ns(P.prec)};
                     if (!both && run_prep(params, B, opts, cv, need, cosmo_status, grad, nullptr, stream) != LCDM_OK)
                         return LCDM_ERR_CUDA;
                     cudaEventRecord(e0, stream);

@@ -61,7 +61,9 @@ enum CoreField {
     CT_QA = 0, CT_QB, CT_QR, CT_QI, CT_B, CT_EPS = 14, CT_K2, CT_K3, CT_A = 17, CT_END = 27,
     NCORE = C_TAN + 6 * C_TSTRIDE
 };
-enum { CORE_NS = 10 };   // series coefficients in the record: degrees 2 to 11
+enum { CORE_NS = 10 };       // room for the series' coefficients in the record: degrees 2 to 11
+enum { CORE_NS_ONCE = 6 };   // used where a record serves one evaluation (the limit at infinity): there the
+                             // coefficients and their tangents cost more than the steps they save
 
 // ------------------------------------------------------------- arithmetic ---
 // 1/sqrt, sqrt and 1/x of positive normal numbers.  Single precision: the
@@ -121,11 +123,11 @@ template <> struct CoreTol<float> {
     // largest deviation left to the series of degree ns + 1 (its truncation:
     // about dup^(ns + 2) / 100); relative deviation s of R_C's; largest z taken
     // without scaling
-    static constexpr float dup = 0.25f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
+    static constexpr float dup = 0.25f, once = 0.15f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
     enum { maxit = 24, ns = 8 };
 };
 template <> struct CoreTol<double> {
-    static constexpr double dup = 0.05, rc = 0.008, big = 1e30, e_series = 0.03;
+    static constexpr double dup = 0.05, once = 0.009, rc = 0.008, big = 1e30, e_series = 0.03;
     enum { maxit = 40, ns = 10 };
 };
 
@@ -275,8 +277,7 @@ LCDM_HD Quad<double> quad(const double* p) {
 // A closing series 1 + w^2 (c_2 + c_3 w + ...) from ns coefficients at rec[i],
 // i = 0 or 1 modulo 4, and with it (D) the derivative of the bracket.
 template <class T> struct SerVal { T v, d; };
-template <bool D, class T> LCDM_HD SerVal<T> series(const T* rec, int i, T w) {
-    constexpr int N = CoreTol<T>::ns;
+template <bool D, int N, class T> LCDM_HD SerVal<T> series(const T* rec, int i, T w) {
     T c[12];
     const int skip = i & 3;
 #pragma unroll
@@ -315,6 +316,7 @@ template <class T, bool REV, bool WT> struct CoreTape {
 // the radiationless case n_A = 0: that term falls off like z^-1/2).
 template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair {
     typedef CoreTape<T, REV, WT> Tape;
+    enum { NS = INF ? (int)CORE_NS_ONCE : (int)CoreTol<T>::ns };
     const T* rc;
     T z, zh, z2, h, cz;
     bool cplx, big;
@@ -426,7 +428,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             dX = -(kX.v[0] * z2) * piX;
         }
         T pX = p0;
-        const float it = (float)(1.0 / CoreTol<T>::dup), z2f = (float)z2 * it;
+        const float it = (float)(1.0 / (INF ? CoreTol<T>::once : CoreTol<T>::dup)), z2f = (float)z2 * it;
         const float dF = (float)rc[C_DF] * z2f * 3.0f, dJ = WT ? (float)kT.v[0] * z2f * 5.0f : 0.0f;
         const float dD = WX ? (float)kX.v[3] * z2f * 5.0f : 0.0f;
         T S1 = s1;
@@ -486,7 +488,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T A = T3 * cst<T>(1.0 / 3);
             rF = rsq(A);
             wF = z2 * (rF * rF);
-            const T s = series<false>(rc, C_B, wF).v;
+            const T s = series<false, NS>(rc, C_B, wF).v;
             sF = one + s * (wF * wF);
             RF = tm * sF * rF;
         }
@@ -496,7 +498,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T A = (T3 + p + p) * cst<T>(0.2);
             rJ = rsq(A);
             wJ = z2 * (rJ * rJ);
-            const T s = series<false>(rc, C_A, wJ).v;
+            const T s = series<false, NS>(rc, C_A, wJ).v;
             sJs = one + s * (wJ * wJ);
             RJ = tm * sJs * (rJ * rJ * rJ) + cst<T>(6.0) * sJ;
             // R_C(s5, p), Carlson's duplication on the square roots a = sqrt(s5), b = sqrt(p)
@@ -642,7 +644,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             }
             p_ = b_ * half * rcp_(bx);                    // b = sqrt(p)
             // R_J: closing series
-            const SerVal<T> sv2 = series<true>(rc, C_A, wJ);
+            const SerVal<T> sv2 = series<true, NS>(rc, C_A, wJ);
             const T s = sv2.v, s2 = sv2.d;
             const T r2 = rJ * rJ, c = RJ_ * tm * r2 * rJ;
             bJ_ = c;
@@ -654,7 +656,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             pf_ = A_ * cst<T>(0.4);
         }
         {
-            const SerVal<T> sv2 = series<true>(rc, C_B, wF);
+            const SerVal<T> sv2 = series<true, NS>(rc, C_B, wF);
             const T s = sv2.v, s2 = sv2.d;
             const T c = RF_ * tm * rF;
             bF_ = c;
@@ -759,10 +761,10 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     LCDM_HD T along(int k) const {
         const T* t = rc + C_TAN + C_TSTRIDE * k;
         const Quad<T> t0 = quad(t);
-        const T b = series<false>(t, CT_B, wF).v;
+        const T b = series<false, NS>(t, CT_B, wF).v;
         T r = qA_ * t0.v[0] + qB_ * t0.v[1] + (qR_ * t0.v[2] + qI_ * t0.v[3]) + bF_ * (wF * wF) * b;
         if (WT) {
-            const T a = series<false>(t, CT_A, wJ).v;
+            const T a = series<false, NS>(t, CT_A, wJ).v;
             r = r + (eps_ * t[CT_EPS] + k2_ * t[CT_K2] + k3_ * t[CT_K3]) + bJ_ * (wJ * wJ) * a;
         }
         return r;

@@ -66,17 +66,46 @@ __device__ __forceinline__ void acc_add(df64& a, float c) {
     a = mkdf(s.hi, LCDM_FADD(a.lo, s.lo));
 }
 
+// The map of a general-limits row: z' = (z2 - z1) / s.  Single precision: hi is
+// exact near z1 (Sterbenz), and its sign decides the domain test; lo is z1 - hi
+// rounded, which keeps the sign of the tie z2 == hi.
+template <class T> struct LimitMap;
+template <> struct LimitMap<float> {
+    float hi, lo, is, s;
+    __device__ __forceinline__ void load(const float4* rowf, const double*, const double*, int row) {
+        const float4 r = __ldg(rowf + row);
+        hi = r.x; lo = r.y; is = r.z; s = r.w;
+    }
+    __device__ __forceinline__ float dz(float z2) const { return (z2 - hi) - lo; }
+    __device__ __forceinline__ float zp(float d) const { return d * is; }
+};
+template <> struct LimitMap<double> {
+    double z1, s;
+    __device__ __forceinline__ void load(const float4*, const double* z1s, const double* scale, int row) {
+        z1 = __ldg(z1s + row); s = __ldg(scale + row);
+    }
+    __device__ __forceinline__ double dz(double z2) const { return z2 - z1; }
+    __device__ __forceinline__ double zp(double d) const { return d / s; }
+};
+
 struct CoreArgs {
     PairArgs p;
     const void* rec;    // [B][NCORE]
     void* grad_z;       // [nnz] derivative with respect to each pair's redshift, optional
+    const float4* rowf; // [B] (z1 hi, z1 lo, 1/s, s) of general limits (single precision)
+    const double* z1;   // [B] lower limits, s = 1 + z1 (double precision)
+    const double* scale;
 };
 
 // What a kernel produces beside the outputs: the per-row sums (of cotangents
 // times derivatives, or of the log-likelihood), per-pair Jacobians, or the
 // sums and the derivatives with respect to each redshift.  (Kernels of their
 // own: the redshift derivatives cost the others 4 % in registers.)
-enum CoreMode { CORE_SUM = 0, CORE_JAC = 1, CORE_DZ = 2 };
+// CORE_BETWEEN: the sums, for pairs given by an upper limit z2 above the row's
+// own lower limit (general limits, lcdm_between.cuh): z' = (z2 - z1) / s, the
+// outputs' factors and the domain test z2 >= z1 are applied here.  (Two maps
+// over the pairs did that before: 0.04 ms of the 0.15 ms of 4 M values.)
+enum CoreMode { CORE_SUM = 0, CORE_JAC = 1, CORE_DZ = 2, CORE_BETWEEN = 3 };
 
 // registers per thread: blocks of 256 threads per SM the compiler aims at
 template <int PREC, int K, bool WT, bool WX, int MODE>
@@ -84,7 +113,7 @@ struct CoreBlocks { enum { value = PREC == 1 ? (K == 0 ? (WX ? 3 : 4) : (MODE ==
 
 template <int PREC, int K, bool WT, bool WX, int MODE>
 __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value) core_kernel(CoreArgs ca) {
-    constexpr bool JAC = MODE == CORE_JAC, DZ = MODE == CORE_DZ;
+    constexpr bool JAC = MODE == CORE_JAC, DZ = MODE == CORE_DZ, BT = MODE == CORE_BETWEEN;
     typedef typename std::conditional<PREC == 0, double, float>::type T;
     typedef typename std::conditional<PREC == 0, double, df64>::type AccT;
     constexpr int NV = K + 2;   // H0, K density directions, log-likelihood
@@ -126,6 +155,7 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
     int row = -1, rend = INT32_MIN, zoff = 0;   // the lane's row, its end, and what takes a pair to its redshift (shared)
     const T* rec = nullptr;
     int st = 0;
+    LimitMap<T> lm;
     // outputs that need the curvature map
     const bool map = loglike || (a.outmask & ((1 << O_DM) | (1 << O_DL) | (1 << O_MU))) ||
                      ((K > 0 || DZ) && (a.cot[O_DM] || a.cot[O_DL] || a.cot[O_MU] || a.jac[O_DM] || a.jac[O_DL] || a.jac[O_MU]));
@@ -165,9 +195,16 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
             rend = e < INT32_MAX ? (int)e : INT32_MAX;
             rec = reinterpret_cast<const T*>(ca.rec) + (int64_t)row * NCORE;
             st = a.status[row];
+            if (BT) lm.load(ca.rowf, ca.z1, ca.scale, row);
         }
         const int64_t zi = a.layout == LAYOUT_SHARED ? o - (int64_t)zoff * a.nrow : o;
-        const T z = __ldg(zs + zi);
+        T z = __ldg(zs + zi);
+        bool inside = true;   // (an interval with z2 < z1 gives NaN and adds nothing)
+        if (BT) {
+            const T d = lm.dz(z);
+            inside = d >= (T)0;
+            z = inside ? lm.zp(d) : (T)0;
+        }
         T gcot[N_OUT];
         T mob = (T)0;
         if constexpr (K > 0 && !JAC) {
@@ -200,11 +237,16 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
             v[O_DM] = DH * S;
             v[O_DL] = z1 * v[O_DM];
             v[O_MU] = want_mu ? mu_of(v[O_DL]) : (T)0;
-            if (fail) {
+            if (BT) {
+                v[O_DC] = v[O_DC] * lm.s;
+                v[O_DM] = v[O_DM] * lm.s;
+                v[O_X] = v[O_X] * (lm.s * lm.s * lm.s);
+            }
+            if (fail || (BT && !inside)) {
                 const T nan = (T)CUDART_NAN;
 #pragma unroll
                 for (int i = 0; i < N_OUT; i++) v[i] = nan;
-                if (active) atomicMax(a.status + row, (int)ST_NOCONV);
+                if (fail && active) atomicMax(a.status + row, (int)ST_NOCONV);
             }
             if (active) {
 #pragma unroll
@@ -268,7 +310,7 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
                 }
                 continue;
             }
-            if (reduce && active && !fail) {
+            if (reduce && active && !fail && inside) {
                 T lin = 0, gm = 0;   // cotangent sums: of H0's linear outputs, of mu
                 T ci = 0, cs = 0, ti = 0;
                 if (loglike) {
@@ -278,11 +320,18 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
                 }
                 if constexpr (K > 0) {
                     if (!loglike) {
+                        if (BT) {
+                            // (v holds the scaled outputs: their sum below keeps the plain cotangents)
+                            lin = gcot[O_DC] * v[O_DC] + gcot[O_DM] * v[O_DM];
+                            gcot[O_DC] = gcot[O_DC] * lm.s;
+                            gcot[O_DM] = gcot[O_DM] * lm.s;
+                        }
                         gm = gcot[O_MU];
                         cs = DH * (gcot[O_DM] + z1 * gcot[O_DL]);
                         ci = DH * gcot[O_DC];
                         if (WT) ti = tH * gcot[O_T];
-                        lin = gcot[O_DC] * v[O_DC] + gcot[O_DM] * v[O_DM] + gcot[O_DL] * v[O_DL];
+                        if (!BT) lin = gcot[O_DC] * v[O_DC] + gcot[O_DM] * v[O_DM];
+                        lin = lin + gcot[O_DL] * v[O_DL];
                         if (WT) lin = lin + gcot[O_T] * v[O_T];
                     }
                     c[0] = -(lin + c5 * gm) * iH0;

@@ -40,7 +40,7 @@ LCDM_HD RowDir row_dir(int ncol, int k) {
     return d;
 }
 
-// The closing series' coefficients, degrees 2 to 11 (single-precision records:
+// The closing series' ns <= 10 coefficients from degree 2 (single-precision records:
 // in single precision; they enter the results times the squared deviation and
 // higher powers, at most a twentieth).  With the arguments' deviations X_i from
 // their mean (sum 0) the series are sum_N c_N T_N, c_N = 1/(2N+1) for R_F and
@@ -51,13 +51,14 @@ template <class S> struct SeriesBase { typedef typename Base<S>::type type; };
 template <class T> struct SeriesBase<DD<T> > { typedef T type; };
 template <class S> LCDM_HD S zero_like(const S& a) { return a * typename SeriesBase<S>::type(0); }
 // R_F: b_2 .. b_11 from (e2, e3)
-template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, S* b) {
+template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, int ns, S* b) {
     typedef typename SeriesBase<S>::type B;
     S t[CORE_NS + 2];
     t[0] = zero_like(e2) + B(1);
     t[1] = zero_like(e2);
 #pragma unroll
     for (int n = 2; n < CORE_NS + 2; n++) {
+        if (n >= ns + 2) break;
         S v = t[n - 2] * e2 * B(-(n - 1.0) / n);
         if (n >= 3) v = v + t[n - 3] * e3 * B((n - 1.5) / n);
         t[n] = v;
@@ -65,7 +66,7 @@ template <class S> LCDM_HD void rf_coefs(const S& e2, const S& e3, S* b) {
     }
 }
 // R_J: a_2 .. a_11; m = (mean of three - p) / z^2
-template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, S* a) {
+template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, int ns, S* a) {
     typedef typename SeriesBase<S>::type B;
     const S m2 = m * m;
     const S E2 = e2 - m2 * B(0.6);
@@ -79,6 +80,7 @@ template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, S
     t[1] = zero_like(E2);
 #pragma unroll
     for (int n = 2; n < CORE_NS + 2; n++) {
+        if (n >= ns + 2) break;
         S v = t[n - 2] * E2 * B(-(n - 1.0) / n);
         if (n >= 3) v = v + t[n - 3] * E3 * B((n - 1.5) / n);
         if (n >= 4) v = v - t[n - 4] * E4 * B((n - 2.0) / n);
@@ -103,7 +105,7 @@ LCDM_HD void put_lo(float* rec, int i, double v) { rec[i] = (float)(v - (double)
 LCDM_HD void put_lo(double* rec, int i, double) { rec[i] = 0.0; }
 
 // values (directions are added by core_tangent)
-template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool absorb, T* rec) {
+template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool absorb, int ns, T* rec) {
     const double Oks = r.Ok + r.Os, S0 = r.S0, iS0 = r.iS0, sS = r.ncol == 4 ? 1.0 : sqrt(S0), isS = sS * iS0;
     const double qA = r.qA, qB = r.qB, q1 = r.q1, q2 = r.q2, eps = r.eps;
     put(rec, C_QA, qA); put(rec, C_QB, qB);
@@ -121,9 +123,10 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
     const double e2 = I * (-1.0 / 3) * (iS0 * iS0), e3 = J * (-1.0 / 27) * (iS0 * iS0 * iS0);
     const T f2 = (T)e2, f3 = (T)e3;
     T b[CORE_NS];
-    rf_coefs<T>(f2, f3, b);
+    rf_coefs<T>(f2, f3, ns, b);
 #pragma unroll
-    for (int j = 0; j < CORE_NS; j++) rec[C_B + j] = b[j];
+    for (int j = 0; j < CORE_NS; j++)
+        if (j < ns) rec[C_B + j] = b[j];
     const float d3 = dev3(e2, e3);
     rec[C_DF] = (T)d3;
     if (time) {
@@ -134,9 +137,10 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
         put(rec, C_EPS, eps);
         put(rec, C_K2, k * (1.0 / 3));
         put(rec, C_K3, r.OL * iS0);
-        rj_coefs<T>((T)m, f2, f3, b);
+        rj_coefs<T>((T)m, f2, f3, ns, b);
 #pragma unroll
-        for (int j = 0; j < CORE_NS; j++) rec[C_A + j] = b[j];
+        for (int j = 0; j < CORE_NS; j++)
+            if (j < ns) rec[C_A + j] = b[j];
         rec[C_DJ] = (T)dev5(d3, m);
     }
     if (!absorb) return;
@@ -183,9 +187,10 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
     else { put(rec, X_SQ, q1 + q2); put(rec, X_PQ, q1 * q2); }
     // the series at p0 (offset X1 + hx) and at x1 (offset X1), and their divided differences
     DD<T> ad[CORE_NS];
-    rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx), (T)X1, (T)1), mkdd<T>(f2, f2, (T)0), mkdd<T>(f3, f3, (T)0), ad);
+    rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx), (T)X1, (T)1), mkdd<T>(f2, f2, (T)0), mkdd<T>(f3, f3, (T)0), ns, ad);
 #pragma unroll
     for (int j = 0; j < CORE_NS; j++) {
+        if (j >= ns) break;
         rec[X_S + 3 * j] = ad[j].v1;
         rec[X_S + 3 * j + 1] = ad[j].v2;
         rec[X_S + 3 * j + 2] = ad[j].d;
@@ -195,7 +200,7 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
 
 // tangents of direction k; dA, dB, (dpr, dpi): the roots' derivatives along it
 template <class T>
-LCDM_HD void core_tangent(const RowRoots& r, bool time, int k, double dA, double dB, double dpr, double dpi, T* rec) {
+LCDM_HD void core_tangent(const RowRoots& r, bool time, int ns, int k, double dA, double dB, double dpr, double dpi, T* rec) {
     T* t = rec + C_TAN + C_TSTRIDE * k;
     const RowDir d = row_dir(r.ncol, k);
     const double Oks = r.Ok + r.Os, iS0 = r.iS0, eps = r.eps;
@@ -227,9 +232,10 @@ LCDM_HD void core_tangent(const RowRoots& r, bool time, int k, double dA, double
                 + fm * fm * fl * cst<T>(27.0) - fr * fc * fl * cst<T>(72.0);
     const F e2 = I * fs * fs * cst<T>(-1.0 / 3), e3 = J * fs * fs * fs * cst<T>(-1.0 / 27);
     F b[CORE_NS];
-    rf_coefs<F>(e2, e3, b);
+    rf_coefs<F>(e2, e3, ns, b);
 #pragma unroll
-    for (int j = 0; j < CORE_NS; j++) t[CT_B + j] = b[j].d[0];
+    for (int j = 0; j < CORE_NS; j++)
+        if (j < ns) t[CT_B + j] = b[j].d[0];
     if (time) {
         // the third-kind integral's constants in double
         ep.v = eps; ep.d[0] = r.quartic ? dA * (eps * eps) : 0.0;
@@ -240,9 +246,10 @@ LCDM_HD void core_tangent(const RowRoots& r, bool time, int k, double dA, double
         put(t, CT_K3, (OL * is).d[0]);
         const F fe = to(ep), f1 = to(g1), f2 = to(g2);
         const F m = (f2 + fe * (fe * fl * cst<T>(3.0) - f1 * cst<T>(2.0))) * fs * cst<T>(1.0 / 3);
-        rj_coefs<F>(m, e2, e3, b);
+        rj_coefs<F>(m, e2, e3, ns, b);
 #pragma unroll
-        for (int j = 0; j < CORE_NS; j++) t[CT_A + j] = b[j].d[0];
+        for (int j = 0; j < CORE_NS; j++)
+            if (j < ns) t[CT_A + j] = b[j].d[0];
     }
     put(t, CT_END, 0.0);
 }

@@ -5,16 +5,16 @@
 
 namespace lcdm {
 
-// One pair kernel: its launch and its resident blocks per SM.  `rec` is the
-// core's record; the kernel of X's tangents reads the records in the arguments.
+// One pair kernel: its launch and its resident blocks per SM.  (The kernel of
+// X's tangents reads the records in PairArgs.)
 struct PairsEntry {
-    cudaError_t (*launch)(const PairArgs& a, const void* rec, void* grad_z, int grid, int block, cudaStream_t s);
+    cudaError_t (*launch)(const CoreArgs& a, int grid, int block, cudaStream_t s);
     int (*occ)(int block);
 };
 
 template <int PREC, int K, bool WT> struct TangentX {
-    static cudaError_t launch(const PairArgs& a, const void*, void*, int grid, int block, cudaStream_t s) {
-        pairs_kernel<PREC, K, WT, true><<<grid, block, 0, s>>>(a);
+    static cudaError_t launch(const CoreArgs& a, int grid, int block, cudaStream_t s) {
+        pairs_kernel<PREC, K, WT, true><<<grid, block, 0, s>>>(a.p);
         return cudaGetLastError();
     }
     static int occ(int block) {
@@ -25,11 +25,7 @@ template <int PREC, int K, bool WT> struct TangentX {
     }
 };
 template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
-    static cudaError_t launch(const PairArgs& a, const void* rec, void* grad_z, int grid, int block, cudaStream_t s) {
-        CoreArgs c;
-        c.p = a;
-        c.rec = rec;
-        c.grad_z = grad_z;
+    static cudaError_t launch(const CoreArgs& c, int grid, int block, cudaStream_t s) {
         core_kernel<PREC, K, WT, WX, MODE><<<grid, block, 0, s>>>(c);
         return cudaGetLastError();
     }
@@ -44,9 +40,11 @@ template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
 // entries by (WT ? 2 : 0) + (WX ? 1 : 0); jac: the kernels of per-pair
 // Jacobians (without X's, whose tangents have a kernel of their own); dz: those
 // that also give the redshift derivatives, by WT (four- and five-column rows;
-// of the value kernels only the one without t and X)
+// of the value kernels only the one without t and X); bt: those of general
+// limits, like e (the shifted rows have four columns, and X's tangents there go
+// through the pair maps)
 struct PairsTable {
-    PairsEntry e[4], jac[4], dz[2];
+    PairsEntry e[4], jac[4], dz[2], bt[4];
 };
 
 template <class E> PairsEntry entry() { PairsEntry e; e.launch = E::launch; e.occ = E::occ; return e; }
@@ -58,6 +56,10 @@ template <int PREC> PairsTable value_table() {
     t.e[2] = entry<Core<PREC, 0, true, false> >();
     t.e[3] = entry<Core<PREC, 0, true, true> >();
     t.dz[0] = entry<Core<PREC, 0, false, false, CORE_DZ> >();
+    t.bt[0] = entry<Core<PREC, 0, false, false, CORE_BETWEEN> >();
+    t.bt[1] = entry<Core<PREC, 0, false, true, CORE_BETWEEN> >();
+    t.bt[2] = entry<Core<PREC, 0, true, false, CORE_BETWEEN> >();
+    t.bt[3] = entry<Core<PREC, 0, true, true, CORE_BETWEEN> >();
     return t;
 }
 template <int PREC, int K> PairsTable tangent_table() {
@@ -70,6 +72,10 @@ template <int PREC, int K> PairsTable tangent_table() {
     t.jac[1] = t.e[1];
     t.jac[2] = entry<Core<PREC, K, true, false, CORE_JAC> >();
     t.jac[3] = t.e[3];
+    if constexpr (K == 3) {
+        t.bt[0] = entry<Core<PREC, K, false, false, CORE_BETWEEN> >();
+        t.bt[2] = entry<Core<PREC, K, true, false, CORE_BETWEEN> >();
+    }
     if constexpr (K < 6) {
         t.dz[0] = entry<Core<PREC, K, false, false, CORE_DZ> >();
         t.dz[1] = entry<Core<PREC, K, true, false, CORE_DZ> >();

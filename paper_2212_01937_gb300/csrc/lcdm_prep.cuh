@@ -197,6 +197,64 @@ LCDM_HD void start_points(const float* c, int n, float* zr, float* zi) {
     for (; r < 4; r++) { zr[r] = 0.5f * r + 0.1f; zi[r] = 0.3f; }  // (zero constant term etc.)
 }
 
+// Starting points in closed form, to about 1e-6: the big root of the quartic by
+// the fixed point A = -(a_3 + a_2/A + a_1/A^2 + a_0/A^3) / a_4 (it contracts by
+// a_4 a_2 / a_3^2, ~1e-4 for any realistic radiation density), the others (all
+// of a cubic's) by Cardano's formulas on the deflated cubic.  Returns false
+// where that is not good: the fixed point has not settled, the other roots are
+// not small beside A, or one of them is so small that the shift a/3 costs its
+// digits.
+LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
+    float g3 = al[3], g2 = al[2], g1 = al[1], g0 = al[0];
+    int k = 0;
+    bool good = true;
+    float A = 0.f;
+    if (n == 4) {
+        const float i4 = -1.0f / al[4];
+        A = al[3] * i4;
+        float prev = A;
+#pragma unroll
+        for (int it = 0; it < 3; it++) {
+            const float iA = 1.0f / A;
+            prev = A;
+            A = (al[3] + iA * (al[2] + iA * (al[1] + iA * al[0]))) * i4;
+        }
+        good = fabsf(A - prev) < 1e-4f * fabsf(A);
+        zr[0] = A;
+        zi[0] = 0.f;
+        k = 1;
+        const float eps = -1.0f / A;
+        g1 = al[1] - eps * g0;
+        g2 = al[2] - eps * g1;
+        g3 = al[3] - eps * g2;
+    }
+    const float i3 = 1.0f / g3, a = g2 * i3, b = g1 * i3, c = g0 * i3;
+    const float sh = a * (1.0f / 3), p3 = (b - a * sh) * (1.0f / 3), h = 0.5f * (c - sh * b) + sh * sh * sh;
+    const float disc = h * h + p3 * p3 * p3;
+    float r0, r1, r2, im = 0.f;
+    if (disc >= 0.f) {
+        const float w = -(h + copysignf(sqrtf(disc), h));
+        const float u = w == 0.f ? 0.f : copysignf(fexp(flog(fabsf(w)) * (1.0f / 3)), w);
+        const float v = u == 0.f ? 0.f : -p3 / u;
+        r0 = (u + v) - sh;
+        r1 = r2 = -0.5f * (u + v) - sh;
+        im = 0.8660254f * fabsf(u - v);
+    } else {
+        const float m = sqrtf(-p3), q = fminf(1.0f, fmaxf(-1.0f, -h / (m * m * m))), th = acosf(q) * (1.0f / 3);
+        r0 = 2.0f * m * fcos(th) - sh;
+        r1 = 2.0f * m * fcos(th + 2.0943951f) - sh;
+        r2 = 2.0f * m * fcos(th - 2.0943951f) - sh;
+    }
+    zr[k] = r0; zi[k] = 0.f;
+    zr[k + 1] = r1; zi[k + 1] = im;
+    zr[k + 2] = r2; zi[k + 2] = -im;
+    if (n == 3) { zr[3] = 0.f; zi[3] = 0.f; }
+    const float q0 = fabsf(r0), q1 = fabsf(r1) + im, q2 = fabsf(r2) + im;
+    const float lo = fminf(q0, fminf(q1, q2)), hi = fmaxf(q0, fmaxf(q1, q2));
+    // (false for anything not finite, too)
+    return good && lo > 1e-2f * (fabsf(sh) + hi) && (n == 3 ? hi < 1e18f : hi < 0.05f * fabsf(A));
+}
+
 // Roots of the monic polynomial c (degree n <= 4) by the simultaneous
 // Aberth-Ehrlich iteration, G lanes per polynomial (G = 1 or 4): lane s of a
 // group of G consecutive lanes owns roots s, s + G, ... and reads the others'
@@ -209,7 +267,10 @@ LCDM_HD void start_points(const float* c, int n, float* zr, float* zi) {
 // On this part every FP64 instruction of a warp holds its sub-partition for
 // 64 cycles (19 per SM when all four issue), whatever the number of active
 // lanes or independent operations, so what counts is the number of FP64
-// instructions.  Hence: single precision first, to about 1e-6; then sweeps in
+// instructions.  Hence: single precision first, to about 1e-6, in closed form
+// where that is good and by the iteration from Newton-polygon circles where it
+// is not (its six to nine sweeps of 250 instructions were most of the kernel's
+// time); then sweeps in
 // which only what decides the accuracy is double, the polynomial's and its
 // derivative's values (26 instructions) and the differences of the roots; the
 // correction itself, a number known to 1e-7 of its size, is single.  A sweep
@@ -239,8 +300,18 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
         usual = usual && fabsf(cf[k]) < 1e6f;
     }
     usual = usual && fabsf(cf[0]) > 1e-20f;
-    float st_r[4], st_i[4];
-    start_points(cf, n, st_r, st_i);
+    float st_r[4], st_i[4], af[5];
+#pragma unroll
+    for (int k = 0; k <= 4; k++) af[k] = (float)alpha[k];
+    const bool good = usual && closed_start(af, n, st_r, st_i);
+    // (a lane beyond the last row, or of an invalid one, takes no part)
+    if (!__all_sync(full, good || !active)) {
+        float pr[4], pi[4];
+        start_points(cf, n, pr, pi);
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (!good) { st_r[k] = pr[k]; st_i[k] = pi[k]; }
+    }
 #pragma unroll
     for (int r = 0; r < R; r++) {
         zr[r] = G == 1 ? st_r[r] : (s == 0 ? st_r[0] : s == 1 ? st_r[1] : s == 2 ? st_r[2] : st_r[3]);
@@ -250,9 +321,10 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
 #pragma unroll
     for (int r = 0; r < R; r++) { zre[r] = zr[r]; zim[r] = zi[r]; }
     {
-        bool done = !active;
+        bool done = !active || good;
 #pragma unroll 1
         for (int itf = 0; itf < 100; itf++) {
+            if (__all_sync(full, done)) break;
             float ar[4], ai[4];
 #pragma unroll
             for (int k = 0; k < 4; k++) {
@@ -298,7 +370,6 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
                 small &= __shfl_xor_sync(full, small, 2, G);
             }
             if (small) done = true;
-            if (__all_sync(full, done)) break;
         }
 #pragma unroll
         for (int r = 0; r < R; r++)
@@ -468,7 +539,8 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
                 const float q = sqrtf(xr * xr + xi * xi) / mz;
                 if (!(q >= d)) d = q;
             }
-            if (!(d > near)) {
+            // (of a conjugate pair only the upper member is used)
+            if (!(d > near) && (zj.im >= 0.0)) {
                 if (d > 1e-4f) polish_once(alpha, n, zj); else polish_root(alpha, n, zj);
             }
             zre[r] = zj.re; zim[r] = zj.im;
@@ -535,43 +607,38 @@ __device__ int prep_roots(const double* p, int ncol, bool active, int tangents, 
         for (int i = 1; i < 4; i++) z[i] = cmk(0.0, 0.0);
     }
     if (st == ST_OK) {
-        // classification: real when the imaginary part is negligible (compared
+        // Classification: real when the imaginary part is negligible (compared
         // in single precision; other comparisons on the bits: a double's
-        // comparison holds the FP64 pipe like any other FP64 instruction)
-        int nreal = 0, ir[4], ic[4], ncx = 0;
-        #pragma unroll 1
-        for (int i = 0; i < n; i++) {
-            if (triple0 || negligible_im(z[i])) {   // (polished on the axis already)
+        // comparison holds the FP64 pipe like any other FP64 instruction).
+        // Reals come first, by decreasing |rho| (fn15: largest roots of
+        // E^2(z+1)), then complex ones, then the cubic's absent fourth.
+        long long key[4];
+        int nreal = 0;
+        #pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const bool real = i < n && (triple0 || negligible_im(z[i]));
+            if (real) {
                 z[i].im = 0;
-                ir[nreal++] = i;
+                nreal++;
+                if (__double_as_longlong(z[i].re) >= __double_as_longlong(1.0)) st = ST_NO_BIG_BANG;   // real root at z >= 0 (Sec. 3, Fig. 1)
             }
-            else ic[ncx++] = i;
+            key[i] = real ? __double_as_longlong(z[i].re) & INT64_MAX : i < n ? -1 : -2;
         }
-        #pragma unroll 1
-        for (int i = 0; i < nreal; i++)
-            if (__double_as_longlong(z[ir[i]].re) >= __double_as_longlong(1.0)) st = ST_NO_BIG_BANG;   // real root at z >= 0 (Sec. 3, Fig. 1)
-        // order reals by decreasing |rho| (fn15: largest roots of E^2(z+1))
-        #pragma unroll 1
-        for (int i = 0; i < nreal; i++)
-            for (int j = i + 1; j < nreal; j++)
-                if ((__double_as_longlong(z[ir[j]].re) & INT64_MAX) > (__double_as_longlong(z[ir[i]].re) & INT64_MAX)) { int t = ir[i]; ir[i] = ir[j]; ir[j] = t; }
+        auto order = [&](int i, int j) {
+            if (key[j] > key[i]) {
+                const long long t = key[i]; key[i] = key[j]; key[j] = t;
+                const cd u = z[i]; z[i] = z[j]; z[j] = u;
+            }
+        };
+        order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
+        const int ncx = n - nreal;
         cd A = cmk(0, 0), Bv = cmk(0, 0), P1 = cmk(0, 0), P2 = cmk(0, 0);
-        bool cpair = false;
-        if (n == 4 && nreal == 2 && ncx == 2) {
-            A = z[ir[0]]; Bv = z[ir[1]]; cpair = true;
-            P1 = z[ic[0]].im > 0 ? z[ic[0]] : z[ic[1]];
-            P1.im = 0.5 * (fabs(z[ic[0]].im) + fabs(z[ic[1]].im));
-            P1.re = 0.5 * (z[ic[0]].re + z[ic[1]].re);
-        } else if (n == 4 && nreal == 4) {
-            A = z[ir[0]]; Bv = z[ir[1]]; P1 = z[ir[2]]; P2 = z[ir[3]];
-        } else if (n == 3 && nreal == 1 && ncx == 2) {
-            Bv = z[ir[0]]; cpair = true;
-            P1 = z[ic[0]].im > 0 ? z[ic[0]] : z[ic[1]];
-            P1.im = 0.5 * (fabs(z[ic[0]].im) + fabs(z[ic[1]].im));
-            P1.re = 0.5 * (z[ic[0]].re + z[ic[1]].re);
-        } else if (n == 3 && nreal == 3) {
-            Bv = z[ir[0]]; P1 = z[ir[1]]; P2 = z[ir[2]];
-        } else if (st == ST_OK) {
+        const bool cpair = ncx == 2 && nreal == n - 2;
+        if (n == 4) { A = z[0]; Bv = z[1]; P1 = z[2]; P2 = z[3]; }
+        else { Bv = z[0]; P1 = z[1]; P2 = z[2]; }
+        if (cpair) {
+            if (__double_as_longlong(P1.im) < 0) P1 = P2;   // the member with the positive imaginary part
+        } else if (ncx != 0 && st == ST_OK) {
             st = ST_UNSUPPORTED;   // e.g. two complex pairs (no real root)
         }
         if (st != ST_OK && st != ST_NO_BIG_BANG) return st;
@@ -801,9 +868,10 @@ __device__ __noinline__ void legacy_record(const RowRoots& r, const cd (*dr)[RF_
 // The core's record of one cosmology: lane 0 of the group writes the values,
 // lane k mod G the tangents of direction k.
 template <int G, class T>
-__device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, bool time, bool absorb, bool tangents, T* rec) {
+__device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, bool time, bool absorb, bool tangents, int ns,
+                           T* rec) {
     if (lane == 0) {
-        core_values<T>(r, time, absorb, rec);
+        core_values<T>(r, time, absorb, ns, rec);
         const double iH0 = r.H0 < 1e-280 ? ddiv(1.0, r.H0) : rcp_(r.H0);
         put(rec, C_DH, LCDM_C_KMS * iH0);
         put(rec, C_TH, LCDM_HUBBLE_GYR * iH0);
@@ -813,7 +881,7 @@ __device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, b
     const int b = r.quartic ? 1 : 0;
     #pragma unroll 1
     for (int k = lane; k < r.ncol - 1; k += G)
-        core_tangent<T>(r, time, k, dr[0][k].re, dr[b][k].re, dr[b + 1][k].re, r.cpair ? dr[b + 1][k].im : dr[b + 2][k].re,
+        core_tangent<T>(r, time, ns, k, dr[0][k].re, dr[b][k].re, dr[b + 1][k].re, r.cpair ? dr[b + 1][k].im : dr[b + 2][k].re,
                         rec);
 }
 
@@ -822,6 +890,7 @@ struct PrepArgs {
     int64_t B;
     int ncol;
     int tangents;           // the root derivatives are needed
+    int ns;                 // series coefficients the core will use
     int time;               // the time coordinate's constants are needed
     int absorb;             // the absorption distance's constants are needed
     double* recD;           // [B][NREC] record of the X-tangent kernel, and its (hi, lo) copy (optional)
@@ -863,8 +932,8 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
     }
     if (st == ST_OK && (a.coreF || a.coreD)) {
         r.finish();
-        if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, a.tangents, a.coreF + b * NCORE);
-        else write_core<G, double>(r, dr, j, a.time, a.absorb, a.tangents, a.coreD + b * NCORE);
+        if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, a.tangents, a.ns, a.coreF + b * NCORE);
+        else write_core<G, double>(r, dr, j, a.time, a.absorb, a.tangents, a.ns, a.coreD + b * NCORE);
     }
     if (j != 0) return;
     a.status[b] = st;
