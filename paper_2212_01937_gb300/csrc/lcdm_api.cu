@@ -348,7 +348,15 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
         }
     }
     P.args.interleave = lane_map == LCDM_MAP_INTERLEAVED ? 1 : 0;
-    if (block == 0) block = 256;   // full-size blocks (the largest kernels step in lockstep, see pairs_kernel)
+    if (block == 0) {
+        // Full-size blocks (the X-tangent kernels step in lockstep, see
+        // pairs_kernel), smaller ones where those would leave SMs idle: a warp
+        // alone on its sub-partition issues an FP64 instruction every 64 cycles,
+        // one of eight on an SM every 152 (10^4 FP64 pairs: 40 blocks of 256,
+        // 20 us; 313 of 32, 10 us).
+        block = 256;
+        while (block > 32 && P.npairs < (int64_t)block * 2 * num_sms()) block /= 2;
+    }
     int occ = cached_occ(t, entry_index(P), P.prec, P.K, block);
     if (occ <= 0) return LCDM_ERR_CUDA;
     if (bps == 0 || bps > occ) bps = occ;
@@ -806,13 +814,11 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     la.age = t_inf;
     la.cot_chi = cot_chi;
     la.cot_age = cot_t;
-    la.gradp = w.gradp;
+    la.jac = w.jac;
+    la.ncol = ncol;
+    la.grad = grad;
     if (launch_limits(la, grad != nullptr, stream) != cudaSuccess) return LCDM_ERR_CUDA;
     g_launches++;
-    if (grad) {
-        if (launch_chain(w.jac, w.gradp, B, ncol, grad, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-        g_launches++;
-    }
     return LCDM_OK;
 }
 

@@ -31,7 +31,7 @@ __global__ void shift_kernel(ShiftArgs a) {
         a.rowf[b] = make_float4(nan, nan, nan, nan);
         return;
     }
-    const double iE = 1.0 / E1, rE = sqrt(E1);
+    const double irE = E1 > 1e-280 && E1 < 1e280 ? rsq(E1) : 1.0 / sqrt(E1), rE = E1 * irE, iE = irE * irE;
     const double pw[4] = {s3, 1.0, s4, s2};       // powers of s for (Om, OL, Or, Ok)
     const double om[4] = {Om, OL, Or, Ok};
     q[0] = H0 * rE;
@@ -46,14 +46,14 @@ __global__ void shift_kernel(ShiftArgs a) {
         if (nc == 4) d[3] = -1.0;
         double dE = 0.0;
         for (int i = 0; i < 4; i++) dE += pw[i] * d[i];
-        J[0 * nc + c] = 0.5 * H0 * dE / rE;
+        J[0 * nc + c] = 0.5 * H0 * dE * irE;
         for (int i = 0; i < 3; i++) J[(1 + i) * nc + c] = (pw[i] * d[i] - q[1 + i] * dE) * iE;
     }
     a.scale[b] = s;
     // z1 as an unevaluated float sum hi + lo, so that z2 - z1 and the sign test
     // z2 >= z1 come out right in float32 arithmetic when z2 is close to z1
     const float hi = (float)z1;
-    a.rowf[b] = make_float4(hi, (float)(z1 - (double)hi), (float)(1.0 / s), (float)s);
+    a.rowf[b] = make_float4(hi, (float)(z1 - (double)hi), (float)rcp_(s), (float)s);
 }
 
 cudaError_t launch_shift(const ShiftArgs& a, cudaStream_t s) {
@@ -185,24 +185,26 @@ cudaError_t launch_pair_post(const PairMapArgs& a, cudaStream_t s) {
 }
 
 // ------------------------------------------------------ gradient chain -----
-// grad[b][c] = sum_a gradp[b][a] d params4[b][a] / d params[b][c].  Entries
+// grad[c] = sum_a gradp[a] d params4[a] / d params[c] of one row.  Entries
 // with a zero Jacobian are skipped, so that the NaN Omega_r' component of a
 // radiationless row (no such direction in the cubic) reaches only the
 // Omega_r column, as on the z1 = 0 path.
-__global__ void chain_kernel(const double* __restrict__ jac, const double* __restrict__ gradp, int64_t B,
-                             int ncol, double* __restrict__ grad) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const double* J = jac + b * 4 * ncol;
-    const double* g = gradp + b * 4;
+__device__ __forceinline__ void chain_row(const double* J, const double* g, int ncol, double* grad) {
     for (int c = 0; c < ncol; c++) {
         double acc = 0.0;
         for (int i = 0; i < 4; i++) {
             const double j = J[i * ncol + c];
             if (j != 0.0) acc += g[i] * j;
         }
-        grad[b * ncol + c] = acc;
+        grad[c] = acc;
     }
+}
+
+__global__ void chain_kernel(const double* __restrict__ jac, const double* __restrict__ gradp, int64_t B,
+                             int ncol, double* __restrict__ grad) {
+    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B) return;
+    chain_row(jac + b * 4 * ncol, gradp + b * 4, ncol, grad + b * ncol);
 }
 
 cudaError_t launch_chain(const double* jac, const double* gradp, int64_t B, int ncol, double* grad,
@@ -237,15 +239,16 @@ template <bool GRAD> __global__ void __launch_bounds__(128) limits_kernel(LimitA
             age = tH * e.It;
             if (GRAD) {
                 const double gc = a.cot_chi ? a.cot_chi[b] : 0.0, ga = a.cot_age ? a.cot_age[b] : 0.0;
-                double* g = a.gradp + b * 4;
+                double g[4];
                 g[0] = -(gc * chi + ga * age) * rec[C_IH0];
                 e.reverse(gc * s * DH, ga * tH, tape);
                 for (int k = 0; k < 3; k++) g[1 + k] = e.along(k);
+                chain_row(a.jac + b * 4 * a.ncol, g, a.ncol, a.grad + b * a.ncol);
             }
         }
     }
-    if (st != ST_OK && GRAD && a.gradp)
-        for (int k = 0; k < 4; k++) a.gradp[b * 4 + k] = nan;
+    if (st != ST_OK && GRAD)
+        for (int k = 0; k < a.ncol; k++) a.grad[b * a.ncol + k] = nan;
     if (a.chi) a.chi[b] = chi;
     if (a.age) a.age[b] = age;
 }

@@ -64,7 +64,9 @@ struct LimitArgs {
     double* age;            // [B] t(z1, inf), Gyr (may be null)
     const double* cot_chi;  // [B] (VJP; may be null)
     const double* cot_age;
-    double* gradp;          // [B][4] gradient w.r.t. the shifted parameters (VJP)
+    const double* jac;      // [B][4][ncol] d (shifted parameters) / d params (VJP)
+    int ncol;
+    double* grad;           // [B][ncol] (VJP)
 };
 
 cudaError_t launch_shift(const ShiftArgs& a, cudaStream_t s);

@@ -63,7 +63,9 @@ enum CoreField {
 };
 enum { CORE_NS = 10 };       // room for the series' coefficients in the record: degrees 2 to 11
 enum { CORE_NS_ONCE = 6 };   // used where a record serves one evaluation (the limit at infinity): there the
-                             // coefficients and their tangents cost more than the steps they save
+                             // coefficients cost more than the steps they save, and instead of their
+                             // tangents the record holds (e2, e3, m) and theirs
+enum { C_E2 = C_B + 6, C_E3 = C_B + 7, C_M = C_A + 6, CT_E2 = CT_B, CT_E3 = CT_B + 1, CT_M = CT_A };
 
 // ------------------------------------------------------------- arithmetic ---
 // 1/sqrt, sqrt and 1/x of positive normal numbers.  Single precision: the
@@ -333,6 +335,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     T Ichi, It;
     // adjoints of the row's constants
     T qA_, qB_, qR_, qI_, bF_, eps_, k2_, k3_, bJ_;
+    T e2_, e3_, m_;   // INF: in the place of the series' coefficients
 
     LCDM_HD void forward(T zin, const T* rec, Tape& tape, int* fail) {
         rc = rec;
@@ -754,12 +757,54 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         }
         qA_ = (nA_ * half * rA + wA_) * z;
         qB_ = nB_ * half * rB * z;
+        if (INF) series_adjoint();
     }
     T pf_;
+
+    // INF: the closing series' adjoints taken through to (e2, e3, m), where a
+    // record of coefficient tangents would be used once.  R_F to degree 7:
+    //   1 - E2/10 + E3/14 + E2^2/24 - 3 E2 E3/44 - 5 E2^3/208 + 3 E3^2/104 + E2^2 E3/16, E_i = e_i w^i;
+    // R_J alike in E2 .. E5 (DLMF 19.36.2), which are polynomials of (m, e2, e3) (rj_coefs).
+    LCDM_HD void series_adjoint() {
+        {
+            const T w = wF, ww = w * w, E2 = rc[C_E2] * ww, E3 = rc[C_E3] * (ww * w);
+            e2_ = bF_ * ww * (cst<T>(-0.1) + E2 * cst<T>(1.0 / 12) - E3 * cst<T>(3.0 / 44) - E2 * E2 * cst<T>(15.0 / 208)
+                              + E2 * E3 * cst<T>(0.125));
+            e3_ = bF_ * ww * w * (cst<T>(1.0 / 14) - E2 * cst<T>(3.0 / 44) + E3 * cst<T>(3.0 / 52) + E2 * E2 * cst<T>(1.0 / 16));
+        }
+        if (WT) {
+            const T w = wJ, ww = w * w, m = rc[C_M] * w, e2 = rc[C_E2] * ww, e3 = rc[C_E3] * (ww * w);
+            const T mm = m * m, P = m * cst<T>(0.6), P2 = P * P, P3 = P2 * P;
+            const T E2 = e2 - mm * cst<T>(0.6);
+            const T Q = e3 - m * e2 * cst<T>(0.4) - mm * m * cst<T>(0.064);
+            const T E3 = Q + cst<T>(2.0) * E2 * P + cst<T>(4.0) * P3;
+            const T W = cst<T>(2.0) * Q + E2 * P + cst<T>(3.0) * P3, E4 = W * P, E5 = Q * P2;
+            const T g5 = cst<T>(3.0 / 26) - E2 * cst<T>(9.0 / 68);
+            const T g4 = cst<T>(-3.0 / 22) + E2 * cst<T>(3.0 / 20) - E3 * cst<T>(9.0 / 68);
+            const T g3 = cst<T>(1.0 / 6) - E2 * cst<T>(9.0 / 52) + E3 * cst<T>(3.0 / 20) + E2 * E2 * cst<T>(45.0 / 272)
+                         - E4 * cst<T>(9.0 / 68);
+            const T gW = g4 * P;
+            const T g2 = cst<T>(-3.0 / 14) + E2 * cst<T>(9.0 / 44) - E3 * cst<T>(9.0 / 52) - E2 * E2 * cst<T>(3.0 / 16)
+                         + E4 * cst<T>(3.0 / 20) + E2 * E3 * cst<T>(45.0 / 136) - E5 * cst<T>(9.0 / 68)
+                         + cst<T>(2.0) * g3 * P + gW * P;
+            const T gQ = g5 * P2 + cst<T>(2.0) * gW + g3;
+            const T gP = cst<T>(2.0) * g5 * Q * P + g4 * W + gW * (E2 + cst<T>(9.0) * P2) + g3 * (cst<T>(2.0) * E2 + cst<T>(12.0) * P2);
+            const T c = bJ_;
+            m_ = c * w * (cst<T>(0.6) * gP - cst<T>(1.2) * m * g2 - gQ * (cst<T>(0.4) * e2 + cst<T>(0.192) * mm));
+            e2_ = e2_ + c * ww * (g2 - cst<T>(0.4) * m * gQ);
+            e3_ = e3_ + c * ww * w * gQ;
+        }
+    }
 
     // sum over the row's constants of adjoint times tangent, direction k
     LCDM_HD T along(int k) const {
         const T* t = rc + C_TAN + C_TSTRIDE * k;
+        if (INF) {
+            const Quad<T> f = quad(t);
+            T r = qA_ * f.v[0] + qB_ * f.v[1] + (qR_ * f.v[2] + qI_ * f.v[3]) + e2_ * t[CT_E2] + e3_ * t[CT_E3];
+            if (WT) r = r + (eps_ * t[CT_EPS] + k2_ * t[CT_K2] + k3_ * t[CT_K3]) + m_ * t[CT_M];
+            return r;
+        }
         const Quad<T> t0 = quad(t);
         const T b = series<false, NS>(t, CT_B, wF).v;
         T r = qA_ * t0.v[0] + qB_ * t0.v[1] + (qR_ * t0.v[2] + qI_ * t0.v[3]) + bF_ * (wF * wF) * b;

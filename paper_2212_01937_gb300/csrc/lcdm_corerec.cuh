@@ -129,6 +129,7 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
         if (j < ns) rec[C_B + j] = b[j];
     const float d3 = dev3(e2, e3);
     rec[C_DF] = (T)d3;
+    if (ns <= CORE_NS_ONCE) { put(rec, C_E2, e2); put(rec, C_E3, e3); }
     if (time) {
         // t: E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
         const double g0 = r.OL, g1 = r.Ox - eps * g0, g2 = Oks - eps * g1, g3 = r.Om - eps * g2;
@@ -137,6 +138,7 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
         put(rec, C_EPS, eps);
         put(rec, C_K2, k * (1.0 / 3));
         put(rec, C_K3, r.OL * iS0);
+        if (ns <= CORE_NS_ONCE) put(rec, C_M, m);
         rj_coefs<T>((T)m, f2, f3, ns, b);
 #pragma unroll
         for (int j = 0; j < CORE_NS; j++)
@@ -215,41 +217,63 @@ LCDM_HD void core_tangent(const RowRoots& r, bool time, int ns, int k, double dA
         put(t, CT_QR, dpr * (r.q1 * r.q1));
         put(t, CT_QI, dpi * (r.q2 * r.q2));
     }
-    typedef Dual<double, 1> D;
-    D Om, OL, Or, c, Ox, is, ep;
-    Om.v = r.Om; Om.d[0] = d.dOm;
-    OL.v = r.OL; OL.d[0] = d.dOL;
-    Or.v = r.Or; Or.d[0] = d.dOr;
-    c.v = Oks; c.d[0] = d.dOk;
-    Ox.v = r.Ox; Ox.d[0] = d.dOx;
-    is.v = iS0; is.d[0] = -d.dS * iS0 * iS0;
-    // the series in the record's precision
+    // e2 = -I / (3 S0^2), e3 = -J / (27 S0^3) by the invariants' partial derivatives
+    const double Om = r.Om, OL = r.OL, Or = r.Or, c = Oks, Ox = r.Ox, c2 = c * c, iS2 = iS0 * iS0;
+    double dI = 2.0 * c * d.dOk, dJ = (6.0 * c2 - 9.0 * Om * Ox - 72.0 * Or * OL) * d.dOk;
+    if (k == 0) { dI -= 3.0 * Ox; dJ += 54.0 * Om * OL - 9.0 * c * Ox; }
+    if (k == 1) { dI += 12.0 * Or; dJ += 27.0 * Om * Om - 72.0 * Or * c; }
+    if (k == 2) { dI += 12.0 * OL; dJ += 27.0 * Ox * Ox - 72.0 * c * OL; }
+    if (k == 5) { dI -= 3.0 * Om; dJ += 54.0 * Or * Ox - 9.0 * Om * c; }
+    double de2 = dI * (-1.0 / 3), de3 = dJ * (-1.0 / 27);
+    T e2, e3;
+    {
+        const double I = 12.0 * Or * OL - 3.0 * Om * Ox + c2;
+        const double J = 2.0 * c2 * c - 9.0 * Om * c * Ox + 27.0 * Or * Ox * Ox + 27.0 * Om * Om * OL - 72.0 * Or * c * OL;
+        const double v2 = I * (-1.0 / 3) * iS2, v3 = J * (-1.0 / 27) * (iS2 * iS0);
+        if (r.ncol != 4) {
+            de2 = (de2 * iS0 - 2.0 * v2) * iS0;
+            de3 = (de3 * iS2 - 3.0 * v3) * iS0;
+        }
+        e2 = (T)v2;
+        e3 = (T)v3;
+    }
     typedef Dual<T, 1> F;
-    auto to = [](const D& x) { F f; f.v = (T)x.v; f.d[0] = (T)x.d[0]; return f; };
-    const F fm = to(Om), fl = to(OL), fr = to(Or), fc = to(c), fx = to(Ox), fs = to(is);
-    const F I = fr * fl * cst<T>(12.0) - fm * fx * cst<T>(3.0) + fc * fc;
-    const F J = fc * fc * fc * cst<T>(2.0) - fm * fc * fx * cst<T>(9.0) + fr * fx * fx * cst<T>(27.0)
-                + fm * fm * fl * cst<T>(27.0) - fr * fc * fl * cst<T>(72.0);
-    const F e2 = I * fs * fs * cst<T>(-1.0 / 3), e3 = J * fs * fs * fs * cst<T>(-1.0 / 27);
-    F b[CORE_NS];
-    rf_coefs<F>(e2, e3, ns, b);
-#pragma unroll
-    for (int j = 0; j < CORE_NS; j++)
-        if (j < ns) t[CT_B + j] = b[j].d[0];
-    if (time) {
-        // the third-kind integral's constants in double
-        ep.v = eps; ep.d[0] = r.quartic ? dA * (eps * eps) : 0.0;
-        const D g1 = Ox - ep * OL, g2 = c - ep * g1, g3 = Om - ep * g2;
-        const D kk = (ep * (g2 - ep * (g1 - ep * OL)) - g3) * is;
-        put(t, CT_EPS, ep.d[0]);
-        put(t, CT_K2, kk.d[0] * (1.0 / 3));
-        put(t, CT_K3, (OL * is).d[0]);
-        const F fe = to(ep), f1 = to(g1), f2 = to(g2);
-        const F m = (f2 + fe * (fe * fl * cst<T>(3.0) - f1 * cst<T>(2.0))) * fs * cst<T>(1.0 / 3);
-        rj_coefs<F>(m, e2, e3, ns, b);
+    F f2, f3, b[CORE_NS];
+    f2.v = e2; f2.d[0] = (T)de2;
+    f3.v = e3; f3.d[0] = (T)de3;
+    const bool once = ns <= CORE_NS_ONCE;
+    if (once) {
+        put(t, CT_E2, de2);
+        put(t, CT_E3, de3);
+    } else {
+        rf_coefs<F>(f2, f3, ns, b);
 #pragma unroll
         for (int j = 0; j < CORE_NS; j++)
-            if (j < ns) t[CT_A + j] = b[j].d[0];
+            if (j < ns) t[CT_B + j] = b[j].d[0];
+    }
+    if (time) {
+        // k S0 = -Om + 2 eps C - 3 eps^2 Ox + 4 eps^3 OL, 3 m S0 = C - 3 eps Ox + 6 eps^2 OL (C = Ok + Os):
+        // the recursion of core_values multiplied out
+        const double ee = eps * eps, de = r.quartic ? dA * ee : 0.0;
+        const double kv = (-Om + eps * (2.0 * c - eps * (3.0 * Ox - 4.0 * eps * OL))) * iS0;
+        const double mv = (c - eps * (3.0 * Ox - 6.0 * eps * OL)) * (iS0 * (1.0 / 3));
+        const double dk = (-d.dOm + 2.0 * eps * d.dOk - ee * (3.0 * d.dOx - 4.0 * eps * d.dOL)
+                           + (2.0 * c - eps * (6.0 * Ox - 12.0 * eps * OL)) * de - kv * d.dS) * iS0;
+        const double dm = (d.dOk - eps * (3.0 * d.dOx - 6.0 * eps * d.dOL) - (3.0 * Ox - 12.0 * eps * OL) * de
+                           - 3.0 * mv * d.dS) * (iS0 * (1.0 / 3));
+        put(t, CT_EPS, de);
+        put(t, CT_K2, dk * (1.0 / 3));
+        put(t, CT_K3, (d.dOL - OL * iS0 * d.dS) * iS0);
+        if (once) {
+            put(t, CT_M, dm);
+        } else {
+            F fm;
+            fm.v = (T)mv; fm.d[0] = (T)dm;
+            rj_coefs<F>(fm, f2, f3, ns, b);
+#pragma unroll
+            for (int j = 0; j < CORE_NS; j++)
+                if (j < ns) t[CT_A + j] = b[j].d[0];
+        }
     }
     put(t, CT_END, 0.0);
 }
