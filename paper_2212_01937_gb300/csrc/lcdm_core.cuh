@@ -67,6 +67,70 @@ enum { CORE_NS_ONCE = 6 };   // used where a record serves one evaluation (the l
                              // tangents the record holds (e2, e3, m) and theirs
 enum { C_E2 = C_B + 6, C_E3 = C_B + 7, C_M = C_A + 6, CT_E2 = CT_B, CT_E3 = CT_B + 1, CT_M = CT_A };
 
+// ----------------------------------------------------- two pairs in a thread ---
+// Two single-precision numbers in one 64-bit register pair: this part's packed
+// add, multiply and fused multiply-add do both in one issue slot (of the two
+// cycles that their 64 lane operations take), and the pair kernels are bound by
+// issue.  Written without a rounding modifier, so that a product and a sum
+// contract as for plain floats.
+struct F2 { float x, y; };
+LCDM_HD F2 mkf2(float x, float y) { F2 r; r.x = x; r.y = y; return r; }
+#ifdef __CUDA_ARCH__
+LCDM_HD uint64_t f2_bits(F2 a) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y)); return r; }
+LCDM_HD F2 f2_of(uint64_t u) { F2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(u)); return r; }
+LCDM_HD F2 operator*(F2 a, F2 b) {
+    uint64_t r;
+    asm("mul.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+LCDM_HD F2 operator+(F2 a, F2 b) {
+    uint64_t r;
+    asm("add.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+LCDM_HD F2 operator-(F2 a, F2 b) {
+    uint64_t r;
+    asm("sub.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return f2_of(r);
+}
+#else
+LCDM_HD F2 operator*(F2 a, F2 b) { return mkf2(a.x * b.x, a.y * b.y); }
+LCDM_HD F2 operator+(F2 a, F2 b) { return mkf2(a.x + b.x, a.y + b.y); }
+LCDM_HD F2 operator-(F2 a, F2 b) { return mkf2(a.x - b.x, a.y - b.y); }
+#endif
+LCDM_HD F2 operator-(F2 a) { return mkf2(-a.x, -a.y); }
+template <> struct CstImpl<F2> { static LCDM_HD F2 make(double v) { return mkf2((float)v, (float)v); } };
+
+// What the core asks of its scalar beside arithmetic: the record's type, a
+// record entry as a scalar, |a|, a selection by sign, and comparisons (of both
+// numbers: all of them, or any).
+template <class T> struct Scalar {
+    typedef T rec;
+    static LCDM_HD T of(T v) { return v; }
+};
+template <> struct Scalar<F2> {
+    typedef float rec;
+    static LCDM_HD F2 of(float v) { return mkf2(v, v); }
+};
+LCDM_HD float abs_(float a) { return fabsf(a); }
+LCDM_HD double abs_(double a) { return fabs(a); }
+LCDM_HD F2 abs_(F2 a) { return mkf2(fabsf(a.x), fabsf(a.y)); }
+template <class T> LCDM_HD T sel_ge0(T c, T a, T b) { return c >= cst<T>(0.0) ? a : b; }
+LCDM_HD F2 sel_ge0(F2 c, F2 a, F2 b) { return mkf2(c.x >= 0.f ? a.x : b.x, c.y >= 0.f ? a.y : b.y); }
+template <class T> LCDM_HD bool all_le(T a, T b) { return a <= b; }
+LCDM_HD bool all_le(F2 a, F2 b) { return a.x <= b.x && a.y <= b.y; }
+template <class T> LCDM_HD bool any_gt(T a, T b) { return a > b; }
+LCDM_HD bool any_gt(F2 a, F2 b) { return a.x > b.x || a.y > b.y; }
+// bits of the numbers that are not <= (NaN included)
+template <class T> LCDM_HD int not_le(T a, T b) { return a <= b ? 0 : 1; }
+LCDM_HD int not_le(F2 a, F2 b) { return (a.x <= b.x ? 0 : 1) | (a.y <= b.y ? 0 : 2); }
+// (in double a comparison would hold the FP64 pipe: both sides in single)
+LCDM_HD float cmp_(float a) { return a; }
+LCDM_HD float cmp_(double a) { return (float)a; }
+LCDM_HD F2 cmp_(F2 a) { return a; }
+LCDM_HD float times_(float k, float a) { return k * a; }
+LCDM_HD F2 times_(float k, F2 a) { return mkf2(k, k) * a; }
+
 // ------------------------------------------------------------- arithmetic ---
 // 1/sqrt, sqrt and 1/x of positive normal numbers.  Single precision: the
 // hardware approximations (within two ulp).  Double precision: one step of
@@ -77,6 +141,8 @@ enum { C_E2 = C_B + 6, C_E3 = C_B + 7, C_M = C_A + 6, CT_E2 = CT_B, CT_E3 = CT_B
 // instructions; CUDA's square root issues about 9, its division 9, rsqrt 5.5.
 LCDM_HD float rsq(float x) { return srsqrt(x); }
 LCDM_HD float sqt(float x) { return x * srsqrt(x); }
+LCDM_HD F2 rsq(F2 x) { return mkf2(srsqrt(x.x), srsqrt(x.y)); }
+LCDM_HD F2 sqt(F2 x) { return x * rsq(x); }
 #ifdef __CUDA_ARCH__
 LCDM_HD double rsq_seed(double x) {
     double y;
@@ -109,6 +175,7 @@ LCDM_HD float rcp_(float x) {
     return 1.0f / x;
 #endif
 }
+LCDM_HD F2 rcp_(F2 x) { return mkf2(rcp_(x.x), rcp_(x.y)); }
 LCDM_HD double rcp_(double x) {
 #ifdef __CUDA_ARCH__
     double y;
@@ -128,6 +195,7 @@ template <> struct CoreTol<float> {
     static constexpr float dup = 0.25f, once = 0.15f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
     enum { maxit = 24, ns = 8 };
 };
+template <> struct CoreTol<F2> : CoreTol<float> {};
 template <> struct CoreTol<double> {
     static constexpr double dup = 0.05, once = 0.009, rc = 0.008, big = 1e30, e_series = 0.03;
     enum { maxit = 40, ns = 10 };
@@ -170,6 +238,25 @@ LCDM_HD RcE<float> rc1_core(float e, bool grad) {
         return r;
     }
     return rc1_far<float>(e, sqt(1.0f + e));
+}
+LCDM_HD RcE<F2> rc1_core(F2 e, bool grad) {
+    RcE<F2> r;
+    if (all_le(abs_(e), cst<F2>(CoreTol<float>::e_series))) {
+        const F2 w = -e;
+        F2 s = cst<F2>(1.0 / 13), ds = cst<F2>(0.0);
+#pragma unroll
+        for (int n = 5; n >= 0; n--) {
+            if (grad) ds = ds * w + s;
+            s = cst<F2>(1.0 / (2 * n + 1)) + w * s;
+        }
+        r.v = s;
+        r.d = -ds;
+        return r;
+    }
+    const RcE<float> a = rc1_core(e.x, grad), b = rc1_core(e.y, grad);
+    r.v = mkf2(a.v, b.v);
+    r.d = mkf2(a.d, b.d);
+    return r;
 }
 LCDM_HD RcE<double> rc1_core(double e, bool grad) {
     // e falls by 64 or more per step: most steps need a few terms only
@@ -243,6 +330,7 @@ LCDM_HD float one_plus(float q, float ql, float z) {
     const df64 s = two_sum(1.0f, p);
     return s.hi + (s.lo + fmaf(ql, z, e1));
 }
+LCDM_HD F2 one_plus(F2 q, F2 ql, F2 z) { return mkf2(one_plus(q.x, ql.x, z.x), one_plus(q.y, ql.y, z.y)); }
 // power of two near 1/z for very large z
 LCDM_HD float scale_of(float z) { return z < 1e38f ? pow2i<float>(-even_exponent(z)) : 0.0f; }
 LCDM_HD double scale_of(double z) {
@@ -250,6 +338,11 @@ LCDM_HD double scale_of(double z) {
     frexp(z, &e);
     return z < 1e300 ? pow2i<double>(-e) : 0.0;
 }
+
+// the scaling of a pair, 1 unless z is very large
+LCDM_HD float scaling(float z) { return z > CoreTol<float>::big ? scale_of(z) : 1.0f; }
+LCDM_HD double scaling(double z) { return z > CoreTol<double>::big ? scale_of(z) : 1.0; }
+LCDM_HD F2 scaling(F2 z) { return mkf2(scaling(z.x), scaling(z.y)); }
 
 // Four consecutive record entries from a multiple of four (records are 16-byte
 // aligned): one 128-bit load in single precision, two in double.
@@ -275,16 +368,24 @@ LCDM_HD Quad<double> quad(const double* p) {
     return q;
 }
 
+template <class T> LCDM_HD Quad<T> quad_as(const typename Scalar<T>::rec* p) {
+    const Quad<typename Scalar<T>::rec> f = quad(p);
+    Quad<T> q;
+#pragma unroll
+    for (int i = 0; i < 4; i++) q.v[i] = Scalar<T>::of(f.v[i]);
+    return q;
+}
+
 // ------------------------------------------------------------------- core ---
 // A closing series 1 + w^2 (c_2 + c_3 w + ...) from ns coefficients at rec[i],
 // i = 0 or 1 modulo 4, and with it (D) the derivative of the bracket.
 template <class T> struct SerVal { T v, d; };
-template <bool D, int N, class T> LCDM_HD SerVal<T> series(const T* rec, int i, T w) {
+template <bool D, int N, class T> LCDM_HD SerVal<T> series(const typename Scalar<T>::rec* rec, int i, T w) {
     T c[12];
     const int skip = i & 3;
 #pragma unroll
     for (int q = 0; q < (N + skip + 3) / 4; q++) {
-        const Quad<T> k = quad(rec + (i - skip) + 4 * q);
+        const Quad<T> k = quad_as<T>(rec + (i - skip) + 4 * q);
 #pragma unroll
         for (int l = 0; l < 4; l++)
             if (4 * q + l >= skip && 4 * q + l - skip < 12) c[4 * q + l - skip] = k.v[l];
@@ -319,7 +420,8 @@ template <class T, bool REV, bool WT> struct CoreTape {
 template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair {
     typedef CoreTape<T, REV, WT> Tape;
     enum { NS = INF ? (int)CORE_NS_ONCE : (int)CoreTol<T>::ns };
-    const T* rc;
+    typedef typename Scalar<T>::rec R;
+    const R* rc;
     T z, zh, z2, h, cz;
     bool cplx, big;
     // square roots of the linear factors and their reciprocals
@@ -337,20 +439,21 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     T qA_, qB_, qR_, qI_, bF_, eps_, k2_, k3_, bJ_;
     T e2_, e3_, m_;   // INF: in the place of the series' coefficients
 
-    LCDM_HD void forward(T zin, const T* rec, Tape& tape, int* fail) {
+    LCDM_HD void forward(T zin, const R* rec, Tape& tape, int* fail) {
         rc = rec;
         z = zin;
         const T one = cst<T>(1.0);
-        const Quad<T> k0 = quad(rc + C_QA), k1 = quad(rc + C_QI);
-        cplx = k1.v[3] != cst<T>(0.0);
+        const Quad<T> k0 = quad_as<T>(rc + C_QA), k1 = quad_as<T>(rc + C_QI);
+        cplx = rc[C_KIND] != R(0);
         const T wA = INF ? k0.v[0] : one + k0.v[0] * z, wB = INF ? k0.v[1] : one + k0.v[1] * z;
-        rA = INF && !(wA > cst<T>(0.0)) ? cst<T>(0.0) : rsq(wA);
+        rA = rsq(wA);
+        if (INF && !any_gt(wA, cst<T>(0.0))) rA = cst<T>(0.0);
         nA = wA * rA;
         rB = rsq(wB);
         nB = wB * rB;
         const T qR = k0.v[2], qI = k1.v[0], c2 = k1.v[2];
         Quad<T> kT;
-        if (WT) kT = quad(rc + C_DJ);
+        if (WT) kT = quad_as<T>(rc + C_DJ);
         T S, P, T30;
         if (cplx) {
             wr = INF ? qR : one_plus(qR, k0.v[3], z);
@@ -359,11 +462,10 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             iP = rsq(r2);
             Pn = r2 * iP;
             // n_P: the larger part by a square root, the other by division
-            const T hh = (Pn + fabs(wr)) * cst<T>(0.5), rh = rsq(hh);
+            const T hh = (Pn + abs_(wr)) * cst<T>(0.5), rh = rsq(hh);
             const T t = hh * rh, o = wi * cst<T>(0.5) * rh;
-            const bool pos = wr >= cst<T>(0.0);
-            nr = pos ? t : o;
-            ni = pos ? o : t;
+            nr = sel_ge0(wr, t, o);
+            ni = sel_ge0(wr, o, t);
             uR = nr * (nA + nB);
             uI = ni * (nA - nB);
         } else {
@@ -388,16 +490,16 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         T aX = cst<T>(0.0), lX = cst<T>(0.0);
         Quad<T> kX;
         if (WX) {
-            kX = quad(rc + X_HX);
+            kX = quad_as<T>(rc + X_HX);
             aX = nA * Pn + nB;
             lX = kX.v[1] * wB;
         }
         // powers of z^6 and d^2 would leave the range for very large z:
         // everything is homogeneous and is scaled by a power of two
-        big = z > CoreTol<T>::big;
+        big = any_gt(z, cst<T>(CoreTol<T>::big));
         h = one;
         if (big) {
-            h = scale_of(z);
+            h = scaling(z);
             s1 = s1 * h; uR = uR * h; uI = uI * h;
             if (WT) a5 = a5 * h;
             if (WX) aX = aX * h;
@@ -431,9 +533,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             dX = -(kX.v[0] * z2) * piX;
         }
         T pX = p0;
-        const float it = (float)(1.0 / (INF ? CoreTol<T>::once : CoreTol<T>::dup)), z2f = (float)z2 * it;
-        const float dF = (float)rc[C_DF] * z2f * 3.0f, dJ = WT ? (float)kT.v[0] * z2f * 5.0f : 0.0f;
-        const float dD = WX ? (float)kX.v[3] * z2f * 5.0f : 0.0f;
+        const float it = (float)(1.0 / (INF ? CoreTol<T>::once : CoreTol<T>::dup));
+        const auto z2c = cmp_(z2);
+        const auto dF = times_((float)rc[C_DF] * it * 3.0f, z2c);
+        const auto dJ = times_(WT ? (float)rc[C_DJ] * it * 5.0f : 0.0f, z2c);
+        const auto dD = times_(WX ? (float)rc[X_DX] * it * 5.0f : 0.0f, z2c);
         T S1 = s1;
         tm = one;
         T q0 = cst<T>(0.0);
@@ -442,9 +546,9 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         for (; m < CoreTol<T>::maxit; m++) {
             // (compared in single precision: in double each comparison would hold
             // the FP64 pipe)
-            bool conv = dF <= (float)T3;
-            if (WT) conv = conv && dJ <= (float)(T3 + p + p);
-            if (WX) conv = conv && dD <= (float)(T3 + pX + pX) && dD <= (float)(T3 + x + x);
+            bool conv = all_le(dF, cmp_(T3));
+            if (WT) conv = conv && all_le(dJ, cmp_(T3 + p + p));
+            if (WX) conv = conv && all_le(dD, cmp_(T3 + pX + pX)) && all_le(dD, cmp_(T3 + x + x));
             if (conv) break;
             const T lam = S1 * S + P;
             const T xl = x + lam;
@@ -458,7 +562,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 if (REV) tape.q[m] = sq;
                 p = p + lam;
             }
-            if (WX) {
+            if constexpr (WX) {
                 // R_D: 1 / (s1 (x + lambda)); divided difference of the p0 track against it
                 const T ix = rcp_(S1 * xl);
                 sD = sD + tm * ix;
@@ -485,7 +589,12 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             S1 = n1;
             tm = tm + tm;
         }
-        if (m == CoreTol<T>::maxit) *fail = 1;
+        if (m == CoreTol<T>::maxit) {
+            // not converged (of two pairs: those that are not)
+            *fail |= not_le(dF, cmp_(T3));
+            if (WT) *fail |= not_le(dJ, cmp_(T3 + p + p));
+            if (WX) *fail |= not_le(dD, cmp_(T3 + pX + pX)) | not_le(dD, cmp_(T3 + x + x));
+        }
         // closing series in w = z^2 / A
         {
             const T A = T3 * cst<T>(1.0 / 3);
@@ -509,18 +618,18 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             U = a * a + cst<T>(2.0) * (b * b);
             tr = one;
             mr = 0;
-            const T ad = fabs(d5);
+            const T ad = abs_(d5);
 #pragma unroll 1
             for (; mr < CoreTol<T>::maxit; mr++) {
                 if (REV) { tape.ra[mr] = a; tape.rb[mr] = b; }
-                if (ad <= CoreTol<T>::rc * U) break;
+                if (all_le(ad, cst<T>(CoreTol<T>::rc) * U)) break;
                 const T n = a + b, q = cst<T>(2.0) * b * n;
                 a = n;
                 b = sqt(q);
                 U = a * a + cst<T>(2.0) * (b * b);
                 tr = tr + tr;
             }
-            if (mr == CoreTol<T>::maxit) *fail = 1;
+            if (mr == CoreTol<T>::maxit) *fail |= not_le(ad, cst<T>(CoreTol<T>::rc) * U);
             const T iA = cst<T>(3.0) * rcp_(U);
             sc = -d5 * iA * cst<T>(1.0 / 3);
             T ser = cst<T>(159.0 / 208) + sc * cst<T>(1.125);
@@ -532,7 +641,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             rcr = rsq(U * cst<T>(1.0 / 3));
             RCp = tr * ser * rcr * izh;
             const T eps = kT.v[1];
-            g = fabs(opE) * nA;
+            g = abs_(opE) * nA;
             if (INF) {
                 It = cz * (RCp * g - eps * RF - kT.v[2] * z2 * RJ);
             } else {
@@ -541,7 +650,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 It = cz * (RCp + eps * (RCp * kB - RF) - kT.v[2] * z2 * RJ);
             }
         }
-        if (WX) {
+        if constexpr (WX) {
             const T iA2 = cst<T>(5.0) * rcp_(T3 + x + x);
             const T A2 = (T3 + x + x) * cst<T>(0.2), A1 = (T3 + pX + pX) * cst<T>(0.2);
             const T r1 = rsq(A1), r2 = rsq(A2);
@@ -553,7 +662,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             T q[3 * CORE_NS + 2];
 #pragma unroll
             for (int j = 0; j < (3 * N + 3) / 4; j++) {
-                const Quad<T> f = quad(rc + X_S + 4 * j);
+                const Quad<T> f = quad_as<T>(rc + X_S + 4 * j);
 #pragma unroll
                 for (int i = 0; i < 4; i++) q[4 * j + i] = f.v[i];
             }
@@ -575,7 +684,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T ih = big ? one / h : one;
             const T s1u = s1 * ih, sp0 = rp0 * ih, zz = z * z, x1 = x0 * (ih * ih);
             const T hRF = RF * h, hRD = RD * (h * h * h), hDJ = DJ * (h * h * h) * (h * h);
-            const Quad<T> c0 = quad(rc + X_C0), c3 = quad(rc + X_G3), cN = quad(rc + X_N0), cB = quad(rc + X_AB);
+            const Quad<T> c0 = quad_as<T>(rc + X_C0), c3 = quad_as<T>(rc + X_G3), cN = quad_as<T>(rc + X_N0), cB = quad_as<T>(rc + X_AB);
             const T irA = rA, syd = c3.v[3] * (nA * Pn * rB + one), isy = rcp_(syd);
             const T T0 = c0.v[0] * irA * (k0.v[1] * Pn * rcp_(nB + one) + (cB.v[2] + z * cB.v[3]) * rcp_(Pn + one)
                                            - k0.v[0] * rcp_(nA + one));
@@ -592,7 +701,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     }
 
     // 1 / E(z) = E(0)^-1 / (n_A n_B |n_P|^2)
-    LCDM_HD T inv_E() const { return rc[C_C2] * cst<T>(0.5) * (rA * rB * iP); }
+    LCDM_HD T inv_E() const { return Scalar<T>::of(rc[C_C2] * R(0.5)) * (rA * rB * iP); }
 
     // Adjoints of the row's constants for the cotangents ci, ti of Ichi, It.
     LCDM_HD void reverse(T ci, T ti, const Tape& tape) {
@@ -600,7 +709,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         T RF_ = ci * cz, T_ = cst<T>(0.0), p_ = cst<T>(0.0), cJ = cst<T>(0.0), del_ = cst<T>(0.0), a_ = cst<T>(0.0),
           b_ = cst<T>(0.0), d_ = cst<T>(0.0), nA_ = cst<T>(0.0), wA_ = cst<T>(0.0);
         Quad<T> kT;
-        if (WT) kT = quad(rc + C_DJ);
+        if (WT) kT = quad_as<T>(rc + C_DJ);
         const T eps = WT ? kT.v[1] : cst<T>(0.0), z1 = INF ? one : one + z;
         eps_ = k2_ = k3_ = bJ_ = cst<T>(0.0);
         if (WT) {
@@ -610,7 +719,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T bk = b * z2;
             const T RJ_ = -bk * kT.v[2];
             k2_ = -bk * RJ;
-            const T opE = one + eps, ao = fabs(opE), sA = opE < cst<T>(0.0) ? -nA : nA;
+            const T opE = one + eps, ao = abs_(opE), sA = sel_ge0(opE, nA, -nA);
             if (INF) {
                 eps_ = b * (RCp * sA - RF);
                 nA_ = b * RCp * ao;
@@ -767,13 +876,13 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
     // R_J alike in E2 .. E5 (DLMF 19.36.2), which are polynomials of (m, e2, e3) (rj_coefs).
     LCDM_HD void series_adjoint() {
         {
-            const T w = wF, ww = w * w, E2 = rc[C_E2] * ww, E3 = rc[C_E3] * (ww * w);
+            const T w = wF, ww = w * w, E2 = Scalar<T>::of(rc[C_E2]) * ww, E3 = Scalar<T>::of(rc[C_E3]) * (ww * w);
             e2_ = bF_ * ww * (cst<T>(-0.1) + E2 * cst<T>(1.0 / 12) - E3 * cst<T>(3.0 / 44) - E2 * E2 * cst<T>(15.0 / 208)
                               + E2 * E3 * cst<T>(0.125));
             e3_ = bF_ * ww * w * (cst<T>(1.0 / 14) - E2 * cst<T>(3.0 / 44) + E3 * cst<T>(3.0 / 52) + E2 * E2 * cst<T>(1.0 / 16));
         }
         if (WT) {
-            const T w = wJ, ww = w * w, m = rc[C_M] * w, e2 = rc[C_E2] * ww, e3 = rc[C_E3] * (ww * w);
+            const T w = wJ, ww = w * w, m = Scalar<T>::of(rc[C_M]) * w, e2 = Scalar<T>::of(rc[C_E2]) * ww, e3 = Scalar<T>::of(rc[C_E3]) * (ww * w);
             const T mm = m * m, P = m * cst<T>(0.6), P2 = P * P, P3 = P2 * P;
             const T E2 = e2 - mm * cst<T>(0.6);
             const T Q = e3 - m * e2 * cst<T>(0.4) - mm * m * cst<T>(0.064);
@@ -796,21 +905,24 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         }
     }
 
+    LCDM_HD T thirds(const R* t) const {
+        return eps_ * Scalar<T>::of(t[CT_EPS]) + k2_ * Scalar<T>::of(t[CT_K2]) + k3_ * Scalar<T>::of(t[CT_K3]);
+    }
     // sum over the row's constants of adjoint times tangent, direction k
     LCDM_HD T along(int k) const {
-        const T* t = rc + C_TAN + C_TSTRIDE * k;
+        const R* t = rc + C_TAN + C_TSTRIDE * k;
         if (INF) {
-            const Quad<T> f = quad(t);
-            T r = qA_ * f.v[0] + qB_ * f.v[1] + (qR_ * f.v[2] + qI_ * f.v[3]) + e2_ * t[CT_E2] + e3_ * t[CT_E3];
-            if (WT) r = r + (eps_ * t[CT_EPS] + k2_ * t[CT_K2] + k3_ * t[CT_K3]) + m_ * t[CT_M];
+            const Quad<T> f = quad_as<T>(t);
+            T r = qA_ * f.v[0] + qB_ * f.v[1] + (qR_ * f.v[2] + qI_ * f.v[3]) + e2_ * Scalar<T>::of(t[CT_E2]) + e3_ * Scalar<T>::of(t[CT_E3]);
+            if (WT) r = r + thirds(t) + m_ * Scalar<T>::of(t[CT_M]);
             return r;
         }
-        const Quad<T> t0 = quad(t);
+        const Quad<T> t0 = quad_as<T>(t);
         const T b = series<false, NS>(t, CT_B, wF).v;
         T r = qA_ * t0.v[0] + qB_ * t0.v[1] + (qR_ * t0.v[2] + qI_ * t0.v[3]) + bF_ * (wF * wF) * b;
         if (WT) {
             const T a = series<false, NS>(t, CT_A, wJ).v;
-            r = r + (eps_ * t[CT_EPS] + k2_ * t[CT_K2] + k3_ * t[CT_K3]) + bJ_ * (wJ * wJ) * a;
+            r = r + thirds(t) + bJ_ * (wJ * wJ) * a;
         }
         return r;
     }

@@ -37,6 +37,19 @@ template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
     }
 };
 
+template <int K, bool WT, int MODE = CORE_SUM> struct Core2 {
+    static cudaError_t launch(const CoreArgs& c, int grid, int block, cudaStream_t s) {
+        core2_kernel<K, WT, MODE><<<grid, block, 0, s>>>(c);
+        return cudaGetLastError();
+    }
+    static int occ(int block) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core2_kernel<K, WT, MODE>, block, 0) != cudaSuccess)
+            return 0;
+        return n;
+    }
+};
+
 // entries by (WT ? 2 : 0) + (WX ? 1 : 0); jac: the kernels of per-pair
 // Jacobians (without X's, whose tangents have a kernel of their own); dz: those
 // that also give the redshift derivatives, by WT (four- and five-column rows;
@@ -45,6 +58,8 @@ template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
 // through the pair maps)
 struct PairsTable {
     PairsEntry e[4], jac[4], dz[2], bt[4];
+    PairsEntry packed[3][2];   // two pairs in a thread (single precision, no X, no gradient of t): sums, redshift
+                               // derivatives and general limits, by WT
 };
 
 template <class E> PairsEntry entry() { PairsEntry e; e.launch = E::launch; e.occ = E::occ; return e; }
@@ -55,6 +70,13 @@ template <int PREC> PairsTable value_table() {
     t.e[1] = entry<Core<PREC, 0, false, true> >();
     t.e[2] = entry<Core<PREC, 0, true, false> >();
     t.e[3] = entry<Core<PREC, 0, true, true> >();
+    if constexpr (PREC == 1) {
+        t.packed[0][0] = entry<Core2<0, false> >();
+        t.packed[0][1] = entry<Core2<0, true> >();
+        t.packed[1][0] = entry<Core2<0, false, CORE_DZ> >();
+        t.packed[2][0] = entry<Core2<0, false, CORE_BETWEEN> >();
+        t.packed[2][1] = entry<Core2<0, true, CORE_BETWEEN> >();
+    }
     t.dz[0] = entry<Core<PREC, 0, false, false, CORE_DZ> >();
     t.bt[0] = entry<Core<PREC, 0, false, false, CORE_BETWEEN> >();
     t.bt[1] = entry<Core<PREC, 0, false, true, CORE_BETWEEN> >();
@@ -72,6 +94,11 @@ template <int PREC, int K> PairsTable tangent_table() {
     t.jac[1] = t.e[1];
     t.jac[2] = entry<Core<PREC, K, true, false, CORE_JAC> >();
     t.jac[3] = t.e[3];
+    if constexpr (PREC == 1) {
+        t.packed[0][0] = entry<Core2<K, false> >();
+        if constexpr (K < 6) t.packed[1][0] = entry<Core2<K, false, CORE_DZ> >();
+        if constexpr (K == 3) t.packed[2][0] = entry<Core2<K, false, CORE_BETWEEN> >();
+    }
     if constexpr (K == 3) {
         t.bt[0] = entry<Core<PREC, K, false, false, CORE_BETWEEN> >();
         t.bt[2] = entry<Core<PREC, K, true, false, CORE_BETWEEN> >();
