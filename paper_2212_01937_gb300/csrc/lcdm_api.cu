@@ -401,13 +401,16 @@ struct PrepNeed {
 };
 
 lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv, const PrepNeed& need,
-                     int32_t* status, double* grad, double* loglike, cudaStream_t s) {
+                     int32_t* status, double* grad, double* loglike, cudaStream_t s,
+                     const ShiftArgs* shift = nullptr) {
     // One warp per block, so that the FP64 work spreads over as many SMs as
     // possible.  Up to LCDM_PREP_GROUP_MAX_B cosmologies the solve is bound by
     // the latency of one cosmology's dependent FP64 chain and four lanes share
     // each root solve; beyond that the FP64 pipe is the bound and one lane per
     // cosmology does no repeated work.
     PrepArgs a;
+    memset(&a.shift, 0, sizeof(a.shift));
+    if (shift) a.shift = *shift;
     a.params = params;
     a.B = B;
     a.ncol = opts->ncol;
@@ -438,12 +441,13 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
 // X-tangent kernel's and that also has value-only outputs prepares the core's
 // records for those first, then its own.
 lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv,
-                     int32_t* status, double* grad, double* loglike, int block, int bps, int lane_map, cudaStream_t s) {
+                     int32_t* status, double* grad, double* loglike, int block, int bps, int lane_map, cudaStream_t s,
+                     const ShiftArgs* shift = nullptr) {
     lcdm_status st;
     const bool dz = separate_dz(P);
     if (P.split_mask || dz || !P.legacy) {
         const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.time != 0, P.absorb != 0, core_ns(P.prec)};
-        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
+        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s, shift);
         if (st != LCDM_OK) return st;
     }
     if (P.split_mask) {
@@ -456,7 +460,7 @@ lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_
     }
     if (P.legacy) {
         const PrepNeed need = {true, P.prec, true, true, true, 0};
-        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s);
+        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s, shift);
         if (st != LCDM_OK) return st;
     }
     return launch_main(P, block, bps, lane_map, s);
@@ -601,7 +605,6 @@ HostCarve host_carve(char* base, int64_t B, int64_t n, int ncol, size_t es) {
 // (d_C, X, d_M).
 struct BetweenCarve {
     Carved rec;
-    double* params4;
     double* jac;
     double* scale;
     float4* rowf;
@@ -619,7 +622,6 @@ BetweenCarve between_carve(char* base, int64_t B, int64_t npairs, int ncol, size
     c.rec.recD = (double*)rec;
     c.rec.core = rec;
     c.rec.recF = rec ? (float2*)(rec + align256((size_t)B * NREC * sizeof(double))) : nullptr;
-    c.params4 = (double*)take((size_t)B * 4 * sizeof(double));
     c.jac = (double*)take((size_t)B * 4 * ncol * sizeof(double));
     c.scale = (double*)take((size_t)B * sizeof(double));
     c.rowf = (float4*)take((size_t)B * sizeof(float4));
@@ -640,21 +642,17 @@ lcdm_status between_npairs(int64_t B, int64_t n, const lcdm_opts* opts, int64_t*
     return LCDM_OK;
 }
 
-// Shift every row to its lower limit.
-lcdm_status between_setup(const double* params, int64_t B, const double* z1, int ncol, const BetweenCarve& w,
-                          cudaStream_t stream) {
+// The shift of every row to its lower limit, for the preparation.
+ShiftArgs between_shift(const double* params, int64_t B, const double* z1, int ncol, const BetweenCarve& w, bool grad) {
     ShiftArgs sa;
     sa.params = params;
     sa.z1 = z1;
     sa.B = B;
     sa.ncol = ncol;
-    sa.params4 = w.params4;
-    sa.jac = w.jac;
+    sa.jac = grad ? w.jac : nullptr;
     sa.scale = w.scale;
     sa.rowf = w.rowf;
-    if (launch_shift(sa, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-    g_launches++;
-    return LCDM_OK;
+    return sa;
 }
 
 }  // namespace
@@ -687,10 +685,9 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
     if (ws_bytes < w.bytes) return LCDM_ERR_WORKSPACE;
     lcdm_opts o4 = *opts;
     o4.ncol = 4;
-    st = between_setup(params, B, z1, ncol, w, stream);
-    if (st != LCDM_OK) return st;
+    const ShiftArgs shift = between_shift(params, B, z1, ncol, w, grad != nullptr);
     Plan P;
-    make_plan(w.params4, B, offsets, z2, n, out, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad ? w.gradp : nullptr,
+    make_plan(params, B, offsets, z2, n, out, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad ? w.gradp : nullptr,
               nullptr, cosmo_status, &o4, w.rec, P);
     PairMapArgs m;
     memset(&m, 0, sizeof(m));
@@ -716,13 +713,15 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
             cotk[i] = cot[i];
             if (cot[i] && w.cotp[i]) { m.cotp[i] = w.cotp[i]; cotk[i] = w.cotp[i]; }
         }
+        // (which need the rows' constants before the preparation has run)
+        if (launch_shift(shift, stream) != cudaSuccess) return LCDM_ERR_CUDA;
         if (launch_pair_pre(m, stream) != cudaSuccess) return LCDM_ERR_CUDA;
-        g_launches++;
-        make_plan(w.params4, B, offsets, w.zp, n, out, nullptr, cotk, nullptr, 0, 1, w.gradp, nullptr, cosmo_status, &o4,
+        g_launches += 2;
+        make_plan(params, B, offsets, w.zp, n, out, nullptr, cotk, nullptr, 0, 1, w.gradp, nullptr, cosmo_status, &o4,
                   w.rec, P);
     }
-    st = run_plan(P, w.params4, B, &o4, w.rec, cosmo_status, grad ? w.gradp : nullptr, nullptr, opts->block,
-                  opts->blocks_per_sm, opts->lane_map, stream);
+    st = run_plan(P, params, B, &o4, w.rec, cosmo_status, grad ? w.gradp : nullptr, nullptr, opts->block,
+                  opts->blocks_per_sm, opts->lane_map, stream, &shift);
     if (st != LCDM_OK) return st;
     if (out && P.legacy) {
         for (int i = 0; i < LCDM_NOUT; i++) m.out[i] = out[i];
@@ -809,10 +808,9 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     if (ws_bytes < w.bytes) return LCDM_ERR_WORKSPACE;
     lcdm_opts o4 = *opts;
     o4.ncol = 4;
-    lcdm_status st = between_setup(params, B, z1, ncol, w, stream);
-    if (st != LCDM_OK) return st;
+    const ShiftArgs shift = between_shift(params, B, z1, ncol, w, grad != nullptr);
     const PrepNeed need = {false, 0, grad != nullptr, true, false, CORE_NS_ONCE};
-    st = run_prep(w.params4, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream);
+    lcdm_status st = run_prep(params, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream, &shift);
     if (st != LCDM_OK) return st;
     LimitArgs la;
     la.rec = (const double*)w.rec.core;

@@ -9,51 +9,12 @@
 
 namespace lcdm {
 
-// ------------------------------------------------------------ row shift ----
+// The row shift alone, for the per-pair maps.
 __global__ void shift_kernel(ShiftArgs a) {
     const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= a.B) return;
-    const int nc = a.ncol;
-    const double* p = a.params + b * nc;
-    const double H0 = p[0], Om = p[1], OL = p[2], Or = p[3];
-    const double Ok = nc == 5 ? p[4] : 1.0 - Om - OL - Or;
-    const double z1 = a.z1[b];
-    const double s = 1.0 + z1, s2 = s * s, s3 = s2 * s, s4 = s2 * s2;
-    // E^2(z1), eq. (2.2); exactly 1 at z1 = 0 under the closure
-    const double E1 = (z1 == 0.0 && nc == 4) ? 1.0 : Or * s4 + Om * s3 + Ok * s2 + OL;
-    double* q = a.params4 + b * 4;
-    double* J = a.jac + b * 4 * nc;
-    if (!(z1 >= 0.0) || !isfinite(z1) || !(E1 > 0.0) || !isfinite(E1)) {
-        const double nan = CUDART_NAN;
-        for (int i = 0; i < 4; i++) q[i] = nan;
-        for (int i = 0; i < 4 * nc; i++) J[i] = nan;
-        a.scale[b] = nan;
-        a.rowf[b] = make_float4(nan, nan, nan, nan);
-        return;
-    }
-    const double irE = E1 > 1e-280 && E1 < 1e280 ? rsq(E1) : 1.0 / sqrt(E1), rE = E1 * irE, iE = irE * irE;
-    const double pw[4] = {s3, 1.0, s4, s2};       // powers of s for (Om, OL, Or, Ok)
-    const double om[4] = {Om, OL, Or, Ok};
-    q[0] = H0 * rE;
-    for (int i = 0; i < 3; i++) q[1 + i] = om[i] * pw[i] * iE;
-    // derivatives: column 0 is H0; the Omega columns act on (Om, OL, Or[, Ok]),
-    // with dOk = -1 for each of the first three under the closure
-    J[0 * nc + 0] = rE;
-    for (int i = 0; i < 3; i++) J[(1 + i) * nc + 0] = 0.0;
-    for (int c = 1; c < nc; c++) {
-        double d[4] = {0.0, 0.0, 0.0, 0.0};
-        d[c - 1] = 1.0;
-        if (nc == 4) d[3] = -1.0;
-        double dE = 0.0;
-        for (int i = 0; i < 4; i++) dE += pw[i] * d[i];
-        J[0 * nc + c] = 0.5 * H0 * dE * irE;
-        for (int i = 0; i < 3; i++) J[(1 + i) * nc + c] = (pw[i] * d[i] - q[1 + i] * dE) * iE;
-    }
-    a.scale[b] = s;
-    // z1 as an unevaluated float sum hi + lo, so that z2 - z1 and the sign test
-    // z2 >= z1 come out right in float32 arithmetic when z2 is close to z1
-    const float hi = (float)z1;
-    a.rowf[b] = make_float4(hi, (float)(z1 - (double)hi), (float)rcp_(s), (float)s);
+    double q[4];
+    shift_row(a, b, true, q);
 }
 
 cudaError_t launch_shift(const ShiftArgs& a, cudaStream_t s) {
@@ -63,6 +24,7 @@ cudaError_t launch_shift(const ShiftArgs& a, cudaStream_t s) {
 }
 
 // ------------------------------------------------------- per-pair maps -----
+// (where X has tangents; other plans map in the pair kernel, see LimitMap)
 // Each warp takes a contiguous run of pairs, lane l every 32nd pair from l
 // (coalesced); the row of a lane's first pair comes from a binary search of
 // the CSR offsets, later rows from stepping forward.

@@ -24,7 +24,10 @@
 // derivatives d/dOmega'_a - d/dOk' (a = m, L, r).
 #pragma once
 #include <cuda_runtime.h>
+#include <math_constants.h>
 #include <stdint.h>
+
+#include "lcdm_core.cuh"
 
 namespace lcdm {
 
@@ -33,11 +36,58 @@ struct ShiftArgs {
     const double* z1;       // [B]
     int64_t B;
     int ncol;
-    double* params4;        // [B][4] (H0', Om', OL', Or'), closure
-    double* jac;            // [B][4][ncol] d params4 / d params
+    double* jac;            // [B][4][ncol] d (H0', Om', OL', Or') / d params, optional
     double* scale;          // [B] s = 1 + z1 (NaN for an invalid row)
     float4* rowf;           // [B] (z1 hi, z1 lo, 1/s, s) in float32 for the FP32 pair maps
 };
+
+// The shifted row q = (H0', Om', OL', Or') of row b (closure form); `write`: also
+// its Jacobian and constants.  Part of the root preparation (a kernel of its
+// own took 7 us of the 97 of 4096 rows x 1024 pairs).
+__device__ __forceinline__ void shift_row(const ShiftArgs& a, int64_t b, bool write, double* q) {
+    const int nc = a.ncol;
+    const double* p = a.params + b * nc;
+    const double H0 = p[0], Om = p[1], OL = p[2], Or = p[3];
+    const double Ok = nc == 5 ? p[4] : 1.0 - Om - OL - Or;
+    const double z1 = a.z1[b];
+    const double s = 1.0 + z1, s2 = s * s, s3 = s2 * s, s4 = s2 * s2;
+    // E^2(z1), eq. (2.2); exactly 1 at z1 = 0 under the closure
+    const double E1 = (z1 == 0.0 && nc == 4) ? 1.0 : Or * s4 + Om * s3 + Ok * s2 + OL;
+    if (!(z1 >= 0.0) || !isfinite(z1) || !(E1 > 0.0) || !isfinite(E1)) {
+        const double nan = CUDART_NAN;
+        for (int i = 0; i < 4; i++) q[i] = nan;
+        if (!write) return;
+        if (a.jac)
+            for (int i = 0; i < 4 * nc; i++) a.jac[b * 4 * nc + i] = nan;
+        a.scale[b] = nan;
+        a.rowf[b] = make_float4(nan, nan, nan, nan);
+        return;
+    }
+    const double irE = E1 > 1e-280 && E1 < 1e280 ? rsq(E1) : 1.0 / sqrt(E1), rE = E1 * irE, iE = irE * irE;
+    const double pw[4] = {s3, 1.0, s4, s2};       // powers of s for (Om, OL, Or, Ok)
+    q[0] = H0 * rE;
+    q[1] = Om * s3 * iE;
+    q[2] = OL * iE;
+    q[3] = Or * s4 * iE;
+    if (!write) return;
+    if (a.jac) {
+        // derivatives: column 0 is H0; the Omega columns act on (Om, OL, Or[, Ok]),
+        // with dOk = -1 for each of the first three under the closure
+        double* J = a.jac + b * 4 * nc;
+        J[0] = rE;
+        for (int i = 0; i < 3; i++) J[(1 + i) * nc] = 0.0;
+        for (int c = 1; c < nc; c++) {
+            const double dE = pw[c - 1] - (nc == 4 ? s2 : 0.0);
+            J[c] = 0.5 * H0 * dE * irE;
+            for (int i = 0; i < 3; i++) J[(1 + i) * nc + c] = ((i == c - 1 ? pw[i] : 0.0) - q[1 + i] * dE) * iE;
+        }
+    }
+    a.scale[b] = s;
+    // z1 as an unevaluated float sum hi + lo, so that z2 - z1 and the sign test
+    // z2 >= z1 come out right in float32 arithmetic when z2 is close to z1
+    const float hi = (float)z1;
+    a.rowf[b] = make_float4(hi, (float)(z1 - (double)hi), (float)rcp_(s), (float)s);
+}
 
 struct PairMapArgs {
     const int64_t* offsets; // CSR offsets, or null for the dense layout

@@ -331,6 +331,10 @@ LCDM_HD float one_plus(float q, float ql, float z) {
     return s.hi + (s.lo + fmaf(ql, z, e1));
 }
 LCDM_HD F2 one_plus(F2 q, F2 ql, F2 z) { return mkf2(one_plus(q.x, ql.x, z.x), one_plus(q.y, ql.y, z.y)); }
+// w - n^2, rounded once
+LCDM_HD float fms_(float n, float w) { return fmaf(-n, n, w); }
+LCDM_HD double fms_(double n, double w) { return fma(-n, n, w); }
+LCDM_HD F2 fms_(F2 n, F2 w) { return mkf2(fms_(n.x, w.x), fms_(n.y, w.y)); }
 // power of two near 1/z for very large z
 LCDM_HD float scale_of(float z) { return z < 1e38f ? pow2i<float>(-even_exponent(z)) : 0.0f; }
 LCDM_HD double scale_of(double z) {
@@ -478,6 +482,13 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             iP = wr * wi;
             uR = nr * nA + ni * nB;
             uI = ni * nA + nr * nB;
+        }
+        if (WX && sizeof(R) == 4) {
+            // the absorption distance is a difference of terms twice its size:
+            // one Newton step takes the approximate square roots to half an ulp
+            const T hf = cst<T>(0.5);
+            nA = nA + hf * rA * fms_(nA, wA);
+            nB = nB + hf * rB * fms_(nB, wB);
         }
         s1 = nA * nB + Pn;
         zh = z;

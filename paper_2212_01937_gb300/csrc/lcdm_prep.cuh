@@ -2,6 +2,7 @@
 // classify the roots, choose the root labels, precompute the per-cosmology
 // constants and the root tangents (App. A, eqs. A.1-A.4).
 #pragma once
+#include "lcdm_between.cuh"
 #include "lcdm_corerec.cuh"
 #include "lcdm_kernels.cuh"
 
@@ -886,6 +887,7 @@ __device__ void write_core(const RowRoots& r, const cd (*dr)[RF_KT], int lane, b
 }
 
 struct PrepArgs {
+    ShiftArgs shift;        // general limits: the rows are shifted first (shift.z1 null: they are not)
     const double* params;   // [B][ncol]
     int64_t B;
     int ncol;
@@ -911,7 +913,10 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
     const bool inb = b < a.B;
     const int ncol = a.ncol;
     // lanes past the end work on a copy of the last row and write nothing
-    const double* prow = a.params + (inb ? b : a.B - 1) * ncol;
+    const int64_t bb = inb ? b : a.B - 1;
+    double shifted[4];
+    if (a.shift.z1) shift_row(a.shift, bb, inb && j == 0, shifted);
+    const double* prow = a.shift.z1 ? shifted : a.params + bb * ncol;
     RowRoots r;
     cd dr[4][RF_KT];
     bool labelled;
