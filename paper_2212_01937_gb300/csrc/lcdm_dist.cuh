@@ -1,6 +1,6 @@
-// Distance assembly for one (cosmology, redshift) pair, written once for any
-// scalar S: a plain number (values only) or Dual<T,K> (values and tangents
-// with respect to the density parameters).
+// Distance assembly for one (cosmology, redshift) pair with tangents carried
+// forward (Dual<T,K>): used where the absorption distance is differentiated
+// (all other pair work: lcdm_core.cuh).
 //
 // Carlson integrals enter through carlson_any / rc_any.  Their tangents are
 // carried through one shared duplication sequence as dual numbers (see
@@ -19,14 +19,9 @@
 namespace lcdm {
 
 
-// ---------------------------------------------------------------- values ----
-template <class T> LCDM_HD T rc_any(T x, T y, int* fail) {
-    if (sval(y) < 0) {
-        T x2 = x - y, y2 = -y;
-        return ssqrt(x / x2) * rc_value(x2, y2, fail);
-    }
-    return rc_value(x, y, fail);
-}
+// --------------------------------------------------------------- tangents ---
+// R_C (see rc_value_grad below)
+template <class T, int K> LCDM_HD Dual<T, K> rc_any(const Dual<T, K>& x, const Dual<T, K>& y, int* fail);
 
 // The triple enters through square roots: x1 = u1^2 and the pair y = u^2
 // (a conjugate pair, or two reals).  The R_J tracks are given by
@@ -155,8 +150,8 @@ template <class S> LCDM_HD S phi_rc(const S& w, int* fail) {
 //   eq. (3.8):  t H0 = 2z [ R_C(k s5, k q5) - eps_A R_F - z^2/3 m_A (1 + eps_A rho_B) |1 + eps_A rho_P|^2 R_J(u~^2, lam u_A5^2) ]
 //   eq. (3.9):  X H0/c = z [ T0 + (2 rho_B^2 - |P-B|^2) R_F + rho_A G ]
 // with u~ = sqrt(lam) u and the terms defined in the code.
-template <class S, class PS, bool WT, bool WX>
-LCDM_HD void quartic_integrals(typename Base<S>::type z, const S& lam, const S& aA, const S& mA, const S& epsA,
+template <class S, class PS, bool WT>
+LCDM_NI void quartic_integrals(typename Base<S>::type z, const S& lam, const S& aA, const S& mA, const S& epsA,
                                const S& rhoA, const S& B, const PS& P, const S& YB, const PS& YP, const S& qA,
                                const S& qB, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX, int* fail) {
     typedef typename Base<S>::type T;
@@ -181,11 +176,11 @@ LCDM_HD void quartic_integrals(typename Base<S>::type z, const S& lam, const S& 
     PS rhoP = padd(P, one);
     S ppPA = pprod(padd(pscale(rhoP, epsA), one));     // |P - A|^2 / rho_A^2
     S ppPB = pprod(padd(P, -B));
-    enum { NJ = (WT ? 1 : 0) + (WX ? 1 : 0) };
-    S p[NJ > 0 ? NJ : 1];
-    int jt = 0, jx = WT ? 1 : 0;
+    enum { NJ = WT ? 2 : 1 };
+    S p[NJ];
+    const int jt = 0, jx = WT ? 1 : 0;
     if (WT) p[jt] = -(mA * ppPA * rhoB * z2);          // lam u_A5^2 - x1
-    if (WX) p[jx] = -(lam * ppPB * z2);                // lam u_B0^2 - x1
+    p[jx] = -(lam * ppPB * z2);                // lam u_B0^2 - x1
     // eq. (3.8), i = A: everything but the R_F and R_J terms before the
     // duplication sequence, so that only three factors stay live across it
     S RCp, kB, cJ;
@@ -205,14 +200,14 @@ LCDM_HD void quartic_integrals(typename Base<S>::type z, const S& lam, const S& 
         kB = (cst<T>(2.0) + z + epsA * (one + z)) / (ssqrt(cA) + one);
         cJ = mA * (one + epsA * rhoB) * ppPA * (z2 * third);
     }
-    S RF, RD1, RJ[NJ > 0 ? NJ : 1], DJ;
-    carlson_any<NJ, WX, WX>(uAB, uAP, p, RF, RD1, RJ, fail, &DJ);
+    S RF, RD1, RJ[NJ], DJ;
+    carlson_any<NJ, true, true>(uAB, uAP, p, RF, RD1, RJ, fail, &DJ);
     Ichi = RF * (z + z);                               // eq. (3.7)
     if (WT) {
         S Bk = RCp * kB - RF;
         It = (RCp + epsA * Bk - cJ * RJ[jt]) * (z + z);
     }
-    if (WX) {                                          // eq. (3.9), i = B, l = A
+    {                                                  // eq. (3.9), i = B, l = A
         // The l = A part of (3.9), rho_A G, is a sum of O(1) terms that cancel to
         // O(lam): written out so that every term is O(1) by itself:
         //   G1 + G4 = z^2/3 |P-B|^2 [c (a_A + lam B) h0 Delta_J + E1 R_D1],
@@ -245,8 +240,8 @@ LCDM_HD void quartic_integrals(typename Base<S>::type z, const S& lam, const S& 
     }
 }
 
-template <class S, class PS, bool WT, bool WX>
-LCDM_HD void cubic_integrals(typename Base<S>::type z, const S& A, const PS& P, const S& YA, const PS& YP,
+template <class S, class PS, bool WT>
+LCDM_NI void cubic_integrals(typename Base<S>::type z, const S& A, const PS& P, const S& YA, const PS& YP,
                              const S& amh, const S& qA, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX,
                              int* fail) {
     typedef typename Base<S>::type T;
@@ -274,10 +269,10 @@ LCDM_HD void cubic_integrals(typename Base<S>::type z, const S& A, const PS& P, 
         RC5 = rc_any(s5 * s5, q5, fail);
     }
     S RF, RD1, RJ[1];
-    carlson_any<NJ, WX, false>(uA, uP, p, RF, RD1, RJ, fail);
+    carlson_any<NJ, true, false>(uA, uP, p, RF, RD1, RJ, fail);
     Ichi = amh * RF * (z + z);                         // eq. (B.1)
     if (WT) It = amh * (z + z) * (RJ[0] * (z2 * cst<T>(1.0 / 3.0)) + RC5);   // eq. (B.2)
-    if (WX) {                                          // eq. (B.3), i = A
+    {                                                  // eq. (B.3), i = A
         S ppPA = pprod(padd(P, -A));
         S eA = one / (XA + YA);
         PS XY = XP + YP;
@@ -287,39 +282,6 @@ LCDM_HD void cubic_integrals(typename Base<S>::type z, const S& A, const PS& P, 
         S T2 = (A + psum(P) + cst<T>(3.0)) * (ppPA * RD1 * (z2 * cst<T>(1.0 / 3.0)) + YA * XA / uA) * cst<T>(2.0);
         IX = amh * (T0 + T1 + T2) * (z + z) * cst<T>(1.0 / 3.0);
     }
-}
-
-// The same integrals as one real call, for the kernels whose tangents or
-// outputs need more registers than the inlined path can hold (seven-column
-// tangents, X's tangents): there the allocator handles the pair in two parts.
-template <class S, class PS, bool WT, bool WX>
-LCDM_NI void quartic_integrals_call(typename Base<S>::type z, const S& lam, const S& aA, const S& mA, const S& epsA,
-                                    const S& rhoA, const S& B, const PS& P, const S& YB, const PS& YP, const S& qA,
-                                    const S& qB, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX, int* fail) {
-    quartic_integrals<S, PS, WT, WX>(z, lam, aA, mA, epsA, rhoA, B, P, YB, YP, qA, qB, wP, nrm, Ichi, It, IX, fail);
-}
-template <class S, class PS, bool WT, bool WX>
-LCDM_NI void cubic_integrals_call(typename Base<S>::type z, const S& A, const PS& P, const S& YA, const PS& YP,
-                                  const S& amh, const S& qA, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX,
-                                  int* fail) {
-    cubic_integrals<S, PS, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
-}
-
-template <bool CALL, class S, class PS, bool WT, bool WX>
-LCDM_HD void quartic_integrals_any(typename Base<S>::type z, const S& lam, const S& aA, const S& mA, const S& epsA,
-                                   const S& rhoA, const S& B, const PS& P, const S& YB, const PS& YP, const S& qA,
-                                   const S& qB, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX, int* fail) {
-    if constexpr (CALL)
-        quartic_integrals_call<S, PS, WT, WX>(z, lam, aA, mA, epsA, rhoA, B, P, YB, YP, qA, qB, wP, nrm, Ichi, It, IX, fail);
-    else
-        quartic_integrals<S, PS, WT, WX>(z, lam, aA, mA, epsA, rhoA, B, P, YB, YP, qA, qB, wP, nrm, Ichi, It, IX, fail);
-}
-template <bool CALL, class S, class PS, bool WT, bool WX>
-LCDM_HD void cubic_integrals_any(typename Base<S>::type z, const S& A, const PS& P, const S& YA, const PS& YP,
-                                 const S& amh, const S& qA, const PS& wP, const S& nrm, S& Ichi, S& It, S& IX,
-                                 int* fail) {
-    if constexpr (CALL) cubic_integrals_call<S, PS, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
-    else cubic_integrals<S, PS, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
 }
 
 }  // namespace lcdm

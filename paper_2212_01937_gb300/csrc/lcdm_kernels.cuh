@@ -1,9 +1,8 @@
-// Kernels of the distance path:
-//   (the root preparation kernel is in lcdm_prep.cuh)
-//   pairs_kernel  persistent warps over contiguous ranges of (cosmology,
-//                 redshift) pairs: distance integrals (3.7)-(3.9) / (B.1)-(B.3),
-//                 observables, tangents, and the per-cosmology reductions of the
-//                 vector-Jacobian product and of the Gaussian log-likelihood.
+// What the pair kernels share (arguments, the curvature map, the per-row
+// reductions), and the kernel of the absorption distance's tangents: forward
+// mode through the duplication, one real call per pair.  All other pair work
+// runs on the core (lcdm_corekernel.cuh); the root preparation is in
+// lcdm_prep.cuh.
 #pragma once
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -147,94 +146,74 @@ template <> LCDM_HD float one_plus_qz<float>(const double*, const float2* rf, in
     return s.hi + (s.lo + fmaf(ql, z, e1));
 }
 
-// Build the root quantities in scalar S and evaluate the integrals.
-template <class T, int K, bool WT, bool WX> struct PairEval {
-    typedef typename std::conditional<(K > 0), Dual<T, K>, T>::type S;
-    // the integrals inline, or as one call (see quartic_integrals_call)
-    static constexpr bool SPLIT = K > 3 || (K > 0 && WX);
+// Build the root quantities as dual numbers and evaluate the integrals.
+template <class T, int K, bool WT> struct PairEval {
+    typedef Dual<T, K> S;
 
     static LCDM_HD S val(const double* rd, const float2* rf, int i, int di) {
         S s;
-        if constexpr (K > 0) {
-            s.v = recv<T>(rd, rf, i);
+        s.v = recv<T>(rd, rf, i);
 #pragma unroll
-            for (int k = 0; k < K; k++) s.d[k] = recv<T>(rd, rf, di + k);
-        } else {
-            s = recv<T>(rd, rf, i);
-        }
+        for (int k = 0; k < K; k++) s.d[k] = recv<T>(rd, rf, di + k);
         return s;
     }
     // Y = sqrt(-r) with its tangent -dr / (2Y)
     static LCDM_HD S yval(const double* rd, const float2* rf, int iy, const S& r) {
         S y;
-        if constexpr (K > 0) {
-            y.v = recv<T>(rd, rf, iy);
-            T h = cst<T>(-0.5) / y.v;
+        y.v = recv<T>(rd, rf, iy);
+        T h = cst<T>(-0.5) / y.v;
 #pragma unroll
-            for (int k = 0; k < K; k++) y.d[k] = r.d[k] * h;
-        } else {
-            y = recv<T>(rd, rf, iy);
-        }
+        for (int k = 0; k < K; k++) y.d[k] = r.d[k] * h;
         return y;
     }
 
-    static LCDM_HD void run(T z, const double* rd, const float2* rf, int kind, S& Ichi,
-                                               S& It, S& IX, int* fail) {
+    template <class PS>
+    static LCDM_HD void integrals(T z, const double* rd, const float2* rf, bool quartic, const PS& P, const PS& YP,
+                                  const PS& wP, S& Ichi, S& It, S& IX, int* fail) {
         S A = val(rd, rf, RF_A, RF_DA);
-        S amh = val(rd, rf, RF_AMH, RF_DAMH);
-        S YA = yval(rd, rf, RF_YA, A);
-        S Pre = val(rd, rf, RF_PRE, RF_DPRE), Pim = val(rd, rf, RF_PIM, RF_DPIM);
         S qA = val(rd, rf, RF_QA, RF_DQA), nrm = val(rd, rf, RF_NRM, RF_DNRM);
+        if (quartic) {
+            S B = val(rd, rf, RF_B, RF_DB);
+            S YB = yval(rd, rf, RF_YB, B);
+            quartic_integrals<S, PS, WT>(z, val(rd, rf, RF_LAM, RF_DLAM), val(rd, rf, RF_AA, RF_DAA),
+                                         val(rd, rf, RF_MA, RF_DMA), val(rd, rf, RF_EPSA, RF_DEPSA),
+                                         val(rd, rf, RF_RHOA, RF_DRHOA), B, P, YB, YP, qA, val(rd, rf, RF_QB, RF_DQB), wP,
+                                         nrm, Ichi, It, IX, fail);
+        } else {
+            S YA = yval(rd, rf, RF_YA, A);
+            cubic_integrals<S, PS, WT>(z, A, P, YA, YP, val(rd, rf, RF_AMH, RF_DAMH), qA, wP, nrm, Ichi, It, IX, fail);
+        }
+    }
+
+    static LCDM_HD void run(T z, const double* rd, const float2* rf, int kind, S& Ichi, S& It, S& IX, int* fail) {
+        S Pre = val(rd, rf, RF_PRE, RF_DPRE), Pim = val(rd, rf, RF_PIM, RF_DPIM);
         S qPre = val(rd, rf, RF_QPRE, RF_DQPRE), qPim = val(rd, rf, RF_QPIM, RF_DQPIM);
         // w_P = 1 + z q_P (its tangent z dq_P), the first member's real part
         // by one_plus_qz
         S wre = qPre * z, wim = qPim * z;
-        if constexpr (K > 0) wre.v = one_plus_qz<T>(rd, rf, RF_QPRE, z);
-        else wre = one_plus_qz<T>(rd, rf, RF_QPRE, z);
+        wre.v = one_plus_qz<T>(rd, rf, RF_QPRE, z);
         if (kind == 0 || kind == 2) {
-            CPair<S> P = mkcp(mkcx<S>(Pre, Pim)), wP = mkcp(mkcx<S>(wre, wim));
             Cx<S> yv;
             yv.re = val(rd, rf, RF_YPRE, RF_YPRE);
             yv.im = val(rd, rf, RF_YPIM, RF_YPIM);
-            if constexpr (K > 0) {
-                // dY = -dP / (2Y), complex
-                Cx<T> y0 = mkcx<T>(yv.re.v, yv.im.v);
-                Cx<T> h = cxrcp(y0);
+            // dY = -dP / (2Y), complex
+            Cx<T> y0 = mkcx<T>(yv.re.v, yv.im.v);
+            Cx<T> h = cxrcp(y0);
 #pragma unroll
-                for (int k = 0; k < K; k++) {
-                    Cx<T> dp = mkcx<T>(Pre.d[k], Pim.d[k]);
-                    Cx<T> dy = dp * h;
-                    yv.re.d[k] = dy.re * cst<T>(-0.5);
-                    yv.im.d[k] = dy.im * cst<T>(-0.5);
-                }
+            for (int k = 0; k < K; k++) {
+                Cx<T> dp = mkcx<T>(Pre.d[k], Pim.d[k]);
+                Cx<T> dy = dp * h;
+                yv.re.d[k] = dy.re * cst<T>(-0.5);
+                yv.im.d[k] = dy.im * cst<T>(-0.5);
             }
-            CPair<S> YP = mkcp(yv);
-            if (kind == 0) {
-                S B = val(rd, rf, RF_B, RF_DB);
-                S YB = yval(rd, rf, RF_YB, B);
-                quartic_integrals_any<SPLIT, S, CPair<S>, WT, WX>(z, val(rd, rf, RF_LAM, RF_DLAM), val(rd, rf, RF_AA, RF_DAA),
-                                                       val(rd, rf, RF_MA, RF_DMA), val(rd, rf, RF_EPSA, RF_DEPSA),
-                                                       val(rd, rf, RF_RHOA, RF_DRHOA), B, P, YB, YP, qA,
-                                                       val(rd, rf, RF_QB, RF_DQB), wP, nrm, Ichi, It, IX, fail);
-            } else {
-                cubic_integrals_any<SPLIT, S, CPair<S>, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
-            }
+            integrals<CPair<S> >(z, rd, rf, kind == 0, mkcp(mkcx<S>(Pre, Pim)), mkcp(yv), mkcp(mkcx<S>(wre, wim)), Ichi, It,
+                                 IX, fail);
         } else {
             wim = wim + cst<T>(1.0);
-            if constexpr (K > 0) wim.v = one_plus_qz<T>(rd, rf, RF_QPIM, z);
-            else wim = one_plus_qz<T>(rd, rf, RF_QPIM, z);
-            RPair<S> P = mkrp<S>(Pre, Pim), wP = mkrp<S>(wre, wim);
-            RPair<S> YP = mkrp<S>(yval(rd, rf, RF_YPRE, Pre), yval(rd, rf, RF_YPIM, Pim));
-            if (kind == 1) {
-                S B = val(rd, rf, RF_B, RF_DB);
-                S YB = yval(rd, rf, RF_YB, B);
-                quartic_integrals_any<SPLIT, S, RPair<S>, WT, WX>(z, val(rd, rf, RF_LAM, RF_DLAM), val(rd, rf, RF_AA, RF_DAA),
-                                                       val(rd, rf, RF_MA, RF_DMA), val(rd, rf, RF_EPSA, RF_DEPSA),
-                                                       val(rd, rf, RF_RHOA, RF_DRHOA), B, P, YB, YP, qA,
-                                                       val(rd, rf, RF_QB, RF_DQB), wP, nrm, Ichi, It, IX, fail);
-            } else {
-                cubic_integrals_any<SPLIT, S, RPair<S>, WT, WX>(z, A, P, YA, YP, amh, qA, wP, nrm, Ichi, It, IX, fail);
-            }
+            wim.v = one_plus_qz<T>(rd, rf, RF_QPIM, z);
+            integrals<RPair<S> >(z, rd, rf, kind == 1, mkrp<S>(Pre, Pim),
+                                 mkrp<S>(yval(rd, rf, RF_YPRE, Pre), yval(rd, rf, RF_YPIM, Pim)), mkrp<S>(wre, wim), Ichi,
+                                 It, IX, fail);
         }
     }
 };
@@ -243,7 +222,7 @@ template <class T, int K, bool WT, bool WX> struct PairEval {
 // per-pair results in the output type TO
 template <class TO, int K> struct PairOut {
     TO v[N_OUT];
-    TO d[N_OUT][K > 0 ? K : 1];   // tangents w.r.t. the Omega directions
+    TO d[N_OUT][K];               // tangents w.r.t. the Omega directions
     TO h0[N_OUT];                 // derivative w.r.t. H0
 };
 
@@ -253,30 +232,14 @@ template <class TO> __device__ __forceinline__ TO load_io(const void* p, int64_t
 
 // Evaluate one pair.  PREC 0: FP64 throughout.  PREC 1: FP32 throughout (the
 // root records come from the FP64 preparation).
-template <int PREC, int K, bool WT, bool WX>
-LCDM_HD void eval_pair(typename std::conditional<PREC == 0, double, float>::type zin,
-                                          const double* rd, const float2* rf, PairOut<
-                                          typename std::conditional<PREC == 0, double, float>::type, K>& o,
-                                          int* fail) {
+template <int PREC, int K, bool WT>
+LCDM_HD void eval_pair(typename std::conditional<PREC == 0, double, float>::type zin, const double* rd, const float2* rf,
+                       PairOut<typename std::conditional<PREC == 0, double, float>::type, K>& o, int* fail) {
     typedef typename std::conditional<PREC == 0, double, float>::type TO;
     const int kind = (int)rf[RF_KIND].x;
-    TO Ichi, It = 0, IX = 0;
-    TO dIchi[K > 0 ? K : 1], dIt[K > 0 ? K : 1], dIX[K > 0 ? K : 1];
-    {
-        typedef PairEval<TO, K, WT, WX> E;
-        typename E::S a, b, c;
-        E::run(zin, rd, rf, kind, a, b, c, fail);
-        if constexpr (K > 0) {
-            Ichi = a.v; It = WT ? b.v : (TO)0; IX = WX ? c.v : (TO)0;
-            for (int k = 0; k < K; k++) {
-                dIchi[k] = a.d[k];
-                dIt[k] = WT ? b.d[k] : (TO)0;
-                dIX[k] = WX ? c.d[k] : (TO)0;
-            }
-        } else {
-            Ichi = a; It = WT ? b : (TO)0; IX = WX ? c : (TO)0;
-        }
-    }
+    typename PairEval<TO, K, WT>::S a, b, c;
+    PairEval<TO, K, WT>::run(zin, rd, rf, kind, a, b, c, fail);
+    const TO Ichi = a.v, It = WT ? b.v : (TO)0, IX = c.v;
     // observables
     const TO z = zin;
     const TO H0 = recv<TO>(rd, rf, RF_H0);
@@ -292,16 +255,14 @@ LCDM_HD void eval_pair(typename std::conditional<PREC == 0, double, float>::type
     o.v[O_MU] = (TO)5 * log10(o.v[O_DL]) + (TO)25;
     for (int i = 0; i < O_MU; i++) o.h0[i] = -o.v[i] / H0;
     o.h0[O_MU] = (TO)-5 / (ln10 * H0);
-    if constexpr (K > 0) {
-        for (int k = 0; k < K; k++) {
-            TO dOk = recv<TO>(rd, rf, RF_DOK + k);
-            o.d[O_DC][k] = DH * dIchi[k];
-            o.d[O_T][k] = tH * dIt[k];
-            o.d[O_X][k] = DH * dIX[k];
-            o.d[O_DM][k] = DH * (SD * dIchi[k] + Sk * dOk);
-            o.d[O_DL][k] = ((TO)1 + z) * o.d[O_DM][k];
-            o.d[O_MU][k] = z == (TO)0 ? (TO)0 : (TO)5 / ln10 * o.d[O_DM][k] / o.v[O_DM];
-        }
+    for (int k = 0; k < K; k++) {
+        TO dOk = recv<TO>(rd, rf, RF_DOK + k);
+        o.d[O_DC][k] = DH * a.d[k];
+        o.d[O_T][k] = WT ? tH * b.d[k] : (TO)0;
+        o.d[O_X][k] = DH * c.d[k];
+        o.d[O_DM][k] = DH * (SD * a.d[k] + Sk * dOk);
+        o.d[O_DL][k] = ((TO)1 + z) * o.d[O_DM][k];
+        o.d[O_MU][k] = z == (TO)0 ? (TO)0 : (TO)5 / ln10 * o.d[O_DM][k] / o.v[O_DM];
     }
 }
 
@@ -371,29 +332,18 @@ __device__ __forceinline__ void flush_row(const AccT* acc, int64_t row, const Pa
     if (lane == 0) add_row(a, row, v, K + 1, warp, wf, wl);
 }
 
-// Register budget: the FP32 kernels are bound by how many warps hide the
-// latency of their dependent chains, so the three-tangent kernel is held to
-// 128 registers (two full blocks per SM) and the value kernel to 85 (three),
-// which measured faster than the unconstrained allocation (the tangent
-// kernel of the benchmark step: 0.51 ms against 0.62 ms, with the pair's
-// integrals inlined).
-// (The kernels with X's tangents need more: they are left unconstrained.)
-template <int PREC, int K, bool WX>
-struct MinBlocks { enum { value = PREC == 1 ? ((K == 3 && !WX) ? 2 : (K == 0 ? 3 : 1)) : 1 }; };
-
-template <int PREC, int K, bool WT, bool WX>
-__global__ void __launch_bounds__(256, MinBlocks<PREC, K, WX>::value) pairs_kernel(PairArgs a) {
+// The kernel of X's tangents (a Jacobian or a cotangent of X is asked for): all
+// outputs of the pair in forward mode, with no register cap (inlined, or
+// capped, the divided-difference track's tangents spill over 1 KB a thread).
+template <int PREC, int K, bool WT>
+__global__ void __launch_bounds__(256, 1) pairs_kernel(PairArgs a) {
     typedef typename std::conditional<PREC == 0, double, float>::type TO;
     constexpr int NV = K + 2;   // H0, K Omega directions, loglike value
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t start = warp * a.chunk;
     const int64_t end = max(start, min(start + a.chunk, a.nnz));   // empty range past the end
-    const bool reduce = (a.grad != nullptr) || (a.loglike != nullptr);
-    const bool loglike = a.mobs != nullptr;
-    const TO inv_sig = (TO)(1.0 / a.sigma);
-    const TO lnorm = (TO)(-log(a.sigma * 2.5066282746310002));
-    const TO Mobs = (TO)a.M;
+    const bool reduce = a.grad != nullptr;
     typedef typename std::conditional<PREC == 0, double, df64>::type AccT;
     int64_t row = -1;
     // The per-lane accumulators live in shared memory (lane-private slots):
@@ -418,13 +368,11 @@ __global__ void __launch_bounds__(256, MinBlocks<PREC, K, WX>::value) pairs_kern
     }
     const int64_t len = end - start, nb = (len + 31) / 32, nb_all = a.chunk / 32;
     const int64_t s_lane = a.interleave ? nb : 1, s_it = a.interleave ? 1 : 32;
-    // With a full-SM block (256 threads) the warps of the kernels whose code per
-    // pair is largest (X's tangents, seven-column tangents) step through their
-    // ranges together, one 32-pair batch at a time: that code is about the size
+    // With a full-SM block (256 threads) the warps step through their ranges
+    // together, one 32-pair batch at a time: the code per pair is about the size
     // of the instruction cache, and warps at the same place in it share each
-    // fetched line.  Every warp then runs nb_all steps (the same number).  For
-    // the other kernels the barrier costs more than it saves (measured).
-    const bool lockstep = blockDim.x == 256 && K > 0 && (WX || K > 3);
+    // fetched line.  Every warp then runs nb_all steps (the same number).
+    const bool lockstep = blockDim.x == 256;
     for (int64_t it = 0; it < nb_all; it++) {
         if (lockstep) __syncthreads();
         if (it >= nb) continue;
@@ -450,36 +398,32 @@ __global__ void __launch_bounds__(256, MinBlocks<PREC, K, WX>::value) pairs_kern
         const float2* rf = a.recF + row * NREC;
         const int st = a.status[row];
         const TO z = load_io<TO>(a.z, zi);
-        // the pair's cotangents (or observed magnitude) are loaded before the
-        // evaluation, so that their latency hides behind it
+        // the pair's cotangents are loaded before the evaluation, so that their
+        // latency hides behind it
         TO gcot[N_OUT];
-        TO mob = (TO)0;
-        if constexpr (K > 0) {
 #pragma unroll
-            for (int i = 0; i < N_OUT; i++) gcot[i] = (reduce && !loglike && a.cot[i]) ? load_io<TO>(a.cot[i], pidx) : (TO)0;
-            if (loglike) mob = load_io<TO>(a.mobs, zi);
-        }
+        for (int i = 0; i < N_OUT; i++) gcot[i] = (reduce && a.cot[i]) ? load_io<TO>(a.cot[i], pidx) : (TO)0;
         PairOut<TO, K> o;
         int fail = 0;
         if (st == ST_OK) {
             if (z == (TO)0) {
-                for (int i = 0; i < N_OUT; i++) { o.v[i] = 0; o.h0[i] = 0; for (int k = 0; k < (K > 0 ? K : 1); k++) o.d[i][k] = 0; }
+                for (int i = 0; i < N_OUT; i++) { o.v[i] = 0; o.h0[i] = 0; for (int k = 0; k < K; k++) o.d[i][k] = 0; }
                 o.v[O_MU] = -CUDART_INF;
                 o.h0[O_MU] = (TO)(-5.0 / (2.302585092994045684 * rd[RF_H0]));
             } else {
-                eval_pair<PREC, K, WT, WX>(z, rd, rf, o, &fail);
+                eval_pair<PREC, K, WT>(z, rd, rf, o, &fail);
             }
         }
         if (st != ST_OK || fail) {
             const TO nan = (TO)CUDART_NAN;
-            for (int i = 0; i < N_OUT; i++) { o.v[i] = nan; o.h0[i] = nan; for (int k = 0; k < (K > 0 ? K : 1); k++) o.d[i][k] = nan; }
+            for (int i = 0; i < N_OUT; i++) { o.v[i] = nan; o.h0[i] = nan; for (int k = 0; k < K; k++) o.d[i][k] = nan; }
             if (fail && active && st == ST_OK) atomicMax(a.status + row, (int)ST_NOCONV);
         }
         if (active) {
 #pragma unroll
             for (int i = 0; i < N_OUT; i++) {
                 if (a.outmask & (1 << i)) reinterpret_cast<TO*>(a.out[i])[pidx] = o.v[i];
-                if (K > 0 && a.jac[i]) {
+                if (a.jac[i]) {
                     TO* jp = reinterpret_cast<TO*>(a.jac[i]) + pidx * a.ncol;
                     jp[0] = o.h0[i];
                     for (int k = 0; k < K; k++) jp[1 + k] = o.d[i][k];
@@ -492,22 +436,13 @@ __global__ void __launch_bounds__(256, MinBlocks<PREC, K, WX>::value) pairs_kern
 #pragma unroll
         for (int i = 0; i < NV; i++) c[i] = 0;
         if (active && st == ST_OK && !fail) {
-            if (loglike) {
-                TO r = ((K > 0 ? mob : load_io<TO>(a.mobs, zi)) - o.v[O_MU] - Mobs) * inv_sig;
-                TO w = r * inv_sig;
-                c[0] = w * o.h0[O_MU];
 #pragma unroll
-                for (int k = 0; k < K; k++) c[1 + k] = w * o.d[O_MU][k];
-                c[K + 1] = (TO)-0.5 * r * r + lnorm;
-            } else {
+            for (int i = 0; i < N_OUT; i++) {
+                if (!a.cot[i]) continue;
+                const TO g = gcot[i];
+                c[0] += g * o.h0[i];
 #pragma unroll
-                for (int i = 0; i < N_OUT; i++) {
-                    if (!a.cot[i]) continue;
-                    TO g = K > 0 ? gcot[i] : load_io<TO>(a.cot[i], pidx);
-                    c[0] += g * o.h0[i];
-#pragma unroll
-                    for (int k = 0; k < K; k++) c[1 + k] += g * o.d[i][k];
-                }
+                for (int k = 0; k < K; k++) c[1 + k] += g * o.d[i][k];
             }
         }
         // register accumulation while the whole warp stays on one row

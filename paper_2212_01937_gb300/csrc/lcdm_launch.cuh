@@ -14,12 +14,12 @@ struct PairsEntry {
 
 template <int PREC, int K, bool WT> struct TangentX {
     static cudaError_t launch(const CoreArgs& a, int grid, int block, cudaStream_t s) {
-        pairs_kernel<PREC, K, WT, true><<<grid, block, 0, s>>>(a.p);
+        pairs_kernel<PREC, K, WT><<<grid, block, 0, s>>>(a.p);
         return cudaGetLastError();
     }
     static int occ(int block) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pairs_kernel<PREC, K, WT, true>, block, 0) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pairs_kernel<PREC, K, WT>, block, 0) != cudaSuccess)
             return 0;
         return n;
     }
