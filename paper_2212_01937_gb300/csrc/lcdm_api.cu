@@ -213,7 +213,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
 // (0.41 against 0.39 ms for 4 M pairs of d_C, t and mu).
 #define LCDM_PACKED_ROW 256
 bool packed_plan(const Plan& P) {
-    return P.prec == 1 && !P.wx && !P.legacy && !(P.K > 0 && P.wt) && P.npairs >= P.args.B * LCDM_PACKED_ROW;
+    return P.prec == 1 && !P.legacy && !(P.K > 0 && P.wt) && P.npairs >= P.args.B * LCDM_PACKED_ROW;
 }
 
 // index of the plan's kernel in its table (4 and up: per-pair Jacobians, 8 and
@@ -222,7 +222,7 @@ bool packed_plan(const Plan& P) {
 int entry_index(const Plan& P) {
     bool jac = false;
     for (int i = 0; i < LCDM_NOUT; i++) jac = jac || P.args.jac[i];
-    if (packed_plan(P) && !jac) return 14 + (P.rowf ? 4 : P.grad_z ? 2 : 0) + (P.wt ? 1 : 0);
+    if (packed_plan(P) && !jac) return 14 + (P.rowf ? 8 : P.grad_z ? 4 : 0) + (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
     if (P.rowf) return 10 + (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
     if (P.grad_z && !P.wx && !P.legacy) return 8 + (P.wt ? 1 : 0);
     return (P.wt ? 2 : 0) + (P.wx ? 1 : 0) + (jac ? 4 : 0);
@@ -240,7 +240,7 @@ CoreArgs core_args(const Plan& P) {
 const PairsEntry& plan_entry(const Plan& P) {
     const int i = entry_index(P);
     const PairsTable& t = table(P.prec, P.K);
-    return i < 4 ? t.e[i] : i < 8 ? t.jac[i - 4] : i < 10 ? t.dz[i - 8] : i < 14 ? t.bt[i - 10] : t.packed[(i - 14) / 2][(i - 14) % 2];
+    return i < 4 ? t.e[i] : i < 8 ? t.jac[i - 4] : i < 10 ? t.dz[i - 8] : i < 14 ? t.bt[i - 10] : t.packed[(i - 14) / 4][(i - 14) % 4];
 }
 
 }  // namespace

@@ -295,6 +295,16 @@ template <class T> LCDM_HD T rc1m1_core(T e) {
     }
     return (rc1_far<T>(e, sqt(cst<T>(1.0) + e)).v - cst<T>(1.0)) / e;
 }
+LCDM_HD F2 rc1m1_core(F2 e) {
+    if (all_le(abs_(e), cst<F2>(CoreTol<float>::e_series))) {
+        const F2 w = -e;
+        F2 s = cst<F2>(-1.0 / 15);
+#pragma unroll
+        for (int n = 6; n >= 1; n--) s = cst<F2>(-1.0 / (2 * n + 1)) + w * s;
+        return s;
+    }
+    return mkf2(rc1m1_core<float>(e.x), rc1m1_core<float>(e.y));
+}
 // [R_C(1, 1-w) - (1-w)^-1/2] / w  (see phi_rc) for 0 <= w < 1, so = sqrt(1-w)
 // (which cancels if formed from w near 1).  Beyond the series' range R_C's
 // duplication is carried on the difference itself: with a = sqrt(x), b =
@@ -302,10 +312,10 @@ template <class T> LCDM_HD T rc1m1_core(T e) {
 //   F = R_C - 1/b = 2 F' - 2 w / ((a + b) b' (2 b + b')),
 // a sum of numbers of one sign.
 template <class T> LCDM_HD T phi_core(T w, T so) {
-    constexpr int NT = sizeof(T) == 4 ? 9 : 17;
+    constexpr int NT = sizeof(typename Scalar<T>::rec) == 4 ? 9 : 17;
     T a = cst<T>(1.0), b = so, sum = cst<T>(0.0), t = cst<T>(1.0), ia = cst<T>(1.0), v = w;
 #pragma unroll 1
-    for (int m = 0; m < CoreTol<T>::maxit && v > cst<T>(0.1); m++) {
+    for (int m = 0; m < CoreTol<T>::maxit && any_gt(v, cst<T>(0.1)); m++) {
         const T n = a + b, q = cst<T>(2.0) * b * n, c = sqt(q);
         sum = sum - cst<T>(2.0) * t * rcp_(n * c * (cst<T>(2.0) * b + c));
         a = n;
@@ -347,6 +357,8 @@ LCDM_HD double scale_of(double z) {
 LCDM_HD float scaling(float z) { return z > CoreTol<float>::big ? scale_of(z) : 1.0f; }
 LCDM_HD double scaling(double z) { return z > CoreTol<double>::big ? scale_of(z) : 1.0; }
 LCDM_HD F2 scaling(F2 z) { return mkf2(scaling(z.x), scaling(z.y)); }
+template <class T> LCDM_HD T unscale(T h) { return cst<T>(1.0) / h; }
+LCDM_HD F2 unscale(F2 h) { return mkf2(1.0f / h.x, 1.0f / h.y); }
 
 // Four consecutive record entries from a multiple of four (records are 16-byte
 // aligned): one 128-bit load in single precision, two in double.
@@ -692,7 +704,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T RD = tm * (one + v2 * (w2 * w2)) * r23 + cst<T>(3.0) * sD;
             if (m == 0) rp0 = sqt(p0);
             // the results belong to arguments scaled by h^2 (h = 1 but for very large z)
-            const T ih = big ? one / h : one;
+            const T ih = big ? unscale(h) : one;
             const T s1u = s1 * ih, sp0 = rp0 * ih, zz = z * z, x1 = x0 * (ih * ih);
             const T hRF = RF * h, hRD = RD * (h * h * h), hDJ = DJ * (h * h * h) * (h * h);
             const Quad<T> c0 = quad_as<T>(rc + X_C0), c3 = quad_as<T>(rc + X_G3), cN = quad_as<T>(rc + X_N0), cB = quad_as<T>(rc + X_AB);

@@ -433,8 +433,8 @@ __device__ __forceinline__ void curv_core(F2 D, float Ok, bool want_d, F2& S, F2
 }
 
 // (one block more or less per SM: 2 and 33 % slower on 25 M pairs' values and
-// gradients)
-template <int K> struct Core2Blocks { enum { value = K == 0 ? 3 : 2 }; };
+// gradients; with X two blocks, at 128 registers)
+template <int K, bool WX> struct Core2Blocks { enum { value = K == 0 && !WX ? 3 : 2 }; };
 
 // The single-precision sums and values with two pairs of a row in a thread:
 // the arithmetic is that of core_kernel on packed numbers (F2), and what it
@@ -442,10 +442,10 @@ template <int K> struct Core2Blocks { enum { value = K == 0 ? 3 : 2 }; };
 // for two.  Bound by issue like core_kernel (75 % of cycles there, at 241
 // instructions per pair of values and 527 with the gradient): 1.42e8 ragged
 // pairs of mu and its gradient 4.43 -> 3.59 ms, 25 M pairs over a shared set
-// 0.78 -> 0.63 ms.  A warp takes two 32-pair batches at a time while every lane's two
+// 0.78 -> 0.63 ms, 1e8 pairs of d_C, t and X 3.18 -> 2.74 ms.  A warp takes two 32-pair batches at a time while every lane's two
 // pairs lie in one row, else one (the second number is then a copy).
-template <int K, bool WT, int MODE>
-__global__ void __launch_bounds__(256, Core2Blocks<K>::value) core2_kernel(CoreArgs ca) {
+template <int K, bool WT, bool WX, int MODE>
+__global__ void __launch_bounds__(256, Core2Blocks<K, WX>::value) core2_kernel(CoreArgs ca) {
     constexpr bool DZ = MODE == CORE_DZ, BT = MODE == CORE_BETWEEN;
     constexpr int NV = K + 2;
     constexpr unsigned full = 0xffffffffu;
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(256, Core2Blocks<K>::value) core2_kernel(CoreA
         if (st == ST_OK) {
             int fail = 0;
             const bool z0 = z.x == 0.f, z1_ = z.y == 0.f;
-            typedef CorePair<F2, WT, false, (K > 0)> E;
+            typedef CorePair<F2, WT, WX, (K > 0)> E;
             E e;
             typename E::Tape tape;
             e.forward(mkf2(z0 ? 1.f : z.x, z1_ ? 1.f : z.y), rec, tape, &fail);
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(256, Core2Blocks<K>::value) core2_kernel(CoreA
             F2 v[N_OUT];
             v[O_DC] = DH * D;
             v[O_T] = WT ? zeroed(tH * e.It) : mkf2(0.f, 0.f);
-            v[O_X] = mkf2(0.f, 0.f);
+            v[O_X] = WX ? zeroed(DH * e.X) : mkf2(0.f, 0.f);
             v[O_DM] = DH * S;
             v[O_DL] = z1 * v[O_DM];
             v[O_MU] = want_mu ? mkf2(mu_of(v[O_DL].x), mu_of(v[O_DL].y)) : mkf2(0.f, 0.f);
@@ -577,6 +577,7 @@ __global__ void __launch_bounds__(256, Core2Blocks<K>::value) core2_kernel(CoreA
                 const F2 s = mkf2(lm.s, lm.s);
                 v[O_DC] = v[O_DC] * s;
                 v[O_DM] = v[O_DM] * s;
+                v[O_X] = v[O_X] * (s * s * s);
             }
             if (fail || (BT && !(in0 && in1))) {
                 const float nan = CUDART_NAN_F;
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(256, Core2Blocks<K>::value) core2_kernel(CoreA
             }
 #pragma unroll
             for (int i = 0; i < N_OUT; i++)
-                if (i != O_X && (i != O_T || WT) && (a.outmask & (1 << i))) {
+                if ((i != O_X || WX) && (i != O_T || WT) && (a.outmask & (1 << i))) {
                     float* p = reinterpret_cast<float*>(a.out[i]) + p0;
                     if (act0) p[o0] = v[i].x;
                     if (act1) p[o1] = v[i].y;

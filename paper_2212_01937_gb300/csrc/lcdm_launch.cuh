@@ -37,14 +37,14 @@ template <int PREC, int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core {
     }
 };
 
-template <int K, bool WT, int MODE = CORE_SUM> struct Core2 {
+template <int K, bool WT, bool WX, int MODE = CORE_SUM> struct Core2 {
     static cudaError_t launch(const CoreArgs& c, int grid, int block, cudaStream_t s) {
-        core2_kernel<K, WT, MODE><<<grid, block, 0, s>>>(c);
+        core2_kernel<K, WT, WX, MODE><<<grid, block, 0, s>>>(c);
         return cudaGetLastError();
     }
     static int occ(int block) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core2_kernel<K, WT, MODE>, block, 0) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, core2_kernel<K, WT, WX, MODE>, block, 0) != cudaSuccess)
             return 0;
         return n;
     }
@@ -58,8 +58,8 @@ template <int K, bool WT, int MODE = CORE_SUM> struct Core2 {
 // through the pair maps)
 struct PairsTable {
     PairsEntry e[4], jac[4], dz[2], bt[4];
-    PairsEntry packed[3][2];   // two pairs in a thread (single precision, no X, no gradient of t): sums, redshift
-                               // derivatives and general limits, by WT
+    PairsEntry packed[3][4];   // two pairs in a thread (single precision, no gradient of t): sums, redshift
+                               // derivatives and general limits, each like e
 };
 
 template <class E> PairsEntry entry() { PairsEntry e; e.launch = E::launch; e.occ = E::occ; return e; }
@@ -71,11 +71,15 @@ template <int PREC> PairsTable value_table() {
     t.e[2] = entry<Core<PREC, 0, true, false> >();
     t.e[3] = entry<Core<PREC, 0, true, true> >();
     if constexpr (PREC == 1) {
-        t.packed[0][0] = entry<Core2<0, false> >();
-        t.packed[0][1] = entry<Core2<0, true> >();
-        t.packed[1][0] = entry<Core2<0, false, CORE_DZ> >();
-        t.packed[2][0] = entry<Core2<0, false, CORE_BETWEEN> >();
-        t.packed[2][1] = entry<Core2<0, true, CORE_BETWEEN> >();
+        t.packed[0][0] = entry<Core2<0, false, false> >();
+        t.packed[0][1] = entry<Core2<0, false, true> >();
+        t.packed[0][2] = entry<Core2<0, true, false> >();
+        t.packed[0][3] = entry<Core2<0, true, true> >();
+        t.packed[1][0] = entry<Core2<0, false, false, CORE_DZ> >();
+        t.packed[2][0] = entry<Core2<0, false, false, CORE_BETWEEN> >();
+        t.packed[2][1] = entry<Core2<0, false, true, CORE_BETWEEN> >();
+        t.packed[2][2] = entry<Core2<0, true, false, CORE_BETWEEN> >();
+        t.packed[2][3] = entry<Core2<0, true, true, CORE_BETWEEN> >();
     }
     t.dz[0] = entry<Core<PREC, 0, false, false, CORE_DZ> >();
     t.bt[0] = entry<Core<PREC, 0, false, false, CORE_BETWEEN> >();
@@ -95,9 +99,9 @@ template <int PREC, int K> PairsTable tangent_table() {
     t.jac[2] = entry<Core<PREC, K, true, false, CORE_JAC> >();
     t.jac[3] = t.e[3];
     if constexpr (PREC == 1) {
-        t.packed[0][0] = entry<Core2<K, false> >();
-        if constexpr (K < 6) t.packed[1][0] = entry<Core2<K, false, CORE_DZ> >();
-        if constexpr (K == 3) t.packed[2][0] = entry<Core2<K, false, CORE_BETWEEN> >();
+        t.packed[0][0] = entry<Core2<K, false, false> >();
+        if constexpr (K < 6) t.packed[1][0] = entry<Core2<K, false, false, CORE_DZ> >();
+        if constexpr (K == 3) t.packed[2][0] = entry<Core2<K, false, false, CORE_BETWEEN> >();
     }
     if constexpr (K == 3) {
         t.bt[0] = entry<Core<PREC, K, false, false, CORE_BETWEEN> >();

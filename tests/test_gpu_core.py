@@ -96,6 +96,33 @@ def test_two_pairs_in_a_thread(lib, lane_map, ncol, radiation):
         assert np.all((np.abs(got_g - g) <= bound)[ok])
 
 
+@pytest.mark.parametrize("names", [("X",), ("t", "X", "mu")])
+@pytest.mark.parametrize("ncol,radiation", [(4, True), (5, True), (4, False)])
+def test_two_pairs_in_a_thread_absorption(lib, names, ncol, radiation):
+    """X beside a pair that needs another number of steps (z over five decades
+    in random order) and beside a NaN; general limits."""
+    P, z, offs, rng = _batch(LENS, 29, ncol, radiation)
+    z = np.where(z > 0, 10.0 ** rng.uniform(-3, 0.5, z.size), 0.0).astype(np.float32)
+    bad = z.copy()
+    bad[5] = np.nan
+    z64 = z.astype(np.float64)
+    ref = lib.distances(_t(P), _t(z64), _t(offs), outputs=names, precision="fp64")
+    for lane_map in ("contiguous", "interleaved"):
+        got = lib.distances(_t(P), _t(z), _t(offs), outputs=names, precision="fp32", lane_map=lane_map)
+        nan = lib.distances(_t(P), _t(bad), _t(offs), outputs=names, precision="fp32", lane_map=lane_map)
+        for o in names:
+            _close(got[o], ref[o], o)
+            assert np.isnan(nan[o][5].item())
+            nan[o][5] = got[o][5]
+            _close(nan[o], ref[o], o)
+    z1 = _t(rng.uniform(0.0, 0.5, len(P)))
+    z2 = (z + z1.cpu().numpy()[np.repeat(np.arange(len(P)), np.diff(offs))] + 0.05).astype(np.float32)
+    got = lib.distances_between(_t(P), z1, _t(z2), _t(offs), outputs=names, precision="fp32")
+    ref = lib.distances_between(_t(P), z1, _t(z2.astype(np.float64)), _t(offs), outputs=names, precision="fp64")
+    for o in names:
+        _close(got[o], ref[o], o)
+
+
 @pytest.mark.parametrize("n", [255, 256, 1001])
 def test_shared_layout_loglike(lib, n):
     """Below and from the packed kernel's line on; a shared redshift set."""
