@@ -13,10 +13,11 @@
  *                                                       (Sec. 2.1.1; fn22)
  * The quartic E^2 of eq. (2.2) is factorised per cosmology (eq. 3.2, FP64) and
  * each integral is reduced to Carlson's R_F, R_J, R_D, R_C (eqs. 2.6-2.9),
- * evaluated by duplication.  Derivatives with respect to the parameters are
- * carried through the duplication sequences as forward-mode tangents (the
- * differentiated form of eqs. 2.6-2.9; eq. 2.10 for R_C) from the root
- * derivatives of App. A (eqs. A.1-A.4).
+ * evaluated by duplication.  Derivatives with respect to the parameters run
+ * backwards through the stored duplication sequence and are contracted with
+ * the row's derivatives, which come from the root derivatives of App. A (eqs.
+ * A.1-A.4); where X is differentiated they are carried through the sequence
+ * as forward-mode tangents.
  *
  * Conventions shared by every entry point
  *   params   [B][ncol] float64, row-major: (H0 [km/s/Mpc], Omega_m0,

@@ -276,8 +276,9 @@ LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
 // derivative's values (26 instructions) and the differences of the roots; the
 // correction itself, a number known to 1e-7 of its size, is single.  A sweep
 // leaves 1e-7 of the error (or its cube), so two usually end it; comparisons
-// are made in single precision or on the bits.  (4096 rows: 0.070 ms with
-// double corrections, confirmations and hypot; see DESIGN for the rest.)
+// are made in single precision or on the bits.  (4096 rows, kernel time: 0.070
+// ms with double corrections, confirmations and hypot; 0.031 ms so, with the
+// closed-form starts, 418 FP64 and 4259 instructions a warp.)
 // Coefficients outside single precision's range (Or0 below about 1e-10, OL0 =
 // 0) take the sweeps in double throughout.
 //
