@@ -38,13 +38,15 @@ template <class T> LCDM_HD void curv_core(T D, T Ok, bool want_d, T& S, T& SD, T
     curv_map<T>(D, Ok, S, SD, Sk);
 }
 
-// mu = 5 log10(d_L) + 25.  Single precision: log10 from the exponent and a
-// series in s = f / (2 + f), f = mantissa - 1 in [-0.29, 0.41] (log(1 + f) =
-// 2 s (1 + s^2/3 + s^4/5 + ...), to 2e-9), 15 instructions; its error is below
-// that of mu's last place at mu ~ 40.  Zero, negative and non-finite distances
-// go to log10f.
+// mu = 5 log10(d_L) + 25.  Single precision: the exponent's part and the special
+// function unit's log2 of the mantissa in [sqrt(1/2), sqrt(2)), whose absolute
+// error of 2^-22 there is a tenth of the last place of mu ~ 40 (applied to d_L
+// itself it would be 2^-22 of a log2 of 14).  8 instructions; 15 with a series
+// in (m - 1) / (m + 1), 3.63 against 3.58 ms for 1.4e8 pairs of mu and its
+// gradient; rms error over z = 0.01 to 10 1.26e-6 mag against 1.28e-6, and
+// 1.41e-6 with log10f.  Zero, negative and non-finite distances go to log10f.
 LCDM_HD double mu_of(double dL) { return 5.0 * log10(dL) + 25.0; }
-LCDM_HD float mu_of(float dL) {
+__device__ __forceinline__ float mu_of(float dL) {
     uint32_t b;
     memcpy(&b, &dL, sizeof b);
     if (b - 0x00800000u >= 0x7f000000u) return 5.0f * log10f(dL) + 25.0f;
@@ -52,9 +54,9 @@ LCDM_HD float mu_of(float dL) {
     const uint32_t mb = b - ((uint32_t)e << 23);
     float m;
     memcpy(&m, &mb, sizeof m);
-    const float f = m - 1.0f, s = f * rcp_(2.0f + f), q = s * s;
-    const float l = s * (2.0f + q * (2.0f / 3 + q * (0.4f + q * (2.0f / 7 + q * (2.0f / 9)))));
-    return fmaf((float)e, 1.50514997831990598f, fmaf(l, 2.17147240951625903f, 25.0f));
+    float l;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(m));
+    return fmaf((float)e, 1.50514997831990598f, fmaf(l, 1.50514997831990598f, 25.0f));
 }
 
 // acc += c.  Double-float: one error-free sum; its error joins the low word,
