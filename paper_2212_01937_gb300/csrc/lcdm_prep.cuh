@@ -400,36 +400,49 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
     const bool iso = sep > 0.1f;
     // (a group's lanes agree; the others take the next block for nothing)
     if (!__all_sync(full, iso || !active)) {
-        // Single precision can merge a complex pair of nearly double roots (near
-        // the no-Big-Bang boundary) into two points on or near the real axis, and
-        // for a real polynomial the iteration keeps real approximations real.
-        // Two such approximations within 1e-3 of each other get imaginary
-        // offsets of opposite sign (far above double precision, far below the
-        // spacing), which lets the double-precision sweeps move them back into
-        // the complex plane if the roots are complex; real ones return to the axis.
-        float cr[4], ci[4];
+        // Single precision (the closed form's discriminant, or the sweeps) knows
+        // two nearly equal roots only to about 1e-3 of their size: it cannot tell
+        // two reals from a conjugate pair, and may return them equal, both real,
+        // or exactly conjugate.  The sweeps keep real approximations real and
+        // mirror images mirror images (the polynomial is real), so from such
+        // starts roots of the other kind are out of reach.  Two approximations
+        // that are each other's nearest, with a mean near the real axis, restart
+        // at 45 degrees to it through that mean: there the iteration is Halley's
+        // for the square root of the pair's discriminant, which reaches either
+        // kind (a distance ten times too large costs two sweeps).
+        float cr[4], ci[4], dist[4];
+        int near_to[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             cr[k] = G == 1 ? (float)zre[k / G] : __shfl_sync(full, (float)zre[k / G], k % G, G);
             ci[k] = G == 1 ? (float)zim[k / G] : __shfl_sync(full, (float)zim[k / G], k % G, G);
         }
 #pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int j = r * G + s;
-            if (j >= n) continue;
-            float xj = 0.f, yj = 0.f;
+        for (int j = 0; j < 4; j++) {
+            dist[j] = 3e38f;
+            near_to[j] = -1;
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (k == j) { xj = cr[k]; yj = ci[k]; }
-            const float m = fabsf(xj) + fabsf(yj);
-            if (!(fabsf(yj) < 1e-6f * m)) continue;
-            float off = 0.f;
-#pragma unroll
-            for (int k = 3; k >= 0; k--) {
-                if (k == j || k >= n || !(fabsf(ci[k]) < 1e-6f * m)) continue;
-                if (fabsf(cr[k] - xj) < 1e-3f * m) off = j < k ? 1e-6f : -1e-6f;
+            for (int k = 0; k < 4; k++) {
+                if (k == j || k >= n) continue;
+                const float xr = cr[j] - cr[k], xi = ci[j] - ci[k], q = sqrtf(xr * xr + xi * xi);
+                if (q < dist[j]) { dist[j] = q; near_to[j] = k; }
             }
-            if (off != 0.f) zim[r] = (double)(yj + off * m);
+        }
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (j != r * G + s || j >= n) continue;
+                const float m = fabsf(cr[j]) + fabsf(ci[j]);
+                if (!(dist[j] < 0.1f * m && fabsf(ci[j]) < 0.1f * m)) continue;
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    if (k != near_to[j] || near_to[k] != j) continue;
+                    const float h = 0.70710678f * fmaxf(0.5f * dist[j], 1e-3f * m), sg = j < k ? h : -h;
+                    zre[r] = (double)(0.5f * (cr[j] + cr[k]) + sg);
+                    zim[r] = (double)sg;
+                }
+            }
         }
     }
     {
