@@ -101,6 +101,20 @@ LCDM_HD void polish_root(const double* a, int n, cd& x) {
     }
 }
 
+// (pr + i pi) / (er + i ei).  Divided by the larger part first: with a root of
+// 1e6 (Om / Or) the polynomial's value is 1e24, and its products with the
+// derivative leave single precision from a root of 3e5 on.
+LCDM_HD void fquot(float pr, float pi, float er, float ei, float& wr, float& wi) {
+    const float i = 1.0f / fmaxf(fabsf(er), fabsf(ei));
+    er *= i;
+    ei *= i;
+    pr *= i;
+    pi *= i;
+    const float ie = 1.0f / (er * er + ei * ei);
+    wr = (pr * er + pi * ei) * ie;
+    wi = (pi * er - pr * ei) * ie;
+}
+
 // One Newton step from one compensated evaluation, the quotient in single
 // precision: enough for a root known to about 1e-15 / separation (the step
 // leaves 1e-7 of that error), without polish_root's confirming evaluations.
@@ -108,8 +122,8 @@ LCDM_HD void polish_once(const double* a, int n, cd& x) {
     cd p, dp;
     horner_comp(a, n, x, p, dp);
     const float pr = (float)p.re, pi = (float)p.im, dr = (float)dp.re, di = (float)dp.im;
-    const float i = 1.0f / (dr * dr + di * di);
-    const float wr = (pr * dr + pi * di) * i, wi = (pi * dr - pr * di) * i;
+    float wr, wi;
+    fquot(pr, pi, dr, di, wr, wi);
     if (!(fabsf(wr) + fabsf(wi) < 1e30f)) return;
     x = cmk(x.re - (double)wr, x.im - (double)wi);
 }
@@ -204,7 +218,7 @@ LCDM_HD void start_points(const float* c, int n, float* zr, float* zi) {
 // of a cubic's) by Cardano's formulas on the deflated cubic.  Returns false
 // where that is not good: the fixed point has not settled, the other roots are
 // not small beside A, or one of them is so small that the shift a/3 costs its
-// digits.
+// digits, or the discriminant, of the roots' sixth power, may leave the range.
 LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
     float g3 = al[3], g2 = al[2], g1 = al[1], g0 = al[0];
     int k = 0;
@@ -253,7 +267,7 @@ LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
     const float q0 = fabsf(r0), q1 = fabsf(r1) + im, q2 = fabsf(r2) + im;
     const float lo = fminf(q0, fminf(q1, q2)), hi = fmaxf(q0, fmaxf(q1, q2));
     // (false for anything not finite, too)
-    return good && lo > 1e-2f * (fabsf(sh) + hi) && (n == 3 ? hi < 1e18f : hi < 0.05f * fabsf(A));
+    return good && lo > 1e-2f * (fabsf(sh) + hi) && lo > 1e-5f && hi < 1e5f && (n == 3 || hi < 0.05f * fabsf(A));
 }
 
 // Roots of the monic polynomial c (degree n <= 4) by the simultaneous
@@ -279,8 +293,9 @@ LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
 // are made in single precision or on the bits.  (4096 rows, kernel time: 0.070
 // ms with double corrections, confirmations and hypot; 0.031 ms so, with the
 // closed-form starts, 418 FP64 and 4259 instructions a warp.)
-// Coefficients outside single precision's range (Or0 below about 1e-10, OL0 =
-// 0) take the sweeps in double throughout.
+// Coefficients of the monic polynomial beyond 1e6 (Or0 below 3e-7 for Om0 = 0.3:
+// |A|^4 would near the end of single precision) or OL0 = 0 take the sweeps in
+// double throughout, from the circles.
 //
 // A root closer than a tenth of its modulus to another (near-multiple roots,
 // as near the no-Big-Bang boundary) is polished on the original coefficients
@@ -346,10 +361,9 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
                     float npr = pr * xr0 - pi * xi0 + cf[k], npi = pr * xi0 + pi * xr0;
                     dr = ndr; di = ndi; pr = npr; pi = npi;
                 }
-                float dn = dr * dr + di * di;
-                if ((pr == 0.f && pi == 0.f) || !(dn > 0.f)) continue;
-                float idn = 1.0f / dn;
-                float rr = (pr * dr + pi * di) * idn, ri = (pi * dr - pr * di) * idn;   // p / p'
+                if ((pr == 0.f && pi == 0.f) || !(fabsf(dr) + fabsf(di) > 1e-30f)) continue;
+                float rr, ri;
+                fquot(pr, pi, dr, di, rr, ri);   // p / p'
                 float sr = 0.f, si = 0.f;
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
@@ -490,8 +504,8 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
                         si -= xi * ix;
                     }
                     // w = p / (p' - p S)
-                    const float er = dr - (pr * sr - pi * si), ei = di - (pr * si + pi * sr), ie = 1.0f / (er * er + ei * ei);
-                    const float wr = (pr * er + pi * ei) * ie, wi = (pi * er - pr * ei) * ie;
+                    float wr, wi;
+                    fquot(pr, pi, dr - (pr * sr - pi * si), di - (pr * si + pi * sr), wr, wi);
                     if (pr == 0.f && pi == 0.f) continue;
                     zre[r] = x - (double)wr;
                     zim[r] = y - (double)wi;

@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from test_gpu_parity import COLS, TOL32, TOL64, _t
-from test_prep_host import _double_root, _exact
+from test_prep_host import _double_root, _exact, _low_radiation
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +57,12 @@ def test_nearly_double_roots(lib, ncol, times, prec):
     well = np.array([max(float(abs(x)) for x in re + cx if abs(x) < 20) < 0.8 for re, cx in map(_exact, P)])
     assert well.sum() >= 10
     _check(lib, P, well, np.array([0.01, 0.3, 1.0, 5.0, 300.0]), prec, times)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("times", [1, 140])
+@pytest.mark.parametrize("ncol", [4, 5, 7])
+def test_low_radiation(lib, ncol, times, prec):
+    rng = np.random.default_rng(12)
+    P = np.array([_low_radiation(rng, ncol) for _ in range(120)])
+    _check(lib, P, np.full(len(P), True), np.array([0.01, 0.3, 1.0, 5.0, 300.0]), prec, times)

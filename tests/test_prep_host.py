@@ -117,6 +117,36 @@ def test_nearly_double_roots(prep, ncol, quartic, near):
     _check(prep, np.array(P), near)
 
 
+def _low_radiation(rng, ncol):
+    """Om / Or from 1e4 to 1e7 (across the root sweeps' two ranges of
+    coefficients) with OL from 1e-12 to 1."""
+    Om = rng.uniform(0.05, 0.6)
+    row = [70.0, Om, 10.0 ** rng.uniform(-12, 0), Om / 10.0 ** rng.uniform(4, 7)]
+    return row + [10.0 ** rng.uniform(-6, 0), 10.0 ** rng.uniform(-6, -1), 10.0 ** rng.uniform(-6, -1)][:ncol - 4]
+
+
+@pytest.mark.parametrize("near", [0.1, 0.01])
+@pytest.mark.parametrize("ncol", [4, 5, 7])
+def test_low_radiation(prep, ncol, near):
+    rng = np.random.default_rng(12)
+    _check(prep, np.array([_low_radiation(rng, ncol) for _ in range(100)]), near)
+
+
+@pytest.mark.parametrize("row", [[70.0, 0.3, 1e-4, 7e-7],
+                                 [70.0, 3.59100770371796, -5.521955913688765e-06, 1.0813750580855664e-05],
+                                 [70.0, 1.1555128340131777, 4.6205600454127664e-08, 3.1582537844621348e-06,
+                                  -0.9848739552881378],
+                                 [70.0, 0.2462031973093668, -1.976969922057992e-25, 1e-05, 8.522853391548514e-10,
+                                  4.967495035992166e-09, 0.0],
+                                 [70.0, 0.8123634327126253, -4.790791447752325e-25, 1e-05, 1.09264510906137e-08,
+                                  2.4156781053752366e-08, 0.0]])
+def test_single_precision_range(prep, row):
+    """A root of 3e5 to 1e6 whose closed-form start is not good (the sweeps'
+    products), and three reals of 1e-8 (the discriminant)."""
+    for near in (0.1, 0.01):
+        _check(prep, np.array([row]), near)
+
+
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 def test_values_inside_the_recollapse_boundary(prep, prec):
     """Two real roots 2e-7 inside the boundary, at x = 0.372."""
