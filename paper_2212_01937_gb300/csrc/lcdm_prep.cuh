@@ -135,8 +135,8 @@ LCDM_HD void polish_once(const double* a, int n, cd& x) {
 LCDM_HD int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
 LCDM_HD float scaled(double v, int e) {
     const long long b = __double_as_longlong(v);
-    const int k = (int)((b >> 52) & 0x7ff) - e;   // biased exponent of the quotient
-    if (k < 1023 - 100) return 0.0f;
+    const int x = (int)((b >> 52) & 0x7ff), k = x - e;   // biased exponents of v and of the quotient
+    if (x == 0 || k < 1023 - 100) return 0.0f;   // (zero has no leading one: a root at exactly zero is real)
     if (k > 1023 + 100) return 1e30f;
     return (float)__longlong_as_double((b & ~(0x7ffLL << 52)) | ((long long)k << 52));
 }
@@ -560,6 +560,9 @@ __device__ void group_roots(const double* c, const double* alpha, int n, bool ac
             const int ez = exponent_of(zj);
             const float mx = scaled(zj.re, ez), my = scaled(zj.im, ez), mz = sqrtf(mx * mx + my * my);
             if (fabsf(my) <= 1e-12f * mz) zj.im = 0.0;
+            // a single root at zero (OL0 = 0 beside Ox0) is one exactly: the sweeps
+            // end somewhere below 1e-100, off the axis
+            if (c[0] == 0.0 && c[1] != 0.0 && fabs(zj.re) + fabs(zj.im) < 1e-100) zj = cmk(0.0, 0.0);
             float d = 1.0f;   // distance to the nearest other root over the modulus
 #pragma unroll
             for (int k = 0; k < 4; k++) {

@@ -6,18 +6,9 @@ import pytest
 
 import oracle
 from test_gpu_parity import COLS, TOL32, TOL64, _t
-from test_prep_host import _double_root, _exact, _low_radiation
+from test_prep_host import _double_root, _exact, _low_radiation, _status, _zero_root
 
 pytestmark = pytest.mark.gpu
-
-
-def _status(P):
-    out = []
-    for row in P:
-        re, cx = _exact(row)
-        n = 3 + (row[3] > 0)
-        out.append(1 if any(x >= 1 for x in re) else 0 if len(re) + 2 * len(cx) == n and len(cx) < 2 else 5)
-    return np.array(out)
 
 
 def _check(lib, P, well, z, prec, times):
@@ -29,7 +20,7 @@ def _check(lib, P, well, z, prec, times):
     zz = zz if prec == "fp64" else zz.astype(np.float32)
     got = lib.distances(_t(P_), _t(zz), _t(off), outputs=("d_C", "t", "X"), precision=prec)
     st = got["status"].cpu().numpy().reshape(times, rows)
-    want = _status(P)
+    want = np.array([_status(row, *_exact(row)) for row in P])
     assert np.all(st == want), (P[(st != want).any(axis=0)].tolist(), want[(st != want).any(axis=0)])
     good = np.nonzero((want == 0) & well)[0]
     ref = oracle.quad_distances(P[good], np.tile(zz[:n].astype(np.float64), good.size),
@@ -65,4 +56,12 @@ def test_nearly_double_roots(lib, ncol, times, prec):
 def test_low_radiation(lib, ncol, times, prec):
     rng = np.random.default_rng(12)
     P = np.array([_low_radiation(rng, ncol) for _ in range(120)])
+    _check(lib, P, np.full(len(P), True), np.array([0.01, 0.3, 1.0, 5.0, 300.0]), prec, times)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("times", [1, 140])
+def test_zero_root(lib, times, prec):
+    rng = np.random.default_rng(13)
+    P = np.array([_zero_root(rng, i % 2) for i in range(120)])
     _check(lib, P, np.full(len(P), True), np.array([0.01, 0.3, 1.0, 5.0, 300.0]), prec, times)

@@ -54,6 +54,13 @@ def _exact(P):
     return [x.real for x in r if abs(x.imag) <= tiny * abs(x)], [x for x in r if x.imag > tiny * abs(x)]
 
 
+def _status(row, re, cx):
+    """1: a real root at z >= 0; 5: two pairs; 3: the cubic's special root at x = 0."""
+    if any(x >= 1 for x in re):
+        return 1
+    return 5 if len(cx) == 2 else 3 if row[3] == 0 and cx and re[0] == 0 else 0
+
+
 def _check(prep, P, near):
     """Status, kind and the roots to 1e-13 (an isolated root is good to a few
     ulp, 1e-15; one of a pair is polished to the same, and its condition number,
@@ -63,10 +70,7 @@ def _check(prep, P, near):
     for b, row in enumerate(P):
         re, cx = _exact(row)
         quartic = row[3] > 0
-        if any(x >= 1 for x in re):
-            assert st[b] == 1, (row.tolist(), st[b])
-        else:
-            assert st[b] == (0 if len(re) + 2 * len(cx) == 3 + quartic and len(cx) < 2 else 5), (row.tolist(), st[b])
+        assert st[b] == _status(row, re, cx), (row.tolist(), st[b])
         if len(cx) == 2:
             continue
         assert kind[b] == (0 if quartic else 2) + (0 if cx else 1), (row.tolist(), kind[b])
@@ -145,6 +149,19 @@ def test_single_precision_range(prep, row):
     products), and three reals of 1e-8 (the discriminant)."""
     for near in (0.1, 0.01):
         _check(prep, np.array([row]), near)
+
+
+def _zero_root(rng, quartic):
+    """Omega_L0 = 0 beside Omega_x0: a single root at exactly x = 0."""
+    return [70.0, rng.uniform(0.05, 0.6), 0.0, 10.0 ** rng.uniform(-6, -3) if quartic else 0.0,
+            10.0 ** rng.uniform(-6, 0), 10.0 ** rng.uniform(-3, -1), 10.0 ** rng.uniform(-6, 0)]
+
+
+@pytest.mark.parametrize("near", [0.1, 0.01])
+@pytest.mark.parametrize("quartic", [True, False])
+def test_zero_root(prep, quartic, near):
+    rng = np.random.default_rng(13)
+    _check(prep, np.array([_zero_root(rng, quartic) for _ in range(60)]), near)
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
