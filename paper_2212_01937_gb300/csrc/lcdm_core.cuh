@@ -559,6 +559,14 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         T p0 = cst<T>(0.0), dX = cst<T>(0.0), piX = cst<T>(0.0), sD = cst<T>(0.0), sDD = cst<T>(0.0), x0 = x, rp0 = cst<T>(0.0);
         if (WX) {
             p0 = aX * aX - lX * z2;
+            if (big) {
+                // the z^3 of both terms cancel (lambda y_B^2 q_B = S0 q_A q_P q_P*): the
+                // polynomial w_A |w_P|^2 - lx w_B z^2 without it
+                const Quad<T> kB = quad_as<T>(rc + X_AB);
+                const T qA = k0.v[0], p1 = qA + kB.v[2], p2 = qA * kB.v[2] + kB.v[3] - kX.v[1];
+                const T pb = p2 * z2 + (p1 * zh + h) * h + cst<T>(2.0) * (nA * (nB * h)) * (Pn * h) + wB * h * h;
+                p0 = sel_ge0(z - cst<T>(CoreTol<T>::big), pb, p0);
+            }
             piX = kX.v[2] * (z2 * z2);
             dX = -(kX.v[0] * z2) * piX;
         }
@@ -710,23 +718,24 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T DJ = tm * (dA * ser1 + r23 * dser) + cst<T>(6.0) * sDD;
             const T RD = tm * (one + v2 * (w2 * w2)) * r23 + cst<T>(3.0) * sD;
             if (m == 0) rp0 = sqt(p0);
-            // the results belong to arguments scaled by h^2 (h = 1 but for very large z)
+            // the arguments, and with them s1, x0, p0 and the integrals, are scaled by
+            // powers of h (1 but for very large z): what falls off like 1/z is formed
+            // from them as they are, with one h in front (unscaled, z^4 and x1 leave
+            // single precision from z = 1e10 on)
             const T ih = big ? unscale(h) : one;
-            const T s1u = s1 * ih, sp0 = rp0 * ih, zz = z * z, x1 = x0 * (ih * ih);
-            const T hRF = RF * h, hRD = RD * (h * h * h), hDJ = DJ * (h * h * h) * (h * h);
             const Quad<T> c0 = quad_as<T>(rc + X_C0), c3 = quad_as<T>(rc + X_G3), cN = quad_as<T>(rc + X_N0), cB = quad_as<T>(rc + X_AB);
             const T irA = rA, syd = c3.v[3] * (nA * Pn * rB + one), isy = rcp_(syd);
             const T T0 = c0.v[0] * irA * (k0.v[1] * Pn * rcp_(nB + one) + (cB.v[2] + z * cB.v[3]) * rcp_(Pn + one)
                                            - k0.v[0] * rcp_(nA + one));
-            const T t1 = zz * (c0.v[2] * hRD + c0.v[3] * zz * hDJ);
-            const T iyd = isy * isy;
+            const T t1 = c0.v[1] * RF + z2 * (c0.v[2] * RD + c0.v[3] * z2 * DJ);
+            const T wy = z * isy, wy2 = wy * wy;
             // y / yd = S0 p0 / (yB^2 n_B^2 yd), the part of yd beside lam z^2
-            const T t2 = c3.v[0] * zz * phi_core(cB.v[1] * zz * iyd, sp0 * c3.v[3] * rB * isy) * iyd * isy;
-            const T as = nA * s1u;
-            const T num = x1 * (cN.v[1] * z + cN.v[0]) + cN.v[2] * zz;
-            const T t3 = c3.v[1] * nB * num * rcp_(sp0 * as * (as + cB.v[0] * sp0));
-            const T t4 = c3.v[2] * nB * irA * rcp_(s1u);
-            X = z * (T0 + c0.v[1] * hRF + t1 + t2 + t3 + t4);
+            const T t2 = c3.v[0] * wy2 * phi_core(cB.v[1] * wy2, (rp0 * rB) * (c3.v[3] * (isy * ih))) * isy;
+            const T as = nA * s1;
+            const T num = x0 * (cN.v[1] * z + cN.v[0]) + cN.v[2] * z2;
+            const T t3 = c3.v[1] * num * (nB * rcp_(rp0 * as * (as + cB.v[0] * rp0)));
+            const T t4 = c3.v[2] * nB * irA * rcp_(s1);
+            X = z * (T0 + t2 + h * (t1 + t3 + t4));
         }
     }
 

@@ -50,3 +50,15 @@ def test_double_precision(core, name, z):
     assert np.all(np.abs(out[:2] / val[:2] - 1) <= 1e-12)
     err = np.abs(grad[:, cols] - jac[:, cols]).max(axis=1) / np.abs(jac[:, cols]).max(axis=1)
     assert np.all(err <= 1e-9)
+
+
+@pytest.mark.parametrize("name", NAMES)
+@pytest.mark.parametrize("fp64,z", [(0, 6.4e4), (0, 6.6e4), (0, 1e9), (0, 1e12), (0, 1e15), (0, 1e18), (1, 0.9e9), (1, 1.1e9),
+                                    (1, 1e20), (1, 2e30), (1, 1e100)])
+def test_absorption_distance(core, name, fp64, z):
+    """X grows like z: finite, and as accurate as at ordinary redshifts, FP64
+    1e-12, FP32 1e-4."""
+    z = z if fp64 else float(np.float32(z))
+    out, _, _ = _run(core, name, z, fp64)
+    val, _ = _exact(ROWS[name], z, False)
+    assert abs(out[2] / val[2] - 1) <= (1e-12 if fp64 else 1e-4)
