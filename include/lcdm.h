@@ -66,7 +66,11 @@
  *                than the cases below, or rho_A == 0)
  *              4 duplication did not converge / principal value not available
  *              5 root configuration not supported (two complex pairs)
- *            and every output of such a cosmology is NaN.
+ *            and every output of such a cosmology is NaN, except with 4: there
+ *            the outputs of the pairs that did not converge are NaN (a
+ *            non-finite redshift, or one beyond a bounce), they add nothing to
+ *            grad and loglike, the other pairs are as in any row, and all
+ *            redshift derivatives (grad_z) of the row are NaN.
  *   triple root  Omega_L0 = Omega_k0 (+ Omega_s0) = Omega_x0 = 0 to within
  *            the rounding of the closure (Einstein-de Sitter, flat matter +
  *            radiation: E^2 = x^3 (Or x + Om), x = 1 + z): the roots are set

@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
             }
             rend = e < INT32_MAX ? (int)e : INT32_MAX;
             rec = reinterpret_cast<const T*>(ca.rec) + (int64_t)row * NCORE;
-            st = a.status[row];
+            st = row_status(a.status, row);
             if (BT) lm.load(ca.rowf, ca.z1, ca.scale, row);
         }
         const int64_t zi = a.layout == LAYOUT_SHARED ? o - (int64_t)zoff * a.nrow : o;
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(256, Core2Blocks<K, WX>::value) core2_kernel(C
             }
             rend = e < INT32_MAX ? (int)e : INT32_MAX;
             rec = reinterpret_cast<const float*>(ca.rec) + (int64_t)row * NCORE;
-            st = a.status[row];
+            st = row_status(a.status, row);
             if (BT) lm.load(ca.rowf, ca.z1, ca.scale, row);
         }
         const int off1 = off + s_it;

@@ -45,6 +45,15 @@ enum CosmoStatus {
     ST_OK = 0, ST_NO_BIG_BANG = 1, ST_INVALID = 2, ST_DEGENERATE = 3, ST_NOCONV = 4, ST_UNSUPPORTED = 5
 };
 
+// A row's status as the pair kernels read it.  A pair whose duplication does not
+// converge marks its row while other warps are still to enter it: that code is
+// no reason to skip a row, or which of its pairs are evaluated would depend on
+// the warps' timing.
+__device__ __forceinline__ int row_status(const int32_t* status, int64_t row) {
+    const int st = status[row];
+    return st == ST_NOCONV ? (int)ST_OK : st;
+}
+
 // ------------------------------------------------------------ observables ---
 LCDM_HD float expm1_(float x) { return expm1f(x); }
 LCDM_HD double expm1_(double x) { return expm1(x); }
@@ -396,7 +405,7 @@ __global__ void __launch_bounds__(256, 1) pairs_kernel(PairArgs a) {
         }
         const double* rd = a.recD + row * NREC;
         const float2* rf = a.recF + row * NREC;
-        const int st = a.status[row];
+        const int st = row_status(a.status, row);
         const TO z = load_io<TO>(a.z, zi);
         // the pair's cotangents are loaded before the evaluation, so that their
         // latency hides behind it
