@@ -22,15 +22,21 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // largest batch whose root preparation uses four lanes per cosmology
 #define LCDM_PREP_GROUP_MAX_B 16384
 
-// Row records: those of the core (NCORE floats or doubles per row), or those
-// of the X-tangent kernel (FP64 and its (hi, lo) copy), in the same memory (a
-// plan that needs both prepares one after the other).
-#define LCDM_RECORD_BYTES(B)                                                                              \
-    (((size_t)(B) * NCORE * sizeof(double) + 255) / 256 * 256 >                                           \
-             ((size_t)(B) * NREC * sizeof(double) + 255) / 256 * 256 + ((size_t)(B) * NREC * sizeof(float2) + 255) / 256 * 256 \
-         ? ((size_t)(B) * NCORE * sizeof(double) + 255) / 256 * 256                                       \
-         : ((size_t)(B) * NREC * sizeof(double) + 255) / 256 * 256 + ((size_t)(B) * NREC * sizeof(float2) + 255) / 256 * 256)
-size_t ws_bytes_for(int64_t B) { return LCDM_RECORD_BYTES(B); }
+// Row records: those of the core (NCORE floats or doubles per row), and beside
+// them those of the X-tangent kernel (FP64, in single precision also their (hi,
+// lo) copy): a call that differentiates X and has other work on the core uses
+// both from one preparation.
+size_t core_bytes(int64_t B, int prec) { return align256((size_t)B * NCORE * (prec == 0 ? sizeof(double) : sizeof(float))); }
+size_t record_bytes(int64_t B, int prec) {
+    return core_bytes(B, prec) + align256((size_t)B * NREC * sizeof(double)) +
+           (prec == 1 ? align256((size_t)B * NREC * sizeof(float2)) : 0);
+}
+// (one size for either precision)
+size_t ws_bytes_for(int64_t B) {
+    const size_t d = record_bytes(B, 0), f = record_bytes(B, 1);
+    return d > f ? d : f;
+}
+int prec_of(const lcdm_opts* o) { return o->precision == LCDM_FP64 ? 0 : 1; }
 
 bool opts_ok(const lcdm_opts* o) {
     return o && (o->ncol == 4 || o->ncol == 5 || o->ncol == 7) &&
@@ -52,21 +58,29 @@ size_t det_bytes() {
 }
 
 struct Carved {
-    double* recD;
-    float2* recF;
-    char* core;                  // the core's records (the same memory)
+    char* core;                  // the core's records
+    double* recD;                // those of the X-tangent kernel
+    float2* recF;                // (null in double precision)
     double* part = nullptr;      // deterministic mode: [warps][2][DET_NV]
     int64_t* wrow = nullptr;     // [warps][2]
 };
 
-lcdm_status carve(void* ws, size_t ws_bytes, int64_t B, Carved& c, int det = 0) {
-    if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < ws_bytes_for(B) + (det ? det_bytes() : 0))
-        return LCDM_ERR_WORKSPACE;
-    c.recD = (double*)ws;
-    c.core = (char*)ws;
-    c.recF = (float2*)((char*)ws + align256((size_t)B * NREC * sizeof(double)));
+Carved carve_records(char* p, int64_t B, int prec) {
+    Carved c;
+    c.core = p;
+    c.recD = p ? (double*)(p + core_bytes(B, prec)) : nullptr;
+    c.recF = p && prec == 1 ? (float2*)((char*)c.recD + align256((size_t)B * NREC * sizeof(double))) : nullptr;
+    return c;
+}
+
+// need: the bytes the call asks of its workspace, 0: those of every record
+lcdm_status carve(void* ws, size_t ws_bytes, int64_t B, int prec, Carved& c, int det = 0, size_t need = 0) {
+    const size_t rec = ws_bytes_for(B);
+    if (need == 0) need = rec + (det ? det_bytes() : 0);
+    if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < need) return LCDM_ERR_WORKSPACE;
+    c = carve_records((char*)ws, B, prec);
     if (det) {
-        c.part = (double*)((char*)ws + ws_bytes_for(B));
+        c.part = (double*)((char*)ws + rec);
         c.wrow = (int64_t*)((char*)c.part + align256(det_warps() * 2 * DET_NV * sizeof(double)));
     }
     return LCDM_OK;
@@ -394,7 +408,8 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
 int core_ns(int prec) { return prec == 0 ? (int)CoreTol<double>::ns : (int)CoreTol<float>::ns; }
 // What a call's records hold.
 struct PrepNeed {
-    bool legacy;     // the X-tangent kernel's records, else the core's
+    bool legacy;     // the X-tangent kernel's records
+    bool core;       // the core's (beside the former: without tangents)
     int prec;        // precision of the core's records
     bool tangents, time, absorb;
     int ns;          // series coefficients of the core's records
@@ -420,8 +435,8 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
     a.absorb = need.absorb;
     a.recD = need.legacy ? cv.recD : nullptr;
     a.recF = need.legacy ? cv.recF : nullptr;
-    a.coreF = !need.legacy && need.prec == 1 ? (float*)cv.core : nullptr;
-    a.coreD = !need.legacy && need.prec == 0 ? (double*)cv.core : nullptr;
+    a.coreF = need.core && need.prec == 1 ? (float*)cv.core : nullptr;
+    a.coreD = need.core && need.prec == 0 ? (double*)cv.core : nullptr;
     a.status = status;
     a.grad = grad;
     a.loglike = loglike;
@@ -437,33 +452,23 @@ lcdm_status run_prep(const double* params, int64_t B, const lcdm_opts* opts, con
     return cudaGetLastError() == cudaSuccess ? LCDM_OK : LCDM_ERR_CUDA;
 }
 
-// Preparation and launches of a plan.  A plan whose tangent launch is the
-// X-tangent kernel's and that also has value-only outputs prepares the core's
-// records for those first, then its own.
+// The plan's preparation: one launch, also where the tangent launch is the
+// X-tangent kernel's and others (value-only outputs, redshift derivatives) run on
+// the core.  (One after the other in the same memory: 737 against 636 us for 65536 rows
+// of 8 pairs of X with its gradient, and t.)
+PrepNeed plan_need(const Plan& P) {
+    const bool legacy = P.legacy != 0;
+    return PrepNeed{legacy, !legacy || P.split_mask || separate_dz(P), P.prec, P.K > 0, P.time != 0, P.absorb != 0, core_ns(P.prec)};
+}
+
+// Preparation and launches of a plan.
 lcdm_status run_plan(const Plan& P, const double* params, int64_t B, const lcdm_opts* opts, const Carved& cv,
                      int32_t* status, double* grad, double* loglike, int block, int bps, int lane_map, cudaStream_t s,
                      const ShiftArgs* shift = nullptr) {
-    lcdm_status st;
-    const bool dz = separate_dz(P);
-    if (P.split_mask || dz || !P.legacy) {
-        const PrepNeed need = {false, P.prec, P.K > 0 && !P.legacy, P.time != 0, P.absorb != 0, core_ns(P.prec)};
-        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s, shift);
-        if (st != LCDM_OK) return st;
-    }
-    if (P.split_mask) {
-        st = launch_values(P, lane_map, s);
-        if (st != LCDM_OK) return st;
-    }
-    if (dz) {
-        st = launch_dz(P, lane_map, s);
-        if (st != LCDM_OK) return st;
-    }
-    if (P.legacy) {
-        const PrepNeed need = {true, P.prec, true, true, true, 0};
-        st = run_prep(params, B, opts, cv, need, status, grad, loglike, s, shift);
-        if (st != LCDM_OK) return st;
-    }
-    return launch_main(P, block, bps, lane_map, s);
+    lcdm_status st = run_prep(params, B, opts, cv, plan_need(P), status, grad, loglike, s, shift);
+    if (st == LCDM_OK && P.split_mask) st = launch_values(P, lane_map, s);
+    if (st == LCDM_OK && separate_dz(P)) st = launch_dz(P, lane_map, s);
+    return st == LCDM_OK ? launch_main(P, block, bps, lane_map, s) : st;
 }
 
 __global__ void extract_roots(const double* __restrict__ recD, int64_t B, int ncol, double* roots, double* droots,
@@ -496,11 +501,11 @@ __global__ void extract_roots(const double* __restrict__ recD, int64_t B, int nc
 lcdm_status pairs_common(const double* params, int64_t B, const int64_t* offsets, const void* z, int64_t n,
                          void* const* out, void* const* jac, const void* const* cot, const void* mobs, double M,
                          double sigma, double* grad, double* loglike, int32_t* status, const lcdm_opts* opts,
-                         void* ws, size_t ws_bytes, cudaStream_t stream) {
+                         void* ws, size_t ws_bytes, cudaStream_t stream, size_t need = 0) {
     lcdm_status st = check_pairs_args(params, B, offsets, z, n, status, opts);
     if (st != LCDM_OK) return st;
     Carved cv;
-    st = carve(ws, ws_bytes, B, cv, opts->deterministic);
+    st = carve(ws, ws_bytes, B, prec_of(opts), cv, opts->deterministic, need);
     if (st != LCDM_OK) return st;
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, jac, cot, mobs, M, sigma, grad, loglike, status, opts, cv, P);
@@ -515,7 +520,8 @@ lcdm_status pairs_common(const double* params, int64_t B, const int64_t* offsets
 // cudaGetSymbolAddress (the host-side name is only a stand-in and must never
 // be handed to a kernel).
 // ----------------------------------------------------------------------------
-#define LCDM_STATIC_WS_BYTES LCDM_RECORD_BYTES(LCDM_STATIC_MAX_COSMOLOGIES)
+// (values only: the core's records)
+#define LCDM_STATIC_WS_BYTES ((size_t)LCDM_STATIC_MAX_COSMOLOGIES * NCORE * sizeof(double))
 static __device__ __align__(256) unsigned char g_static_ws[LCDM_STATIC_WS_BYTES];
 
 static void* g_static_ptr[LCDM_MAX_DEVICES];
@@ -583,10 +589,7 @@ HostCarve host_carve(char* base, int64_t B, int64_t n, int ncol, size_t es) {
     HostCarve c;
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align256(bytes); return p; };
-    char* rec = take(ws_bytes_for(B));
-    c.rec.recD = (double*)rec;
-    c.rec.core = take((size_t)B * NCORE * es);
-    c.rec.recF = rec ? (float2*)(rec + align256((size_t)B * NREC * sizeof(double))) : nullptr;
+    c.rec = carve_records(take(ws_bytes_for(B)), B, es == 8 ? 0 : 1);
     c.params = (double*)take((size_t)B * ncol * sizeof(double));
     c.offsets = (int64_t*)take((size_t)(B + 1) * sizeof(int64_t));
     c.status = (int32_t*)take((size_t)B * sizeof(int32_t));
@@ -618,10 +621,7 @@ BetweenCarve between_carve(char* base, int64_t B, int64_t npairs, int ncol, size
     BetweenCarve c;
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align256(bytes); return p; };
-    char* rec = take(ws_bytes_for(B));
-    c.rec.recD = (double*)rec;
-    c.rec.core = rec;
-    c.rec.recF = rec ? (float2*)(rec + align256((size_t)B * NREC * sizeof(double))) : nullptr;
+    c.rec = carve_records(take(ws_bytes_for(B)), B, es == 8 ? 0 : 1);
     c.jac = (double*)take((size_t)B * 4 * ncol * sizeof(double));
     c.scale = (double*)take((size_t)B * sizeof(double));
     c.rowf = (float4*)take((size_t)B * sizeof(float4));
@@ -739,7 +739,7 @@ lcdm_status lcdm_loglike_dz_workspace_size(int64_t B, int64_t n, const lcdm_opts
     if (!opts_ok(opts) || B <= 0 || n < 0 || !bytes) return LCDM_ERR_INVALID;
     const int64_t npairs = opts->layout == LCDM_LAYOUT_CSR ? n : B * n;
     const size_t es = opts->precision == LCDM_FP64 ? 8 : 4;
-    *bytes = align256(ws_bytes_for(B)) + 2 * align256((size_t)npairs * es);
+    *bytes = ws_bytes_for(B) + 2 * align256((size_t)npairs * es);
     return LCDM_OK;
 }
 
@@ -756,7 +756,7 @@ lcdm_status lcdm_gauss_loglike_dz(const double* params, int64_t B, const int64_t
     lcdm_loglike_dz_workspace_size(B, n, opts, &need);
     if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < need) return LCDM_ERR_WORKSPACE;
     Carved cv;
-    carve(ws, ws_bytes, B, cv);
+    carve(ws, ws_bytes, B, prec_of(opts), cv);
     void* out[LCDM_NOUT] = {nullptr, nullptr, nullptr, nullptr, nullptr, mu_out};
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, nullptr, nullptr, m_obs, M, sigma, grad, loglike, cosmo_status,
@@ -782,7 +782,7 @@ lcdm_status lcdm_distances_vjp_dz(const double* params, int64_t B, const int64_t
     lcdm_loglike_dz_workspace_size(B, n, opts, &need);
     if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < need) return LCDM_ERR_WORKSPACE;
     Carved cv;
-    carve(ws, ws_bytes, B, cv);
+    carve(ws, ws_bytes, B, prec_of(opts), cv);
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, nullptr, grad ? cot : nullptr, nullptr, 0, 1, grad, nullptr,
                    cosmo_status, opts, cv, P);
@@ -809,7 +809,7 @@ lcdm_status lcdm_limits(const double* params, int64_t B, const double* z1, doubl
     lcdm_opts o4 = *opts;
     o4.ncol = 4;
     const ShiftArgs shift = between_shift(params, B, z1, ncol, w, grad != nullptr);
-    const PrepNeed need = {false, 0, grad != nullptr, true, false, CORE_NS_ONCE};
+    const PrepNeed need = {false, true, 0, grad != nullptr, true, false, CORE_NS_ONCE};
     lcdm_status st = run_prep(params, B, &o4, w.rec, need, cosmo_status, nullptr, nullptr, stream, &shift);
     if (st != LCDM_OK) return st;
     LimitArgs la;
@@ -841,7 +841,7 @@ lcdm_status lcdm_distances_static(const double* params, int64_t B, const int64_t
     lcdm_opts o = *opts;
     o.deterministic = 0;   // forward values only: there is no reduction
     return pairs_common(params, B, offsets, z, n, out, nullptr, nullptr, nullptr, 0, 1, nullptr, nullptr,
-                        cosmo_status, &o, ws, LCDM_STATIC_WS_BYTES, stream);
+                        cosmo_status, &o, ws, LCDM_STATIC_WS_BYTES, stream, core_bytes(B, prec_of(&o)));
 }
 
 
@@ -882,23 +882,14 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
     chk(cudaEventRecord(ev[1], hs->up));
     chk(cudaStreamWaitEvent(stream, ev[1], 0));
     if (!ok) return LCDM_ERR_CUDA;
-    // one preparation of all rows for every chunk (both kinds of records when a
-    // plan of X's tangents also has value-only outputs)
+    // one preparation of all rows for every chunk
     {
         Plan P;
         void* const* outs = out;
         make_plan(d.params, B, d.offsets, d.z, n, outs, nullptr, cot, nullptr, 0, 1, d.grad, nullptr, d.status, opts,
                   d.rec, P);
-        if (P.legacy) {
-            const PrepNeed need = {true, P.prec, true, true, true, 0};
-            st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
-            if (st != LCDM_OK) return st;
-        }
-        if (P.split_mask || !P.legacy) {
-            const PrepNeed need = {false, P.prec, !P.legacy, P.time != 0, P.absorb != 0, core_ns(P.prec)};
-            st = run_prep(d.params, B, opts, d.rec, need, d.status, d.grad, nullptr, stream);
-            if (st != LCDM_OK) return st;
-        }
+        st = run_prep(d.params, B, opts, d.rec, plan_need(P), d.status, d.grad, nullptr, stream);
+        if (st != LCDM_OK) return st;
     }
     // chunk c covers rows [rb[c], rb[c+1]); its share of the pairs ramps up and
     // down, weights min(c + 1, nchunks - c, 3) (1 2 3 ... 3 2 1): the first
@@ -944,7 +935,7 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
         if (!ok) return LCDM_ERR_CUDA;
         Carved rc;
         rc.recD = d.rec.recD + r0 * NREC;
-        rc.recF = d.rec.recF + r0 * NREC;
+        rc.recF = d.rec.recF ? d.rec.recF + r0 * NREC : nullptr;
         rc.core = d.rec.core + (size_t)r0 * NCORE * es;
         Plan P;
         make_plan(d.params + r0 * ncol, r1 - r0, d.offsets + r0, d.z, o1 - o0, outd, nullptr, cotd, nullptr, 0, 1,
@@ -980,9 +971,9 @@ lcdm_status lcdm_roots(const double* params, int64_t B, const lcdm_opts* opts, d
                        int32_t* kind, int32_t* cosmo_status, void* ws, size_t ws_bytes, cudaStream_t stream) {
     if (!opts_ok(opts) || !params || !cosmo_status || B <= 0) return LCDM_ERR_INVALID;
     Carved cv;
-    lcdm_status st = carve(ws, ws_bytes, B, cv);
+    lcdm_status st = carve(ws, ws_bytes, B, prec_of(opts), cv);
     if (st != LCDM_OK) return st;
-    const PrepNeed need = {true, 0, true, true, false, 0};
+    const PrepNeed need = {true, false, 0, true, true, false, 0};
     st = run_prep(params, B, opts, cv, need, cosmo_status, nullptr, nullptr, stream);
     if (st != LCDM_OK) return st;
     extract_roots<<<(unsigned)((B + 127) / 128), 128, 0, stream>>>(cv.recD, B, opts->ncol, roots, droots, kind);
@@ -1034,7 +1025,7 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
     if (st != LCDM_OK) return st;
     if (!grad) cot = nullptr;   // forward-only shape
     Carved cv;
-    st = carve(ws, ws_bytes, B, cv, opts->deterministic);
+    st = carve(ws, ws_bytes, B, prec_of(opts), cv, opts->deterministic);
     if (st != LCDM_OK) return st;
     Plan P;
     st = make_plan(params, B, offsets, z, n, out, nullptr, cot, nullptr, 0, 1, grad, nullptr, cosmo_status, opts, cv,
@@ -1053,19 +1044,12 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
             for (int bps = 1; bps <= occ; bps = (bps * 2 > occ && bps < occ) ? occ : bps * 2) {
                 float tot = 0;
                 for (int rep = 0; rep < 3; rep++) {
-                    // (the preparation is not timed, but where it comes between the launches)
-                    const bool both = P.legacy && P.split_mask;
-                    const PrepNeed need = {P.legacy != 0, P.prec, P.K > 0, P.time != 0, P.absorb != 0, core_ns(P.prec)};
-                    if (!both && run_prep(params, B, opts, cv, need, cosmo_status, grad, nullptr, stream) != LCDM_OK)
+                    // (the preparation is not timed)
+                    if (run_prep(params, B, opts, cv, plan_need(P), cosmo_status, grad, nullptr, stream) != LCDM_OK)
                         return LCDM_ERR_CUDA;
                     cudaEventRecord(e0, stream);
-                    if (both) {
-                        if (run_plan(P, params, B, opts, cv, cosmo_status, grad, nullptr, block, bps, map, stream) != LCDM_OK)
-                            return LCDM_ERR_CUDA;
-                    } else {
-                        if (P.split_mask && launch_values(P, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
-                        if (launch_main(P, block, bps, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
-                    }
+                    if (P.split_mask && launch_values(P, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
+                    if (launch_main(P, block, bps, map, stream) != LCDM_OK) return LCDM_ERR_CUDA;
                     cudaEventRecord(e1, stream);
                     cudaEventSynchronize(e1);
                     float ms = 0;

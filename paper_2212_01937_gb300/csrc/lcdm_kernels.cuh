@@ -245,7 +245,7 @@ template <int PREC, int K, bool WT>
 LCDM_HD void eval_pair(typename std::conditional<PREC == 0, double, float>::type zin, const double* rd, const float2* rf,
                        PairOut<typename std::conditional<PREC == 0, double, float>::type, K>& o, int* fail) {
     typedef typename std::conditional<PREC == 0, double, float>::type TO;
-    const int kind = (int)rf[RF_KIND].x;
+    const int kind = (int)recv<TO>(rd, rf, RF_KIND);
     typename PairEval<TO, K, WT>::S a, b, c;
     PairEval<TO, K, WT>::run(zin, rd, rf, kind, a, b, c, fail);
     const TO Ichi = a.v, It = WT ? b.v : (TO)0, IX = c.v;

@@ -928,7 +928,8 @@ struct PrepArgs {
     int absorb;             // the absorption distance's constants are needed
     double* recD;           // [B][NREC] record of the X-tangent kernel, and its (hi, lo) copy (optional)
     float2* recF;
-    float* coreF;           // [B][NCORE] record of the core, single or double precision (optional)
+    float* coreF;           // [B][NCORE] record of the core, single or double precision (optional; beside
+                            // recD without tangents)
     double* coreD;
     int32_t* status;
     double* grad;           // [B][ncol], [B]: initialised to 0 (NaN for a bad status), optional
@@ -951,7 +952,7 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
     RowRoots r;
     cd dr[4][RF_KT];
     bool labelled;
-    const int st = prep_roots<G>(prow, ncol, inb, a.tangents ? (a.recD ? 2 : 1) : 0, a.coreF ? 0.01f : 0.1f, r, dr,
+    const int st = prep_roots<G>(prow, ncol, inb, a.tangents ? (a.recD ? 2 : 1) : 0, a.coreF && !a.recD ? 0.01f : 0.1f, r, dr,
                                  labelled);
     if (!inb) return;
     if (a.recD) {
@@ -962,14 +963,16 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
         #pragma unroll 1
         for (int i = j; i < NREC; i += G) {
             rd[i] = rec[i];
+            if (!a.recF) continue;
             float h = (float)rec[i];
             rf[i] = make_float2(h, (float)(rec[i] - (double)h));
         }
     }
     if (st == ST_OK && (a.coreF || a.coreD)) {
         r.finish();
-        if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, a.tangents, a.ns, a.coreF + b * NCORE);
-        else write_core<G, double>(r, dr, j, a.time, a.absorb, a.tangents, a.ns, a.coreD + b * NCORE);
+        const bool tangents = a.tangents && !a.recD;
+        if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, tangents, a.ns, a.coreF + b * NCORE);
+        else write_core<G, double>(r, dr, j, a.time, a.absorb, tangents, a.ns, a.coreD + b * NCORE);
     }
     if (j != 0) return;
     a.status[b] = st;
