@@ -116,8 +116,8 @@ const PairsTable& table(int prec, int K) {
     return t[prec][K == 0 ? 0 : (K == 3 ? 1 : (K == 4 ? 2 : 3))];
 }
 
-// tuned launch shapes: key (device, precision, K, WT, WX, layout, log2 npairs)
-typedef std::tuple<int, int, int, int, int, int, int> TuneKey;
+// tuned launch shapes: key (device, precision, K, kernel (entry_index), layout, log2 npairs)
+typedef std::tuple<int, int, int, int, int, int> TuneKey;
 struct Tuned { int block, bps, lane_map; };
 std::map<TuneKey, Tuned> g_tuned;
 std::mutex g_tune_mu;
@@ -139,7 +139,6 @@ struct Plan {
     int time, absorb;       // the core's records need the constants of t, of the absorption distance
     int prec, K, wt, wx;
     int64_t npairs;
-    TuneKey key;
     // outputs wanted as values only while other outputs need tangents: the
     // time coordinate and the absorption distance each run their own R_J
     // track, whose tangents would be computed for nothing; such outputs are
@@ -215,7 +214,6 @@ lcdm_status make_plan(const double* params, int64_t B, const int64_t* offsets, c
     P.legacy = P.K > 0 && wx;
     P.time = (P.split_mask >> LCDM_T) & 1 || (!P.legacy && wt);
     P.absorb = (P.split_mask >> LCDM_X) & 1 || (P.K == 0 && wx);
-    P.key = TuneKey(current_device(), P.prec, P.K, wt, wx, opts->layout, log2_bucket(P.npairs));
     return LCDM_OK;
 }
 
@@ -240,6 +238,9 @@ int entry_index(const Plan& P) {
     if (P.rowf) return 10 + (P.wt ? 2 : 0) + (P.wx ? 1 : 0);
     if (P.grad_z && !P.wx && !P.legacy) return 8 + (P.wt ? 1 : 0);
     return (P.wt ? 2 : 0) + (P.wx ? 1 : 0) + (jac ? 4 : 0);
+}
+TuneKey tune_key(const Plan& P) {
+    return TuneKey(current_device(), P.prec, P.K, entry_index(P), P.args.layout, log2_bucket(P.npairs));
 }
 CoreArgs core_args(const Plan& P) {
     CoreArgs c;
@@ -304,9 +305,6 @@ lcdm_status launch_values(const Plan& P, int lane_map, cudaStream_t s) {
     V.wt = (P.split_mask >> LCDM_T) & 1;
     V.wx = (P.split_mask >> LCDM_X) & 1;
     V.split_mask = 0;
-    std::get<2>(V.key) = 0;
-    std::get<3>(V.key) = V.wt;
-    std::get<4>(V.key) = V.wx;
     return launch_one(V, 0, 0, lane_map, s);
 }
 // The redshift derivatives alone: a value launch of chi without outputs.
@@ -316,7 +314,6 @@ lcdm_status launch_dz(const Plan& P, int lane_map, cudaStream_t s) {
     D.args.outmask = 0;
     D.args.grad = nullptr;
     D.K = D.legacy = D.wt = D.wx = D.split_mask = 0;
-    std::get<2>(D.key) = std::get<3>(D.key) = std::get<4>(D.key) = 0;
     return launch_one(D, 0, 0, lane_map, s);
 }
 // The redshift derivatives come with the plan's main launch, unless that is
@@ -365,7 +362,7 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
     const PairsEntry& t = plan_entry(P);
     if (block == 0 || bps == 0 || lane_map == LCDM_MAP_TUNED) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tuned.find(P.key);
+        auto it = g_tuned.find(tune_key(P));
         if (it != g_tuned.end()) {
             if (block == 0) block = it->second.block;
             if (bps == 0) bps = it->second.bps;
@@ -1065,7 +1062,7 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
     cudaEventDestroy(e1);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tuned[P.key] = Tuned{bb, bbps, bmap};
+        g_tuned[tune_key(P)] = Tuned{bb, bbps, bmap};
     }
     if (best_block) *best_block = bb;
     if (best_bps) *best_bps = bbps;
