@@ -602,7 +602,7 @@ HostCarve host_carve(char* base, int64_t B, int64_t n, int ncol, size_t es) {
 // shifted cosmologies, shifted parameters (closure form, four columns), their
 // Jacobian, the scale s = 1+z1,
 // the gradient w.r.t. the shifted parameters, z' and three scaled cotangents
-// (d_C, X, d_M).
+// (d_C, X, d_M; these four only where X is differentiated, see RowMap).
 struct BetweenCarve {
     Carved rec;
     double* jac;
@@ -734,9 +734,7 @@ lcdm_status lcdm_distances_between(const double* params, int64_t B, const double
 
 lcdm_status lcdm_loglike_dz_workspace_size(int64_t B, int64_t n, const lcdm_opts* opts, size_t* bytes) {
     if (!opts_ok(opts) || B <= 0 || n < 0 || !bytes) return LCDM_ERR_INVALID;
-    const int64_t npairs = opts->layout == LCDM_LAYOUT_CSR ? n : B * n;
-    const size_t es = opts->precision == LCDM_FP64 ? 8 : 4;
-    *bytes = ws_bytes_for(B) + 2 * align256((size_t)npairs * es);
+    *bytes = ws_bytes_for(B);   // (the redshift derivatives come with the pair kernel)
     return LCDM_OK;
 }
 
@@ -747,7 +745,7 @@ lcdm_status lcdm_gauss_loglike_dz(const double* params, int64_t B, const int64_t
     if (!m_obs || !loglike || !grad_z || !(sigma > 0) || !std::isfinite(M)) return LCDM_ERR_INVALID;
     lcdm_status st = check_pairs_args(params, B, offsets, z, n, cosmo_status, opts);
     if (st != LCDM_OK) return st;
-    if (opts->ncol > 5) return LCDM_ERR_UNSUPPORTED;   // E(z) of the redshift kernel: 4 or 5 columns
+    if (opts->ncol > 5) return LCDM_ERR_UNSUPPORTED;   // no kernel with redshift derivatives for seven columns
     if (opts->deterministic) return LCDM_ERR_UNSUPPORTED;
     size_t need = 0;
     lcdm_loglike_dz_workspace_size(B, n, opts, &need);
@@ -773,7 +771,7 @@ lcdm_status lcdm_distances_vjp_dz(const double* params, int64_t B, const int64_t
     if (!cot || !grad_z) return LCDM_ERR_INVALID;
     lcdm_status st = check_pairs_args(params, B, offsets, z, n, cosmo_status, opts);
     if (st != LCDM_OK) return st;
-    if (opts->ncol > 5) return LCDM_ERR_UNSUPPORTED;   // E(z) of the redshift kernel: 4 or 5 columns
+    if (opts->ncol > 5) return LCDM_ERR_UNSUPPORTED;   // no kernel with redshift derivatives for seven columns
     if (opts->deterministic && grad) return LCDM_ERR_UNSUPPORTED;
     size_t need = 0;
     lcdm_loglike_dz_workspace_size(B, n, opts, &need);
