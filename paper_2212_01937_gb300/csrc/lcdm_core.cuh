@@ -24,8 +24,12 @@
 // Consequences for the duplication (Carlson's algorithm, the paper's ref. [10]):
 //  * the sequence is carried without the division by four (x <- x + lambda):
 //    differences are then constant and the truncated series are polynomials
-//    in w = z^2 / A with constants of the row as coefficients, so a degree more
-//    costs one multiply-add (and a larger deviation may be left: fewer steps);
+//    in w = z^2 dev / A with constants of the row as coefficients, so a degree more
+//    costs one multiply-add (and a larger deviation may be left: fewer steps).
+//    dev is the row's largest deviation over z^2: with it in w the coefficients
+//    are at most of order one (a power of dev up to the eleventh leaves single
+//    precision where E^2(0) is small, a sum of densities of 1e-5 or a lower limit
+//    at which the universe loiters);
 //  * the stopping rule is one multiplication: z^2 max|deviation| <= tol A;
 //  * y y* = x1 S^2 after the first step, so a step takes two square roots
 //    (one more per third-kind track) and no division by a difference;
@@ -190,7 +194,7 @@ LCDM_HD double rcp_(double x) {
 template <class T> struct CoreTol;
 template <> struct CoreTol<float> {
     // largest deviation left to the series of degree ns + 1 (its truncation:
-    // about dup^(ns + 2) / 100); relative deviation s of R_C's; largest z taken
+    // about dup^(ns + 2) / 100); relative deviation s of R_C's; largest s1 taken
     // without scaling
     static constexpr float dup = 0.25f, once = 0.15f, rc = 0.1f, big = 65536.0f, e_series = 0.1f;
     enum { maxit = 24, ns = 8 };
@@ -346,7 +350,7 @@ LCDM_HD F2 one_plus(F2 q, F2 ql, F2 z) { return mkf2(one_plus(q.x, ql.x, z.x), o
 LCDM_HD float fms_(float n, float w) { return fmaf(-n, n, w); }
 LCDM_HD double fms_(double n, double w) { return fma(-n, n, w); }
 LCDM_HD F2 fms_(F2 n, F2 w) { return mkf2(fms_(n.x, w.x), fms_(n.y, w.y)); }
-// power of two near 1/z for very large z
+// power of two near 1/z for very large z (or s1, which is of z's size where E^2(0) is 1)
 LCDM_HD float scale_of(float z) { return z < 1e38f ? pow2i<float>(-even_exponent(z)) : 0.0f; }
 LCDM_HD double scale_of(double z) {
     int e;
@@ -354,7 +358,7 @@ LCDM_HD double scale_of(double z) {
     return z < 1e300 ? pow2i<double>(-e) : 0.0;
 }
 
-// the scaling of a pair, 1 unless z is very large
+// the scaling of a pair, 1 unless its s1 is very large
 LCDM_HD float scaling(float z) { return z > CoreTol<float>::big ? scale_of(z) : 1.0f; }
 LCDM_HD double scaling(double z) { return z > CoreTol<double>::big ? scale_of(z) : 1.0; }
 LCDM_HD F2 scaling(F2 z) { return mkf2(scaling(z.x), scaling(z.y)); }
@@ -524,12 +528,12 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             aX = nA * Pn + nB;
             lX = kX.v[1] * wB;
         }
-        // powers of z^6 and d^2 would leave the range for very large z:
-        // everything is homogeneous and is scaled by a power of two
-        big = any_gt(z, cst<T>(CoreTol<T>::big));
+        // powers of large arguments (very large z, or a small E^2(0)) would leave
+        // the range: everything is homogeneous and is scaled by a power of two
+        big = any_gt(s1, cst<T>(CoreTol<T>::big));
         h = one;
         if (big) {
-            h = scaling(z);
+            h = scaling(s1);
             s1 = s1 * h; uR = uR * h; uI = uI * h;
             if (WT) a5 = a5 * h;
             if (WX) aX = aX * h;
@@ -548,15 +552,16 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         }
         T x = s1 * s1;
         T3 = x + T30;
-        T sJ = cst<T>(0.0), delta = cst<T>(0.0), opE = cst<T>(0.0);
+        T sJ = cst<T>(0.0), kz = cst<T>(0.0), k9 = kz, opE = cst<T>(0.0);
         p = cst<T>(0.0);
         if (WT) {
             opE = one + kT.v[1];
             d5 = kT.v[3] * z2 * (opE * opE) * (wA * (izh * izh));
             p = a5 * a5 - d5;
-            delta = cst<T>(-9.0) * kT.v[2] * kT.v[2] * kT.v[3] * (z2 * z2 * z2);
+            kz = kT.v[2] * (z2 * zh);
+            k9 = cst<T>(-9.0) * kT.v[3];
         }
-        T p0 = cst<T>(0.0), dX = cst<T>(0.0), piX = cst<T>(0.0), sD = cst<T>(0.0), sDD = cst<T>(0.0), x0 = x, rp0 = cst<T>(0.0);
+        T p0 = cst<T>(0.0), hX = cst<T>(0.0), piX = cst<T>(0.0), sD = cst<T>(0.0), sDD = cst<T>(0.0), x0 = x, rp0 = cst<T>(0.0);
         if (WX) {
             p0 = aX * aX - lX * z2;
             if (big) {
@@ -568,7 +573,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 p0 = sel_ge0(z - cst<T>(CoreTol<T>::big), pb, p0);
             }
             piX = kX.v[2] * (z2 * z2);
-            dX = -(kX.v[0] * z2) * piX;
+            hX = -(kX.v[0] * z2);
         }
         T pX = p0;
         const float it = (float)(1.0 / (INF ? CoreTol<T>::once : CoreTol<T>::dup));
@@ -595,7 +600,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 if (m == 0) q0 = sq;
                 const T gg = p + (sq * S + P);
                 const T id = rcp_((sq + S1) * gg);
-                const T e = (delta * id) * id;
+                const T v = kz * id, e = k9 * (v * v);
                 sJ = sJ + tm * rc1_core(e, false).v * id;
                 if (REV) tape.q[m] = sq;
                 p = p + lam;
@@ -608,7 +613,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 if (m == 0) rp0 = sq;
                 const T gg = pX + (sq * S + P), qs = sq + S1;
                 const T id = rcp_(qs * gg);
-                const T e = (dX * id) * id, eh = (piX * id) * id;
+                const T eh = (piX * id) * id, e = hX * eh;
                 sDD = sDD + tm * (eh * rc1m1_core(e) * id
                                   - (gg + cst<T>(2.0) * S1 * (qs + S)) * (id * id) * gg * ix * cst<T>(0.5));
                 pX = pX + lam;
@@ -637,7 +642,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         {
             const T A = T3 * cst<T>(1.0 / 3);
             rF = rsq(A);
-            wF = z2 * (rF * rF);
+            wF = (INF ? z2 : z2 * Scalar<T>::of(rc[C_DF])) * (rF * rF);
             const T s = series<false, NS>(rc, C_B, wF).v;
             sF = one + s * (wF * wF);
             RF = tm * sF * rF;
@@ -647,7 +652,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         if (WT) {
             const T A = (T3 + p + p) * cst<T>(0.2);
             rJ = rsq(A);
-            wJ = z2 * (rJ * rJ);
+            wJ = (INF ? z2 : z2 * kT.v[0]) * (rJ * rJ);
             const T s = series<false, NS>(rc, C_A, wJ).v;
             sJs = one + s * (wJ * wJ);
             RJ = tm * sJs * (rJ * rJ * rJ) + cst<T>(6.0) * sJ;
@@ -692,7 +697,8 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             const T iA2 = cst<T>(5.0) * rcp_(T3 + x + x);
             const T A2 = (T3 + x + x) * cst<T>(0.2), A1 = (T3 + pX + pX) * cst<T>(0.2);
             const T r1 = rsq(A1), r2 = rsq(A2);
-            const T i1 = r1 * r1, w1 = z2 * i1, w2 = z2 * iA2, ww = cst<T>(-0.4) * w1 * w2;
+            const T sx = Scalar<T>::of(rc[X_DX]);
+            const T i1 = r1 * r1, w1 = (z2 * sx) * i1, u2 = z2 * iA2, w2 = u2 * sx, ww = cst<T>(-0.4) * w1 * u2;
             // series at p0 and at x1, and the divided difference of the brackets
             // (coefficients by degree: at p0, at x1, their divided difference)
             constexpr int N = CoreTol<T>::ns;
@@ -711,7 +717,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 v2 = horner(v2, w2, q[3 * j + 1]);
             }
             const T ser1 = one + v1 * (w1 * w1);
-            const T dser = cst<T>(-0.4) * (w1 + w2) * z2 * i1 * iA2 * v1 + w2 * iA2 * e;
+            const T dser = iA2 * (cst<T>(-0.4) * (w1 + w2) * w1 * v1 + w2 * (sx * e));
             const T q1 = A1 * r1, q2 = A2 * r2;
             const T r13 = r1 * i1, r23 = r2 * iA2;
             const T dA = cst<T>(-0.4) * (A1 + q1 * q2 + A2) * rcp_(q1 + q2) * r13 * r23;
@@ -816,8 +822,11 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
         // the duplication in reverse: cotangents of (s1, S, P), x and p
         T s_ = cst<T>(0.0), S_ = cst<T>(0.0), P_ = cst<T>(0.0), x_ = cst<T>(0.0);
         T ps_ = WT ? pf_ : cst<T>(0.0);
-        T delta = cst<T>(0.0), tk = tm;
-        if (WT) delta = cst<T>(-9.0) * kT.v[2] * kT.v[2] * kT.v[3] * (z2 * z2 * z2);
+        T kz = cst<T>(0.0), k9 = kz, tk = tm;
+        if (WT) {
+            kz = kT.v[2] * (z2 * zh);
+            k9 = cst<T>(-9.0) * kT.v[3];
+        }
         T n1 = one, n1s = one;   // the next step's sqrt(x) and S
 #pragma unroll 1
         for (int i = m - 1; i >= 0; i--) {
@@ -841,10 +850,10 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
             P_ = lam_;
             if (WT) {
                 const T sq = tape.q[i], gg = sq * (sq + Sm) + Pm, qs = sq + a;
-                const T id = rcp_(qs * gg), e = (delta * id) * id;
+                const T id = rcp_(qs * gg), v = kz * id, vv = v * v, e = k9 * vv;
                 const RcE<T> r = rc1_core(e, true);
                 const T c = cJ * tk * id;                 // cotangent of rc
-                del_ = del_ + c * r.d * id * id;
+                del_ = del_ + c * r.d * vv;
                 // 1/d: rc d(1/d) + rc' 2 delta id d(1/d), d(1/d) = -id^2 dd
                 const T dd = -c * id * (r.v + two * e * r.d);
                 const T g_ = dd * qs, q_ = dd * gg + g_ * Sm;
@@ -854,18 +863,19 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 ps_ = ps_ + g_ + q_ * half * rcp_(sq);
             }
         }
-        // initial values: x = s1^2, 3 A = x + y + y*, p = a5^2 - d5, delta = -9 k2^2 k3 z^6
+        // initial values: x = s1^2, 3 A = x + y + y*, p = a5^2 - d5; e = -9 k3 v^2, v = k2 z^3 / d
         s_ = s_ + two * s1 * (x_ + T_);
         T nB_, Pn_ = cst<T>(0.0), h5_ = cst<T>(0.0);
         if (WT) {
             p_ = p_ + ps_;
             a_ = a_ + two * a5 * p_;
             d_ = d_ - p_;
-            const T z6 = z2 * z2 * z2, k2 = kT.v[2], k3 = kT.v[3];
-            k2_ = k2_ - cst<T>(18.0) * k2 * k3 * z6 * del_;
+            const R k2 = rc[C_K2];
+            const T ik2 = Scalar<T>::of(fabs(k2) > R(1e-30) ? rcp_(k2) : R(0)), k3 = kT.v[3];
+            k2_ = k2_ - cst<T>(18.0) * k3 * del_ * ik2;
             const T opE = one + eps, wA = nA * nA;
             const T f = z2 * (izh * izh) * opE;
-            k3_ = -cst<T>(9.0) * k2 * k2 * z6 * del_ + d_ * f * opE * wA;
+            k3_ = d_ * f * opE * wA - cst<T>(9.0) * del_;
             eps_ = eps_ + d_ * k3 * two * f * wA;
             wA_ = d_ * k3 * f * opE;
             h5_ = a_ * izh;

@@ -4,6 +4,17 @@
 
 namespace lcdm {
 
+// largest deviation of the three, and of the five, arguments from their mean, over z^2
+LCDM_HD float dev3(double e2, double e3) {
+    const float a = sqrtf((float)fabs(e2)), b = cbrtf(4.0f * (float)fabs(e3));
+    return a > b ? a : b;
+}
+LCDM_HD float dev5(float d3, double m) {
+    const float am = (float)fabs(m);
+    const float a = 0.6f * am, b = d3 + 0.4f * am;
+    return a > b ? a : b;
+}
+
 // Roots of E^2(x), x = 1 + z, as classified by the preparation: the big root A
 // (quartic only), B, and the pair (conjugate: P = (pr, +-pi); two reals: pr, pi),
 // with derivatives along the K density directions.
@@ -14,9 +25,14 @@ struct RowRoots {
     // set by finish(): q_j = -1/(rho_j - 1) (0 for the cubic's absent root; the
     // pair: real and imaginary part, or the two), eps = -1/rho_A, 1/S0
     double qA, qB, q1, q2, eps, S0, iS0;
+    // the invariants e2 = -I / (3 S0^2), e3 = -J / (27 S0^3), the largest deviation
+    // of the three arguments over z^2; with `time` also k (k2 = k / 3), m and the
+    // five's.  (Every lane of a group needs them.)
+    double e2, e3, k, m;
+    float d3, d5;
 
     // (for a valid row: every real root below 1, S0 > 0)
-    LCDM_HD void finish() {
+    LCDM_HD void finish(bool time = true) {
         qA = quartic ? rcp_(1.0 - A) : 0.0;
         eps = quartic ? -1.0 / A : 0.0;
         qB = rcp_(1.0 - B);
@@ -27,6 +43,18 @@ struct RowRoots {
         q2 = (cpair ? -b : a) * i;
         S0 = ncol == 4 ? 1.0 : Om + OL + Or + Ok + Os + Ox;
         iS0 = ncol == 4 ? 1.0 : rcp_(S0);
+        const double C = Ok + Os, iS2 = iS0 * iS0;
+        const double I = 12.0 * Or * OL - 3.0 * Om * Ox + C * C;
+        const double J = 2.0 * C * C * C - 9.0 * Om * C * Ox + 27.0 * Or * Ox * Ox + 27.0 * Om * Om * OL - 72.0 * Or * C * OL;
+        e2 = I * (-1.0 / 3) * iS2;
+        e3 = J * (-1.0 / 27) * (iS2 * iS0);
+        d3 = dev3(e2, e3);
+        if (!time) return;
+        // E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
+        const double g0 = OL, g1 = Ox - eps * g0, g2 = C - eps * g1, g3 = Om - eps * g2;
+        k = (-g3 + eps * (g2 - eps * (g1 - eps * g0))) * iS0;
+        m = (g2 + eps * (3.0 * eps * g0 - 2.0 * g1)) * (iS0 * (1.0 / 3));
+        d5 = dev5(d3, m);
     }
 };
 
@@ -89,15 +117,10 @@ template <class S> LCDM_HD void rj_coefs(const S& m, const S& e2, const S& e3, i
         a[n - 2] = v * B(3.0 / (2 * n + 3));
     }
 }
-// largest deviation of the three, and of the five, arguments from their mean, over z^2
-LCDM_HD float dev3(double e2, double e3) {
-    const float a = sqrtf((float)fabs(e2)), b = cbrtf(4.0f * (float)fabs(e3));
-    return a > b ? a : b;
-}
-LCDM_HD float dev5(float d3, double m) {
-    const float am = (float)fabs(m);
-    const float a = 0.6f * am, b = d3 + 0.4f * am;
-    return a > b ? a : b;
+// 1 / dev, the scale of the series' variable (1 where a record serves one
+// evaluation; 0 without deviations)
+template <class T> LCDM_HD T dev_scale(float dev, int ns) {
+    return ns <= CORE_NS_ONCE ? (T)1 : dev > 0.0f ? (T)1 / (T)dev : (T)0;
 }
 
 template <class T> LCDM_HD void put(T* rec, int i, double v) { rec[i] = (T)v; }
@@ -116,34 +139,27 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
     put(rec, C_KIND, r.cpair ? 1.0 : 0.0);
     put(rec, C_RS, r.ncol == 4 ? 0.0 : -0.5 * iS0);
     put(rec, C_FREE0, 0.0); put(rec, C_FREE1, 0.0);
-    // invariants
-    const double I = 12.0 * r.Or * r.OL - 3.0 * r.Om * r.Ox + Oks * Oks;
-    const double J = 2.0 * Oks * Oks * Oks - 9.0 * r.Om * Oks * r.Ox + 27.0 * r.Or * r.Ox * r.Ox
-                     + 27.0 * r.Om * r.Om * r.OL - 72.0 * r.Or * Oks * r.OL;
-    const double e2 = I * (-1.0 / 3) * (iS0 * iS0), e3 = J * (-1.0 / 27) * (iS0 * iS0 * iS0);
-    const T f2 = (T)e2, f3 = (T)e3;
+    const T f2 = (T)r.e2, f3 = (T)r.e3;
     T b[CORE_NS];
-    rf_coefs<T>(f2, f3, ns, b);
+    // (normalised by the largest deviation: see lcdm_core.cuh)
+    const T u3 = dev_scale<T>(r.d3, ns);
+    rf_coefs<T>((f2 * u3) * u3, ((f3 * u3) * u3) * u3, ns, b);
 #pragma unroll
     for (int j = 0; j < CORE_NS; j++)
         if (j < ns) rec[C_B + j] = b[j];
-    const float d3 = dev3(e2, e3);
-    rec[C_DF] = (T)d3;
-    if (ns <= CORE_NS_ONCE) { put(rec, C_E2, e2); put(rec, C_E3, e3); }
+    rec[C_DF] = (T)r.d3;
+    if (ns <= CORE_NS_ONCE) { put(rec, C_E2, r.e2); put(rec, C_E3, r.e3); }
     if (time) {
-        // t: E^2(x) / (1 - x / rho_A) = g0 + g1 x + g2 x^2 + g3 x^3
-        const double g0 = r.OL, g1 = r.Ox - eps * g0, g2 = Oks - eps * g1, g3 = r.Om - eps * g2;
-        const double k = (-g3 + eps * (g2 - eps * (g1 - eps * g0))) * iS0;
-        const double m = (g2 + eps * (3.0 * eps * g0 - 2.0 * g1)) * (iS0 * (1.0 / 3));
         put(rec, C_EPS, eps);
-        put(rec, C_K2, k * (1.0 / 3));
+        put(rec, C_K2, r.k * (1.0 / 3));
         put(rec, C_K3, r.OL * iS0);
-        if (ns <= CORE_NS_ONCE) put(rec, C_M, m);
-        rj_coefs<T>((T)m, f2, f3, ns, b);
+        if (ns <= CORE_NS_ONCE) put(rec, C_M, r.m);
+        const T u5 = dev_scale<T>(r.d5, ns);
+        rj_coefs<T>((T)r.m * u5, (f2 * u5) * u5, ((f3 * u5) * u5) * u5, ns, b);
 #pragma unroll
         for (int j = 0; j < CORE_NS; j++)
             if (j < ns) rec[C_A + j] = b[j];
-        rec[C_DJ] = (T)dev5(d3, m);
+        rec[C_DJ] = (T)r.d5;
     }
     if (!absorb) return;
     const double S = r.cpair ? 2.0 * r.pr : r.pr + r.pi, Q = r.cpair ? r.pr * r.pr + r.pi * r.pi : r.pr * r.pi;
@@ -183,13 +199,14 @@ template <class T> LCDM_HD void core_values(const RowRoots& r, bool time, bool a
     }
     put(rec, X_FREE, 0.0);
     put(rec, X_HX, hx);
-    const float dA = dev5(d3, X1 + hx), dD = dev5(d3, X1);
-    rec[X_DX] = (T)(dA > dD ? dA : dD);
+    const float dA = dev5(r.d3, X1 + hx), dD = dev5(r.d3, X1), dX = dA > dD ? dA : dD;
+    rec[X_DX] = (T)dX;
     if (r.cpair) { put(rec, X_SQ, 2.0 * q1); put(rec, X_PQ, q1 * q1 + q2 * q2); }
     else { put(rec, X_SQ, q1 + q2); put(rec, X_PQ, q1 * q2); }
     // the series at p0 (offset X1 + hx) and at x1 (offset X1), and their divided differences
     DD<T> ad[CORE_NS];
-    rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx), (T)X1, (T)1), mkdd<T>(f2, f2, (T)0), mkdd<T>(f3, f3, (T)0), ns, ad);
+    const T uX = dev_scale<T>(dX, ns), g2 = (f2 * uX) * uX, g3 = ((f3 * uX) * uX) * uX;
+    rj_coefs<DD<T> >(mkdd<T>((T)(X1 + hx) * uX, (T)X1 * uX, uX), mkdd<T>(g2, g2, (T)0), mkdd<T>(g3, g3, (T)0), ns, ad);
 #pragma unroll
     for (int j = 0; j < CORE_NS; j++) {
         if (j >= ns) break;
@@ -225,38 +242,32 @@ LCDM_HD void core_tangent(const RowRoots& r, bool time, int ns, int k, double dA
     if (k == 2) { dI += 12.0 * OL; dJ += 27.0 * Ox * Ox - 72.0 * c * OL; }
     if (k == 5) { dI -= 3.0 * Om; dJ += 54.0 * Or * Ox - 9.0 * Om * c; }
     double de2 = dI * (-1.0 / 3), de3 = dJ * (-1.0 / 27);
-    T e2, e3;
-    {
-        const double I = 12.0 * Or * OL - 3.0 * Om * Ox + c2;
-        const double J = 2.0 * c2 * c - 9.0 * Om * c * Ox + 27.0 * Or * Ox * Ox + 27.0 * Om * Om * OL - 72.0 * Or * c * OL;
-        const double v2 = I * (-1.0 / 3) * iS2, v3 = J * (-1.0 / 27) * (iS2 * iS0);
-        if (r.ncol != 4) {
-            de2 = (de2 * iS0 - 2.0 * v2) * iS0;
-            de3 = (de3 * iS2 - 3.0 * v3) * iS0;
-        }
-        e2 = (T)v2;
-        e3 = (T)v3;
+    if (r.ncol != 4) {
+        de2 = (de2 * iS0 - 2.0 * r.e2) * iS0;
+        de3 = (de3 * iS2 - 3.0 * r.e3) * iS0;
     }
+    const T e2 = (T)r.e2, e3 = (T)r.e3;
     typedef Dual<T, 1> F;
-    F f2, f3, b[CORE_NS];
-    f2.v = e2; f2.d[0] = (T)de2;
-    f3.v = e3; f3.d[0] = (T)de3;
+    F b[CORE_NS];
+    // the invariants and their derivatives, normalised by dev u = 1 (a constant of the row here)
+    auto f2 = [&](T u) { F f; f.v = (e2 * u) * u; f.d[0] = ((T)de2 * u) * u; return f; };
+    auto f3 = [&](T u) { F f; f.v = ((e3 * u) * u) * u; f.d[0] = ((T)(de3 * u) * u) * u; return f; };
     const bool once = ns <= CORE_NS_ONCE;
     if (once) {
         put(t, CT_E2, de2);
         put(t, CT_E3, de3);
     } else {
-        rf_coefs<F>(f2, f3, ns, b);
+        const T u = dev_scale<T>(r.d3, ns);
+        rf_coefs<F>(f2(u), f3(u), ns, b);
 #pragma unroll
         for (int j = 0; j < CORE_NS; j++)
             if (j < ns) t[CT_B + j] = b[j].d[0];
     }
     if (time) {
         // k S0 = -Om + 2 eps C - 3 eps^2 Ox + 4 eps^3 OL, 3 m S0 = C - 3 eps Ox + 6 eps^2 OL (C = Ok + Os):
-        // the recursion of core_values multiplied out
+        // the recursion of finish() multiplied out
         const double ee = eps * eps, de = r.quartic ? dA * ee : 0.0;
-        const double kv = (-Om + eps * (2.0 * c - eps * (3.0 * Ox - 4.0 * eps * OL))) * iS0;
-        const double mv = (c - eps * (3.0 * Ox - 6.0 * eps * OL)) * (iS0 * (1.0 / 3));
+        const double kv = r.k, mv = r.m;
         const double dk = (-d.dOm + 2.0 * eps * d.dOk - ee * (3.0 * d.dOx - 4.0 * eps * d.dOL)
                            + (2.0 * c - eps * (6.0 * Ox - 12.0 * eps * OL)) * de - kv * d.dS) * iS0;
         const double dm = (d.dOk - eps * (3.0 * d.dOx - 6.0 * eps * d.dOL) - (3.0 * Ox - 12.0 * eps * OL) * de
@@ -268,8 +279,9 @@ LCDM_HD void core_tangent(const RowRoots& r, bool time, int ns, int k, double dA
             put(t, CT_M, dm);
         } else {
             F fm;
-            fm.v = (T)mv; fm.d[0] = (T)dm;
-            rj_coefs<F>(fm, f2, f3, ns, b);
+            const T u = dev_scale<T>(r.d5, ns);
+            fm.v = (T)mv * u; fm.d[0] = (T)dm * u;
+            rj_coefs<F>(fm, f2(u), f3(u), ns, b);
 #pragma unroll
             for (int j = 0; j < CORE_NS; j++)
                 if (j < ns) t[CT_A + j] = b[j].d[0];

@@ -969,7 +969,7 @@ template <int G> __global__ void prep_kernel(PrepArgs a) {
         }
     }
     if (st == ST_OK && (a.coreF || a.coreD)) {
-        r.finish();
+        r.finish(a.time);
         const bool tangents = a.tangents && !a.recD;
         if (a.coreF) write_core<G, float>(r, dr, j, a.time, a.absorb, tangents, a.ns, a.coreF + b * NCORE);
         else write_core<G, double>(r, dr, j, a.time, a.absorb, tangents, a.ns, a.coreD + b * NCORE);
