@@ -601,8 +601,10 @@ HostCarve host_carve(char* base, int64_t B, int64_t n, int ncol, size_t es) {
 // Device workspace of the general-limits entry points: records of the
 // shifted cosmologies, shifted parameters (closure form, four columns), their
 // Jacobian, the scale s = 1+z1,
-// the gradient w.r.t. the shifted parameters, z' and three scaled cotangents
-// (d_C, X, d_M; these four only where X is differentiated, see RowMap).
+// the gradient w.r.t. the shifted parameters, z' and the mapped cotangents of
+// d_C, X, d_M (scaled) and mu (0 for a pair outside the domain: at z' = 0, where
+// such a pair is evaluated, mu alone has a derivative); these five only where X is
+// differentiated, see RowMap.
 struct BetweenCarve {
     Carved rec;
     double* jac;
@@ -628,6 +630,7 @@ BetweenCarve between_carve(char* base, int64_t B, int64_t npairs, int ncol, size
     c.cotp[LCDM_DC] = take((size_t)npairs * es);
     c.cotp[LCDM_X] = take((size_t)npairs * es);
     c.cotp[LCDM_DM] = take((size_t)npairs * es);
+    c.cotp[LCDM_MU] = take((size_t)npairs * es);
     c.bytes = off;
     return c;
 }

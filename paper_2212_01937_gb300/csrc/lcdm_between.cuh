@@ -101,7 +101,7 @@ struct PairMapArgs {
     const void* z2;         // [nnz]
     void* zp;               // [nnz] z' = (z2 - z1) / s
     const void* cot[6];     // user cotangents
-    void* cotp[6];          // scaled cotangents (d_C, X, d_M; null = not needed)
+    void* cotp[6];          // mapped cotangents (d_C, X, d_M, mu; null = not needed)
     void* out[6];           // outputs scaled in place
 };
 
