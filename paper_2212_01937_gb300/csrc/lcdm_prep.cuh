@@ -876,7 +876,7 @@ __device__ __noinline__ void legacy_record(const RowRoots& r, const cd (*dr)[RF_
     const double iH0 = ddiv(1.0, H0);
     rec[RF_DH] = LCDM_C_KMS * iH0;
     rec[RF_TH] = LCDM_HUBBLE_GYR * iH0;
-    rec[RF_KIND] = n == 4 ? (cpair ? 0 : 1) : (cpair ? 2 : 3);
+    rec[RF_KIND] = !labelled ? 0 : n == 4 ? (cpair ? 0 : 1) : (cpair ? 2 : 3);
     // N = sqrt(E^2(0) / alpha_n): E^2(0) = Om + OL + Or + Ok (+ Os + Ox), exactly 1 under the closure
     const double S0 = ncol == 4 ? 1.0 : Om + OL + Or + Ok + Os + Ox;
     const double iOm = ddiv(1.0, Om);
