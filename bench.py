@@ -40,12 +40,12 @@ COT_OUTPUTS = ("d_C", "t", "mu")
 ALG_FLOP_PER_PAIR = 7033.1
 ALG_MUFU_PER_PAIR = 390.3
 # FP32 floating-point operations the step's two pair launches execute per pair
-# (FFMA counted as 2, FADD and FMUL as 1: 364 in the value launch + 783 in the
+# (FFMA counted as 2, FADD and FMUL as 1: 355 in the value launch + 772 in the
 # gradient launch; a packed instruction counts for both its numbers) and their DRAM bytes (read + write) per step, from one ncu
 # capture of both launches on this workload (profiles/pairs_kernel_fp32_vjp_
 # 4096x1024.md; to be set to None whenever the kernels change until re-taken).
-EXEC_FLOP_PER_PAIR = 1146.5
-TRAFFIC_BYTES = 114.4e6
+EXEC_FLOP_PER_PAIR = 1126.5
+TRAFFIC_BYTES = 114.3e6
 # Derived peaks (unit counts x maximum SM clock): FP32 FMA, 152 SMs x 128 lanes
 # x 2 flops; special-function unit, 152 SMs x 16 per clock.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12

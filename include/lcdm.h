@@ -41,7 +41,11 @@
  *            n redshifts z[n]; pair (b, i) has index b*n + i.
  *            npairs = n (CSR) or B*n (DENSE, SHARED).
  *   dtype    precision LCDM_FP64: z, outputs, cotangents, Jacobians and
- *            m_obs are float64 and every step is FP64.  LCDM_FP32_MIXED: they
+ *            m_obs are float64 and so is the arithmetic; single precision only
+ *            starts the root iteration, forms its corrections (known to 1e-7
+ *            of what is left to correct) and decides where iterations stop.
+ *            Square roots and reciprocals are within about an ulp.
+ *            LCDM_FP32_MIXED: they
  *            are float32 and the per-pair arithmetic is FP32 (division and
  *            square root within 2 ulp, subnormal results flushed to zero);
  *            the root solve and all per-cosmology reductions stay FP64.
@@ -263,7 +267,7 @@ lcdm_status lcdm_distances_vjp_host(const double* params, int64_t B, const int64
  * allocator at hand.  (The paper has no counterpart; this is a convenience of
  * this library.)
  *   Scratch lives in a fixed device array inside the library, sized for
- *   LCDM_STATIC_MAX_COSMOLOGIES cosmologies (about 6 MB), which stays
+ *   LCDM_STATIC_MAX_COSMOLOGIES cosmologies (8.5 MB), which stays
  *   allocated on every device that loads the library until the process exits.
  *   B larger than that is rejected with LCDM_ERR_INVALID; nothing is enqueued.
  *   The function calls no cudaMalloc, cudaFree or other allocating routine.
@@ -307,7 +311,8 @@ lcdm_status lcdm_autotune(const double* params, int64_t B, const int64_t* offset
  * ------------------------------------------------------------------------- */
 
 /* Workspace bytes of lcdm_distances_between (B rows, n as in the layout) and
- * of lcdm_limits (n = 0).                                                   */
+ * of lcdm_limits (n = 0).  The part that grows with the pairs is used only
+ * where X is differentiated.                                                */
 lcdm_status lcdm_between_workspace_size(int64_t B, int64_t n, const lcdm_opts* opts, size_t* bytes);
 
 /* Distances between z1[b] and each pair's z2 (layouts LCDM_LAYOUT_CSR and

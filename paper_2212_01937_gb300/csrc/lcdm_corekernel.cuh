@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256, CoreBlocks<PREC, K, WT, WX, MODE>::value)
 #pragma unroll
         for (int i = 0; i < NV; i++) acc[i * ACC_STRIDE] = cst<AccT>(0.0);
     }
-    int acc_row = -1;   // (a row's index fits 32 bits: its record alone takes 768 bytes)
+    int acc_row = -1;   // (a row's index fits 32 bits: its record alone takes 1040 bytes)
     int64_t wf = -1, wl = -1;
     if (a.part && reduce && warp < a.det_cap) {
         // deterministic reduction: the warp's first and last rows, its slots zeroed
@@ -443,8 +443,8 @@ template <int K, bool WX> struct Core2Blocks { enum { value = K == 0 && !WX ? 3 
 // does per pair beside arithmetic (the row, the record, the loop) is done once
 // for two.  Bound by issue like core_kernel (75 % of cycles there, at 241
 // instructions per pair of values and 527 with the gradient): 1.42e8 ragged
-// pairs of mu and its gradient 4.43 -> 3.59 ms, 25 M pairs over a shared set
-// 0.78 -> 0.63 ms, 1e8 pairs of d_C, t and X 3.18 -> 2.74 ms.  A warp takes two 32-pair batches at a time while every lane's two
+// pairs of mu and its gradient 4.43 -> 3.49 ms, 25 M pairs over a shared set
+// 0.78 -> 0.62 ms, 1e8 pairs of d_C, t and X 3.18 -> 2.75 ms.  A warp takes two 32-pair batches at a time while every lane's two
 // pairs lie in one row, else one (the second number is then a copy).
 template <int K, bool WT, bool WX, int MODE>
 __global__ void __launch_bounds__(256, Core2Blocks<K, WX>::value) core2_kernel(CoreArgs ca) {

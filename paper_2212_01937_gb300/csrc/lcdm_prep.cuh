@@ -294,7 +294,7 @@ LCDM_HD bool closed_start(const float* al, int n, float* zr, float* zi) {
 // leaves 1e-7 of the error (or its cube), so two usually end it; comparisons
 // are made in single precision or on the bits.  (4096 rows, kernel time: 0.070
 // ms with double corrections, confirmations and hypot; 0.031 ms so, with the
-// closed-form starts, 418 FP64 and 4259 instructions a warp.)
+// closed-form starts.)
 // Coefficients of the monic polynomial beyond 1e6 (Or0 below 3e-7 for Om0 = 0.3:
 // |A|^4 would near the end of single precision) or OL0 = 0 take the sweeps in
 // double throughout, from the circles.
