@@ -221,7 +221,10 @@ lcdm_status launch_one(Plan& P, int block, int bps, int lane_map, cudaStream_t s
 
 // Two pairs in a thread where rows are long (a mean of LCDM_PACKED_ROW pairs):
 // a batch that crosses a row runs one pair at a time, at the packed kernel's
-// registers.  Not with t's gradient: two pairs of that do not fit the registers
+// registers.  The line is the gradient's (us for 4 M pairs of mu and its gradient
+// in rows of 128 / 256 / 512 / 1024, packed and not: 255 222, 220 216, 144 152, 122
+// 135); d_C and mu as values cross at 64 (181 190, at 48 221 200; at 1024 66 76).
+// Not with t's gradient: two pairs of that do not fit the registers
 // (0.41 against 0.39 ms for 4 M pairs of d_C, t and mu).
 #define LCDM_PACKED_ROW 256
 bool packed_plan(const Plan& P) {
