@@ -615,7 +615,7 @@ template <class T, bool WT, bool WX, bool REV, bool INF = false> struct CorePair
                 const T id = rcp_(qs * gg);
                 const T eh = (piX * id) * id, e = hX * eh;
                 sDD = sDD + tm * (eh * rc1m1_core(e) * id
-                                  - (gg + cst<T>(2.0) * S1 * (qs + S)) * (id * id) * gg * ix * cst<T>(0.5));
+                                  - ((gg + cst<T>(2.0) * S1 * (qs + S)) * id) * (id * gg) * ix * cst<T>(0.5));   // (id^2 may flush to zero)
                 pX = pX + lam;
             }
             if (REV) {

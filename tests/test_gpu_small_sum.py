@@ -74,3 +74,21 @@ def test_small_sum(lib, n):
         return lib.distances(_t(P), zz, off, outputs=outs, precision=prec)
 
     _compare(run, np.array(S))
+
+
+def test_small_sum_absorption(lib):
+    """X far out: no product on the way flushes to zero (within 5e-6; 1e-6 is
+    usual at sums of 1e-6 and more)."""
+    rng = np.random.default_rng(16)
+    P = []
+    while len(P) < 300:
+        Om, OL, Or, s = rng.uniform(0.05, 1.0), rng.uniform(-0.3, 0.3), 10.0 ** rng.uniform(-5, -3), 10.0 ** rng.uniform(-9, -6)
+        Ok = s - Om - OL - Or
+        if 4 * Or + 3 * Om + 2 * Ok > 0.05:
+            P.append([70.0, Om, OL, Or, Ok])
+    P, n = np.array(P), 8
+    z = (10.0 ** rng.uniform(1.5, 3, len(P) * n)).astype(np.float32)
+    off = _t(np.arange(len(P) + 1, dtype=np.int64) * n)
+    a, b = (lib.distances(_t(P), _t(v), off, outputs=("X",), precision=p)["X"]
+            for v, p in ((z, "fp32"), (z.astype(np.float64), "fp64")))
+    assert (a.double() / b - 1).abs().max().item() <= 5e-6
